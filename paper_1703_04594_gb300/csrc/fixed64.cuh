@@ -93,6 +93,14 @@ __host__ __device__ __forceinline__ double fx_to_double_dp_pos(long long X, int 
 #endif
 }
 
+// X 2^-(K / 2^20) for a float64 conversion of X and K >= 0 in units of the exponent field, as
+// fx_to_double_dp_pos.
+__device__ __forceinline__ double fx_lower_exponent(long long X, int K) {
+  const double d = __ll2double_rn(X);
+  const unsigned h = (unsigned)__double2hiint(d);
+  return __hiloint2double((int)(h - min(h, (unsigned)K)), __double2loint(d));
+}
+
 // f' = f 2^(59 + e) for a population whose value is an integer there: with the exponent
 // field E, sh = E - 1016 + e is the left shift of the 53-bit significand, and
 // 2^-7 <= f 2^e < 8 is 0 <= sh <= 9 (one unsigned compare, which also fails for negative

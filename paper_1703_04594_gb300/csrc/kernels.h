@@ -5,6 +5,7 @@
 
 #include "../../include/lbm_d2q37.h"
 #include "collide_fp64.cuh"
+#include "site_fix64.cuh"
 
 namespace d2q37 {
 
@@ -15,6 +16,7 @@ struct StepScalars {
   long long pop;        // elements per population plane = lx * pitch
   int periodic;         // 1: y wraps (test mode), 0: thermal walls
   CollideConst cc;
+  FixConsts fx;         // the fixed-point collision's constants (site_fix64.cuh)
   double rho0;          // FP32 shifted storage: g_i = f_i - w_i rho0
   // Float copies of cc for the FP32 collision.  Their rounding must not bias the
   // collision: a relative bias e of the equilibrium's momentum multiplies the momentum by

@@ -86,6 +86,7 @@ StepArgs d2q37::make_step_args(const lbm_params* p) {
   a.cc.cgx = C * tau * p->gx;
   a.cc.cgy = C * tau * p->gy;
   a.cc.tshift = tau * (1.0 - tau) * (p->gx * p->gx + p->gy * p->gy) / D - 1.0;
+  a.fx = make_fix_consts(tau, p->gx, p->gy);
   a.rho0 = p->rho0;
   a.f_omega = (float)a.cc.omega;
   a.f_om1 = 1.0f - a.f_omega;  // exact for 1/2 <= omega <= 2

@@ -1,0 +1,386 @@
+// Collision of one site in 64-bit fixed point on the integer pipes.
+//
+// The update is collide_site's (Sec. 3, eq. "lbequation"; equilibrium and moments as in
+// collide_fp64.cuh).  GB300 runs float64 at 1/64 of its float32 rate, and a float64
+// collision needs ~260 operations of that pipe per site; here only the 37 conversions of the
+// results back to float64 run on it.
+//
+// The equilibrium is expanded in the monomials vx^p vy^q, p + q <= 4, of the integer
+// velocities: omega f^eq_i = w_i sum_pq c_pq vx^p vy^q, with 15 coefficients c_pq that
+// depend on the site alone (X = c u_s,x, Y = c u_s,y, t = T_s - 1, U = |u_s|^2,
+// R = omega rho, h = R c^2 t / 4):
+//   c00 = R (1 - U/2 - t + U^2/8 + t U + t^2)
+//   c10 = R (1 - U/2 - 2t) X                      c01: Y
+//   c20 = R c^2 (t/2 - t U/4 - t^2) + R20 X^2     c02: Y^2     R20 = R (1/2 - U/4 - 3t/2)
+//   c11 = 2 R20 X Y
+//   c30 = X (2h + R X^2/6)   c21 = Y (2h + R X^2/2)   c12 = X (2h + R Y^2/2)   c03: Y, Y^2/6
+//   c40 = R c^4 t^2/8 + X^2 (h + R X^2/24)            c04: Y
+//   c22 = R c^4 t^2/4 + h (X^2 + Y^2) + R X^2 Y^2/4
+//   c31 = X Y (2h + R X^2/6)                          c13 = X Y (2h + R Y^2/6)
+// The velocity set is closed under sign changes, so the populations come in quads
+// (a, b), (-a, -b), (a, -b), (-a, b) that share four sums S (even, even), D (odd, odd),
+// Ox and Oy: p = S + D + Ox + Oy, S + D - Ox - Oy, S - D + Ox - Oy, S - D - Ox + Oy.  With
+// |a|, |b| <= 3 every multiple is a shift or two and an add: 30 full 64-bit products make
+// the coefficients of a site, and a population costs about eight 64-bit adds and two
+// products, w_s p and (1 - omega) f.  (Evaluating the polynomial in s = v.u_s per opposite
+// pair took 6 products per pair and 5 per shell, 4387 instructions per site in all.)
+//
+// Scales.  Populations of shell s are scaled by 2^e_s (w_s 2^e_s in [0.5, 1)), and the whole
+// site by 2^-k, with k read off the rest population's exponent, f_0 2^(e_0 - k) in [1/4, 1/2):
+// the path is the same at every density.  Numbers in [] below are fraction bits.
+//   f_i 2^(e_s - k) [60], in [2^-8, 2): exact (a shift of the significand); moments [60]
+//   omega f^eq / w_s [59], below 14; (1 - omega) [62]; w_s 2^e_s [63]; outputs [58]
+// With every rounding counted an output carries about one unit of 2^-58 at a scaled size of
+// 1/4 to 1/2 or more, below a float64 rounding (2^-54 of it); the coefficients that large
+// integers multiply carry 62 to 65 bits.
+//
+// Range: 2^-8 <= f_i 2^(e_s - k) < 2, 9/64 <= rho 2^-k < 1, |X|, |Y| < 1/4, |t| < 1/4,
+// 1/2 < tau < 1e6 with |tau g| small (fix_consts); other sites take the float64 collision.
+#pragma once
+#include "collide_fix64.cuh"
+
+namespace d2q37 {
+
+// ---- products of signed fixed-point numbers ------------------------------------------------
+// a = hi 2^32 + lo with a signed low word: three signed 32 x 32 -> 64 products then give the
+// high half of a 64-bit product (the low words' product, at most 1/4 unit and as often
+// negative as positive, is left out), half a unit below the exact value on average.
+struct FxHalves {
+  int h, l;
+};
+__host__ __device__ __forceinline__ FxHalves fx_halves(long long a) {
+  const unsigned lo = (unsigned)a;
+  return FxHalves{(int)((unsigned)((unsigned long long)a >> 32) + (lo >> 31)), (int)lo};
+}
+__host__ __device__ __forceinline__ long long fx_smul(FxHalves a, FxHalves b) {
+  const long long t = (long long)a.h * b.l + (long long)a.l * b.h;
+  return (long long)a.h * b.h + (t >> 32);
+}
+__host__ __device__ __forceinline__ long long fx_smul(long long a, FxHalves b) { return fx_smul(fx_halves(a), b); }
+__host__ __device__ __forceinline__ long long fx_smul(long long a, long long b) {
+  return fx_smul(fx_halves(a), fx_halves(b));
+}
+// v 2^k as an integer, |v| 2^k < 2^62, at compile time or on the host.
+__host__ __device__ constexpr long long fx_signed(double v, int k) {
+  return v == 0.0 ? 0LL : v > 0.0 ? (long long)fx_const(v, 1.0, k) : -(long long)fx_const(-v, 1.0, k);
+}
+
+constexpr long long kFxC2_62 = (long long)fx_const(C2, 1.0, 62);
+constexpr long long kFxC2_63q = (long long)fx_const(C2, 0.25, 64);         // c^2 / 4 [64]
+constexpr long long kFxC4_64 = (long long)fx_const(C2, C2 * 0.125, 64);    // c^4 / 8 [64]
+constexpr long long kFxInvC2_63 = (long long)(kInvC2 >> 1);                // 1 / c^2 [63]
+constexpr long long kFxTwoThirds_63 = 6148914691236517205LL;               // round(2^64 / 3)
+// w_s 2^e_s [63]: the constants kCw (correctly rounded from the float64 weights)
+
+// ---- per-lattice constants -------------------------------------------------------------------
+struct FixConsts {
+  int usable;              // 0: the lattice's constants are outside the formats
+  int neg;                 // 1 - omega < 0 (the common case, tau < 1)
+  unsigned long long om1;  // |1 - omega| [62]
+  long long om;            // omega [62]
+  long long cgx, cgy;      // c tau g [60]
+  long long hgx, hgy;      // 2 c tau g / c^2 [63]
+  long long tc;            // tau (1 - tau) |g|^2 / 2 - |c tau g|^2 / (2 c^2) [60]
+};
+
+inline FixConsts make_fix_consts(double tau, double gx, double gy) {
+  FixConsts r = {};
+  const double om = 1.0 / tau, sx = C * tau * gx, sy = C * tau * gy;
+  const double tc = tau * (1.0 - tau) * (gx * gx + gy * gy) / 2.0 - (sx * sx + sy * sy) / (2.0 * C2);
+  const double om1 = 1.0 - om;  // as CollideConst::om1
+  const auto small = [](double v) { return v > -0.125 && v < 0.125; };
+  r.usable = om > 0.0 && om < 2.0 && om1 > -1.0 && om1 < 1.0 && small(sx) && small(sy) && small(tc);
+  if (!r.usable) return r;
+  r.neg = om1 < 0.0;
+  // (doubles of this size are multiples of 2^-60 or round there; conversions are exact or
+  // round to nearest)
+  const auto fix = [](double v, int k) {
+    bool unused = false;
+    return fx_from_double(v, k, 64, unused);
+  };
+  r.om1 = (unsigned long long)fix(om1 < 0.0 ? -om1 : om1, 62);
+  r.om = fix(om, 62);
+  r.cgx = fix(sx, 60);
+  r.cgy = fix(sy, 60);
+  r.hgx = fix(2.0 * sx / C2, 63);
+  r.hgy = fix(2.0 * sy / C2, 63);
+  r.tc = fix(tc, 60);
+  return r;
+}
+
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+
+// ---- index of a velocity -----------------------------------------------------------------------
+__host__ __device__ constexpr int pop_index(int a, int b) {
+  for (int i = 0; i < Q; ++i)
+    if (vx(i) == a && vy(i) == b) return i;
+  return -1;
+}
+
+// ---- 1. populations to fixed point, and the moments ---------------------------------------------
+struct FixMoments {
+  long long R, E, X, Y;  // sum f, sum |v|^2 f, sum vx f, sum vy f, times 2^-k [60]
+  int kb;                // k << 20 (the exponent field's unit), for the results
+  bool ok;               // every population in range
+};
+
+// `load(i)` returns f_i as a float64, `keep(i, f')` stores its fixed-point form; each is called
+// once per population, load(i) before keep(i).
+template <class Load, class Keep>
+__host__ __device__ __forceinline__ FixMoments fix_moments(Load&& load, Keep&& keep) {
+  // shift of the significand: exponent field + e_s - k + (60 - 52 - 1023); k from f_0, whose
+  // field E0 gives f_0 2^(2 - k) in [1/4, 1/2):  k = E0 - 1023 + 2 + 2
+  const double f0 = load(0);
+  const unsigned E0 = fx_hi_word(f0) >> 20;
+  const unsigned base = 4u - E0;  // + E + e_s: with k = E0 - 1019 the shift is E - E0 + e_s + 4
+  unsigned worst = 0;
+  const auto conv = [&](int i, double f) {
+    const int e = shell_exp(shell(i));
+    const unsigned sh = (fx_hi_word(f) >> 20) + (base + (unsigned)e);
+    worst = worst > sh ? worst : sh;
+    const long long q = fx_from_double_shifted(f, sh);
+    keep(i, q);
+    return q;
+  };
+  FixMoments m;
+  m.kb = (int)((E0 - 1019u) << 20);
+  long long R = (conv(0, f0) + 2) >> 2, E = 0, X = 0, Y = 0;  // e_0 = 2
+  const auto axis = [&](auto ac) {
+    constexpr int a = decltype(ac)::value, e = shell_exp(shell_of_v2(a * a));
+    constexpr long long half = 1LL << (e - 1);
+    constexpr int ix = pop_index(a, 0), jx = pop_index(-a, 0), iy = pop_index(0, a), jy = pop_index(0, -a);
+    const long long p = conv(ix, load(ix)), q = conv(jx, load(jx));
+    const long long r = conv(iy, load(iy)), s = conv(jy, load(jy));
+    const long long T = (long long)(((unsigned long long)(p + q) + (unsigned long long)(r + s) + half) >> e);
+    R += T;
+    E += (long long)(a * a) * T;
+    X += (long long)a * ((p - q + half) >> e);
+    Y += (long long)a * ((r - s + half) >> e);
+  };
+  const auto quad = [&](auto ac, auto bc) {
+    constexpr int a = decltype(ac)::value, b = decltype(bc)::value, e = shell_exp(shell_of_v2(a * a + b * b));
+    constexpr long long half = 1LL << (e - 1);
+    constexpr int i1 = pop_index(a, b), i2 = pop_index(-a, -b), i3 = pop_index(a, -b), i4 = pop_index(-a, b);
+    const long long f1 = conv(i1, load(i1)), f2 = conv(i2, load(i2));
+    const long long f3 = conv(i3, load(i3)), f4 = conv(i4, load(i4));
+    const long long T =
+        (long long)(((unsigned long long)(f1 + f2) + (unsigned long long)(f3 + f4) + half) >> e);
+    const long long d = f1 - f2, g = f3 - f4;
+    R += T;
+    E += (long long)(a * a + b * b) * T;
+    X += (long long)a * ((d + g + half) >> e);
+    Y += (long long)b * ((d - g + half) >> e);
+  };
+  axis(IntC<1>());
+  quad(IntC<1>(), IntC<1>());
+  axis(IntC<2>());
+  quad(IntC<2>(), IntC<1>());
+  quad(IntC<1>(), IntC<2>());
+  quad(IntC<2>(), IntC<2>());
+  axis(IntC<3>());
+  quad(IntC<3>(), IntC<1>());
+  quad(IntC<1>(), IntC<3>());
+  m.R = R;
+  m.E = E;
+  m.X = X;
+  m.Y = Y;
+  // shifts 0 .. 8; E0 in [128, 1078], f_0 below 2^56, keeps every result a normal float64 and
+  // k below 60 (fx_lower_exponent), and rules out a sign bit, zeros, infinities and NaNs (with
+  // f_0 ordinary, the others' shifts rule theirs out)
+  m.ok = worst <= 8u && E0 - 128u <= 950u;
+  return m;
+}
+
+// ---- 2. site scalars ------------------------------------------------------------------------------
+struct FixScalars {
+  long long R;         // omega rho 2^-k [61]
+  long long X, Y;      // c u_s [64]
+  long long XX, YY, U; // X^2, Y^2, |u_s|^2 [64]
+  long long t;         // T_s - 1 [65]
+  bool ok;
+};
+
+// 1 / a float32 to within a few units in its last place.
+__host__ __device__ __forceinline__ float fx_rcp_seed(float v) {
+#ifdef __CUDA_ARCH__
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+#else
+  return 1.0f / v;
+#endif
+}
+
+// 1 / rho [60] of rho [60] in [1/8, 1): a float32 seed of 24 bits (its integer form has 30,
+// so the residual is two exact 32 x 64 products) and one step y (1 + e + e^2), e^3 < 2^-63.
+__host__ __device__ __forceinline__ long long fx_reciprocal(long long R) {
+  const unsigned rh = (unsigned)((unsigned long long)R >> 32), rl = (unsigned)R;  // rh in [2^25, 2^28)
+  const unsigned yh = (unsigned)(fx_rcp_seed((float)rh) * 36028797018963968.0f);  // [27], <= 2^30
+  // rho y = (rh 2^32 + rl) yh 2^-87
+  const unsigned long long pl = (unsigned long long)rl * yh;
+  const unsigned long long ph = (unsigned long long)rh * yh + (pl >> 32);  // [55]
+  const long long e = (((1LL << 55) - (long long)ph) << 22) - (long long)((unsigned)pl >> 10);  // 1 - rho y [77]
+  const int eh = (int)(e >> 32);                                                                  // [45]
+  const long long g = e + (((long long)eh * eh) >> 13);                                           // e + e^2 [77]
+  const long long d = (long long)(int)(g >> 32) * (int)yh + (long long)(((unsigned long long)(unsigned)g * yh) >> 32);
+  return ((long long)yh << 33) + ((d + (1LL << 11)) >> 12);  // y + y g, the latter [72] -> [60]
+}
+
+__host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, const FixConsts& k) {
+  FixScalars s;
+  // rho in [9/64, 1), |j| < 1/4, |sum |v|^2 f - 2 rho / c^2| < 1/2 (2 rho |t| / c^2 + ... < 0.4 in
+  // range): what the formats below hold; unsigned compares of the offset values
+  const long long W = fx_smul(m.R << 3, fx_halves(kFxInvC2_63));  // rho / c^2 [62] = 2 rho / c^2 [61]
+  const long long dev = m.E * 2 - W;                               // [61]
+  bool ok = m.ok & ((unsigned long long)(m.R - (9LL << 54)) < (55ull << 54)) &
+            ((unsigned long long)(m.X + (1LL << 58)) < (1ull << 59)) &
+            ((unsigned long long)(m.Y + (1LL << 58)) < (1ull << 59)) &
+            ((unsigned long long)(dev + (1LL << 60)) < (1ull << 61));
+  const long long yc = fx_smul(fx_reciprocal(m.R) , fx_halves(kFxC2_62)) * 2;  // c^2 / rho [58] -> [59]
+  const FxHalves y = fx_halves(yc);
+  const long long X = fx_smul(m.X << 5, y) + k.cgx, Y = fx_smul(m.Y << 5, y) + k.cgy;  // [60]
+  const long long e2 = fx_smul(dev << 3, y);  // 2 (T - 1) + |u|^2 [59], so half of it [60]
+  ok = ok & ((unsigned long long)(X + (1LL << 58)) < (1ull << 59)) &
+       ((unsigned long long)(Y + (1LL << 58)) < (1ull << 59));
+  s.X = X << 4;
+  s.Y = Y << 4;
+  const FxHalves xh = fx_halves(s.X), yh = fx_halves(s.Y);
+  s.XX = fx_smul(xh, xh);
+  s.YY = fx_smul(yh, yh);
+  s.U = fx_smul((s.XX + s.YY) << 1, fx_halves(kFxInvC2_63));
+  // |u|^2 of the unshifted velocity from that of the shifted one
+  const long long g = fx_smul(xh, fx_halves(k.hgx)) + fx_smul(yh, fx_halves(k.hgy));  // [63]
+  const long long t = e2 + k.tc - (s.U >> 5) + (g >> 4);                              // [60]
+  ok = ok & ((unsigned long long)(t + (1LL << 58)) < (1ull << 59));
+  s.t = t << 5;
+  s.R = fx_smul(m.R << 3, fx_halves(k.om));
+  s.ok = ok;
+  return s;
+}
+
+// ---- 3. coefficients, and the populations -------------------------------------------------------
+// Added to omega f^eq / w (between -2 and 14 in range) or to its negative, so that the unsigned
+// products take positive numbers: 2 or 14 [59].
+template <bool NEG>
+constexpr long long kFixB = NEG ? 7LL << 60 : 1LL << 60;
+// What the shifts and products below round off on average, put back: units of 2^-59 on the even
+// sum, and of 2^-58 on a result.
+template <bool NEG>
+constexpr long long kFixEvenMean = NEG ? 0 : 2;
+template <bool NEG>
+constexpr long long kFixOutMean = 1;
+
+// NEG: 1 - omega < 0.  `fixed(i)` returns f_i' [60]; `out(i, v, s)` takes f_i^{new} 2^(e_s - k)
+// [58] of population i (shell s).  For NEG the sums are formed for -omega f^eq, so that both
+// products of a population stay positive: w (B - p) + |1 - omega| f = w B - f^{new}.
+template <bool NEG, class Fixed, class Out>
+__host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, unsigned long long om1, Fixed&& fixed,
+                                                   Out&& out) {
+  const FxHalves Rh = fx_halves(v.R), th = fx_halves(v.t), Uh = fx_halves(v.U);
+  const FxHalves xh = fx_halves(v.X), yh = fx_halves(v.Y), xxh = fx_halves(v.XX), yyh = fx_halves(v.YY);
+  const long long Rt = fx_smul(th, Rh);                              // [62]
+  const FxHalves Rth = fx_halves(Rt);
+  const long long RU = fx_smul(Uh, Rh);                              // [61]
+  const long long h = fx_smul(Rth, fx_halves(kFxC2_63q));            // [62]
+  const long long Rt2 = fx_smul(Rth, th);                            // [63]
+  const long long RtU = fx_smul(Rth, Uh);                            // [62]
+  const long long RU2 = fx_smul(fx_halves(RU), Uh);                  // [61]
+  const long long a01 = fx_smul(Rt - (RtU >> 1) - Rt2, fx_halves(kFxC2_62));  // [63] c^2 [62] -> [61]
+  const long long a02 = fx_smul(Rt2 << 2, fx_halves(kFxC4_64));      // [65]
+  const long long R1 = v.R - (RU >> 1);
+  const long long R10 = R1 - Rt;                                     // [61]
+  const FxHalves R20 = fx_halves(R10 - (Rt >> 1));                   // [62]
+  const long long c00 = ((R1 - (Rt >> 1) + (RU2 >> 3) + (RtU >> 1) + (Rt2 >> 2)) >> 2);  // [59]
+  const long long XY = fx_smul(xh, yh);                              // [64]
+  const FxHalves xyh = fx_halves(XY);
+  const long long c20 = a01 * 2 + fx_smul(R20, xxh), c02 = a01 * 2 + fx_smul(R20, yyh);  // [62]
+  const long long c11 = fx_smul(R20, xyh) * 2;                                            // [62]
+  const FxHalves q = fx_halves(fx_smul(Rh, fx_halves(kFxTwoThirds_63)) << 2);             // R / 6 [64]
+  const long long A = fx_smul(q, xxh), B = fx_smul(q, yyh);                               // [64]
+  const long long h2 = h << 3, h1 = h << 2;                                               // 2h, h [64]
+  const FxHalves alpha = fx_halves(h2 + A), beta = fx_halves(h2 + B);
+  const FxHalves R10h = fx_halves(R10);
+  const long long c10 = fx_smul(xh, R10h), c01 = fx_smul(yh, R10h);                       // [61]
+  const long long c30 = fx_smul(xh, alpha), c03 = fx_smul(yh, beta);                      // [64]
+  const long long c21 = fx_smul(yh, fx_halves(h2 + A * 3)), c12 = fx_smul(xh, fx_halves(h2 + B * 3));
+  const long long c31 = fx_smul(xyh, alpha), c13 = fx_smul(xyh, beta);
+  const long long c40 = (a02 >> 1) + 1 + fx_smul(xxh, fx_halves(h1 + (A >> 2)));
+  const long long c04 = (a02 >> 1) + 1 + fx_smul(yyh, fx_halves(h1 + (B >> 2)));
+  const long long c22 = a02 + 1 + fx_smul(xxh, fx_halves(h1)) + fx_smul(yyh, fx_halves(h1 + A + (A >> 1)));
+  // multiples, all [59]: S_a = a^2 c20 + a^4 c40, O_a = a c10 + a^3 c30 (and the same in y)
+  const auto even = [](long long c2, long long c4, int a) {
+    if (a == 1) return (c2 + (c4 >> 2)) >> 3;
+    if (a == 2) return (c2 + c4) >> 1;
+    const long long w = c2 + ((c4 * 9) >> 2);
+    return w + (w >> 3);
+  };
+  const auto odd = [](long long c1, long long c3, int a) {
+    if (a == 1) return (c1 + (c3 >> 3)) >> 2;
+    if (a == 2) return (c1 + (c3 >> 1)) >> 1;
+    const long long w = c1 + c3 + (c3 >> 3);
+    return w - (w >> 2);
+  };
+  const long long S0 = NEG ? kFixB<true> - c00 + kFixEvenMean<true> : kFixB<false> + c00 + kFixEvenMean<false>;
+  const unsigned o1 = (unsigned)(om1 >> 32), o0 = (unsigned)om1;
+  // one result from p = omega f^eq / w + B (or B - it for NEG) [59]
+  const auto emit = [&](int i, long long p) {
+    const int s = shell(i);
+    const unsigned long long w = (unsigned long long)kCw(s);
+    const unsigned w1 = (unsigned)(w >> 32), w0 = (unsigned)w;
+    const unsigned long long wB = NEG ? (w >> 1) - (w >> 4) - kFixOutMean<true> : (w >> 4) - kFixOutMean<false>;  // w B [58]
+    const unsigned p1 = (unsigned)((unsigned long long)p >> 32), p0 = (unsigned)p;
+    const unsigned long long f = (unsigned long long)fixed(i);
+    const unsigned f1 = (unsigned)(f >> 32), f0 = (unsigned)f;
+    // two 64 x 64 -> high 64 products without their low words' product; the cross terms of
+    // each fit 64 bits (p, w < 2^63, f < 2^61, om1 < 2^62)
+    const unsigned long long t1 = (unsigned long long)p1 * w0 + (unsigned long long)p0 * w1;
+    const unsigned long long t2 = (unsigned long long)f1 * o0 + (unsigned long long)f0 * o1;
+    const unsigned long long r =
+        (unsigned long long)p1 * w1 + (unsigned long long)f1 * o1 + (unsigned)(t1 >> 32) + (unsigned)(t2 >> 32);
+    out(i, NEG ? (long long)(wB - r) : (long long)(r - wB), s);
+  };
+  const auto four = [&](int a, int b, long long S, long long D, long long Ox, long long Oy) {
+    const long long P = S + D, M = S - D, u = Ox + Oy, w = Ox - Oy;
+    emit(pop_index(a, b), P + u);
+    emit(pop_index(-a, -b), P - u);
+    emit(pop_index(a, -b), M + w);
+    emit(pop_index(-a, b), M - w);
+  };
+  const auto sg = [](long long z) { return NEG ? -z : z; };
+  emit(0, S0);
+  long long Sx[4], Sy[4], Ox[4], Oy[4];
+  const auto tables = [&](int a) {
+    Sx[a] = even(c20, c40, a);
+    Sy[a] = even(c02, c04, a);
+    Ox[a] = odd(c10, c30, a);
+    Oy[a] = odd(c01, c03, a);
+  };
+  const auto axes = [&](int a) {
+    const long long P = S0 + sg(Sx[a]), M = S0 + sg(Sy[a]);
+    emit(pop_index(a, 0), P + sg(Ox[a]));
+    emit(pop_index(-a, 0), P - sg(Ox[a]));
+    emit(pop_index(0, a), M + sg(Oy[a]));
+    emit(pop_index(0, -a), M - sg(Oy[a]));
+  };
+  const auto quad = [&](int a, int b, long long ds, long long d, long long dx, long long dy) {
+    four(a, b, S0 + sg(Sx[a] + Sy[b] + ds), sg(d), sg(Ox[a] + dx), sg(Oy[b] + dy));
+  };
+  tables(1);
+  axes(1);
+  quad(1, 1, c22 >> 5, (c11 + ((c31 + c13) >> 2)) >> 3, c12 >> 5, c21 >> 5);
+  tables(2);
+  axes(2);
+  quad(2, 1, c22 >> 3, (c11 + c31 + (c13 >> 2)) >> 2, c12 >> 4, c21 >> 3);
+  quad(1, 2, c22 >> 3, (c11 + c13 + (c31 >> 2)) >> 2, c12 >> 3, c21 >> 4);
+  quad(2, 2, c22 >> 1, (c11 + c31 + c13) >> 1, c12 >> 2, c21 >> 2);
+  tables(3);
+  axes(3);
+  const long long s31 = (c22 + (c22 >> 3)) >> 2;
+  quad(3, 1, s31, ((c11 + ((c31 * 9 + c13) >> 2)) * 3) >> 3, (c12 * 3) >> 5, (c21 + (c21 >> 3)) >> 2);
+  quad(1, 3, s31, ((c11 + ((c13 * 9 + c31) >> 2)) * 3) >> 3, (c12 + (c12 >> 3)) >> 2, (c21 * 3) >> 5);
+}
+
+}  // namespace d2q37

@@ -47,20 +47,18 @@ extern "C" {
 #endif
 
 enum lbm_status { LBM_OK = 0, LBM_EINVAL = 1, LBM_ECUDA = 2, LBM_ETIMEOUT = 3, LBM_ENOMEM = 4, LBM_ESIZE = 5 };
-/* LBM_FP64: float64 populations, float64 collision arithmetic (moment sums in exact 64-bit
- * fixed point for sites whose populations are all below 8 in magnitude, plain float64 sums
- * for any other site, so every finite state is handled; a non-finite population makes its
- * site's outputs NaN; the sums' conversion and the products by powers of two run on the
- * integer pipe, with the bits of their float64 counterparts).  LBM_FP32_SHIFTED: float32 storage of g_i = f_i - w_i rho0, for
- * states with every |g_i| < 8 (choose rho0 near the state's density); a site holding a
- * larger deviation, an infinity or a NaN gets NaN moments, and every population it
- * produces is NaN.  LBM_FP64_FIXED:
- * float64 populations as LBM_FP64 (same buffers, interchangeable states); the fused step
- * evaluates the equilibrium polynomial and the relaxation of every population in 64-bit
- * fixed point on the integer pipes, with errors below one float64 rounding unit, for sites
- * in a stated physical range (float64 elsewhere).  lbm_step, lbm_run, lbm_init, lbm_moments,
- * lbm_kinetic_energy*, lbm_simulate_host and the batch entry points accept it; the separate
- * kernels, layouts and adjoint entry points take LBM_FP64 (its states are the same). */
+/* LBM_FP64: float64 populations.  The fused step evaluates the collision (moments, site
+ * scalars, equilibrium and relaxation) of a site in 64-bit fixed point scaled by the site's
+ * density, with errors below one float64 rounding unit of each result (about a tenth of a
+ * float64 evaluation's), when its populations are within a factor of the equilibrium at rest
+ * and |u_s| < 0.31, |T_s - 1| < 0.4; every other site (fast or hot fluid, zero or negative
+ * populations) is evaluated in float64, so every finite state is handled, and a non-finite
+ * population makes its site's outputs NaN.  LBM_FP64_FIXED: the same step (the name is kept
+ * for callers of earlier versions; the separate kernels, layouts and adjoint entry points take
+ * LBM_FP64 only, its states are the same).  LBM_FP32_SHIFTED: float32 storage of
+ * g_i = f_i - w_i rho0, for states with every |g_i| < 8 (choose rho0 near the state's density);
+ * a site holding a larger deviation, an infinity or a NaN gets NaN moments, and every
+ * population it produces is NaN. */
 /* LBM_FP32_CONSERVED: the FP32_SHIFTED storage (same buffers, interchangeable states) with a
  * collision that restores the exact post-collision mass, momentum and energy of every site
  * after its float32 arithmetic (a second, exact moment sum over the outputs and a correction

@@ -5,9 +5,8 @@
 // are laid end to end in one tile index space (prefix sums in BatchLattice::tile_begin, y
 // fastest inside a lattice) and a device table gives each tile's lattice, so everything a
 // block reads about its lattice is uniform across the block.  Each warp runs the same strip
-// step as the single-lattice kernels (step_fp64.cuh / step_fp32.cuh), so results are
-// bit-identical to lbm_run per lattice (all three forms: FP64, FP64 with the fixed-point
-// relaxation, whose blocks stage their strips in dynamic shared memory, and FP32).
+// step as the single-lattice kernels (step_fix64.cuh, which stages its strips in dynamic
+// shared memory, and step_fp32.cuh), so results are bit-identical to lbm_run per lattice.
 //
 // Modes:
 //   LBM_BATCH_PER_STEP   one launch per step over all tiles of all lattices;
@@ -60,8 +59,7 @@ namespace {
 // kFp32Scaled: FP32 storage where some lattice has a reference density of 2 or more (the
 // moment sums read each lattice's scale constants; see step_fp32.cuh); kFp32Cons and
 // kFp32ConsScaled: the same with the conserved-moment correction (LBM_FP32_CONSERVED).
-enum BatchKind { kFp64 = 0, kFp32 = 1, kFix64 = 2, kFp32Scaled = 3, kFp32Cons = 4, kFp32ConsScaled = 5 };
-constexpr bool kind_fp32(int k) { return k == kFp32 || k == kFp32Scaled || k == kFp32Cons || k == kFp32ConsScaled; }
+enum BatchKind { kFp32 = 1, kFix64 = 2, kFp32Scaled = 3, kFp32Cons = 4, kFp32ConsScaled = 5 };
 
 template <int K>
 struct KindOf {
@@ -105,8 +103,7 @@ __device__ __forceinline__ void batch_tile(const BatchLattice* __restrict__ L, c
   if (x >= B.a.lx) return;  // uniform per warp
   const T* src = (const T*)B.f[parity];
   T* dst = (T*)B.f[parity ^ 1];
-  if constexpr (KIND == kFp64) step_strip_fp64<PERIODIC>(src, dst, B.a, B.a, x, ty * 32, ld);
-  else if constexpr (KIND == kFix64)
+  if constexpr (KIND == kFix64)
     step_strip_fix64<PERIODIC>(src, dst, B.a, B.a, x, ty * 32, ld, staged + threadIdx.y * (Q * 32));
   else
     step_strip_fp32<PERIODIC, KIND == kFp32Scaled || KIND == kFp32ConsScaled, KIND == kFp32Cons || KIND == kFp32ConsScaled>(
@@ -159,11 +156,10 @@ __device__ __forceinline__ bool grid_barrier(BatchSync* sync, unsigned target, l
 }  // namespace
 
 // Register caps, with at most 256 threads per block (8 warps): the FP32 step keeps three
-// such blocks resident per SM (80 registers), the float64 step two (128 registers, as its
-// single-lattice kernel), the fixed-point FP64 step and the conserved-moment FP32 step the
-// 96 registers of their single-lattice kernels (5 blocks of 4 warps per SM).
+// such blocks resident per SM (80 registers), the float64-state step and the conserved-moment
+// FP32 step the 96 registers of their single-lattice kernels (5 blocks of 4 warps per SM).
 constexpr int batch_max_regs(int kind) {
-  return kind == kFp64 ? 128 : (kind == kFix64 || kind == kFp32Cons || kind == kFp32ConsScaled ? 96 : 80);
+  return kind == kFix64 || kind == kFp32Cons || kind == kFp32ConsScaled ? 96 : 80;
 }
 
 extern __shared__ double batch_staged[];
@@ -228,7 +224,7 @@ int32_t cuda_status(cudaError_t e) {
 int kind_of(const lbm_batch* b) {
   if (b->precision == LBM_FP32_SHIFTED) return b->fp32_scaled ? kFp32Scaled : kFp32;
   if (b->precision == LBM_FP32_CONSERVED) return b->fp32_scaled ? kFp32ConsScaled : kFp32Cons;
-  return b->precision == LBM_FP64_FIXED ? kFix64 : kFp64;
+  return kFix64;  // LBM_FP64 and LBM_FP64_FIXED
 }
 
 template <int K>
@@ -242,22 +238,20 @@ void* per_step_fn(bool periodic) {
 
 void* persistent_kernel(const lbm_batch* b) {
   switch (kind_of(b)) {
-    case kFix64: return persistent_fn<kFix64>(b->periodic);
     case kFp32: return persistent_fn<kFp32>(b->periodic);
     case kFp32Scaled: return persistent_fn<kFp32Scaled>(b->periodic);
     case kFp32Cons: return persistent_fn<kFp32Cons>(b->periodic);
     case kFp32ConsScaled: return persistent_fn<kFp32ConsScaled>(b->periodic);
-    default: return persistent_fn<kFp64>(b->periodic);
+    default: return persistent_fn<kFix64>(b->periodic);
   }
 }
 void* per_step_kernel(const lbm_batch* b) {
   switch (kind_of(b)) {
-    case kFix64: return per_step_fn<kFix64>(b->periodic);
     case kFp32: return per_step_fn<kFp32>(b->periodic);
     case kFp32Scaled: return per_step_fn<kFp32Scaled>(b->periodic);
     case kFp32Cons: return per_step_fn<kFp32Cons>(b->periodic);
     case kFp32ConsScaled: return per_step_fn<kFp32ConsScaled>(b->periodic);
-    default: return per_step_fn<kFp64>(b->periodic);
+    default: return per_step_fn<kFix64>(b->periodic);
   }
 }
 

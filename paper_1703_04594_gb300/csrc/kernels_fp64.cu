@@ -1,4 +1,4 @@
-// FP64 kernels: fused pull step, the separate propagate / bc / collide kernels,
+// Kernels of float64 states: fused pull step, the separate propagate / bc / collide kernels,
 // equilibrium initialisation, moments and the kinetic-energy reduction.
 //
 // Thread mapping (all site kernels): block = 32 x 4 threads; threadIdx.x runs along y
@@ -28,26 +28,18 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 }  // namespace
 
 // ---------------------------------------------------------------------------------------
-// Fused step: gather (propagate + bc) -> collide -> streaming store (step_fp64.cuh).
-template <bool PERIODIC>
-__global__ void __launch_bounds__(128, 4) k_step_fp64(const double* __restrict__ fin, double* __restrict__ fout,
-                                                   StepArgs a) {
-  const int x = blockIdx.y * 4 + threadIdx.y;
-  if (x >= a.lx) return;  // uniform per warp
-  step_strip_fp64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly());
-}
-
-// The same fused step with the fixed-point relaxation of collide_fix64.cuh.
+// Fused step of float64 states: gather (propagate + bc) -> collide -> streaming store
+// (step_fix64.cuh).
 #ifndef LBM_FIX64_MIN_BLOCKS
 #define LBM_FIX64_MIN_BLOCKS 5
 #endif
+extern __shared__ double step_staged[];  // 37 populations x 32 sites per warp
 template <bool PERIODIC>
 __global__ void __launch_bounds__(128, LBM_FIX64_MIN_BLOCKS) k_step_fix64(const double* __restrict__ fin,
                                                                          double* __restrict__ fout, StepArgs a) {
-  __shared__ double staged[kFixWarps][Q * 32];  // 37 populations x 32 sites per warp
-  const int x = blockIdx.y * 4 + threadIdx.y;
-  if (x >= a.lx) return;  // uniform per warp
-  step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly(), staged[threadIdx.y]);
+  const int x = blockIdx.y + blockIdx.z * 65535, y0 = (blockIdx.x * blockDim.y + threadIdx.y) * 32;
+  if (x >= a.lx || y0 >= a.ly) return;  // uniform per warp
+  step_strip_fix64<PERIODIC>(fin, fout, a, a, x, y0, LdReadOnly(), step_staged + threadIdx.y * (Q * 32));
 }
 
 // ---------------------------------------------------------------------------------------
@@ -213,15 +205,17 @@ __global__ void __launch_bounds__(256) k_reduce_sum(const double* __restrict__ p
 static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, (a.lx + 3) / 4); }
 static const dim3 kSiteBlock(32, 4);
 
-cudaError_t launch_step_fp64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s) {
-  if (a.periodic) k_step_fp64<true><<<site_grid(a), kSiteBlock, 0, s>>>(fin, fout, a);
-  else k_step_fp64<false><<<site_grid(a), kSiteBlock, 0, s>>>(fin, fout, a);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s) {
-  if (a.periodic) k_step_fix64<true><<<site_grid(a), kSiteBlock, 0, s>>>(fin, fout, a);
-  else k_step_fix64<false><<<site_grid(a), kSiteBlock, 0, s>>>(fin, fout, a);
+  // warps per block: as many as fit a column without idle ones, 4 preferred
+  const int strips = (a.ly + 31) / 32;
+  int w = 4;
+  for (int c = 4; c >= 2; --c)
+    if ((strips + c - 1) / c * c - strips < (strips + w - 1) / w * w - strips) w = c;
+  if (strips < w) w = strips;
+  const dim3 grid((strips + w - 1) / w, a.lx < 65535 ? a.lx : 65535, (a.lx + 65534) / 65535);
+  const size_t smem = (size_t)w * Q * 32 * sizeof(double);
+  if (a.periodic) k_step_fix64<true><<<grid, dim3(32, w), smem, s>>>(fin, fout, a);
+  else k_step_fix64<false><<<grid, dim3(32, w), smem, s>>>(fin, fout, a);
   return cudaGetLastError();
 }
 

@@ -147,8 +147,7 @@ StepArgs d2q37::make_step_args(const lbm_params* p) {
 cudaError_t d2q37::launch_step(const void* fin, void* fout, const StepArgs& a, int32_t precision, cudaStream_t s) {
   if (precision == LBM_FP32_SHIFTED || precision == LBM_FP32_CONSERVED)
     return launch_step_fp32((const float*)fin, (float*)fout, a, s);
-  if (precision == LBM_FP64_FIXED) return launch_step_fix64((const double*)fin, (double*)fout, a, s);
-  return launch_step_fp64((const double*)fin, (double*)fout, a, s);
+  return launch_step_fix64((const double*)fin, (double*)fout, a, s);  // LBM_FP64 and LBM_FP64_FIXED
 }
 
 namespace {

@@ -29,13 +29,13 @@
 // site by 2^-k, with k read off the rest population's exponent, f_0 2^(e_0 - k) in [1/4, 1/2):
 // the path is the same at every density.  Numbers in [] below are fraction bits.
 //   f_i 2^(e_s - k) [60], in [2^-8, 2): exact (a shift of the significand); moments [60]
-//   omega f^eq / w_s [59], below 14; (1 - omega) [62]; w_s 2^e_s [63]; outputs [58]
-// With every rounding counted an output carries about one unit of 2^-58 at a scaled size of
+//   omega f^eq / w_s [58], below 32; (1 - omega) [61]; w_s 2^e_s [63]; outputs [57]
+// With every rounding counted an output carries less than one unit of 2^-57 at a scaled size of
 // 1/4 to 1/2 or more, below a float64 rounding (2^-54 of it); the coefficients that large
-// integers multiply carry 62 to 65 bits.
+// integers multiply carry 61 to 64 bits.
 //
-// Range: 2^-8 <= f_i 2^(e_s - k) < 2, 9/64 <= rho 2^-k < 1, |X|, |Y| < 1/4, |t| < 1/4,
-// 1/2 < tau < 1e6 with |tau g| small (fix_consts); other sites take the float64 collision.
+// Range: 2^-8 <= f_i 2^(e_s - k) < 2, 9/64 <= rho 2^-k < 1, omega rho 2^-k < 1.8, |X|, |Y| < 3/8
+// (|u_s| < 0.31), |t| < 2/5, and |c tau g| < 1/8; other sites take the float64 collision.
 #pragma once
 #include "collide_fix64.cuh"
 
@@ -45,12 +45,12 @@ namespace d2q37 {
 // a = hi 2^32 + lo with a signed low word: three signed 32 x 32 -> 64 products then give the
 // high half of a 64-bit product (the low words' product, at most 1/4 unit and as often
 // negative as positive, is left out), half a unit below the exact value on average.
-struct FxHalves {
-  int h, l;
+struct __align__(8) FxHalves {
+  int l, h;
 };
 __host__ __device__ __forceinline__ FxHalves fx_halves(long long a) {
   const unsigned lo = (unsigned)a;
-  return FxHalves{(int)((unsigned)((unsigned long long)a >> 32) + (lo >> 31)), (int)lo};
+  return FxHalves{(int)lo, (int)((unsigned)((unsigned long long)a >> 32) + (lo >> 31))};
 }
 __host__ __device__ __forceinline__ long long fx_smul(FxHalves a, FxHalves b) {
   const long long t = (long long)a.h * b.l + (long long)a.l * b.h;
@@ -66,7 +66,7 @@ __host__ __device__ constexpr long long fx_signed(double v, int k) {
 }
 
 constexpr long long kFxC2_62 = (long long)fx_const(C2, 1.0, 62);
-constexpr long long kFxC2_63q = (long long)fx_const(C2, 0.25, 64);         // c^2 / 4 [64]
+constexpr long long kFxC2q_64 = (long long)fx_const(C2, 0.25, 64);          // c^2 / 4 [64]
 constexpr long long kFxC4_64 = (long long)fx_const(C2, C2 * 0.125, 64);    // c^4 / 8 [64]
 constexpr long long kFxInvC2_63 = (long long)(kInvC2 >> 1);                // 1 / c^2 [63]
 constexpr long long kFxTwoThirds_63 = 6148914691236517205LL;               // round(2^64 / 3)
@@ -74,13 +74,12 @@ constexpr long long kFxTwoThirds_63 = 6148914691236517205LL;               // ro
 
 // ---- per-lattice constants -------------------------------------------------------------------
 struct FixConsts {
-  int usable;              // 0: the lattice's constants are outside the formats
-  int neg;                 // 1 - omega < 0 (the common case, tau < 1)
-  unsigned long long om1;  // |1 - omega| [62]
-  long long om;            // omega [62]
-  long long cgx, cgy;      // c tau g [60]
-  long long hgx, hgy;      // 2 c tau g / c^2 [63]
-  long long tc;            // tau (1 - tau) |g|^2 / 2 - |c tau g|^2 / (2 c^2) [60]
+  int usable;          // 0: the lattice's constants are outside the formats
+  FxHalves om1;        // 1 - omega [61]
+  FxHalves om;         // omega [62]
+  FxHalves hgx, hgy;   // 2 c tau g / c^2 [63]
+  long long cgx, cgy;  // c tau g [60]
+  long long tc;        // tau (1 - tau) |g|^2 / 2 - |c tau g|^2 / (2 c^2) [60]
 };
 
 inline FixConsts make_fix_consts(double tau, double gx, double gy) {
@@ -91,19 +90,18 @@ inline FixConsts make_fix_consts(double tau, double gx, double gy) {
   const auto small = [](double v) { return v > -0.125 && v < 0.125; };
   r.usable = om > 0.0 && om < 2.0 && om1 > -1.0 && om1 < 1.0 && small(sx) && small(sy) && small(tc);
   if (!r.usable) return r;
-  r.neg = om1 < 0.0;
   // (doubles of this size are multiples of 2^-60 or round there; conversions are exact or
   // round to nearest)
   const auto fix = [](double v, int k) {
     bool unused = false;
     return fx_from_double(v, k, 64, unused);
   };
-  r.om1 = (unsigned long long)fix(om1 < 0.0 ? -om1 : om1, 62);
-  r.om = fix(om, 62);
+  r.om1 = fx_halves(fix(om1, 61));
+  r.om = fx_halves(fix(om, 62));
   r.cgx = fix(sx, 60);
   r.cgy = fix(sy, 60);
-  r.hgx = fix(2.0 * sx / C2, 63);
-  r.hgy = fix(2.0 * sy / C2, 63);
+  r.hgx = fx_halves(fix(2.0 * sx / C2, 63));
+  r.hgy = fx_halves(fix(2.0 * sy / C2, 63));
   r.tc = fix(tc, 60);
   return r;
 }
@@ -127,8 +125,8 @@ struct FixMoments {
   bool ok;               // every population in range
 };
 
-// `load(i)` returns f_i as a float64, `keep(i, f')` stores its fixed-point form; each is called
-// once per population, load(i) before keep(i).
+// `load(i)` returns f_i as a float64, `keep(i, h)` stores its fixed-point form as halves; each is
+// called once per population, load(i) before keep(i).
 template <class Load, class Keep>
 __host__ __device__ __forceinline__ FixMoments fix_moments(Load&& load, Keep&& keep) {
   // shift of the significand: exponent field + e_s - k + (60 - 52 - 1023); k from f_0, whose
@@ -142,7 +140,7 @@ __host__ __device__ __forceinline__ FixMoments fix_moments(Load&& load, Keep&& k
     const unsigned sh = (fx_hi_word(f) >> 20) + (base + (unsigned)e);
     worst = worst > sh ? worst : sh;
     const long long q = fx_from_double_shifted(f, sh);
-    keep(i, q);
+    keep(i, fx_halves(q));
     return q;
   };
   FixMoments m;
@@ -199,7 +197,7 @@ struct FixScalars {
   long long R;         // omega rho 2^-k [61]
   long long X, Y;      // c u_s [64]
   long long XX, YY, U; // X^2, Y^2, |u_s|^2 [64]
-  long long t;         // T_s - 1 [65]
+  long long t;         // T_s - 1 [64]
   bool ok;
 };
 
@@ -243,114 +241,99 @@ __host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, 
   const FxHalves y = fx_halves(yc);
   const long long X = fx_smul(m.X << 5, y) + k.cgx, Y = fx_smul(m.Y << 5, y) + k.cgy;  // [60]
   const long long e2 = fx_smul(dev << 3, y);  // 2 (T - 1) + |u|^2 [59], so half of it [60]
-  ok = ok & ((unsigned long long)(X + (1LL << 58)) < (1ull << 59)) &
-       ((unsigned long long)(Y + (1LL << 58)) < (1ull << 59));
+  ok = ok & ((unsigned long long)(X + (3LL << 57)) < (3ull << 58)) &
+       ((unsigned long long)(Y + (3LL << 57)) < (3ull << 58));
   s.X = X << 4;
   s.Y = Y << 4;
   const FxHalves xh = fx_halves(s.X), yh = fx_halves(s.Y);
   s.XX = fx_smul(xh, xh);
   s.YY = fx_smul(yh, yh);
-  s.U = fx_smul((s.XX + s.YY) << 1, fx_halves(kFxInvC2_63));
+  s.U = fx_smul(s.XX + s.YY, fx_halves(kFxInvC2_63)) * 2;
   // |u|^2 of the unshifted velocity from that of the shifted one
-  const long long g = fx_smul(xh, fx_halves(k.hgx)) + fx_smul(yh, fx_halves(k.hgy));  // [63]
-  const long long t = e2 + k.tc - (s.U >> 5) + (g >> 4);                              // [60]
-  ok = ok & ((unsigned long long)(t + (1LL << 58)) < (1ull << 59));
-  s.t = t << 5;
-  s.R = fx_smul(m.R << 3, fx_halves(k.om));
+  const long long g = fx_smul(xh, k.hgx) + fx_smul(yh, k.hgy);  // [63]
+  const long long t = e2 + k.tc - (s.U >> 5) + (g >> 4);        // [60]
+  constexpr long long kT = (1LL << 61) / 5;                     // 2/5
+  ok = ok & ((unsigned long long)(t + kT) < 2ull * kT);
+  s.t = t << 4;
+  s.R = fx_smul(m.R << 3, k.om);
+  ok = ok & (s.R < (9LL << 58) / 5 * 8);
   s.ok = ok;
   return s;
 }
 
 // ---- 3. coefficients, and the populations -------------------------------------------------------
-// Added to omega f^eq / w (between -2 and 14 in range) or to its negative, so that the unsigned
-// products take positive numbers: 2 or 14 [59].
-template <bool NEG>
-constexpr long long kFixB = NEG ? 7LL << 60 : 1LL << 60;
-// What the shifts and products below round off on average, put back: units of 2^-59 on the even
-// sum, and of 2^-58 on a result.
-template <bool NEG>
-constexpr long long kFixEvenMean = NEG ? 0 : 2;
-template <bool NEG>
-constexpr long long kFixOutMean = 1;
+// What the shifts and products below round off on average, put back in the even sum [58].
+constexpr long long kFixMean = 3;
 
-// NEG: 1 - omega < 0.  `fixed(i)` returns f_i' [60]; `out(i, v, s)` takes f_i^{new} 2^(e_s - k)
-// [58] of population i (shell s).  For NEG the sums are formed for -omega f^eq, so that both
-// products of a population stay positive: w (B - p) + |1 - omega| f = w B - f^{new}.
-template <bool NEG, class Fixed, class Out>
-__host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, unsigned long long om1, Fixed&& fixed,
-                                                   Out&& out) {
+// `fixed(i)` returns the halves of f_i' [60]; `out(i, v, s)` takes f_i^{new} 2^(e_s - k) [57] of
+// population i (shell s).
+template <class Fixed, class Out>
+__host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, FxHalves om1, Fixed&& fixed, Out&& out) {
   const FxHalves Rh = fx_halves(v.R), th = fx_halves(v.t), Uh = fx_halves(v.U);
   const FxHalves xh = fx_halves(v.X), yh = fx_halves(v.Y), xxh = fx_halves(v.XX), yyh = fx_halves(v.YY);
-  const long long Rt = fx_smul(th, Rh);                              // [62]
+  const long long Rt = fx_smul(th, Rh) * 2;                          // [62]
   const FxHalves Rth = fx_halves(Rt);
   const long long RU = fx_smul(Uh, Rh);                              // [61]
-  const long long h = fx_smul(Rth, fx_halves(kFxC2_63q));            // [62]
-  const long long Rt2 = fx_smul(Rth, th);                            // [63]
+  const long long h = fx_smul(Rth, fx_halves(kFxC2q_64));            // [62]
+  const long long Rt2 = fx_smul(Rth, th);                            // [62]
   const long long RtU = fx_smul(Rth, Uh);                            // [62]
   const long long RU2 = fx_smul(fx_halves(RU), Uh);                  // [61]
-  const long long a01 = fx_smul(Rt - (RtU >> 1) - Rt2, fx_halves(kFxC2_62));  // [63] c^2 [62] -> [61]
-  const long long a02 = fx_smul(Rt2 << 2, fx_halves(kFxC4_64));      // [65]
+  const long long a01 = fx_smul(Rt - (RtU >> 1) - Rt2 * 2, fx_halves(kFxC2_62));  // [63] c^2 [62] -> [61]
+  const long long a02 = fx_smul(Rt2 << 2, fx_halves(kFxC4_64));      // [64]
   const long long R1 = v.R - (RU >> 1);
   const long long R10 = R1 - Rt;                                     // [61]
   const FxHalves R20 = fx_halves(R10 - (Rt >> 1));                   // [62]
-  const long long c00 = ((R1 - (Rt >> 1) + (RU2 >> 3) + (RtU >> 1) + (Rt2 >> 2)) >> 2);  // [59]
+  const long long S0 = ((R1 - (Rt >> 1) + (RU2 >> 3) + (RtU >> 1) + (Rt2 >> 1)) >> 3) + kFixMean;  // c00 [58]
   const long long XY = fx_smul(xh, yh);                              // [64]
   const FxHalves xyh = fx_halves(XY);
-  const long long c20 = a01 * 2 + fx_smul(R20, xxh), c02 = a01 * 2 + fx_smul(R20, yyh);  // [62]
-  const long long c11 = fx_smul(R20, xyh) * 2;                                            // [62]
-  const FxHalves q = fx_halves(fx_smul(Rh, fx_halves(kFxTwoThirds_63)) << 2);             // R / 6 [64]
-  const long long A = fx_smul(q, xxh), B = fx_smul(q, yyh);                               // [64]
-  const long long h2 = h << 3, h1 = h << 2;                                               // 2h, h [64]
-  const FxHalves alpha = fx_halves(h2 + A), beta = fx_halves(h2 + B);
+  const long long c20 = a01 + (fx_smul(R20, xxh) >> 1), c02 = a01 + (fx_smul(R20, yyh) >> 1);  // [61]
+  const long long c11 = fx_smul(R20, xyh) * 2;                                                  // [62]
+  const FxHalves q = fx_halves(fx_smul(Rh, fx_halves(kFxTwoThirds_63)) << 2);                   // R / 6 [64]
+  const long long A = fx_smul(q, xxh), B = fx_smul(q, yyh);                                     // [64]
+  const long long h1 = h << 2;                                                                  // h [64], 2h [63]
+  const FxHalves alpha = fx_halves(h1 + (A >> 1)), beta = fx_halves(h1 + (B >> 1));             // [63]
   const FxHalves R10h = fx_halves(R10);
-  const long long c10 = fx_smul(xh, R10h), c01 = fx_smul(yh, R10h);                       // [61]
-  const long long c30 = fx_smul(xh, alpha), c03 = fx_smul(yh, beta);                      // [64]
-  const long long c21 = fx_smul(yh, fx_halves(h2 + A * 3)), c12 = fx_smul(xh, fx_halves(h2 + B * 3));
-  const long long c31 = fx_smul(xyh, alpha), c13 = fx_smul(xyh, beta);
-  const long long c40 = (a02 >> 1) + 1 + fx_smul(xxh, fx_halves(h1 + (A >> 2)));
-  const long long c04 = (a02 >> 1) + 1 + fx_smul(yyh, fx_halves(h1 + (B >> 2)));
-  const long long c22 = a02 + 1 + fx_smul(xxh, fx_halves(h1)) + fx_smul(yyh, fx_halves(h1 + A + (A >> 1)));
-  // multiples, all [59]: S_a = a^2 c20 + a^4 c40, O_a = a c10 + a^3 c30 (and the same in y)
+  const long long c10 = fx_smul(xh, R10h) + 4, c01 = fx_smul(yh, R10h) + 4;  // [61], half a unit of [58] up
+  const long long c30 = fx_smul(xh, alpha), c03 = fx_smul(yh, beta);                            // [63]
+  const long long c21 = fx_smul(yh, fx_halves(h1 + ((A * 3) >> 1)));                            // [63]
+  const long long c12 = fx_smul(xh, fx_halves(h1 + ((B * 3) >> 1)));
+  const long long c31 = fx_smul(xyh, alpha), c13 = fx_smul(xyh, beta);                          // [63]
+  const long long c40 = a02 + 1 + fx_smul(xxh, fx_halves(h1 + (A >> 2)));                       // [64]
+  const long long c04 = a02 + 1 + fx_smul(yyh, fx_halves(h1 + (B >> 2)));
+  const long long c22 = a02 * 2 + 1 + fx_smul(xxh, fx_halves(h1)) + fx_smul(yyh, fx_halves(h1 + A + (A >> 1)));
+  // multiples, all [58]: S_a = a^2 c20 + a^4 c40, O_a = a c10 + a^3 c30 (and the same in y)
   const auto even = [](long long c2, long long c4, int a) {
-    if (a == 1) return (c2 + (c4 >> 2)) >> 3;
-    if (a == 2) return (c2 + c4) >> 1;
-    const long long w = c2 + ((c4 * 9) >> 2);
+    if (a == 1) return (c2 + (c4 >> 3)) >> 3;
+    if (a == 2) return (c2 + (c4 >> 1)) >> 1;
+    const long long w = c2 + c4 + (c4 >> 3);
     return w + (w >> 3);
   };
   const auto odd = [](long long c1, long long c3, int a) {
-    if (a == 1) return (c1 + (c3 >> 3)) >> 2;
-    if (a == 2) return (c1 + (c3 >> 1)) >> 1;
-    const long long w = c1 + c3 + (c3 >> 3);
-    return w - (w >> 2);
+    if (a == 1) return (c1 + (c3 >> 2)) >> 3;
+    if (a == 2) return (c1 + c3) >> 2;
+    const long long w = c1 + c3 * 2 + (c3 >> 2);
+    return (w >> 2) + (w >> 3);
   };
-  const long long S0 = NEG ? kFixB<true> - c00 + kFixEvenMean<true> : kFixB<false> + c00 + kFixEvenMean<false>;
-  const unsigned o1 = (unsigned)(om1 >> 32), o0 = (unsigned)om1;
-  // one result from p = omega f^eq / w + B (or B - it for NEG) [59]
-  const auto emit = [&](int i, long long p) {
-    const int s = shell(i);
-    const unsigned long long w = (unsigned long long)kCw(s);
-    const unsigned w1 = (unsigned)(w >> 32), w0 = (unsigned)w;
-    const unsigned long long wB = NEG ? (w >> 1) - (w >> 4) - kFixOutMean<true> : (w >> 4) - kFixOutMean<false>;  // w B [58]
-    const unsigned p1 = (unsigned)((unsigned long long)p >> 32), p0 = (unsigned)p;
-    const unsigned long long f = (unsigned long long)fixed(i);
-    const unsigned f1 = (unsigned)(f >> 32), f0 = (unsigned)f;
-    // two 64 x 64 -> high 64 products without their low words' product; the cross terms of
-    // each fit 64 bits (p, w < 2^63, f < 2^61, om1 < 2^62)
-    const unsigned long long t1 = (unsigned long long)p1 * w0 + (unsigned long long)p0 * w1;
-    const unsigned long long t2 = (unsigned long long)f1 * o0 + (unsigned long long)f0 * o1;
-    const unsigned long long r =
-        (unsigned long long)p1 * w1 + (unsigned long long)f1 * o1 + (unsigned)(t1 >> 32) + (unsigned)(t2 >> 32);
-    out(i, NEG ? (long long)(wB - r) : (long long)(r - wB), s);
+  // one result, w p + (1 - omega) f, from p = omega f^eq / w [58]: the cross terms of both
+  // products share one sum (|p| < 25 2^58 with |w| < 0.6 2^63 in the outer shells, below
+  // 2^61 in the others; |f|, |1 - omega| < 2^61: the sum stays below 2^63)
+  const auto emit = [&](int i, int s, long long pv) {
+    const FxHalves w = fx_halves(kCw(s)), p = fx_halves(pv), f = fixed(i);
+    const long long t = (long long)p.h * w.l + (long long)p.l * w.h + (long long)f.h * om1.l + (long long)f.l * om1.h;
+    out(i, (long long)p.h * w.h + (long long)f.h * om1.h + (t >> 32), s);
   };
-  const auto four = [&](int a, int b, long long S, long long D, long long Ox, long long Oy) {
-    const long long P = S + D, M = S - D, u = Ox + Oy, w = Ox - Oy;
-    emit(pop_index(a, b), P + u);
-    emit(pop_index(-a, -b), P - u);
-    emit(pop_index(a, -b), M + w);
-    emit(pop_index(-a, b), M - w);
+  // two opposite pairs (v, -v), p = P +- u, then M +- w; rolled, for the instruction cache
+  const auto pairs = [&](int i, int j, int s, long long P, long long u, long long M, long long w) {
+#pragma unroll 1
+    for (int r = 0; r < 2; ++r) {
+      emit(i, s, P + u);
+      emit(i + NPAIR, s, P - u);
+      i = j;
+      P = M;
+      u = w;
+    }
   };
-  const auto sg = [](long long z) { return NEG ? -z : z; };
-  emit(0, S0);
+  emit(0, 0, S0 - 2);  // its share of the sums' mean is less
   long long Sx[4], Sy[4], Ox[4], Oy[4];
   const auto tables = [&](int a) {
     Sx[a] = even(c20, c40, a);
@@ -359,28 +342,31 @@ __host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, unsigned
     Oy[a] = odd(c01, c03, a);
   };
   const auto axes = [&](int a) {
-    const long long P = S0 + sg(Sx[a]), M = S0 + sg(Sy[a]);
-    emit(pop_index(a, 0), P + sg(Ox[a]));
-    emit(pop_index(-a, 0), P - sg(Ox[a]));
-    emit(pop_index(0, a), M + sg(Oy[a]));
-    emit(pop_index(0, -a), M - sg(Oy[a]));
+    pairs(pop_index(a, 0), pop_index(0, a), shell_of_v2(a * a), S0 + Sx[a], Ox[a], S0 + Sy[a], Oy[a]);
   };
-  const auto quad = [&](int a, int b, long long ds, long long d, long long dx, long long dy) {
-    four(a, b, S0 + sg(Sx[a] + Sy[b] + ds), sg(d), sg(Ox[a] + dx), sg(Oy[b] + dy));
+  const auto quad = [&](int a, int b, long long ds, long long D, long long dx, long long dy) {
+    const long long S = S0 + Sx[a] + Sy[b] + ds, ox = Ox[a] + dx, oy = Oy[b] + dy;
+    pairs(pop_index(a, b), pop_index(a, -b), shell_of_v2(a * a + b * b), S + D, ox + oy, S - D, ox - oy);
   };
   tables(1);
   axes(1);
-  quad(1, 1, c22 >> 5, (c11 + ((c31 + c13) >> 2)) >> 3, c12 >> 5, c21 >> 5);
+  quad(1, 1, c22 >> 6, (c11 + ((c31 + c13) >> 1)) >> 4, c12 >> 5, c21 >> 5);
   tables(2);
   axes(2);
-  quad(2, 1, c22 >> 3, (c11 + c31 + (c13 >> 2)) >> 2, c12 >> 4, c21 >> 3);
-  quad(1, 2, c22 >> 3, (c11 + c13 + (c31 >> 2)) >> 2, c12 >> 3, c21 >> 4);
-  quad(2, 2, c22 >> 1, (c11 + c31 + c13) >> 1, c12 >> 2, c21 >> 2);
+  quad(2, 1, c22 >> 4, (c11 + c31 * 2 + (c13 >> 1)) >> 3, c12 >> 4, c21 >> 3);
+  quad(1, 2, c22 >> 4, (c11 + c13 * 2 + (c31 >> 1)) >> 3, c12 >> 3, c21 >> 4);
+  quad(2, 2, c22 >> 2, (c11 + (c31 + c13) * 2) >> 2, c12 >> 2, c21 >> 2);
   tables(3);
   axes(3);
-  const long long s31 = (c22 + (c22 >> 3)) >> 2;
-  quad(3, 1, s31, ((c11 + ((c31 * 9 + c13) >> 2)) * 3) >> 3, (c12 * 3) >> 5, (c21 + (c21 >> 3)) >> 2);
-  quad(1, 3, s31, ((c11 + ((c13 * 9 + c31) >> 2)) * 3) >> 3, (c12 + (c12 >> 3)) >> 2, (c21 * 3) >> 5);
+  const long long s9 = (c22 + (c22 >> 3)) >> 3;
+  const auto d9 = [&](long long c9, long long c1) {  // 3 (c11 + 9 c9 + c1)
+    const long long d = c11 + c9 * 4 + ((c9 + c1) >> 1);
+    return (d >> 3) + (d >> 4);
+  };
+  const auto times3 = [](long long c) { return (c >> 4) + (c >> 5); };
+  const auto times9 = [](long long c) { return (c >> 2) + (c >> 5); };
+  quad(3, 1, s9, d9(c31, c13), times3(c12), times9(c21));
+  quad(1, 3, s9, d9(c13, c31), times9(c12), times3(c21));
 }
 
 }  // namespace d2q37

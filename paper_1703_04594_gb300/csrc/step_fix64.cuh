@@ -93,7 +93,7 @@ __device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin,
   } else {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const double* src = fin + i * a.pop + (off[vx(i) + 3] - vy(i));
+      const double* src = fin + (i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch) - vy(i) + (unsigned)yc;
       if (Ld::kL1) cp_async8(sf + i * 32, src);
       else sf[i * 32] = ld(src);
     }
@@ -123,20 +123,18 @@ __device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin,
     }
   }
   if (!active) return;
-  long long* const sx = reinterpret_cast<long long*>(sf);  // the same slots, as fixed point
-  const FixMoments m = fix_moments([&](int i) { return sf[i * 32]; }, [&](int i, long long q) { sx[i * 32] = q; });
+  FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);  // the same slots, as fixed point
+  const FixMoments m = fix_moments([&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
   const FixScalars v = fix_scalars(m, a.fx);
   const unsigned self = (unsigned)((long long)x * a.pitch + y);
   if (!v.ok || !a.fx.usable) {
     collide_site_reloaded<PERIODIC, Ld>(fin, fout, a, w, x, yc, self);
     return;
   }
-  const auto fixed = [&](int i) { return sx[i * 32]; };
-  const auto out = [&](int i, long long X, int s) {
-    __stcs(fout + i * a.pop + self, fx_lower_exponent(X, ((58 + shell_exp(s)) << 20) - m.kb));
-  };
-  if (a.fx.neg) fix_relax<true>(v, a.fx.om1, fixed, out);
-  else fix_relax<false>(v, a.fx.om1, fixed, out);
+  fix_relax(v, a.fx.om1, [&](int i) { return sx[i * 32]; }, [&](int i, long long X, int s) {
+    double* dst = fout + (i * a.pop + (long long)x * a.pitch) + (unsigned)y;
+    __stcs(dst, fx_lower_exponent(X, ((57 + shell_exp(s)) << 20) - m.kb));
+  });
 }
 
 }  // namespace d2q37

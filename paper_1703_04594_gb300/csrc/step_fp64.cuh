@@ -1,7 +1,5 @@
-// One warp-strip of the fused FP64 pull step: 32 consecutive sites (x, y0 .. y0+31) of
-// one column, gathered (propagate + bc, Sec. 3 eq. "master2", Sec. 5), collided
-// (collide_fp64.cuh) and stored.  Shared by the single-lattice kernel and the batched
-// kernels; `Ld` chooses the load path (read-only cache, or L2-only inside a persistent
+// Pieces of the float64 pull step on a warp-strip, 32 consecutive sites (x, y0 .. y0+31) of
+// one column.  `Ld` chooses the load path (read-only cache, or L2-only inside a persistent
 // kernel whose source buffers were written earlier in the same launch).
 #pragma once
 #include "collide_fp64.cuh"
@@ -75,21 +73,6 @@ __device__ __forceinline__ void gather_strip_fp64(const double* __restrict__ fin
       f[i] = ld(fin + i * a.pop + col[vx(i) + 3] + ys);
     }
   }
-}
-
-// One warp-strip of the fused step.  Must be called by all 32 lanes of a warp
-// (lane = y - y0).  Lanes with y >= ly gather clamped data and store nothing.
-template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void step_strip_fp64(const double* __restrict__ fin, double* __restrict__ fout,
-                                                const StepScalars& a, const StepWalls& w, int x, int y0, Ld ld) {
-  const int y = y0 + (threadIdx.x & 31);
-  const bool active = y < a.ly;
-  const int yc = active ? y : a.ly - 1;
-  double f[Q];
-  gather_strip_fp64<PERIODIC>(fin, a, w, x, y0, yc, f, ld);
-  if (!active) return;
-  double* dst = fout + (long long)x * a.pitch + y;
-  collide_site(f, a.cc, [&](int i, double v) { __stcs(dst + i * a.pop, v); });
 }
 
 }  // namespace d2q37

@@ -21,14 +21,14 @@
 //   2. (k_adj_walls) the wall rows: every population of (x_s, 0) receives the sum of the
 //      bottom slots of column x_s, each times its ghost's weight w_i P_i(T_wall) (the
 //      transpose of rho_w = sum_j f_j(x_s, 0)), and likewise at the top.
-// dL/dtau partials are summed per block and then in a fixed order (deterministic).
+// dL/dtau partials are summed per strip and then in a fixed order (deterministic).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include "../../include/lbm_d2q37.h"
 #include "adjoint_fix64.cuh"
 #include "kernels.h"
-#include "step_fp64.cuh"
+#include "step_fix64.cuh"
 
 namespace d2q37 {
 
@@ -101,22 +101,6 @@ __device__ __forceinline__ EqVjp eq_vjp_pairs(double rho, double usx, double usy
   return {Gr, rho * Gx, rho * Gy, rho * Gt};
 }
 
-// The float64 VJP for sites outside the fixed-point range, not inlined so that its
-// unrolled arithmetic does not weigh on the register allocation of the fixed-point path.
-__device__ __noinline__ EqVjp eq_vjp_float64(double rho, double usx, double usy, double t, const double* mu_staged) {
-  return eq_vjp_pairs(rho, usx, usy, t, [&](int i) { return mu_staged[i * 32]; });
-}
-
-__device__ __forceinline__ double block_sum_128(double v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-  __shared__ double ws[4];
-  const int w = (threadIdx.y * blockDim.x + threadIdx.x) >> 5;
-  if ((threadIdx.x & 31) == 0) ws[w] = v;
-  __syncthreads();
-  return (ws[0] + ws[1]) + (ws[2] + ws[3]);
-}
-
 // Ghost slots of one column: population i with vy_i > 0 fed rows 0 .. vy_i - 1 of column
 // x_s + vx_i from the bottom ghosts of column x_s; those entries take bottom slots
 // ghost_base(i, +1) + row of column x_s.  The top mirrors it with -vy_i and row ly - 1 - y.
@@ -151,30 +135,6 @@ __host__ __device__ constexpr int ghost_base(int i, int sign) {
   return sign > 0 ? b[i] : t[i];
 }
 
-// The pull-gather of a warp's strip into its shared-memory slots sf[i * 32 + lane] through
-// registers (wall bc and periodic wrap included); not inlined, so that its 37 live values
-// do not weigh on the register allocation of the collide kernel.
-template <bool PERIODIC>
-__device__ __noinline__ void gather_to_shared(const double* __restrict__ fin, const StepArgs& a, int x, int y0,
-                                              int yc, double* sf) {
-  double f[Q];
-  gather_strip_fp64<PERIODIC>(fin, a, a, x, y0, yc, f, LdReadOnly());
-#pragma unroll
-  for (int i = 0; i < Q; ++i) sf[i * 32] = f[i];
-}
-
-// Float64 moments of a staged site (populations sf[i * 32]), for sites outside the
-// fixed-point sums' range; not inlined, so the common path keeps its registers.
-__device__ __noinline__ void moments_float64_staged(const double* sf, double& rho, double& jx, double& jy,
-                                                     double& e) {
-  moments_float64([&](int i) { return sf[i * 32]; }, rho, jx, jy, e);
-}
-
-__device__ __forceinline__ void cp_async8_adj(double* smem_dst, const double* gmem_src) {
-  const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-
 }  // namespace
 
 // The lattice-wide scalars of the adjoint collision, formed once on the host.
@@ -187,148 +147,182 @@ struct AdjConsts {
   double tshift;        // tau (1 - tau) |g|^2 / D - 1:  t = T + tshift
   double gx, gy;
   double dts_dtau;      // d T_s / d tau = (1 - 2 tau) |g|^2 / D
+  AdjFixConsts fx;
 };
 
-// Step 1: per-site adjoint of the collision with the transposed propagate as its store
-// (block 32 x 4 as the forward kernels).  `side` holds 2 * lx * kGhostSlots doubles: the
-// bottom slots of every column, then the top slots.
-#ifndef LBM_ADJ_MIN_BLOCKS
-#define LBM_ADJ_MIN_BLOCKS 5  // 96 registers, 20 warps per SM (with 37.9 KB of staging per block)
-#endif
+// The adjoint collision of one site in float64 (sites outside the fixed-point range), not inlined
+// so that its arithmetic does not weigh on the register allocation of the fixed-point path: the
+// site's outputs to its slots, and its part of dL/dtau returned.
 template <bool PERIODIC>
-__global__ void __launch_bounds__(128, LBM_ADJ_MIN_BLOCKS) k_adj_collide(const double* __restrict__ fin,
+__device__ __noinline__ double adj_site_float64(const double* __restrict__ fin, const double* __restrict__ lam,
+                                                const StepArgs& a, const AdjConsts& k, int x, int y, double* sf) {
+  double mu_ft = 0.0, rho, jx, jy, e;
+  {
+    double f[Q];
+    gather_site<PERIODIC>(fin, a, a, x, y, f, LdReadOnly());
+    moments_int(f, rho, jx, jy, e);
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const double l = __ldg(lam + i * a.pop);
+      mu_ft = fma(l, f[i], mu_ft);
+      sf[i * 32] = l;
+    }
+  }
+  const auto mu = [&](int i) { return sf[i * 32]; };
+  const double inv = 1.0 / rho;
+  const double Jx = C * jx, Jy = C * jy, E = C2 * e;  // xi-unit moments
+  const double ux = Jx * inv, uy = Jy * inv;
+  const double uu = fma(ux, ux, uy * uy);
+  const double TD = fma(E, inv, -uu);  // D T
+  const double t = fma(TD, 1.0 / D, k.tshift);
+  const EqVjp G = eq_vjp_pairs(1.0, ux + k.tgx, uy + k.tgy, t, mu);  // per unit density
+  // nu = (d f^eq / d(rho, J, E))^T mu through u = J / rho, T = (E / rho - |u|^2) / D:
+  // the factors rho of G and 1 / rho of the chain rule cancel, and E / rho = D T + |u|^2
+  const double nuE = pow2_scale(G.Gt, -1);      // gt / D, D = 2 (exact scalings on the integer pipe)
+  const double m2nuE = pow2_scale(-nuE, 1);
+  const double nuJx = fma(ux, m2nuE, G.Gux);
+  const double nuJy = fma(uy, m2nuE, G.Guy);
+  const double nuR = fma(nuE, uu - TD, G.Grho - fma(G.Gux, ux, G.Guy * uy));
+  // out_{+-v} = (1-w) mu + A_s +- B_v with A_s = w (nuR + nuE c^2 |v|^2) (one per shell)
+  // and B_v = w c nuJ . v (from the multiples of w c nuJ)
+  const double om1 = k.om1;
+  const double wR = k.om * nuR, wE = k.om_c2 * nuE;
+  const Multiples wJ = make_multiples(k.om_c * nuJx, k.om_c * nuJy);
+  sf[0] = fma(om1, mu(0), wR);
+#pragma unroll
+  for (int j = 1; j <= NPAIR; ++j) {
+    const double A = fma(wE, (double)v2(j), wR);
+    const double B = dot_v(wJ, rep_vx(j), rep_vy(j));
+    sf[j * 32] = fma(om1, mu(j), A + B);
+    sf[(j + NPAIR) * 32] = fma(om1, mu(j + NPAIR), A - B);
+  }
+  // sum_i mu_i f^eq_i = rho * Grho
+  return fma(-k.om2, fma(rho, G.Grho, -mu_ft),
+             (k.om * rho) * fma(G.Gux, k.gx, fma(G.Guy, k.gy, G.Gt * k.dts_dtau)));
+}
+
+// Scatter of a strip's outputs next to a wall or across the periodic seam.  out_i(z) is
+// lambda_i(z - v_i) of the previous step (the transposed pull), or goes to the wall slot of its
+// source column when z - v_i is a ghost; entries of the site whose source z + v_i lies beyond a
+// wall get no push and are set to zero.
+template <bool PERIODIC>
+__device__ __noinline__ void push_strip_edge(const double* sf, double* __restrict__ lam_out, double* __restrict__ side,
+                                             const StepArgs& a, int x, int y) {
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const int xs = wrap_index(x - vx(i), a.lx), yd = y - vy(i);
+    const double val = sf[i * 32];
+    if (!PERIODIC && yd < 0) {
+      __stcs(side + ((long long)xs * kGhostSlots + ghost_base(i, 1) + y), val);
+    } else if (!PERIODIC && yd >= a.ly) {
+      __stcs(side + (((long long)a.lx + xs) * kGhostSlots + ghost_base(i, -1) + (a.ly - 1 - y)), val);
+    } else {
+      __stcs(lam_out + (i * a.pop + (long long)xs * a.pitch + (PERIODIC ? wrap_index(yd, a.ly) : yd)), val);
+    }
+    const int ys = y + vy(i);
+    if (!PERIODIC && (ys < 0 || ys >= a.ly)) __stcs(lam_out + (i * a.pop + (long long)x * a.pitch + y), 0.0);
+  }
+}
+
+// The fixed-point adjoint's view of a site: its slots, and its lambda (planes below 2^32 elements).
+struct AdjIo {
+  FxHalves* slots;
+  const double* lam;
+  unsigned pop;
+  int K;  // exponent units of the outputs
+  struct At {
+    FxHalves* f;
+    const double* lam;
+  };
+  __device__ __forceinline__ At at(int i) const { return At{slots + i * 32, lam + (unsigned long long)pop * (unsigned)i}; }
+  __device__ __forceinline__ double mu(At h, int k) const { return __ldg(k ? h.lam + (unsigned long long)pop * NPAIR : h.lam); }
+  __device__ __forceinline__ FxHalves fixed(At h, int k) const { return h.f[k * (NPAIR * 32)]; }
+  __device__ __forceinline__ void keep(At h, int k, FxHalves q) const { h.f[k * (NPAIR * 32)] = q; }
+  __device__ __forceinline__ FxHalves held(int i) const { return slots[i * 32]; }
+  __device__ __forceinline__ void out(int i, long long v) const {
+    reinterpret_cast<double*>(slots)[i * 32] = fx_lower_exponent(v, K);
+  }
+};
+
+// Step 1: per-site adjoint of the collision with the transposed propagate as its store.  Blocks run
+// along a column (column_launch).  `side` holds 2 * lx * kGhostSlots doubles: the bottom slots of
+// every column, then the top slots.  The strip's pull-gather is staged in shared memory (9.5 KB
+// per warp); a slot holds f~_i, then its fixed-point form, then mu_i's, then the output.  What bounds
+// it: 6.1 k instructions per strip, more code than the instruction cache holds (hit rate 83 %), and
+// latency at 16 warps per SM.  So the loops over populations are rolled, and block barriers keep a
+// block's four warps, one per scheduler, on the same code (512 x 1024: 0.236 ms without them,
+// 0.221 with; fully unrolled 0.247; blocks of 8 to 20 warps 0.238 to 0.338; the float64-pipe
+// version it replaces 0.334).
+extern __shared__ double adj_staged[];
+template <bool PERIODIC>
+__global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict__ fin,
                                                      const double* __restrict__ lam_next, double* __restrict__ lam_out,
                                                      double* __restrict__ side, double* __restrict__ dtau_part,
                                                      StepArgs a, AdjConsts k) {
-  const int x = blockIdx.y * 4 + threadIdx.y;
-  const int y0 = blockIdx.x * 32;
+  const int x = blockIdx.y + blockIdx.z * 65535;
+  if (x >= a.lx) return;  // uniform per block
+  const int y0 = (blockIdx.x * blockDim.y + threadIdx.y) * 32;
+  if (y0 >= a.ly) return;  // uniform per warp
   const int y = y0 + threadIdx.x;
+  const bool active = y < a.ly;  // the other lanes work on the last row's data and store nothing
+  const int yc = active ? y : a.ly - 1;
+  double* const sf = adj_staged + threadIdx.y * (Q * 32) + threadIdx.x;
+  FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);
+  const double* lam = lam_next + (long long)x * a.pitch + (unsigned)yc;
+  stage_strip<PERIODIC>(fin, a, a, x, y0, yc, sf, LdReadOnly());
+  // the block exponent of lambda, from the high words alone (the values are loaded again below,
+  // when their fixed-point forms can go to the slots at once)
+  unsigned top = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i)
+    top = max(top, __ldg(reinterpret_cast<const unsigned*>(lam + i * a.pop) + 1) & 0x7fffffffu);
+  __syncthreads();
+  const FixMoments m = fix_moments_rolled(c_fix_axes, c_fix_quads, [&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
+  const FixScalars v = fix_scalars(m, a.fx);
+  const unsigned E = top == 0u ? 512u : top >> 20;  // all zero: any exponent
+  __syncthreads();
+  const int K = (1080 - (int)E) << 20;
+  const bool ok = v.ok && a.fx.usable && k.fx.usable && E - 100u < 978u;
+  const AdjIo io = {sx, lam, (unsigned)a.pop, K};
+  const FixMu mm = fix_mu_moments(K + (1 << 20), c_fix_axes, c_fix_quads, io);
+  __syncthreads();
+  FixVjp r = fix_vjp(m, v, mm, a.fx, k.fx);
+  if (top == 0u) r = FixVjp{};  // lambda = 0: no rounding residue
+  __syncthreads();
+  fix_adj_outputs(r, k.fx.om1, c_pair_fix, io);
   double contrib = 0.0;
-  if (x < a.lx) {  // uniform per warp
-    const bool active = y < a.ly;
-    const int yc = active ? y : a.ly - 1;
-    // the strip's pull-gather staged in shared memory (9.5 KB per warp): no registers held
-    // for it, which lets 5 blocks of 4 warps share an SM (389 against 399 us per step with
-    // the gather in registers at 4 blocks)
-    __shared__ double staged[4][Q * 32];
-    double* const sf = &staged[threadIdx.y][0] + (threadIdx.x & 31);
-    if (PERIODIC || y0 < 3 || y0 + 32 > a.ly - 3) {
-      gather_to_shared<PERIODIC>(fin, a, x, y0, yc, sf);
+  if (active) {
+    if (ok) contrib = k.om2 * fx_lower_exponent(r.D, K + (1 << 20) - m.kb);
+    else contrib = adj_site_float64<PERIODIC>(fin, lam, a, k, x, y, sf);
+    if (PERIODIC || fix64_wall_strip<PERIODIC>(a, y0)) {
+      push_strip_edge<PERIODIC>(sf, lam_out, side, a, x, y);
     } else {
-      unsigned off[7];  // column x_s, row yc within a population plane
 #pragma unroll
-      for (int d = 0; d < 7; ++d) off[d] = (unsigned)((long long)wrap_index(x - (d - 3), a.lx) * a.pitch + yc);
-#pragma unroll
-      for (int i = 0; i < Q; ++i) cp_async8_adj(sf + i * 32, fin + i * a.pop + (off[vx(i) + 3] - vy(i)));
-      asm volatile("cp.async.wait_all;\n" ::: "memory");
-    }
-    const auto fget = [&](int i) { return sf[i * 32]; };
-    if (active) {
-      double rho, jx, jy, e;
-      moments_get_or(fget, rho, jx, jy, e, [](int, int) {},
-                     [&](double& r, double& mx, double& my, double& me) { moments_float64_staged(sf, r, mx, my, me); });
-      const double inv = 1.0 / rho;
-      const double Jx = C * jx, Jy = C * jy, E = C2 * e;  // xi-unit moments
-      const double ux = Jx * inv, uy = Jy * inv;
-      const double uu = fma(ux, ux, uy * uy);
-      const double TD = fma(E, inv, -uu);  // D T
-      const double usx = ux + k.tgx, usy = uy + k.tgy;
-      const double t = fma(TD, 1.0 / D, k.tshift);
-      const long long o = (long long)x * a.pitch + y;
-      const double* lam = lam_next + o;
-      // sum_i mu_i f~_i; each staging slot, once its f~_i is read, takes mu_i = lambda_i, so
-      // the three later passes over mu (the VJP's exponent scan and conversion, the outputs)
-      // read shared memory instead of re-reading lambda, whose 37.9 KB per block do not stay
-      // in the L1 that the staging leaves
-      double mu_ft = 0.0;
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        const double l = __ldg(lam + i * a.pop);
-        mu_ft = fma(l, fget(i), mu_ft);
-        sf[i * 32] = l;
-      }
-      const auto mu = [&](int i) { return sf[i * 32]; };
-      // the VJP in fixed point (adjoint_fix64.cuh), in float64 outside its range, per unit
-      // density: g = G / rho for G_u and G_t (G_rho has no factor rho)
-      double gr, gux, guy, gt;
-      {
-        VjpSums V;
-        if (eq_vjp_sums_fix(usx, usy, t, mu, V)) {
-          gr = V.Gr;
-          const double Wu2 = pow2_scale(V.Wu, 1);  // 2 Wu, exactly
-          gux = fma(C, V.Ax, usx * Wu2);
-          guy = fma(C, V.Ay, usy * Wu2);
-          gt = V.Gt;
-        } else {
-          const EqVjp G = eq_vjp_float64(1.0, usx, usy, t, sf);
-          gr = G.Grho;
-          gux = G.Gux;
-          guy = G.Guy;
-          gt = G.Gt;
-        }
-      }
-      // nu = (d f^eq / d(rho, J, E))^T mu through u = J / rho, T = (E / rho - |u|^2) / D:
-      // the factors rho of G and 1 / rho of the chain rule cancel, and E / rho = D T + |u|^2
-      const double nuE = pow2_scale(gt, -1);      // gt / D, D = 2 (exact scalings on the integer pipe)
-      const double m2nuE = pow2_scale(-nuE, 1);   // -2 nuE
-      const double nuJx = fma(ux, m2nuE, gux);
-      const double nuJy = fma(uy, m2nuE, guy);
-      const double nuR = fma(nuE, uu - TD, gr - fma(gux, ux, guy * uy));
-      // out_i(z) is lambda_i(z - v_i) of the previous step (the transposed pull), or the
-      // wall slot of its source column when z - v_i is a ghost
-      // (the destination is selected, not branched on, to keep the kernel's code small)
-      const auto push = [&](int i, double val) {
-        const int xs = wrap_index(x - vx(i), a.lx), yd = y - vy(i);
-        const long long in_fluid = i * a.pop + (long long)xs * a.pitch + (PERIODIC ? wrap_index(yd, a.ly) : yd);
-        bool ghost = false;
-        long long slot = 0;
-        if (!PERIODIC && vy(i) > 0) {
-          ghost = yd < 0;
-          slot = (long long)xs * kGhostSlots + ghost_base(i, 1) + y;
-        } else if (!PERIODIC && vy(i) < 0) {
-          ghost = yd >= a.ly;
-          slot = ((long long)a.lx + xs) * kGhostSlots + ghost_base(i, -1) + (a.ly - 1 - y);
-        }
-        // only the selected address is formed (the other offset may be out of its buffer)
-        __stcs(ghost ? side + slot : lam_out + in_fluid, val);
-      };
-      // out_{+-v} = (1-w) mu + A_s +- B_v with A_s = w (nuR + nuE c^2 |v|^2) (one per shell)
-      // and B_v = w c nuJ . v (from the multiples of w c nuJ)
-      const double om1 = k.om1;
-      const double wR = k.om * nuR, wE = k.om_c2 * nuE;
-      const Multiples wJ = make_multiples(k.om_c * nuJx, k.om_c * nuJy);
-      push(0, fma(om1, mu(0), wR));
-#pragma unroll
-      for (int j = 1; j <= NPAIR; ++j) {
-        const double A = fma(wE, (double)v2(j), wR);
-        const double B = dot_v(wJ, rep_vx(j), rep_vy(j));
-        push(j, fma(om1, mu(j), A + B));
-        push(j + NPAIR, fma(om1, mu(j + NPAIR), A - B));
-      }
-      // entries of this site whose source z + v_i lies beyond a wall get no push
-      if (!PERIODIC && (y < 3 || y >= a.ly - 3)) {
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-          const int ys = y + vy(i);
-          if (ys < 0 || ys >= a.ly) __stcs(lam_out + i * a.pop + o, 0.0);
-        }
-      }
-      // sum_i mu_i f^eq_i = rho * Grho
-      contrib = fma(-k.om2, fma(rho, gr, -mu_ft), (k.om * rho) * fma(gux, k.gx, fma(guy, k.gy, gt * k.dts_dtau)));
+      for (int i = 0; i < Q; ++i)
+        __stcs(lam_out + (i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch) - vy(i) + (unsigned)y,
+               sf[i * 32]);
     }
   }
-  const double s = block_sum_128(contrib);
-  if (threadIdx.x == 0 && threadIdx.y == 0) dtau_part[blockIdx.y * gridDim.x + blockIdx.x] = s;
+  // one partial per strip (a sum over the block would hold its early warps' registers and slots)
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) contrib += __shfl_down_sync(0xffffffffu, contrib, off);
+  if (threadIdx.x == 0) dtau_part[(long long)x * ((a.ly + 31) >> 5) + (y0 >> 5)] = contrib;
 }
 
-// Adds sum(part[0..n)) to *acc in a fixed order; one block of 256 threads.
+// Adds sum(part[0..n)) to *acc in a fixed order; one block of 256 threads.  Eight independent sums
+// per thread keep as many loads in flight (one at a time, 16384 partials took ~20 us).
 __device__ __forceinline__ void reduce_add_256(const double* __restrict__ part, long long n, double* acc) {
-  double s = 0.0;
-  for (long long i = threadIdx.x; i < n; i += 256) s += part[i];
+  double s[8] = {};
+  for (long long i = threadIdx.x; i < n; i += 8 * 256) {
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+    for (int j = 0; j < 8; ++j)
+      if (i + j * 256 < n) s[j] += part[i + j * 256];
+  }
+  double v = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
   __shared__ double ws[8];
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
@@ -418,15 +412,16 @@ __global__ void __launch_bounds__(128) k_init_adjoint(const double* __restrict__
 static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, (a.lx + 3) / 4); }
 
 long long adjoint_partial_count(const StepArgs& a) {
-  const dim3 g = site_grid(a);
-  return (long long)g.x * g.y;
+  return (long long)((a.ly + 31) / 32) * a.lx;  // one per strip
 }
 
 long long adjoint_side_count(const StepArgs& a) { return 2LL * a.lx * kGhostSlots; }
 
 cudaError_t launch_adjoint_step(const double* fin, const double* lam_next, double* lam, double* side, double* part,
                                 double* dtau, const StepArgs& a, double tau, double gx, double gy, cudaStream_t s) {
-  const dim3 blk(32, 4);
+  const ColumnLaunch c = column_launch(a);
+  const dim3 blk(32, c.warps);
+  const size_t smem = (size_t)c.warps * Q * 32 * sizeof(double);
   AdjConsts k;
   k.tau = tau;
   k.om = 1.0 / tau;
@@ -441,10 +436,11 @@ cudaError_t launch_adjoint_step(const double* fin, const double* lam_next, doubl
   k.gx = gx;
   k.gy = gy;
   k.dts_dtau = (1.0 - 2.0 * tau) * gg / D;
+  k.fx = make_adj_fix_consts(tau, gx, gy);
   if (a.periodic) {
-    k_adj_collide<true><<<site_grid(a), blk, 0, s>>>(fin, lam_next, lam, side, part, a, k);
+    k_adj_collide<true><<<c.grid, blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
   } else {
-    k_adj_collide<false><<<site_grid(a), blk, 0, s>>>(fin, lam_next, lam, side, part, a, k);
+    k_adj_collide<false><<<c.grid, blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
     const long long items = 2LL * a.lx * Q;  // (column, wall, population), plus one block for the dtau sum
     k_adj_walls<<<(unsigned)((items + 255) / 256) + 1, 256, 0, s>>>(side, lam, a, part, adjoint_partial_count(a),
                                                                     dtau);

@@ -1,181 +1,320 @@
-// Vector-Jacobian product of the equilibrium in 64-bit fixed point (the adjoint's
-// counterpart of collide_fix64.cuh).
+// The adjoint (vector-Jacobian product) of one site's collision in 64-bit fixed point, the
+// counterpart of site_fix64.cuh.
 //
-// The VJP of f^eq_i = w_i rho P_i(s_i, U, t) against the adjoint vector mu (adjoint.cu,
-// eq_vjp_pairs) costs ~32 float64 operations per opposite pair, which bounds the adjoint
-// step by GB300's float64 pipe.  Here the per-shell polynomial coefficients, the per-pair
-// polynomial values (P, dP/ds, dP/dU, dP/dt for the even and odd parts) and their
-// contraction with mu run in fixed point on the integer pipes; only the site scalars and
-// the final combination stay in float64.
+// With f^eq_i = w_i rho sum_pq b_pq(X, Y, t) vx^p vy^q (X = c u_s,x, Y = c u_s,y, t = T_s - 1;
+// b_pq are c_pq / (omega rho) of site_fix64.cuh) the adjoint vector mu enters the product only
+// through its 15 weighted moments m_pq = sum_i w_i mu_i vx^p vy^q:
+//   G_rho = sum b_pq m_pq,  G_X = sum (db_pq/dX) m_pq,  G_Y,  G_t likewise (per unit density),
+// and the derivatives are again low polynomials in X, Y, t, most of them coefficients b_pq of
+// lower order (db40/dX = b30, db22/dX = b12, db31/dX = b21, ...).  So a site costs 37
+// weightings, 53 terms of four scalar products and ~45 products for the coefficients; a
+// population then costs one product, (1 - w) mu_i, and adds (evaluating four polynomials and
+// their products with mu per opposite pair took 12.9 k instructions per site).
 //
-// Formats.  mu is block floating point: every mu_i of the site is scaled by the same power
-// of two, chosen from the largest exponent among the 37 values so that |mu'| < 2^57.
-// Polynomial values have 59 fraction bits (all below 16 in the range of the path), s has
-// 63 and s^2 62 (as in the forward path).  A product of mu' with a polynomial value keeps
-// the high 64 bits, mu' P / 32; sums over a shell are multiplied by the shell weight w_s
-// (64 fraction bits) and the four results are converted back to float64 with the block
-// exponent.  The sums' unit is 2^-52 to 2^-51 of max_i |mu_i|; each high product rounds
-// down by less than one unit, half a unit on average, which the sums add back (+1 per
-// two products, +4 for the eight shell products), so a result carries an unbiased error
-// of a few units, comparable to the float64 rounding of the same sums.  (Uncompensated,
-// that bias is the same sign at every site and adds up in dL/dtau.)
+// Formats ([] = fraction bits).  mu is block floating point: all 37 values share the power of
+// two 2^K with max |mu_i| 2^K in [2^57, 2^58) (held with one bit more).  m_pq are in units of
+// 2^(-1-K), the four products of 2^(-4-K) and outputs of 2^-K.  Over the range |G| < 1.1 max|mu|
+// and |out_i| < 20.4 max|mu| (the largest absolute row sums of the derivatives, omega = 2),
+// below 2^62.4 units.  The error of an output is about a unit, 2^-57 of max |mu|.
+// The scalar products share their cross terms (FxDot), so a term costs three multiply-adds.
 //
-// Range: |c u_s,x|, |c u_s,y| < 0.15 and |t| < 0.25 (as the forward path) and mu finite
-// with max_i |mu_i| in [2^-922, 2^876] (or all zero); other sites use the float64 VJP.
+// Range: that of the forward path (fix_scalars), and 100 <= biased exponent of max |mu| < 1078
+// (or every mu zero); other sites use float64.
 #pragma once
-#include "collide_fix64.cuh"
+#include "site_fix64.cuh"
 
 namespace d2q37 {
 
-// Per-shell constants: q = c^2 |v|^2 (59 fraction bits), q^2 (55), (q - D - 4)/4 (61),
-// (q - D - 2)/2 (60), w_s (64, unsigned).
-struct AdjShellFix {
-  long long q, q2, kq1, kq2;
-  unsigned long long w;
-};
-__host__ __device__ constexpr long long fx_signed_const(double v, int k) {
-  return v >= 0.0 ? (long long)fx_const(v, 1.0, k) : -(long long)fx_const(-v, 1.0, k);
-}
-#define LBM_ADJ_SHELL(s)                                                                          \
-  {                                                                                               \
-    s ? (long long)fx_const(q_shell(s), 1.0, 59) : 0LL,                                           \
-        s ? (long long)fx_const(q_shell(s), q_shell(s), 55) : 0LL,                                \
-        fx_signed_const((q_shell(s) - D - 4.0) / 4.0, 61), fx_signed_const((q_shell(s) - D - 2.0) / 2.0, 60), \
-        fx_const(w_shell(s), 1.0, 64)                                                             \
-  }
-static __constant__ AdjShellFix c_adj_shell[8] = {LBM_ADJ_SHELL(0), LBM_ADJ_SHELL(1), LBM_ADJ_SHELL(2),
-                                                  LBM_ADJ_SHELL(3), LBM_ADJ_SHELL(4), LBM_ADJ_SHELL(5),
-                                                  LBM_ADJ_SHELL(6), LBM_ADJ_SHELL(7)};
-#undef LBM_ADJ_SHELL
+constexpr long long kFxSixth_64 = 3074457345618258603LL;  // round(2^64 / 6)
 
-constexpr unsigned long long kInv6 = 3074457345618258603ull;   // round(2^64 / 6)
-constexpr unsigned long long kInv24 = 768614336404564651ull;   // round(2^64 / 24)
-
-// Sums of the VJP before the site factors: G = {Grho, sum w v_x X, sum w v_y X, sum w W,
-// sum w T} (see eq_vjp_pairs in adjoint.cu for X, W, T), as float64.
-struct VjpSums {
-  double Gr, Ax, Ay, Wu, Gt;
+// The lattice's constants of the adjoint that FixConsts does not hold.
+struct AdjFixConsts {
+  int usable;
+  FxHalves om1;         // 1 - omega [63]
+  FxHalves omc2;        // omega c^2 [61]
+  FxHalves sx, sy, st;  // c tau gx, c tau gy, tau d T_s / d tau = tau (1 - 2 tau) |g|^2 / 2 [63]
+  long long tg;         // tau (1 - tau) |g|^2 / 2 [60]
 };
 
-__device__ __forceinline__ bool zero_sums(VjpSums& out) {
-  out = VjpSums{0.0, 0.0, 0.0, 0.0, 0.0};
-  return true;
-}
-
-// Returns false (and leaves `out` untouched) when the site is outside the fixed-point range.
-// `mu(i)` returns mu_i; it is called twice per population (a scan for the block exponent,
-// then the conversion).
-template <class Mu>
-__device__ __forceinline__ bool eq_vjp_sums_fix(double usx, double usy, double t, Mu&& mu, VjpSums& out) {
-  const double Uxd = C * usx, Uyd = C * usy;
-  const long long kU = 0x3FC3333333333333LL, kT = 0x3FD0000000000000LL, kA = 0x7FFFFFFFFFFFFFFFLL;
-  if ((__double_as_longlong(Uxd) & kA) >= kU || (__double_as_longlong(Uyd) & kA) >= kU ||
-      (__double_as_longlong(t) & kA) >= kT)
-    return false;
-  // block exponent of mu
-  unsigned emax = 0;
-#pragma unroll 1
-  for (int i = 0; i < Q; ++i) {
-    const unsigned e = (unsigned)((unsigned long long)__double_as_longlong(mu(i)) >> 52) & 0x7ffu;
-    emax = e > emax ? e : emax;
-  }
-  // inf or NaN; or magnitudes whose sums could leave the normal float64 range
-  if (emax >= 1900u || emax < 100u) return emax == 0u ? zero_sums(out) : false;
-  const int kmu = 1079 - (int)emax;  // |mu| < 2^(emax - 1022)  =>  |mu 2^kmu| < 2^57
-  bool unused = false;
-  const long long X1 = fx_from_double(Uxd, 63, 64, unused), Y1 = fx_from_double(Uyd, 63, 64, unused);
-  // the forward coefficients of c0, c1, c2 (collide_fix64.cuh), and those in q of dP/dU and
-  // dP/dt at s = 0:  pue0 = b0 + b1 q,  pt0 = p0 + p1 q + p2 q^2
-  const HermiteFix h = hermite_fix(X1, Y1, t);
-  const long long U62 = h.U62, t63 = h.t63;
-  const long long a00 = h.a00, a01 = h.a01, a02 = h.a02, a10 = h.a10, a11 = h.a11, a20 = h.a20;
-  const long long a21 = h.a11;                                                                   // 66
-  const long long b0 = -(1LL << 60) + (U62 >> 3) + (t63 >> 2);                                   // 61
-  const long long b1 = -t63;                                                                     // 65
-  const long long p0 = -(1LL << 61) + (U62 >> 1) + (t63 >> 1);                                   // 61
-  const long long p1 = (1LL << 60) - (U62 >> 3) - (t63 >> 1);                                    // 61
-  const long long p2 = t63 * 2;                                                                  // 66
-  long long Gr = 0, Ax = 0, Ay = 0, Wu = 0, Gt = 0;
-  int cur = -1;
-  long long c0 = 0, c1 = 0, c2 = 0, pue0 = 0, pt0 = 0, kq1 = 0, kq2 = 0;
-  unsigned long long w = 0;
-  long long Rs = 0, Axs = 0, Ays = 0, Ws = 0, Ts = 0;
-  const auto flush = [&]() {
-    Gr += fx_mulhi_su(Rs, w);
-    Ax += fx_mulhi_su(Axs, w);
-    Ay += fx_mulhi_su(Ays, w);
-    Wu += fx_mulhi_su(Ws, w);
-    Gt += fx_mulhi_su(Ts, w);
-    Rs = Axs = Ays = Ws = Ts = 0;
+inline AdjFixConsts make_adj_fix_consts(double tau, double gx, double gy) {
+  AdjFixConsts r = {};
+  const double om1 = 1.0 - 1.0 / tau, gg = gx * gx + gy * gy;
+  const double sx = C * tau * gx, sy = C * tau * gy, st = tau * (1.0 - 2.0 * tau) * gg / 2.0,
+               tg = tau * (1.0 - tau) * gg / 2.0;
+  const auto small = [](double v) { return v > -0.125 && v < 0.125; };
+  r.usable = om1 > -0.999 && om1 < 0.999 && small(sx) && small(sy) && small(st) && small(tg);
+  if (!r.usable) return r;
+  const auto fix = [](double v, int k) {
+    bool unused = false;
+    return fx_from_double(v, k, 64, unused);
   };
-  {  // rest population: s = 0, only E = c0, dP/dU = pue0 and dP/dt = pt0 at q = 0
-    const long long m = fx_from_double(mu(0), kmu, 64, unused);
-    const AdjShellFix& c = c_adj_shell[0];
-    Rs = fx_mulhi(m, a00 >> 2);       // 59 fraction bits each
-    Ws = fx_mulhi(m, b0 >> 2);
-    Ts = fx_mulhi(m, p0 >> 2);
-    w = c.w;
-    flush();
+  r.om1 = fx_halves(fix(om1, 63));
+  r.omc2 = fx_halves(fix(C2 / tau, 61));
+  r.sx = fx_halves(fix(sx, 63));
+  r.sy = fx_halves(fix(sy, 63));
+  r.st = fx_halves(fix(st, 63));
+  r.tg = fix(tg, 60);
+  return r;
+}
+
+// A sum of products a b, high and cross parts apart (the low words' products left out).
+struct FxDot {
+  long long h = 0, t = 0;
+  __host__ __device__ __forceinline__ void add(FxHalves a, FxHalves b) {
+    h = fx_wide(a.h, b.h, h);
+    t = fx_wide(a.l, b.h, fx_wide(a.h, b.l, t));
+  }
+  // the sum times 2^(s - 64)
+  __host__ __device__ __forceinline__ long long high(int s) const { return (h << s) + (t >> (32 - s)); }
+};
+
+// mu 2^(K + 1) rounded to an integer, by an addition to the exponent field and the float64 pipe's
+// conversion (that pipe is otherwise idle but for the outputs' conversions).  K1 = (K + 1) << 20
+// with 3 <= K + 1 <= 981: a field of the block's largest exponent or less stays below 1082, and a
+// zero or subnormal becomes a number below 2^-41, which rounds to 0.
+__host__ __device__ __forceinline__ long long fx_block(double v, int K1) {
+#ifdef __CUDA_ARCH__
+  return __double2ll_rn(__hiloint2double(__double2hiint(v) + K1, __double2loint(v)));
+#else
+  unsigned long long b;
+  __builtin_memcpy(&b, &v, 8);
+  b += (unsigned long long)K1 << 32;
+  __builtin_memcpy(&v, &b, 8);
+  return (long long)__builtin_rint(v);
+#endif
+}
+
+// ---- 1. the moments of mu -----------------------------------------------------------------------
+struct FixMu {
+  long long m00, m10, m01, m20, m11, m02, m30, m21, m12, m03, m40, m31, m22, m13, m04;  // units 2^(-1 - K)
+  long long mf;  // sum mu_i f_i, in units of 2^(k - K - 1)
+};
+
+// `io.at(i)` returns a handle of population i's pair (i, i + NPAIR), and for population i + k NPAIR
+// `io.mu(h, k)` its mu, `io.fixed(h, k)` the halves of f' (fix_moments); `io.keep(h, k, q)` takes the
+// halves of its mu 2^(K + 1), after the other two calls.  `axes` and `quads` are the tables above (the
+// host tests pass their own copies).
+template <class Io>
+__host__ __device__ __forceinline__ FixMu fix_mu_moments(int K1, const FixGroup* axes, const FixGroup* quads,
+                                                                Io&& io) {
+  FixMu r;
+  r.mf = 5;
+  FxDot mf;
+  const auto get = [&](auto at, int k) {
+    const long long q = fx_block(io.mu(at, k), K1);
+    const FxHalves h = fx_halves(q);
+    mf.add(h, io.fixed(at, k));
+    io.keep(at, k, h);
+    return q;
+  };
+  const auto flush = [&](int e) {  // the populations' scale 2^e taken off
+    r.mf += mf.high(4) >> e;
+    mf = FxDot();
+  };
+  // w_s v: the weights are scaled by 2^e_s [63], so the product has e_s - 1 more bits than v; taking
+  // e_s - 1 off leaves the sums' unit
+  const auto weigh = [](long long v, FxHalves w, int e) { return fx_smul(v, w) >> (e - 1); };
+  // every weighting rounds down, half a unit on average: the sums start with what they lack (the
+  // sum of half their multiples); without it the bias, times |v|^2 c^2 / 2 in the outputs, is
+  // 2^-53 of max |mu|
+  unsigned long long m00 = 6, m20 = 17, m02 = 17, m40 = 107, m04 = 107, m22 = 21, m11 = 7, m31 = 28, m13 = 28;
+  unsigned long long m10 = 8, m01 = 8, m30 = 41, m03 = 41, m12 = 13, m21 = 13;
+  m00 += (unsigned long long)weigh(get(io.at(0), 0), fx_halves_ct(kCw(0)), shell_exp(0));
+  flush(shell_exp(0));
+#pragma unroll 1
+  for (int n = 0; n < 3; ++n) {
+    const FixGroup& g = axes[n];
+    const auto ai = io.at(g.i), aj = io.at(g.j);
+    const long long p = get(ai, 0), q = get(ai, 1), u = get(aj, 0), v = get(aj, 1);
+    flush(g.sh);
+    const unsigned long long ex = (unsigned long long)weigh(p + q, g.w, g.sh), ox = (unsigned long long)weigh(p - q, g.w, g.sh);
+    const unsigned long long ey = (unsigned long long)weigh(u + v, g.w, g.sh), oy = (unsigned long long)weigh(u - v, g.w, g.sh);
+    m00 += ex + ey;
+    m20 += g.a2 * ex;
+    m02 += g.a2 * ey;
+    m40 += g.a4 * ex;
+    m04 += g.a4 * ey;
+    m10 += g.a * ox;
+    m01 += g.a * oy;
+    m30 += g.a3 * ox;
+    m03 += g.a3 * oy;
   }
 #pragma unroll 1
-  for (int k = 1; k <= NPAIR; ++k) {
-    const PairFix pk = c_pair_fix[k];
-    if (pk.sh != cur) {  // uniform across the warp
-      if (cur > 0) flush();
-      cur = pk.sh;
-      const AdjShellFix& c = c_adj_shell[cur];
-      const unsigned long long q = (unsigned long long)c.q, q2 = (unsigned long long)c.q2;
-      // values at 59 fraction bits: q (59) x a (65) -> 60, q^2 (55) x a (69) -> 60, ...
-      c0 = (a00 >> 2) + (fx_mulhi_su(a01, q) >> 1) + (fx_mulhi_su(a02, q2) >> 1);
-      c1 = (a10 >> 3) + (fx_mulhi_su(a11, q) >> 1);
-      c2 = (a20 >> 4) + (fx_mulhi_su(a21, q) >> 2);
-      pue0 = (b0 >> 2) + (fx_mulhi_su(b1, q) >> 1);
-      pt0 = (p0 >> 2) + fx_mulhi_su(p1, q) * 8 + fx_mulhi_su(p2, q2) * 4;
-      kq1 = c.kq1;
-      kq2 = c.kq2;
-      w = c.w;
-    }
-    const long long s = pk.vx * X1 + pk.vy * Y1;                                   // 63
-    const unsigned long long as = (unsigned long long)(s < 0 ? -s : s);
-    const unsigned long long s2 = fx_umulhi(as, as);                                // 62
-    const long long h24 = (long long)(fx_umulhi(s2, kInv24) >> 3);                  // s^2/24, 59
-    const long long h6 = (long long)(fx_umulhi(s2, kInv6) >> 3);                    // s^2/6, 59
-    const long long E = c0 + fx_mulhi_su(c2 + h24, s2) * 4;                          // 57 -> 59
-    const long long O = fx_mulhi(c1 + h6, s) * 2;                                    // 58 -> 59
-    const long long Pse = c1 + (long long)(s2 >> 4);                                 // + s^2/2
-    const long long Pso = fx_mulhi(2 * c2 + h6, s) * 2;                              // s (2 c2 + s^2/6)
-    const long long PUe = pue0 - (long long)(s2 >> 5);                               // - s^2/4
-    const long long PUo = -(s >> 5);                                                 // - s/2
-    const long long Pte = pt0 + fx_mulhi_su(kq1, s2);                                // + (q-D-4)/4 s^2
-    const long long Pto = fx_mulhi(s, kq2);                                          // (q-D-2)/2 s
-    const long long mp = fx_from_double(mu(k), kmu, 64, unused);
-    const long long mm = fx_from_double(mu(k + NPAIR), kmu, 64, unused);
-    const long long S = mp + mm, Dm = mp - mm;
-    // each high product rounds down, half a unit low on average: + 1 per two products
-    // (without it the bias, ~2^-51 max|mu| per site, adds up over the sites of dL/dtau)
-    Rs += fx_mulhi(S, E) + fx_mulhi(Dm, O) + 1;
-    const long long X = fx_mulhi(Dm, Pse) + fx_mulhi(S, Pso) + 1;
-    Axs += pk.vx * X;
-    Ays += pk.vy * X;
-    Ws += fx_mulhi(S, PUe) + fx_mulhi(Dm, PUo) + 1;
-    Ts += fx_mulhi(S, Pte) + fx_mulhi(Dm, Pto) + 1;
+  for (int n = 0; n < 6; ++n) {
+    const FixGroup& g = quads[n];
+    const auto ai = io.at(g.i), aj = io.at(g.j);
+    const long long p = get(ai, 0), q = get(ai, 1), u = get(aj, 0), v = get(aj, 1);
+    flush(g.sh);
+    const long long pp = p + q, pm = p - q, up = u + v, um = u - v;
+    const unsigned long long S = (unsigned long long)weigh(pp + up, g.w, g.sh), D = (unsigned long long)weigh(pp - up, g.w, g.sh);
+    const unsigned long long x = (unsigned long long)weigh(pm + um, g.w, g.sh), y = (unsigned long long)weigh(pm - um, g.w, g.sh);
+    m00 += S;
+    m20 += g.a2 * S;
+    m02 += g.b2 * S;
+    m40 += g.a4 * S;
+    m04 += g.b4 * S;
+    m22 += (g.a2 * g.b2) * S;
+    m11 += (g.a * g.b) * D;
+    m31 += (g.a3 * g.b) * D;
+    m13 += (g.a * g.b3) * D;
+    m10 += g.a * x;
+    m30 += g.a3 * x;
+    m12 += (g.a * g.b2) * x;
+    m01 += g.b * y;
+    m03 += g.b3 * y;
+    m21 += (g.a2 * g.b) * y;
   }
-  flush();
-  // the eight shell products of each sum (one per flush) likewise
-  Gr += 4;
-  Ax += 4;
-  Ay += 4;
-  Wu += 4;
-  Gt += 4;
-  // mu' P / 32 with mu' = mu 2^kmu: the sums are their values times 2^(kmu - 5)
-  const int k = kmu - 5;
-  // -826 < k <= 974: on the integer pipe, rounded to nearest even
-  out.Gr = fix_to_double_rn(Gr, k);
-  out.Ax = fix_to_double_rn(Ax, k);
-  out.Ay = fix_to_double_rn(Ay, k);
-  out.Wu = fix_to_double_rn(Wu, k);
-  out.Gt = fix_to_double_rn(Gt, k);
-  return true;
+  r.m00 = (long long)m00, r.m10 = (long long)m10, r.m01 = (long long)m01, r.m20 = (long long)m20;
+  r.m11 = (long long)m11, r.m02 = (long long)m02, r.m30 = (long long)m30, r.m21 = (long long)m21;
+  r.m12 = (long long)m12, r.m03 = (long long)m03, r.m40 = (long long)m40, r.m31 = (long long)m31;
+  r.m22 = (long long)m22, r.m13 = (long long)m13, r.m04 = (long long)m04;
+  return r;
+}
+
+// ---- 2. the products with the equilibrium's derivatives, and the outputs' terms ---------------------
+struct FixVjp {
+  // out_i = (1 - w) mu_i + R + E |v_i|^2 + Bx vx + By vy
+  long long R, E;    // w nu_rho and w c^2 nu_E, in units of 2^(-1-K)
+  long long Bx, By;  // w c nu_J, in units of 2^-K
+  long long D;       // tau^2 d/dtau of the site, in units of 2^(k - K - 1)
+};
+
+__host__ __device__ __forceinline__ FixVjp fix_vjp(const FixMoments& f, const FixScalars& v, const FixMu& m,
+                                                   const FixConsts& k, const AdjFixConsts& ka) {
+  const long long X = v.X, Y = v.Y, XX = v.XX, YY = v.YY, U = v.U, t = v.t;
+  const FxHalves xh = fx_halves(X), yh = fx_halves(Y), xxh = fx_halves(XX), yyh = fx_halves(YY), th = fx_halves(t),
+                 uh = fx_halves(U);
+  const FxHalves ic2 = fx_halves(kFxInvC2_63);
+  constexpr long long one = 1LL << 60;
+  const long long XY = fx_smul(xh, yh);
+  const FxHalves xyh = fx_halves(XY);
+  const long long t2 = fx_smul(th, th), tU = fx_smul(th, uh), U2 = fx_smul(uh, uh);       // [64]
+  const long long h = fx_smul(th, fx_halves(kFxC2q_64)), h2 = h * 2;                       // c^2 t / 4, twice [64]
+  const long long a01 = fx_smul((t >> 1) - (tU >> 2) - t2, fx_halves(kFxC2_62)) >> 2;      // [62] -> [60]
+  const long long a02 = fx_smul(t2, fx_halves(kFxC4_64));                                  // [64]
+  const long long a10 = one - (U >> 5) - (t >> 3), a20 = (one >> 1) - (U >> 6) - (t >> 4) - (t >> 5);  // [60]
+  const FxHalves a10h = fx_halves(a10), a20h = fx_halves(a20);
+  const long long ax = fx_smul(xxh, fx_halves(kFxSixth_64)), ay = fx_smul(yyh, fx_halves(kFxSixth_64));  // X^2/6 [64]
+  const FxHalves alpha = fx_halves(h2 + ax), beta = fx_halves(h2 + ay);                    // [64]
+  const long long gx = h2 + (XX >> 1), gy = h2 + (YY >> 1);                                // [64]
+  const long long b10 = fx_smul(xh, a10h), b01 = fx_smul(yh, a10h);                        // [60]
+  // coefficients at 60 bits, as halves
+  const auto h60 = [](long long c64) { return fx_halves(c64 >> 4); };
+  const FxHalves B30 = h60(fx_smul(xh, alpha)), B03 = h60(fx_smul(yh, beta));
+  const FxHalves B21 = h60(fx_smul(yh, fx_halves(gx))), B12 = h60(fx_smul(xh, fx_halves(gy)));
+  const FxHalves XYh = h60(XY), GX2 = h60(gx), GY2 = h60(gy);
+  const FxHalves m00 = fx_halves(m.m00), m10 = fx_halves(m.m10), m01 = fx_halves(m.m01), m20 = fx_halves(m.m20),
+                 m11 = fx_halves(m.m11), m02 = fx_halves(m.m02), m30 = fx_halves(m.m30), m21 = fx_halves(m.m21),
+                 m12 = fx_halves(m.m12), m03 = fx_halves(m.m03), m40 = fx_halves(m.m40), m31 = fx_halves(m.m31),
+                 m22 = fx_halves(m.m22), m13 = fx_halves(m.m13), m04 = fx_halves(m.m04);
+  // every sum below in units of 2^(-4 - K)
+  FxDot g;  // G_rho
+  g.add(m00, fx_halves(one - (U >> 5) - (t >> 4) + (U2 >> 7) + (tU >> 4) + (t2 >> 4)));
+  g.add(m10, fx_halves(b10));
+  g.add(m01, fx_halves(b01));
+  g.add(m20, fx_halves(a01 + fx_smul(a20h, xxh)));
+  g.add(m02, fx_halves(a01 + fx_smul(a20h, yyh)));
+  g.add(m11, fx_halves(fx_smul(a20h, xyh) * 2));
+  g.add(m30, B30);
+  g.add(m21, B21);
+  g.add(m12, B12);
+  g.add(m03, B03);
+  g.add(m40, h60(a02 + fx_smul(xxh, fx_halves(h + (ax >> 2)))));
+  g.add(m04, h60(a02 + fx_smul(yyh, fx_halves(h + (ay >> 2)))));
+  g.add(m22, h60(a02 * 2 + fx_smul(xxh, fx_halves(h)) + fx_smul(yyh, fx_halves(h + (XX >> 2)))));
+  g.add(m31, h60(fx_smul(xyh, alpha)));
+  g.add(m13, h60(fx_smul(xyh, beta)));
+  const long long Gr = g.high(7);
+  const long long cxx = fx_smul(xxh, ic2) >> 3, cyy = fx_smul(yyh, ic2) >> 3, cxy = fx_smul(xyh, ic2) >> 3;  // / c^2 [60]
+  const FxHalves ncxy = fx_halves(-cxy);
+  g = FxDot();  // G_X
+  g.add(m00, fx_halves(fx_smul(fx_halves(b10), ic2) * -2));
+  g.add(m10, fx_halves(a10 - cxx));
+  g.add(m01, ncxy);
+  g.add(m20, fx_halves(fx_smul(xh, fx_halves(2 * a20 - (t >> 5) - (cxx >> 1)))));
+  g.add(m02, fx_halves(-(fx_smul(xh, fx_halves((t >> 4) + cyy)) >> 1)));
+  g.add(m11, fx_halves(fx_smul(yh, fx_halves(2 * a20 - cxx))));
+  g.add(m30, GX2);
+  g.add(m21, XYh);
+  g.add(m12, GY2);
+  g.add(m40, B30);
+  g.add(m22, B12);
+  g.add(m31, B21);
+  g.add(m13, B03);
+  const long long GX = g.high(7);
+  g = FxDot();  // G_Y
+  g.add(m00, fx_halves(fx_smul(fx_halves(b01), ic2) * -2));
+  g.add(m01, fx_halves(a10 - cyy));
+  g.add(m10, ncxy);
+  g.add(m02, fx_halves(fx_smul(yh, fx_halves(2 * a20 - (t >> 5) - (cyy >> 1)))));
+  g.add(m20, fx_halves(-(fx_smul(yh, fx_halves((t >> 4) + cxx)) >> 1)));
+  g.add(m11, fx_halves(fx_smul(xh, fx_halves(2 * a20 - cyy))));
+  g.add(m03, GY2);
+  g.add(m12, XYh);
+  g.add(m21, GX2);
+  g.add(m04, B03);
+  g.add(m22, B21);
+  g.add(m13, B12);
+  g.add(m31, B30);
+  const long long GY = g.high(7);
+  // G_t: the orders above two share the factor c^2 / 2
+  g = FxDot();
+  g.add(fx_halves(m.m30 + m.m12), h60(X));
+  g.add(fx_halves(m.m03 + m.m21), h60(Y));
+  g.add(fx_halves(m.m31 + m.m13), XYh);
+  g.add(fx_halves(m.m40 + m.m22), fx_halves(XX >> 5));
+  g.add(fx_halves(m.m04 + m.m22), fx_halves(YY >> 5));
+  g.add(fx_halves(m.m40 + m.m04 + 2 * m.m22), h60(h2));
+  const long long high2 = fx_smul(g.high(7), fx_halves(kFxC2_62)) * 2;  // c^2 / 2
+  g = FxDot();
+  const long long e0 = fx_smul((one >> 1) - (U >> 6) - (t >> 3), fx_halves(kFxC2_62)) * 4;  // c^2 (1/2 - U/4 - 2t) [58]
+  g.add(m00, fx_halves((U >> 4) + (t >> 3) - one));
+  g.add(m10, fx_halves(-(X >> 3)));
+  g.add(m01, fx_halves(-(Y >> 3)));
+  g.add(m20, fx_halves(e0 - (XX >> 4) - (XX >> 5)));
+  g.add(m02, fx_halves(e0 - (YY >> 4) - (YY >> 5)));
+  g.add(m11, fx_halves(-((XY * 3) >> 4)));
+  const long long Gt = g.high(7) + high2;
+  // nu = (d f^eq / d(rho, J, E))^T mu through u = J / rho, T = (E / rho - |u|^2) / D (per unit
+  // density): nu_rho = G_rho - G_X X0 - G_Y Y0 + G_t (|u|^2 - D T) / 2 ..., with
+  // |u|^2 - (E / rho) / 2 = kap; c nu_J = c^2 G_X - X0 G_t; nu_E = G_t / 2
+  const FxHalves gxh = fx_halves(GX), gyh = fx_halves(GY), gth = fx_halves(Gt);
+  const FxHalves x0 = fx_halves(v.X0), y0 = fx_halves(v.Y0);
+  const long long kap = (v.e + 2 * ka.tg - (t >> 3) - one) << 2;                 // [62], below 1.6
+  const long long nR = Gr - fx_smul(gxh, x0) - fx_smul(gyh, y0) + fx_smul(gth, fx_halves(kap)) * 4;
+  const FxHalves c2 = fx_halves(kFxC2_62);
+  const FxHalves nx = fx_halves(fx_smul(gxh, c2) * 4 - fx_smul(gth, x0));
+  const FxHalves ny = fx_halves(fx_smul(gyh, c2) * 4 - fx_smul(gth, y0));
+  FixVjp r;
+  r.R = (fx_smul(fx_halves(nR), k.om) + 1) >> 1;
+  r.Bx = (fx_smul(nx, k.om) + 2) >> 2;
+  r.By = (fx_smul(ny, k.om) + 2) >> 2;
+  r.E = (fx_smul(gth, ka.omc2) + 1) >> 1;  // omega c^2 G_t / 2
+  // sum mu f - rho (G_rho - (tau g) . G - tau (dT_s/dtau) G_t)
+  const long long V = Gr - (fx_smul(gxh, ka.sx) + fx_smul(gyh, ka.sy) + fx_smul(gth, ka.st)) * 2;
+  r.D = m.mf - (fx_smul(V, f.R << 3) >> 2);
+  return r;
+}
+
+// ---- 3. the outputs ----------------------------------------------------------------------------------
+// `io.held(i)` returns the halves of mu_i 2^(K + 1); `io.out(i, v)` takes the site's out_i in units
+// of 2^-K.  One rolled loop over the opposite pairs (v, -v), out = (1 - w) mu + A +- B; `pairs` is
+// the table c_pair_fix.
+template <class Io>
+__host__ __device__ __forceinline__ void fix_adj_outputs(const FixVjp& v, FxHalves om1, const PairFix* pairs, Io&& io) {
+  const auto emit = [&](int i, long long add) {
+    const FxHalves m = io.held(i);
+    const long long t = fx_wide(m.l, om1.h, fx_wide(m.h, om1.l));
+    io.out(i, fx_wide(m.h, om1.h, add) + (t >> 32));
+  };
+  emit(0, v.R >> 1);
+#pragma unroll 2
+  for (int j = 1; j <= NPAIR; ++j) {
+    const PairFix p = pairs[j];
+    const long long A = (v.R + v.E * p.v2) >> 1, B = v.Bx * p.vx + v.By * p.vy;
+    emit(j, A + B);
+    emit(j + NPAIR, A - B);
+  }
 }
 
 }  // namespace d2q37

@@ -1,31 +1,6 @@
-// FP64 collision with the equilibrium polynomial and the relaxation in 64-bit fixed point.
-//
-// The same update as collide_site (Sec. 3, eq. "lbequation"; equilibrium and moments as in
-// collide_fp64.cuh), with a different split of the work between the GPU's pipes.  The site
-// scalars (moments, 1/rho, u, T and the gravity shift) stay in float64.  Everything after
-// them runs in signed 64-bit fixed point on the integer pipes: the Hermite coefficients
-// a_jk and their products with omega rho, the shell coefficients K0..K3 of
-// omega rho w_s (C0 + C1 s + C2 s^2 + s^3/6 + s^4/24), and for each opposite pair
-// s = xi . u_s, s^2, h = K3 s^2, the odd part O = s (K1 + h), the even part
-// E = K0 + s^2 (K2 + h/4) and f_+/-' = (1 - omega) f_+/- + E +/- O.
-//
-// Formats.  Shell s is scaled by 2^e_s with w_s 2^e_s in [0.5, 1), so every scaled
-// population and coefficient is of order rho whatever the weight.  A product keeps the
-// high 64 bits of the 128-bit result (a truncation).  Each quantity has the number of
-// fraction bits that makes its products land on their consumers' binary points with no
-// shift:
-//   outputs, E, O, K0, (1 - omega) f   58  (|v| < 32)      K2, K2 + h/4      60
-//   K1, h = K3 s^2, K1 + h             59                  K3 61
-//   s 63, s^2 62, |1 - omega| 63, f 59 + e_s
-// Each output carries a few units of 2^-58 relative to its scaled size, below the 2^-53
-// rounding unit of a float64 result.  The truncations (each -1/2 unit on average) are
-// re-centred by small constant offsets to within half a unit of 2^-58, far below the
-// systematic error that the float64 weights themselves put on mass conservation.
-//
-// Range.  The path is taken for sites with 2^-7 <= f_i 2^e_s < 8 for all i,
-// 0 < omega rho < 3, |c u_s,x| and |c u_s,y| below 0.15 (so |s| < 0.6) and
-// |T_s - 1| < 0.25; then every intermediate stays inside its format.  All other sites (and
-// NaNs) take the float64 collision of collide_site, so results never depend on the range.
+// Compile-time constants of the fixed-point collision (site_fix64.cuh, adjoint_fix64.cuh): the
+// shells' scales, their weights as correctly rounded fixed-point numbers, and the table of opposite
+// pairs.
 #pragma once
 #include "collide_fp64.cuh"
 #include "fixed64.cuh"
@@ -130,47 +105,5 @@ static __constant__ PairFix c_pair_fix[NPAIR + 1] = {
     LBM_PAIR_FIX(10), LBM_PAIR_FIX(11), LBM_PAIR_FIX(12), LBM_PAIR_FIX(13), LBM_PAIR_FIX(14),
     LBM_PAIR_FIX(15), LBM_PAIR_FIX(16), LBM_PAIR_FIX(17), LBM_PAIR_FIX(18)};
 #undef LBM_PAIR_FIX
-
-// The Hermite coefficients of C0 = a00 + a01 q + a02 q^2, C1 = a10 + a11 q, C2 = a20 + a21 q
-// (collide_fp64.cuh) in fixed point, from X1 = c u_s,x and Y1 = c u_s,y (63 fraction bits)
-// and t = T_s - 1, each with the fraction bits (in brackets) that its size allows in the
-// range of the fixed-point path (|X1|, |Y1| < 0.15, |t| < 0.25):
-//   a00 = 1 - U/2 - t + U^2/8 + tU + t^2 [61]   a01 = t/2 - tU/4 - t^2 [65]   a02 = t^2/8 [69]
-//   a10 = 1 - U/2 - 2t [62]   a11 = t/2 [65]   a20 = 1/2 - U/4 - 3t/2 [63]   a21 = t/4 [66]
-// with U = |u_s|^2 = (Ux^2 + Uy^2) / c^2 [62]; a21 is the same integer as a11.
-struct HermiteFix {
-  long long U62, t63, a00, a01, a02, a10, a11, a20;
-};
-
-__device__ __forceinline__ HermiteFix hermite_fix(long long X1, long long Y1, double t) {
-  bool unused = false;
-  HermiteFix h;
-  h.t63 = fx_from_double(t, 63, 64, unused);
-  const unsigned long long ax = (unsigned long long)(X1 < 0 ? -X1 : X1), ay = (unsigned long long)(Y1 < 0 ? -Y1 : Y1);
-  h.U62 = (long long)fx_umulhi(fx_umulhi(ax, ax) + fx_umulhi(ay, ay), kInvC2);
-  const unsigned long long at = (unsigned long long)(h.t63 < 0 ? -h.t63 : h.t63);
-  const long long tU = fx_mulhi_su(h.t63, (unsigned long long)h.U62);                             // 61
-  const long long t2 = (long long)fx_umulhi(at, at);                                                // 62
-  const long long U2 = (long long)fx_umulhi((unsigned long long)h.U62, (unsigned long long)h.U62);  // 60
-  h.a00 = (1LL << 61) - (h.U62 >> 2) - (h.t63 >> 2) + (U2 >> 2) + tU + (t2 >> 1);
-  h.a01 = h.t63 * 2 - tU * 4 - t2 * 8;
-  h.a02 = t2 * 16;
-  h.a10 = (1LL << 62) - (h.U62 >> 1) - h.t63;
-  h.a11 = h.t63 * 2;
-  h.a20 = (1LL << 62) - (h.U62 >> 1) - h.t63 - (h.t63 >> 1);
-  return h;
-}
-
-// Positive float64 values order like their bit patterns.
-constexpr long long kBitsR = 0x4008000000000000LL;  // 3.0
-constexpr long long kBitsU = 0x3FC3333333333333LL;  // 0.15
-constexpr long long kBitsT = 0x3FD0000000000000LL;  // 0.25
-constexpr long long kAbs = 0x7FFFFFFFFFFFFFFFLL;
-
-__device__ __forceinline__ bool fixed_range_ok(const SiteScalars& v) {
-  const long long r = __double_as_longlong(v.R);
-  return r > 0 && r < kBitsR && (__double_as_longlong(v.Ux) & kAbs) < kBitsU &&
-         (__double_as_longlong(v.Uy) & kAbs) < kBitsU && (__double_as_longlong(v.t) & kAbs) < kBitsT;
-}
 
 }  // namespace d2q37

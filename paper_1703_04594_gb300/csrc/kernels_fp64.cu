@@ -205,17 +205,20 @@ __global__ void __launch_bounds__(256) k_reduce_sum(const double* __restrict__ p
 static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, (a.lx + 3) / 4); }
 static const dim3 kSiteBlock(32, 4);
 
-cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s) {
-  // warps per block: as many as fit a column without idle ones, 4 preferred
+ColumnLaunch column_launch(const StepArgs& a, int most) {
   const int strips = (a.ly + 31) / 32;
-  int w = 4;
-  for (int c = 4; c >= 2; --c)
-    if ((strips + c - 1) / c * c - strips < (strips + w - 1) / w * w - strips) w = c;
-  if (strips < w) w = strips;
-  const dim3 grid((strips + w - 1) / w, a.lx < 65535 ? a.lx : 65535, (a.lx + 65534) / 65535);
-  const size_t smem = (size_t)w * Q * 32 * sizeof(double);
-  if (a.periodic) k_step_fix64<true><<<grid, dim3(32, w), smem, s>>>(fin, fout, a);
-  else k_step_fix64<false><<<grid, dim3(32, w), smem, s>>>(fin, fout, a);
+  const auto idle = [&](int c) { return (strips + c - 1) / c * c - strips; };
+  int w = strips < most ? strips : most;
+  for (int c = w - 1; c >= 2; --c)
+    if (idle(c) < idle(w)) w = c;
+  return {dim3((strips + w - 1) / w, a.lx < 65535 ? a.lx : 65535, (a.lx + 65534) / 65535), w};
+}
+
+cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s) {
+  const ColumnLaunch c = column_launch(a);
+  const size_t smem = (size_t)c.warps * Q * 32 * sizeof(double);
+  if (a.periodic) k_step_fix64<true><<<c.grid, dim3(32, c.warps), smem, s>>>(fin, fout, a);
+  else k_step_fix64<false><<<c.grid, dim3(32, c.warps), smem, s>>>(fin, fout, a);
   return cudaGetLastError();
 }
 

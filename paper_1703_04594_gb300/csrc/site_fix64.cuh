@@ -52,9 +52,29 @@ __host__ __device__ __forceinline__ FxHalves fx_halves(long long a) {
   const unsigned lo = (unsigned)a;
   return FxHalves{(int)lo, (int)((unsigned)((unsigned long long)a >> 32) + (lo >> 31))};
 }
+// 32 x 32 -> 64 multiply(-add) of signed numbers, as the one instruction each is (from C++ sums of
+// widened products the compiler makes about twice the instructions).
+__host__ __device__ __forceinline__ long long fx_wide(int a, int b) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+#else
+  return (long long)a * b;
+#endif
+}
+__host__ __device__ __forceinline__ long long fx_wide(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
+  long long r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return (long long)a * b + c;
+#endif
+}
 __host__ __device__ __forceinline__ long long fx_smul(FxHalves a, FxHalves b) {
-  const long long t = (long long)a.h * b.l + (long long)a.l * b.h;
-  return (long long)a.h * b.h + (t >> 32);
+  const long long t = fx_wide(a.l, b.h, fx_wide(a.h, b.l));
+  return fx_wide(a.h, b.h, t >> 32);
 }
 __host__ __device__ __forceinline__ long long fx_smul(long long a, FxHalves b) { return fx_smul(fx_halves(a), b); }
 __host__ __device__ __forceinline__ long long fx_smul(long long a, long long b) {
@@ -117,6 +137,30 @@ __host__ __device__ constexpr int pop_index(int a, int b) {
     if (vx(i) == a && vy(i) == b) return i;
   return -1;
 }
+
+// The groups of four populations (a, b), (-a, -b), (a, -b), (-a, b), and for the axes (a, 0),
+// (-a, 0), (0, a), (0, -a), as tables for rolled loops.
+struct FixGroup {
+  int i, j;                               // first population of each opposite pair (the other is + 18)
+  int sh;                                 // e_s
+  FxHalves w;                             // w_s 2^e_s [63]
+  unsigned a, b, a2, b2, a3, b3, a4, b4;  // powers of a and b
+};
+#define LBM_FIX_GROUP(A, B, J)                                                                                      \
+  {                                                                                                               \
+    pop_index(A, B), J, shell_exp(shell_of_v2(A * A + B * B)), fx_halves_ct(kCw(shell_of_v2(A * A + B * B))), A, B, \
+        A *A, B *B, A *A *A, B *B *B, A *A *A *A, B *B *B *B                                                       \
+  }
+__host__ __device__ constexpr FxHalves fx_halves_ct(long long a) {
+  return FxHalves{(int)(unsigned)a, (int)((a >> 32) + ((unsigned)a >> 31))};
+}
+#define LBM_FIX_AXES                                                                               \
+  {LBM_FIX_GROUP(1, 0, pop_index(0, 1)), LBM_FIX_GROUP(2, 0, pop_index(0, 2)), LBM_FIX_GROUP(3, 0, pop_index(0, 3))}
+#define LBM_FIX_QUADS \
+  {LBM_FIX_GROUP(1, 1, pop_index(1, -1)), LBM_FIX_GROUP(2, 1, pop_index(2, -1)), LBM_FIX_GROUP(1, 2, pop_index(1, -2)), \
+   LBM_FIX_GROUP(2, 2, pop_index(2, -2)), LBM_FIX_GROUP(3, 1, pop_index(3, -1)), LBM_FIX_GROUP(1, 3, pop_index(1, -3))}
+static __constant__ FixGroup c_fix_axes[3] = LBM_FIX_AXES;
+static __constant__ FixGroup c_fix_quads[6] = LBM_FIX_QUADS;
 
 // ---- 1. populations to fixed point, and the moments ---------------------------------------------
 struct FixMoments {
@@ -192,12 +236,67 @@ __host__ __device__ __forceinline__ FixMoments fix_moments(Load&& load, Keep&& k
   return m;
 }
 
+// The same in loops over the tables above, for kernels whose code overflows the instruction cache
+// (about 150 more instructions executed, 400 fewer stored).
+template <class Load, class Keep>
+__host__ __device__ __forceinline__ FixMoments fix_moments_rolled(const FixGroup* axes, const FixGroup* quads, Load&& load, Keep&& keep) {
+  const double f0 = load(0);
+  const unsigned E0 = fx_hi_word(f0) >> 20;
+  const unsigned base = 4u - E0;
+  unsigned worst = 0;
+  const auto conv = [&](int i, int e, double f) {
+    const unsigned sh = (fx_hi_word(f) >> 20) + (base + (unsigned)e);
+    worst = worst > sh ? worst : sh;
+    const long long q = fx_from_double_shifted(f, sh);
+    keep(i, fx_halves(q));
+    return (unsigned long long)q;
+  };
+  FixMoments m;
+  m.kb = (int)((E0 - 1019u) << 20);
+  unsigned long long R = (conv(0, 2, f0) + 2) >> 2, E = 0, X = 0, Y = 0;
+#pragma unroll 1
+  for (int n = 0; n < 3; ++n) {
+    const FixGroup& g = axes[n];
+    const int e = g.sh;
+    const unsigned long long half = 1ull << (e - 1);
+    const double a = load(g.i), b = load(g.i + NPAIR), c = load(g.j), d = load(g.j + NPAIR);
+    const unsigned long long p = conv(g.i, e, a), q = conv(g.i + NPAIR, e, b), r = conv(g.j, e, c), s = conv(g.j + NPAIR, e, d);
+    const unsigned long long T = (p + q + r + s + half) >> e;
+    R += T;
+    E += g.a2 * T;
+    X += g.a * (unsigned long long)((long long)(p - q + half) >> e);
+    Y += g.a * (unsigned long long)((long long)(r - s + half) >> e);
+  }
+#pragma unroll 1
+  for (int n = 0; n < 6; ++n) {
+    const FixGroup& g = quads[n];
+    const int e = g.sh;
+    const unsigned long long half = 1ull << (e - 1);
+    const double a = load(g.i), b = load(g.i + NPAIR), c = load(g.j), dd = load(g.j + NPAIR);
+    const unsigned long long f1 = conv(g.i, e, a), f2 = conv(g.i + NPAIR, e, b), f3 = conv(g.j, e, c), f4 = conv(g.j + NPAIR, e, dd);
+    const unsigned long long T = (f1 + f2 + f3 + f4 + half) >> e;
+    const unsigned long long d = f1 - f2, h = f3 - f4;
+    R += T;
+    E += (g.a2 + g.b2) * T;
+    X += g.a * (unsigned long long)((long long)(d + h + half) >> e);
+    Y += g.b * (unsigned long long)((long long)(d - h + half) >> e);
+  }
+  m.R = (long long)R;
+  m.E = (long long)E;
+  m.X = (long long)X;
+  m.Y = (long long)Y;
+  m.ok = worst <= 8u && E0 - 128u <= 950u;
+  return m;
+}
+
 // ---- 2. site scalars ------------------------------------------------------------------------------
 struct FixScalars {
   long long R;         // omega rho 2^-k [61]
   long long X, Y;      // c u_s [64]
   long long XX, YY, U; // X^2, Y^2, |u_s|^2 [64]
   long long t;         // T_s - 1 [64]
+  long long X0, Y0;    // c u [64], before the gravity shift
+  long long e;         // (T - 1) + |u|^2 / 2 [60]
   bool ok;
 };
 
@@ -222,8 +321,8 @@ __host__ __device__ __forceinline__ long long fx_reciprocal(long long R) {
   const unsigned long long ph = (unsigned long long)rh * yh + (pl >> 32);  // [55]
   const long long e = (((1LL << 55) - (long long)ph) << 22) - (long long)((unsigned)pl >> 10);  // 1 - rho y [77]
   const int eh = (int)(e >> 32);                                                                  // [45]
-  const long long g = e + (((long long)eh * eh) >> 13);                                           // e + e^2 [77]
-  const long long d = (long long)(int)(g >> 32) * (int)yh + (long long)(((unsigned long long)(unsigned)g * yh) >> 32);
+  const long long g = e + (fx_wide(eh, eh) >> 13);                                           // e + e^2 [77]
+  const long long d = fx_wide((int)(g >> 32), (int)yh, (long long)(((unsigned long long)(unsigned)g * yh) >> 32));
   return ((long long)yh << 33) + ((d + (1LL << 11)) >> 12);  // y + y g, the latter [72] -> [60]
 }
 
@@ -239,7 +338,8 @@ __host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, 
             ((unsigned long long)(dev + (1LL << 60)) < (1ull << 61));
   const long long yc = fx_smul(fx_reciprocal(m.R) , fx_halves(kFxC2_62)) * 2;  // c^2 / rho [58] -> [59]
   const FxHalves y = fx_halves(yc);
-  const long long X = fx_smul(m.X << 5, y) + k.cgx, Y = fx_smul(m.Y << 5, y) + k.cgy;  // [60]
+  const long long X0 = fx_smul(m.X << 5, y), Y0 = fx_smul(m.Y << 5, y);  // [60]
+  const long long X = X0 + k.cgx, Y = Y0 + k.cgy;
   const long long e2 = fx_smul(dev << 3, y);  // 2 (T - 1) + |u|^2 [59], so half of it [60]
   ok = ok & ((unsigned long long)(X + (3LL << 57)) < (3ull << 58)) &
        ((unsigned long long)(Y + (3LL << 57)) < (3ull << 58));
@@ -257,6 +357,9 @@ __host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, 
   s.t = t << 4;
   s.R = fx_smul(m.R << 3, k.om);
   ok = ok & (s.R < (9LL << 58) / 5 * 8);
+  s.X0 = X0 << 4;
+  s.Y0 = Y0 << 4;
+  s.e = e2;
   s.ok = ok;
   return s;
 }
@@ -265,10 +368,12 @@ __host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, 
 // What the shifts and products below round off on average, put back in the even sum [58].
 constexpr long long kFixMean = 3;
 
-// `fixed(i)` returns the halves of f_i' [60]; `out(i, v, s)` takes f_i^{new} 2^(e_s - k) [57] of
-// population i (shell s).
-template <class Fixed, class Out>
-__host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, FxHalves om1, Fixed&& fixed, Out&& out) {
+// `io.at(i)` returns a handle h of population i's pair (i, i + NPAIR); `io.fixed(h, k)` returns the
+// halves of f' [60] and `io.put(h, k, v, s)` takes the new value 2^(e_s - k) [57] (shell s) of
+// population i + k NPAIR.  (Handles, so that a rolled loop over pairs carries addresses rather than
+// multiplying them out.)
+template <class Io>
+__host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, FxHalves om1, Io&& io) {
   const FxHalves Rh = fx_halves(v.R), th = fx_halves(v.t), Uh = fx_halves(v.U);
   const FxHalves xh = fx_halves(v.X), yh = fx_halves(v.Y), xxh = fx_halves(v.XX), yyh = fx_halves(v.YY);
   const long long Rt = fx_smul(th, Rh) * 2;                          // [62]
@@ -317,23 +422,25 @@ __host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, FxHalves
   // one result, w p + (1 - omega) f, from p = omega f^eq / w [58]: the cross terms of both
   // products share one sum (|p| < 25 2^58 with |w| < 0.6 2^63 in the outer shells, below
   // 2^61 in the others; |f|, |1 - omega| < 2^61: the sum stays below 2^63)
-  const auto emit = [&](int i, int s, long long pv) {
-    const FxHalves w = fx_halves(kCw(s)), p = fx_halves(pv), f = fixed(i);
-    const long long t = (long long)p.h * w.l + (long long)p.l * w.h + (long long)f.h * om1.l + (long long)f.l * om1.h;
-    out(i, (long long)p.h * w.h + (long long)f.h * om1.h + (t >> 32), s);
+  const auto emit = [&](auto at, int k, int s, long long pv) {
+    const FxHalves w = fx_halves(kCw(s)), p = fx_halves(pv), f = io.fixed(at, k);
+    const long long t = fx_wide(f.l, om1.h, fx_wide(f.h, om1.l, fx_wide(p.l, w.h, fx_wide(p.h, w.l))));
+    io.put(at, k, fx_wide(f.h, om1.h, fx_wide(p.h, w.h, t >> 32)), s);
   };
   // two opposite pairs (v, -v), p = P +- u, then M +- w; rolled, for the instruction cache
   const auto pairs = [&](int i, int j, int s, long long P, long long u, long long M, long long w) {
+    auto at = io.at(i);
+    const auto at_j = io.at(j);
 #pragma unroll 1
     for (int r = 0; r < 2; ++r) {
-      emit(i, s, P + u);
-      emit(i + NPAIR, s, P - u);
-      i = j;
+      emit(at, 0, s, P + u);
+      emit(at, 1, s, P - u);
+      at = at_j;
       P = M;
       u = w;
     }
   };
-  emit(0, 0, S0 - 2);  // its share of the sums' mean is less
+  emit(io.at(0), 0, 0, S0 - 2);  // its share of the sums' mean is less
   long long Sx[4], Sy[4], Ox[4], Oy[4];
   const auto tables = [&](int a) {
     Sx[a] = even(c20, c40, a);

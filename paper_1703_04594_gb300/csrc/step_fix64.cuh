@@ -15,14 +15,11 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Shared staging: one warp holds sf[i * 32 + lane] for its 32 sites.
 constexpr int kFixWarps = 4;  // warps per block (block = 32 x 4 threads)
 
-// The float64 collision of a staged site (its fixed-point forms converted back would not be
-// exact for sites out of range, so its values are gathered again).  Not inlined, so that its
-// 37 live float64 values do not weigh on the register allocation of the fixed-point path.
+// The pulled populations of one site, wall values included, loaded from global memory: for
+// sites that leave the fixed-point path, whose staged slots hold their fixed-point forms by then.
 template <bool PERIODIC, class Ld>
-__device__ __noinline__ void collide_site_reloaded(const double* __restrict__ fin, double* __restrict__ fout,
-                                                   const StepScalars& a, const StepWalls& w, int x, int yc,
-                                                   unsigned self) {
-  const Ld ld;
+__device__ __forceinline__ void gather_site(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
+                                            int x, int yc, double (&f)[Q], Ld ld) {
   const auto wall_density = [&](int i, int row) {  // of the source column of population i
     const double* src = fin + (long long)wrap_index(x - vx(i), a.lx) * a.pitch + row;
     double r = 0.0;
@@ -30,7 +27,6 @@ __device__ __noinline__ void collide_site_reloaded(const double* __restrict__ fi
     for (int j = 0; j < Q; ++j) r += ld(src + j * a.pop);
     return r;
   };
-  double f[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const double* src = fin + i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch;
@@ -39,6 +35,16 @@ __device__ __noinline__ void collide_site_reloaded(const double* __restrict__ fi
     else if (!PERIODIC && vy(i) < 0 && ys >= a.ly) f[i] = wall_density(i, a.ly - 1) * w.wall_t[i];
     else f[i] = ld(src + ys);
   }
+}
+
+// The float64 collision of such a site.  Not inlined, so that its 37 live float64 values do not
+// weigh on the register allocation of the fixed-point path.
+template <bool PERIODIC, class Ld>
+__device__ __noinline__ void collide_site_reloaded(const double* __restrict__ fin, double* __restrict__ fout,
+                                                   const StepScalars& a, const StepWalls& w, int x, int yc,
+                                                   unsigned self) {
+  double f[Q];
+  gather_site<PERIODIC>(fin, a, w, x, yc, f, Ld());
   collide_site(f, a.cc, [&](int i, double val) { __stcs(fout + i * a.pop + self, val); });
 }
 
@@ -69,24 +75,18 @@ __device__ __forceinline__ bool fix64_wall_strip(const StepScalars& a, int y0) {
   return !PERIODIC && (y0 < 3 || y0 + 32 > a.ly - 3);
 }
 
+// The pull-gather of a strip into its slots sf[i * 32] (sf: the lane's first slot), walls
+// included; yc is the lane's row clamped into the lattice.  Asynchronous copies when Ld caches in
+// L1, waited for here.  In a block along one column the addresses are uniform but for the lane's row.
 template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin, double* __restrict__ fout,
-                                                 const StepScalars& a, const StepWalls& w, int x, int y0, Ld ld,
-                                                 double* __restrict__ sf) {
-  const int lane = threadIdx.x & 31;
-  const int y = y0 + lane;
-  const bool active = y < a.ly;
-  const int yc = active ? y : a.ly - 1;
-  sf += lane;
-  unsigned off[7];  // column x_s, row yc within a population plane (planes < 2^32 elements)
-#pragma unroll
-  for (int d = 0; d < 7; ++d) off[d] = (unsigned)((long long)wrap_index(x - (d - 3), a.lx) * a.pitch + yc);
+__device__ __forceinline__ void stage_strip(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
+                                            int x, int y0, int yc, double* __restrict__ sf, Ld ld) {
   const bool wall = fix64_wall_strip<PERIODIC>(a, y0);
   if (wall || PERIODIC) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       const int ys = PERIODIC ? wrap_index(yc - vy(i), a.ly) : min(max(yc - vy(i), 0), a.ly - 1);
-      const double* src = fin + i * a.pop + (off[vx(i) + 3] - yc + ys);
+      const double* src = fin + (i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch) + (unsigned)ys;
       if (Ld::kL1) cp_async8(sf + i * 32, src);
       else sf[i * 32] = ld(src);
     }
@@ -122,6 +122,35 @@ __device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin,
       }
     }
   }
+}
+
+// The relaxation's view of a site: its slots, and its column of the output state.
+struct StepIo {
+  const FxHalves* slots;
+  double* out;
+  long long pop;
+  int kb;
+  struct At {
+    const FxHalves* f;
+    double* out;
+  };
+  __device__ __forceinline__ At at(int i) const { return At{slots + i * 32, out + i * pop}; }
+  __device__ __forceinline__ FxHalves fixed(At h, int k) const { return h.f[k * (NPAIR * 32)]; }
+  __device__ __forceinline__ void put(At h, int k, long long v, int s) const {
+    __stcs(k ? h.out + NPAIR * pop : h.out, fx_lower_exponent(v, ((57 + shell_exp(s)) << 20) - kb));
+  }
+};
+
+template <bool PERIODIC, class Ld>
+__device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin, double* __restrict__ fout,
+                                                 const StepScalars& a, const StepWalls& w, int x, int y0, Ld ld,
+                                                 double* __restrict__ sf) {
+  const int lane = threadIdx.x & 31;
+  const int y = y0 + lane;
+  const bool active = y < a.ly;
+  const int yc = active ? y : a.ly - 1;
+  sf += lane;
+  stage_strip<PERIODIC>(fin, a, w, x, y0, yc, sf, ld);
   if (!active) return;
   FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);  // the same slots, as fixed point
   const FixMoments m = fix_moments([&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
@@ -131,10 +160,7 @@ __device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin,
     collide_site_reloaded<PERIODIC, Ld>(fin, fout, a, w, x, yc, self);
     return;
   }
-  fix_relax(v, a.fx.om1, [&](int i) { return sx[i * 32]; }, [&](int i, long long X, int s) {
-    double* dst = fout + (i * a.pop + (long long)x * a.pitch) + (unsigned)y;
-    __stcs(dst, fx_lower_exponent(X, ((57 + shell_exp(s)) << 20) - m.kb));
-  });
+  fix_relax(v, a.fx.om1, StepIo{sx, fout + (long long)x * a.pitch + (unsigned)y, a.pop, m.kb});
 }
 
 }  // namespace d2q37

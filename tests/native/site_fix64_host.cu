@@ -10,6 +10,15 @@
 
 using namespace d2q37;
 
+struct Io {
+  const FxHalves* f;
+  double* r;
+  int scale;
+  int at(int i) const { return i; }
+  FxHalves fixed(int i, int k) const { return f[i + k * NPAIR]; }
+  void put(int i, int k, long long v, int s) const { r[i + k * NPAIR] = std::ldexp((double)v, scale - 57 - shell_exp(s)); }
+};
+
 static bool read_double(double& v) {
   unsigned long long bits;
   if (std::scanf("%llx", &bits) != 1) return false;
@@ -31,8 +40,7 @@ int main() {
       continue;
     }
     const int scale = m.kb / (1 << 20);
-    fix_relax(v, k.om1, [&](int i) { return fixed[i]; },
-              [&](int i, long long x, int s) { r[i] = std::ldexp((double)x, scale - 57 - shell_exp(s)); });
+    fix_relax(v, k.om1, Io{fixed, r, scale});
     std::printf("1 %d", scale);
     for (int i = 0; i < Q; ++i) {
       unsigned long long bits;

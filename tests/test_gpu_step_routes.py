@@ -1,11 +1,14 @@
-"""The fused float64 step (fixed-point collision in range, float64 elsewhere) against the separate
+"""The fixed-point routes of the float64 step and its adjoint.
+
+The fused float64 step (fixed-point collision in range, float64 elsewhere) against the separate
 kernels (float64 throughout), over sizes that give every block and strip shape, both relaxation
 signs, both y boundaries, and states of which some sites leave the fixed-point range."""
 import pytest
 import torch
 
 from paper_1703_04594_gb300 import lbm
-from tests.gpu_util import device_init, require_gpu, rt_fields
+from tests.gpu_util import device_init, require_gpu, rt_fields, to_host
+from tests.test_gpu_adjoint import oracle_vjp, reach_max
 
 pytestmark = pytest.mark.gpu
 
@@ -29,7 +32,47 @@ def test_fused_step_equals_the_separate_kernels(lx, ly, bc, tau, drift, hot):
     got = torch.full_like(f, -7.0)
     lbm.step(p, f, got)
     a, b = got[:, :, :ly], want[:, :, :ly]
-    # both round every population within a few units of its shell's scale: the populations of
-    # these states stay above a hundredth of it, and a float64 collision's error is ~1e-14 of it
-    assert float(((a - b).abs() / b.abs().clamp_min(1e-7)).max()) <= 2e-12
+    # errors on the scale of the population's shell, w_i rho (an over-relaxed population may itself
+    # cancel to nothing): a float64 collision's stays below ~1e-13 of it
+    w = torch.tensor(lbm.model()[1], dtype=torch.float64, device="cuda")[:, None, None]
+    assert float(((a - b).abs() / (w * b.sum(0))).max()) <= 2e-12
     assert bool((got[:, :, ly:] == -7.0).all())        # the padding is not written
+
+
+@pytest.mark.parametrize("lx,ly", [(5, 31), (4, 32), (7, 33), (6, 97), (4, 161), (5, 64)])
+@pytest.mark.parametrize("bc", [lbm.BC_WALLS, lbm.BC_PERIODIC_Y])
+@pytest.mark.parametrize("tau,drift,heat,scale", [(0.7, 0.02, 1.0, 1.0), (1.4, 0.2, 1.25, 1e-9), (0.9, 0.28, 1.3, 1e3),
+                                                  (0.8, 0.02, 1.0, 1e20), (0.8, 0.02, 1.0, 1e-290)])
+def test_adjoint_step_on_both_routes(lx, ly, bc, tau, drift, heat, scale):
+    """The adjoint step against autograd through the oracle's step, with sites on both sides of the
+    fixed-point range (speeds and temperatures beyond it, lambda above and below its block range),
+    over sizes that give every block and strip shape.  The bar is that of the adjoint's own
+    per-element test, 1e-13 of the largest lambda within reach."""
+    require_gpu()
+    p = lbm.Params(lx, ly, tau=tau, gx=1e-4, gy=-2e-4, bc=bc)
+    rho, ux, uy, T = rt_fields(p, seed=5)
+    x = torch.arange(lx, dtype=torch.float64)[:, None]
+    f = device_init(p, [t.contiguous() for t in (rho, ux + drift * (1 + 0.3 * torch.cos(x)), uy, T * heat)])
+    g = torch.Generator().manual_seed(17)
+    lam = torch.randn(37, lx, ly, dtype=torch.float64, generator=g)
+    lam_dev = torch.zeros_like(f)
+    lam_dev[:, :, :ly] = lam.cuda() * scale
+    lam_n = torch.full_like(f, -7.0)
+    dtau = torch.zeros((), dtype=torch.float64, device="cuda")
+    lbm.adjoint_step(p, f, lam_dev, lam_n, dtau, lbm.adjoint_work(p))
+    want, want_tau = oracle_vjp(p, to_host(p, f), lam)
+    got = to_host(p, lam_n) / scale
+    assert float(((got - want).abs() / reach_max(lam.abs().amax(0), bc)[None]).max()) <= 1e-13
+    assert abs(float(dtau) / scale - want_tau) <= 1e-10 * max(abs(want_tau), float(lam.abs().sum()) * 1e-3)
+    assert bool((lam_n[:, :, ly:] == -7.0).all())
+
+
+def test_adjoint_of_zero_is_zero():
+    require_gpu()
+    p = lbm.Params(6, 97, tau=0.7, gx=1e-4)
+    f = device_init(p, rt_fields(p, seed=5))
+    lam = torch.zeros_like(f)
+    lam_n = torch.full_like(f, 3.0)
+    dtau = torch.zeros((), dtype=torch.float64, device="cuda")
+    lbm.adjoint_step(p, f, lam, lam_n, dtau, lbm.adjoint_work(p))
+    assert bool((lam_n[:, :, :97] == 0).all()) and float(dtau) == 0.0

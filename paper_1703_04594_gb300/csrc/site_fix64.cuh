@@ -364,6 +364,29 @@ __host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, 
   return s;
 }
 
+// The scalars of an equilibrium with the given fields (omega = 1): rho in [1/4, 1/2) 2^k, with k << 20
+// in kb.  v.ok as for a collision.
+__host__ __device__ __forceinline__ FixScalars fix_scalars_of(double rho, double ux, double uy, double T, int& kb) {
+  FixScalars s;
+  const unsigned E = fx_hi_word(rho) >> 20;  // rho 2^-k in [1/4, 1/2): k = E - 1021
+  kb = (int)((E - 1021u) << 20);
+  s.R = (long long)((((unsigned long long)((fx_hi_word(rho) & 0xFFFFFu) | 0x100000u) << 32) | fx_lo_word(rho)) << 7);
+  const double X = C * ux, Y = C * uy, t = T - 1.0;
+  // positive doubles order like their bit patterns
+  const auto below = [](double v, unsigned hi) { return (fx_hi_word(v) & 0x7fffffffu) < hi; };
+  s.ok = E - 128u <= 950u && below(X, 0x3FD80000u) && below(Y, 0x3FD80000u) && below(t, 0x3FD99999u);  // 3/8, 3/8, 2/5
+  bool unused = false;
+  s.X = fx_from_double(s.ok ? X : 0.0, 64, 64, unused);
+  s.Y = fx_from_double(s.ok ? Y : 0.0, 64, 64, unused);
+  s.t = fx_from_double(s.ok ? t : 0.0, 64, 64, unused);
+  const FxHalves xh = fx_halves(s.X), yh = fx_halves(s.Y);
+  s.XX = fx_smul(xh, xh);
+  s.YY = fx_smul(yh, yh);
+  s.U = fx_smul(s.XX + s.YY, fx_halves(kFxInvC2_63)) * 2;
+  s.X0 = s.Y0 = s.e = 0;
+  return s;
+}
+
 // ---- 3. coefficients, and the populations -------------------------------------------------------
 // What the shifts and products below round off on average, put back in the even sum [58].
 constexpr long long kFixMean = 3;
@@ -372,7 +395,8 @@ constexpr long long kFixMean = 3;
 // halves of f' [60] and `io.put(h, k, v, s)` takes the new value 2^(e_s - k) [57] (shell s) of
 // population i + k NPAIR.  (Handles, so that a rolled loop over pairs carries addresses rather than
 // multiplying them out.)
-template <class Io>
+// PLAIN: no population to relax, the results are omega f^eq alone (io.fixed is not called).
+template <bool PLAIN = false, class Io>
 __host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, FxHalves om1, Io&& io) {
   const FxHalves Rh = fx_halves(v.R), th = fx_halves(v.t), Uh = fx_halves(v.U);
   const FxHalves xh = fx_halves(v.X), yh = fx_halves(v.Y), xxh = fx_halves(v.XX), yyh = fx_halves(v.YY);
@@ -423,7 +447,12 @@ __host__ __device__ __forceinline__ void fix_relax(const FixScalars& v, FxHalves
   // products share one sum (|p| < 25 2^58 with |w| < 0.6 2^63 in the outer shells, below
   // 2^61 in the others; |f|, |1 - omega| < 2^61: the sum stays below 2^63)
   const auto emit = [&](auto at, int k, int s, long long pv) {
-    const FxHalves w = fx_halves(kCw(s)), p = fx_halves(pv), f = io.fixed(at, k);
+    const FxHalves w = fx_halves(kCw(s)), p = fx_halves(pv);
+    if constexpr (PLAIN) {
+      io.put(at, k, fx_smul(p, w), s);
+      return;
+    }
+    const FxHalves f = io.fixed(at, k);
     const long long t = fx_wide(f.l, om1.h, fx_wide(f.h, om1.l, fx_wide(p.l, w.h, fx_wide(p.h, w.l))));
     io.put(at, k, fx_wide(f.h, om1.h, fx_wide(p.h, w.h, t >> 32)), s);
   };

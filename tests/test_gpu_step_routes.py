@@ -6,6 +6,7 @@ signs, both y boundaries, and states of which some sites leave the fixed-point r
 import pytest
 import torch
 
+from oracle import lbm as OL
 from paper_1703_04594_gb300 import lbm
 from tests.gpu_util import device_init, require_gpu, rt_fields, to_host
 from tests.test_gpu_adjoint import oracle_vjp, reach_max
@@ -76,3 +77,27 @@ def test_adjoint_of_zero_is_zero():
     dtau = torch.zeros((), dtype=torch.float64, device="cuda")
     lbm.adjoint_step(p, f, lam, lam_n, dtau, lbm.adjoint_work(p))
     assert bool((lam_n[:, :, :97] == 0).all()) and float(dtau) == 0.0
+
+
+@pytest.mark.parametrize("lx,ly", [(4, 6), (5, 33), (9, 64), (70, 131)])
+@pytest.mark.parametrize("rho0", [1.0, 1600.0, 1e-3])
+def test_initial_state_and_fields_on_both_routes(lx, ly, rho0):
+    """lbm_init, lbm_moments and lbm_kinetic_energy on fields of which some leave the fixed-point range
+    (|u| to 0.45, T from 0.5 to 1.5): the state against the oracle's equilibrium at 1e-13 of its
+    shell's scale, the fields of a state back at 1e-12 (the parity tests' bar)."""
+    require_gpu()
+    p = lbm.Params(lx, ly)
+    g = torch.Generator().manual_seed(23)
+    rho = rho0 * (0.5 + torch.rand(lx, ly, dtype=torch.float64, generator=g))
+    ux, uy = ((torch.rand(2, lx, ly, dtype=torch.float64, generator=g) - 0.5) * 0.9).unbind(0)
+    T = 0.5 + torch.rand(lx, ly, dtype=torch.float64, generator=g)
+    fields = [t.contiguous() for t in (rho, ux, uy, T)]
+    f = device_init(p, fields)
+    host = to_host(p, f)
+    w = torch.tensor(lbm.model()[1], dtype=torch.float64)[:, None, None]
+    assert float(((host - OL.init_equilibrium(*fields)).abs() / (w * rho)).max()) <= 1e-13
+    want = OL.fields(host)
+    for a, b in zip(lbm.moments(p, f), want):
+        assert float((a.cpu() - b).abs().max()) <= 1e-12 * float(b.abs().max())
+    ke = float(OL.kinetic_energy(host))
+    assert abs(float(lbm.kinetic_energy(p, f)) - ke) <= 1e-12 * ke

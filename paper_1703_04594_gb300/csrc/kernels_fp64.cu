@@ -148,22 +148,15 @@ __global__ void __launch_bounds__(128, 4) k_init_fp64(const double* __restrict__
   else init_site_float64(r, u, v, t, dst, a.pop);
 }
 
-__device__ __forceinline__ void site_fields(const double (&f)[Q], double& rho, double& ux, double& uy, double& T) {
+// The fields of a site in float64, for sites outside the fixed-point range.
+__device__ __noinline__ void site_fields_float64(const double* __restrict__ f, long long pop, double& rho, double& ux,
+                                                 double& uy, double& T) {
   double jx, jy, e;
-  moments_int(f, rho, jx, jy, e);
+  moments_float64([&](int i) { return __ldg(f + i * pop); }, rho, jx, jy, e);
   const double inv_rho = 1.0 / rho;
   ux = C * jx * inv_rho;
   uy = C * jy * inv_rho;
   T = (C2 * e * inv_rho - fma(ux, ux, uy * uy)) / D;
-}
-
-// The same loaded from memory, for sites outside the fixed-point range.
-__device__ __noinline__ void site_fields_reloaded(const double* __restrict__ f, long long pop, double& rho, double& ux,
-                                                  double& uy, double& T) {
-  double g[Q];
-#pragma unroll
-  for (int i = 0; i < Q; ++i) g[i] = __ldg(f + i * pop);
-  site_fields(g, rho, ux, uy, T);
 }
 
 // rho, c u and T of a site by the fixed-point moments and scalars of site_fix64.cuh: exact sums, four
@@ -200,7 +193,7 @@ __global__ void __launch_bounds__(128) k_moments_fp64(const double* __restrict__
     uy[fi] = cy * (1.0 / C);
     T[fi] = t;
   } else {
-    site_fields_reloaded(src, a.pop, rho[fi], ux[fi], uy[fi], T[fi]);
+    site_fields_float64(src, a.pop, rho[fi], ux[fi], uy[fi], T[fi]);
   }
 }
 
@@ -216,7 +209,7 @@ __global__ void __launch_bounds__(128) k_ke_partial_fp64(const double* __restric
     if (site_fields_fix(src, a.pop, rho, ux, uy, T)) {
       ke = (0.5 / C2) * (rho * fma(ux, ux, uy * uy));
     } else {
-      site_fields_reloaded(src, a.pop, rho, ux, uy, T);
+      site_fields_float64(src, a.pop, rho, ux, uy, T);
       ke = 0.5 * rho * fma(ux, ux, uy * uy);
     }
   }

@@ -318,28 +318,26 @@ __device__ __forceinline__ void collide_site_fp32(float (&g)[Q], const StepScala
   }
 }
 
-// Wall deviations sum_j g_j at (x_s, 0) and (x_s, ly-1) of the seven source columns
-// (lanes 0..6 bottom, 8..14 top), summed in float64, broadcast to the warp.
+// Wall deviation sum_j g_j at (x_s, row) of the seven source columns, summed in float64: lane l takes
+// every fourth population of column l % 8, and two shuffles add the four parts (the same value in the
+// column's four lanes).
 template <class Ld>
-__device__ __forceinline__ void wall_drho(const float* __restrict__ fin, int x, const StepScalars& a, float (&rb)[7],
-                                          float (&rt)[7], Ld ld) {
+__device__ __forceinline__ float wall_drho_lane(const float* __restrict__ fin, int x, const StepScalars& a, int row, Ld ld) {
   const int lane = threadIdx.x & 31;
-  const int d = lane & 7;
-  const int row = lane < 8 ? 0 : a.ly - 1;
+  const int d = lane & 7, part = lane >> 3;
   double r = 0.0;
-  if (d < 7 && lane < 16) {
+  if (d < 7) {
     const float* src = fin + (long long)wrap_index(x - (d - 3), a.lx) * a.pitch + row;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) r += (double)ld(src + i * a.pop);
+    for (int n = 0; n < 10; ++n) {
+      const int i = 4 * n + part;
+      if (i < Q) r += (double)ld(src + i * a.pop);
+    }
   }
-  const float rf = (float)r;
-#pragma unroll
-  for (int j = 0; j < 7; ++j) {
-    rb[j] = __shfl_sync(0xffffffffu, rf, j);
-    rt[j] = __shfl_sync(0xffffffffu, rf, 8 + j);
-  }
+  r += __shfl_xor_sync(0xffffffffu, r, 8);
+  r += __shfl_xor_sync(0xffffffffu, r, 16);
+  return (float)r;
 }
-
 
 // One warp-strip of the FP32 shifted step (see step_fp64.cuh for the strip contract).
 // SCALED: the lattice's reference density is 2 or more (see moments_fix); CONSERVE: the
@@ -356,15 +354,29 @@ __device__ __forceinline__ void step_strip_fp32(const float* __restrict__ fin, f
   float g[Q];
   const bool wall_warp = !PERIODIC && (y0 < 3 || y0 + 32 > a.ly - 3);
   if (wall_warp) {
-    float rb[7], rt[7];
-    wall_drho(fin, x, a, rb, rt, ld);
+    // clamped rows, then the ghost values over them; each wall only where the strip reaches it
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const int ys = yc - vy(i);
-      const float* src = fin + i * a.pop + col[vx(i) + 3];
-      if (vy(i) > 0 && ys < 0) g[i] = fmaf(rb[vx(i) + 3], w.gb_scale[i], w.gb_bias[i]);
-      else if (vy(i) < 0 && ys >= a.ly) g[i] = fmaf(rt[vx(i) + 3], w.gt_scale[i], w.gt_bias[i]);
-      else g[i] = ld(src + ys);
+    for (int i = 0; i < Q; ++i)
+      g[i] = ld(fin + i * a.pop + col[vx(i) + 3] + min(max(yc - vy(i), 0), a.ly - 1));
+    if (y0 < 3) {
+      const float b = wall_drho_lane(fin, x, a, 0, ld);
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        if (vy(i) > 0) {
+          const float r = __shfl_sync(0xffffffffu, b, vx(i) + 3);
+          if (yc < vy(i)) g[i] = fmaf(r, w.gb_scale[i], w.gb_bias[i]);
+        }
+      }
+    }
+    if (y0 + 32 > a.ly - 3) {
+      const float t = wall_drho_lane(fin, x, a, a.ly - 1, ld);
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        if (vy(i) < 0) {
+          const float r = __shfl_sync(0xffffffffu, t, vx(i) + 3);
+          if (yc >= a.ly + vy(i)) g[i] = fmaf(r, w.gt_scale[i], w.gt_bias[i]);
+        }
+      }
     }
   } else if (PERIODIC) {
 #pragma unroll

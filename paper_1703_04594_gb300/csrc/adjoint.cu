@@ -244,8 +244,8 @@ struct AdjIo {
   }
 };
 
-// Step 1: per-site adjoint of the collision with the transposed propagate as its store.  Blocks run
-// along a column (column_launch).  `side` holds 2 * lx * kGhostSlots doubles: the bottom slots of
+// Step 1: per-site adjoint of the collision with the transposed propagate as its store.
+// (block 32 x 4 as the forward kernels).  `side` holds 2 * lx * kGhostSlots doubles: the bottom slots of
 // every column, then the top slots.  The strip's pull-gather is staged in shared memory (9.5 KB
 // per warp); a slot holds f~_i, then its fixed-point form, then mu_i's, then the output.  What bounds
 // it: 6.1 k instructions per strip, more code than the instruction cache holds (hit rate 83 %), and
@@ -259,10 +259,9 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
                                                      const double* __restrict__ lam_next, double* __restrict__ lam_out,
                                                      double* __restrict__ side, double* __restrict__ dtau_part,
                                                      StepArgs a, AdjConsts k) {
-  const int x = blockIdx.y + blockIdx.z * 65535;
-  if (x >= a.lx) return;  // uniform per block
-  const int y0 = (blockIdx.x * blockDim.y + threadIdx.y) * 32;
-  if (y0 >= a.ly) return;  // uniform per warp
+  const int x = blockIdx.y * 4 + threadIdx.y;
+  if (x >= a.lx) return;  // uniform per warp
+  const int y0 = blockIdx.x * 32;
   const int y = y0 + threadIdx.x;
   const bool active = y < a.ly;  // the other lanes work on the last row's data and store nothing
   const int yc = active ? y : a.ly - 1;
@@ -419,9 +418,8 @@ long long adjoint_side_count(const StepArgs& a) { return 2LL * a.lx * kGhostSlot
 
 cudaError_t launch_adjoint_step(const double* fin, const double* lam_next, double* lam, double* side, double* part,
                                 double* dtau, const StepArgs& a, double tau, double gx, double gy, cudaStream_t s) {
-  const ColumnLaunch c = column_launch(a);
-  const dim3 blk(32, c.warps);
-  const size_t smem = (size_t)c.warps * Q * 32 * sizeof(double);
+  const dim3 blk(32, 4);
+  constexpr size_t smem = 4 * Q * 32 * sizeof(double);
   AdjConsts k;
   k.tau = tau;
   k.om = 1.0 / tau;
@@ -438,9 +436,9 @@ cudaError_t launch_adjoint_step(const double* fin, const double* lam_next, doubl
   k.dts_dtau = (1.0 - 2.0 * tau) * gg / D;
   k.fx = make_adj_fix_consts(tau, gx, gy);
   if (a.periodic) {
-    k_adj_collide<true><<<c.grid, blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
+    k_adj_collide<true><<<site_grid(a), blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
   } else {
-    k_adj_collide<false><<<c.grid, blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
+    k_adj_collide<false><<<site_grid(a), blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
     const long long items = 2LL * a.lx * Q;  // (column, wall, population), plus one block for the dtau sum
     k_adj_walls<<<(unsigned)((items + 255) / 256) + 1, 256, 0, s>>>(side, lam, a, part, adjoint_partial_count(a),
                                                                     dtau);

@@ -57,15 +57,6 @@ struct StepWalls {
 // Everything a site kernel needs, passed by value as the kernel parameter.
 struct StepArgs : StepScalars, StepWalls {};
 
-// Launch shape of the kernels whose blocks run along one column, one warp per strip of 32 rows:
-// grid (strips / warps, columns, columns / 65535), block (32, warps).  As many warps as split the
-// column's strips with the fewest idle ones, 4 preferred (5 such blocks share an SM).
-struct ColumnLaunch {
-  dim3 grid;
-  int warps;
-};
-ColumnLaunch column_launch(const StepArgs& a, int most = 4);
-
 cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s);
 cudaError_t launch_propagate_fp64(const double* fin, double* ftmp, const StepArgs& a, cudaStream_t s);
 cudaError_t launch_propagate_push_fp64(const double* fin, double* ftmp, const StepArgs& a, cudaStream_t s);

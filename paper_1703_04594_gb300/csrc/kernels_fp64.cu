@@ -37,9 +37,9 @@ extern __shared__ double step_staged[];  // 37 populations x 32 sites per warp
 template <bool PERIODIC>
 __global__ void __launch_bounds__(128, LBM_FIX64_MIN_BLOCKS) k_step_fix64(const double* __restrict__ fin,
                                                                          double* __restrict__ fout, StepArgs a) {
-  const int x = blockIdx.y + blockIdx.z * 65535, y0 = (blockIdx.x * blockDim.y + threadIdx.y) * 32;
-  if (x >= a.lx || y0 >= a.ly) return;  // uniform per warp
-  step_strip_fix64<PERIODIC>(fin, fout, a, a, x, y0, LdReadOnly(), step_staged + threadIdx.y * (Q * 32));
+  const int x = blockIdx.y * 4 + threadIdx.y;
+  if (x >= a.lx) return;  // uniform per warp
+  step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly(), step_staged + threadIdx.y * (Q * 32));
 }
 
 // ---------------------------------------------------------------------------------------
@@ -251,20 +251,10 @@ __global__ void __launch_bounds__(1024) k_reduce_sum(const double* __restrict__ 
 static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, (a.lx + 3) / 4); }
 static const dim3 kSiteBlock(32, 4);
 
-ColumnLaunch column_launch(const StepArgs& a, int most) {
-  const int strips = (a.ly + 31) / 32;
-  const auto idle = [&](int c) { return (strips + c - 1) / c * c - strips; };
-  int w = strips < most ? strips : most;
-  for (int c = w - 1; c >= 2; --c)
-    if (idle(c) < idle(w)) w = c;
-  return {dim3((strips + w - 1) / w, a.lx < 65535 ? a.lx : 65535, (a.lx + 65534) / 65535), w};
-}
-
 cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s) {
-  const ColumnLaunch c = column_launch(a);
-  const size_t smem = (size_t)c.warps * Q * 32 * sizeof(double);
-  if (a.periodic) k_step_fix64<true><<<c.grid, dim3(32, c.warps), smem, s>>>(fin, fout, a);
-  else k_step_fix64<false><<<c.grid, dim3(32, c.warps), smem, s>>>(fin, fout, a);
+  constexpr size_t smem = 4 * Q * 32 * sizeof(double);
+  if (a.periodic) k_step_fix64<true><<<site_grid(a), kSiteBlock, smem, s>>>(fin, fout, a);
+  else k_step_fix64<false><<<site_grid(a), kSiteBlock, smem, s>>>(fin, fout, a);
   return cudaGetLastError();
 }
 

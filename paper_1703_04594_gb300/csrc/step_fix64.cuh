@@ -77,7 +77,7 @@ __device__ __forceinline__ bool fix64_wall_strip(const StepScalars& a, int y0) {
 
 // The pull-gather of a strip into its slots sf[i * 32] (sf: the lane's first slot), walls
 // included; yc is the lane's row clamped into the lattice.  Asynchronous copies when Ld caches in
-// L1, waited for here.  In a block along one column the addresses are uniform but for the lane's row.
+// L1, waited for here.
 template <bool PERIODIC, class Ld>
 __device__ __forceinline__ void stage_strip(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
                                             int x, int y0, int yc, double* __restrict__ sf, Ld ld) {

@@ -259,6 +259,7 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
                                                      const double* __restrict__ lam_next, double* __restrict__ lam_out,
                                                      double* __restrict__ side, double* __restrict__ dtau_part,
                                                      StepArgs a, AdjConsts k) {
+  pdl_wait();
   const int x = blockIdx.y * 4 + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
   const int y0 = blockIdx.x * 32;
@@ -342,6 +343,7 @@ __device__ __forceinline__ void reduce_add_256(const double* __restrict__ part, 
 __global__ void __launch_bounds__(256) k_adj_walls(const double* __restrict__ side, double* __restrict__ lam,
                                                    StepArgs a, const double* __restrict__ part, long long n_part,
                                                    double* dtau) {
+  pdl_wait();
   if (blockIdx.x == gridDim.x - 1) {  // uniform per block
     reduce_add_256(part, n_part, dtau);
     return;
@@ -435,17 +437,16 @@ cudaError_t launch_adjoint_step(const double* fin, const double* lam_next, doubl
   k.gy = gy;
   k.dts_dtau = (1.0 - 2.0 * tau) * gg / D;
   k.fx = make_adj_fix_consts(tau, gx, gy);
+  const cudaError_t e = launch_dependent(a.periodic ? k_adj_collide<true> : k_adj_collide<false>, site_grid(a), blk, smem,
+                                         s, fin, lam_next, lam, side, part, a, k);
+  if (e != cudaSuccess) return e;
   if (a.periodic) {
-    k_adj_collide<true><<<site_grid(a), blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
-  } else {
-    k_adj_collide<false><<<site_grid(a), blk, smem, s>>>(fin, lam_next, lam, side, part, a, k);
-    const long long items = 2LL * a.lx * Q;  // (column, wall, population), plus one block for the dtau sum
-    k_adj_walls<<<(unsigned)((items + 255) / 256) + 1, 256, 0, s>>>(side, lam, a, part, adjoint_partial_count(a),
-                                                                    dtau);
+    k_reduce_add<<<1, 256, 0, s>>>(part, adjoint_partial_count(a), dtau);
     return cudaGetLastError();
   }
-  k_reduce_add<<<1, 256, 0, s>>>(part, adjoint_partial_count(a), dtau);
-  return cudaGetLastError();
+  const long long items = 2LL * a.lx * Q;  // (column, wall, population), plus one block for the dtau sum
+  return launch_dependent(k_adj_walls, dim3((unsigned)((items + 255) / 256) + 1), dim3(256), 0, s, side, lam, a, part,
+                          adjoint_partial_count(a), dtau);
 }
 
 cudaError_t launch_ke_grad(const double* f, double* lam, const StepArgs& a, cudaStream_t s) {

@@ -168,6 +168,8 @@ template <int KIND, bool PERIODIC>
 __global__ void __launch_bounds__(256) __maxnreg__(batch_max_regs(KIND)) k_batch_step(const BatchLattice* __restrict__ L,
                                                     const unsigned short* __restrict__ tl, long long total,
                                                     int parity) {
+  pdl_trigger();
+  pdl_wait();
   const long long t = blockIdx.x;
   if (t >= total) return;
   batch_tile<KIND, PERIODIC>(L, tl, t, parity, LdReadOnly(), batch_staged);
@@ -231,9 +233,10 @@ template <int K>
 void* persistent_fn(bool periodic) {
   return periodic ? (void*)k_batch_persistent<K, true> : (void*)k_batch_persistent<K, false>;
 }
+using PerStepKernel = void (*)(const BatchLattice*, const unsigned short*, long long, int);
 template <int K>
-void* per_step_fn(bool periodic) {
-  return periodic ? (void*)k_batch_step<K, true> : (void*)k_batch_step<K, false>;
+PerStepKernel per_step_fn(bool periodic) {
+  return periodic ? k_batch_step<K, true> : k_batch_step<K, false>;
 }
 
 void* persistent_kernel(const lbm_batch* b) {
@@ -245,7 +248,7 @@ void* persistent_kernel(const lbm_batch* b) {
     default: return persistent_fn<kFix64>(b->periodic);
   }
 }
-void* per_step_kernel(const lbm_batch* b) {
+PerStepKernel per_step_kernel(const lbm_batch* b) {
   switch (kind_of(b)) {
     case kFp32: return per_step_fn<kFp32>(b->periodic);
     case kFp32Scaled: return per_step_fn<kFp32Scaled>(b->periodic);
@@ -262,7 +265,7 @@ int32_t allow_batch_smem(const lbm_batch* b) {
   if (smem <= 48 * 1024) return LBM_OK;
   if (cudaFuncSetAttribute(persistent_kernel(b), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess ||
-      cudaFuncSetAttribute(per_step_kernel(b), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+      cudaFuncSetAttribute((const void*)per_step_kernel(b), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess)
     return cuda_status(cudaGetLastError());
   return LBM_OK;
@@ -285,9 +288,8 @@ int32_t launch_per_step(lbm_batch* b, int steps, cudaStream_t s) {
   long long total = b->total_tiles;
   for (int st = 0; st < steps; ++st) {
     int par = (b->parity + st) & 1;
-    void* args[] = {(void*)&L, (void*)&tl, &total, &par};
-    const int32_t st_ = cuda_status(cudaLaunchKernel(per_step_kernel(b), dim3((unsigned)total),
-                                                     dim3(32, b->warps_per_block), args, smem, s));
+    const int32_t st_ = cuda_status(launch_dependent(per_step_kernel(b), dim3((unsigned)total),
+                                                     dim3(32, b->warps_per_block), smem, s, L, tl, total, par));
     if (st_ != LBM_OK) return st_;
   }
   return LBM_OK;

@@ -57,6 +57,34 @@ struct StepWalls {
 // Everything a site kernel needs, passed by value as the kernel parameter.
 struct StepArgs : StepScalars, StepWalls {};
 
+// Programmatic dependent launch: a kernel launched by launch_dependent may become resident while the
+// kernel before it in the stream drains, which hides the launch; pdl_wait(), its first statement before
+// any access to global memory, waits until that kernel has completed and its writes are visible.
+// pdl_trigger() lets the next kernel in as soon as every block of this one has started: 64 x 128, 10
+// steps 104 -> 84 us, 501 x 1003 78.0 -> 74.7 us.  The adjoint's kernels do without it (their
+// successors' blocks then hold slots that the recomputation on the other stream could use: gradient
+// 5.92 against 6.10 ms, adjoint step 0.195 against 0.209).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                    const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  const cudaError_t last = cudaGetLastError();  // as after <<<>>>: reported once, and cleared
+  return e != cudaSuccess ? e : last;
+}
+
 cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s);
 cudaError_t launch_propagate_fp64(const double* fin, double* ftmp, const StepArgs& a, cudaStream_t s);
 cudaError_t launch_propagate_push_fp64(const double* fin, double* ftmp, const StepArgs& a, cudaStream_t s);

@@ -20,6 +20,8 @@ template <bool PERIODIC, bool SCALED, bool CONSERVE>
 __global__ void __launch_bounds__(128, CONSERVE ? LBM_FP32C_MIN_BLOCKS : LBM_FP32_MIN_BLOCKS) k_step_fp32(
     const float* __restrict__ fin,
                                                                        float* __restrict__ fout, StepArgs a) {
+  pdl_trigger();
+  pdl_wait();
   const int x = blockIdx.y * 4 + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
   step_strip_fp32<PERIODIC, SCALED, CONSERVE>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly());
@@ -95,21 +97,15 @@ static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, 
 static const dim3 kSiteBlock(32, 4);
 
 template <bool PERIODIC, bool SCALED>
-static void launch_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {
-  if (a.conserve) k_step_fp32<PERIODIC, SCALED, true><<<site_grid(a), kSiteBlock, 0, s>>>(fin, fout, a);
-  else k_step_fp32<PERIODIC, SCALED, false><<<site_grid(a), kSiteBlock, 0, s>>>(fin, fout, a);
+static cudaError_t launch_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {
+  return launch_dependent(a.conserve ? k_step_fp32<PERIODIC, SCALED, true> : k_step_fp32<PERIODIC, SCALED, false>,
+                          site_grid(a), kSiteBlock, 0, s, fin, fout, a);
 }
 
 cudaError_t launch_step_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {
   const bool scaled = a.fix_back != 1.0 / 4503599627370496.0;
-  if (a.periodic) {
-    if (scaled) launch_fp32<true, true>(fin, fout, a, s);
-    else launch_fp32<true, false>(fin, fout, a, s);
-  } else {
-    if (scaled) launch_fp32<false, true>(fin, fout, a, s);
-    else launch_fp32<false, false>(fin, fout, a, s);
-  }
-  return cudaGetLastError();
+  if (a.periodic) return scaled ? launch_fp32<true, true>(fin, fout, a, s) : launch_fp32<true, false>(fin, fout, a, s);
+  return scaled ? launch_fp32<false, true>(fin, fout, a, s) : launch_fp32<false, false>(fin, fout, a, s);
 }
 
 cudaError_t launch_init_fp32(const double* rho, const double* ux, const double* uy, const double* T, float* f,

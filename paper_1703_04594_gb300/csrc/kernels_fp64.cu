@@ -37,6 +37,8 @@ extern __shared__ double step_staged[];  // 37 populations x 32 sites per warp
 template <bool PERIODIC>
 __global__ void __launch_bounds__(128, LBM_FIX64_MIN_BLOCKS) k_step_fix64(const double* __restrict__ fin,
                                                                          double* __restrict__ fout, StepArgs a) {
+  pdl_trigger();
+  pdl_wait();
   const int x = blockIdx.y * 4 + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
   step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly(), step_staged + threadIdx.y * (Q * 32));
@@ -253,9 +255,8 @@ static const dim3 kSiteBlock(32, 4);
 
 cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s) {
   constexpr size_t smem = 4 * Q * 32 * sizeof(double);
-  if (a.periodic) k_step_fix64<true><<<site_grid(a), kSiteBlock, smem, s>>>(fin, fout, a);
-  else k_step_fix64<false><<<site_grid(a), kSiteBlock, smem, s>>>(fin, fout, a);
-  return cudaGetLastError();
+  return launch_dependent(a.periodic ? k_step_fix64<true> : k_step_fix64<false>, site_grid(a), kSiteBlock, smem, s, fin,
+                          fout, a);
 }
 
 cudaError_t launch_propagate_fp64(const double* fin, double* ftmp, const StepArgs& a, cudaStream_t s) {

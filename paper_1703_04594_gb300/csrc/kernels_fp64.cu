@@ -5,6 +5,7 @@
 // (the contiguous axis, Sec. 4 "column-major, Y innermost"), so each warp owns 32
 // consecutive sites of one column x and every population load/store of a warp is one
 // contiguous 256-byte run (shifted by the hop's vy for loads).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -163,7 +164,8 @@ __device__ __noinline__ void site_fields_float64(const double* __restrict__ f, l
 
 // rho, c u and T of a site by the fixed-point moments and scalars of site_fix64.cuh: exact sums, four
 // conversions on the float64 pipe.  false outside their range.  The kernels below then run at the
-// copy rate: k_moments_fp64 reads and writes 2.75 GB (2048 x 4096) in 0.405 ms, 6.8 TB/s; with
+// copy rate, given the 128 registers that keep a site's 37 loads in flight (left to itself the
+// compiler took 66 and 0.48 ms): k_moments_fp64 reads and writes 2.75 GB (2048 x 4096) in 0.405 ms, 6.8 TB/s; with
 // rounding sums and float64 scalars it took ~0.85 ms.
 __device__ __forceinline__ bool site_fields_fix(const double* __restrict__ f, long long pop, double& rho, double& cux,
                                                 double& cuy, double& T) {
@@ -180,7 +182,7 @@ __device__ __forceinline__ bool site_fields_fix(const double* __restrict__ f, lo
   return v.ok;
 }
 
-__global__ void __launch_bounds__(128) k_moments_fp64(const double* __restrict__ fin, double* __restrict__ rho,
+__global__ void __launch_bounds__(128, 4) k_moments_fp64(const double* __restrict__ fin, double* __restrict__ rho,
                                                       double* __restrict__ ux, double* __restrict__ uy,
                                                       double* __restrict__ T, StepArgs a) {
   const int x = blockIdx.y * 4 + threadIdx.y;
@@ -200,7 +202,7 @@ __global__ void __launch_bounds__(128) k_moments_fp64(const double* __restrict__
 }
 
 // Kinetic energy: per-block partial sums (fixed order), then one block sums the partials.
-__global__ void __launch_bounds__(128) k_ke_partial_fp64(const double* __restrict__ fin, double* __restrict__ part,
+__global__ void __launch_bounds__(128, 4) k_ke_partial_fp64(const double* __restrict__ fin, double* __restrict__ part,
                                                          StepArgs a) {
   const int x = blockIdx.y * 4 + threadIdx.y;
   const int y = blockIdx.x * 32 + threadIdx.x;
@@ -224,10 +226,9 @@ __global__ void __launch_bounds__(128) k_ke_partial_fp64(const double* __restric
     part[blockIdx.y * gridDim.x + blockIdx.x] = (warp_sum[0] + warp_sum[1]) + (warp_sum[2] + warp_sum[3]);
 }
 
-// Sums n doubles in a fixed order: one block, eight independent sums per thread (65536 partials in
-// 8 rounds of loads; with one sum in each of 256 threads it took 256).
-__global__ void __launch_bounds__(1024) k_reduce_sum(const double* __restrict__ part, long long n,
-                                                    double* __restrict__ out) {
+// Sum of part[0..n) over one block of 1024 threads in a fixed order, valid in thread 0: eight
+// independent sums per thread keep as many loads in flight.
+__device__ __forceinline__ double block_sum_1024(const double* __restrict__ part, long long n) {
   double v[8] = {};
   for (long long i = threadIdx.x; i < n; i += 8 * 1024) {
 #pragma unroll
@@ -240,11 +241,33 @@ __global__ void __launch_bounds__(1024) k_reduce_sum(const double* __restrict__ 
   __shared__ double ws[32];
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    double t = ws[threadIdx.x];
+  double t = threadIdx.x < 32 ? ws[threadIdx.x] : 0.0;
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(FULL, t, off);
+  for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(FULL, t, off);
+  return t;
+}
+
+// One cluster of CLUSTER blocks, each summing its part of the array; block 0 adds their sums in order
+// through distributed shared memory.
+template <int CLUSTER>
+__global__ void __launch_bounds__(1024) k_reduce_sum(const double* __restrict__ part, long long n,
+                                                    double* __restrict__ out) {
+  if constexpr (CLUSTER == 1) {
+    const double t = block_sum_1024(part, n);
     if (threadIdx.x == 0) *out = t;
+  } else {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    __shared__ double sums[CLUSTER];
+    const long long each = (n + CLUSTER - 1) / CLUSTER, begin = each * blockIdx.x;
+    const double t = block_sum_1024(part + begin, begin < n ? (n - begin < each ? n - begin : each) : 0);
+    if (threadIdx.x == 0) cluster.map_shared_rank(sums, 0)[blockIdx.x] = t;
+    cluster.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      double s = 0.0;
+      for (int c = 0; c < CLUSTER; ++c) s += sums[c];
+      *out = s;
+    }
   }
 }
 
@@ -300,9 +323,26 @@ long long ke_partial_count(const StepArgs& a) {
   return (long long)g.x * g.y;
 }
 
+// One block reads at most ~60 GB/s: from 8192 partials (one round of its loads) on, a cluster of eight
+// (65536 partials: 26 -> 11 us).
 cudaError_t launch_reduce_sum(const double* part, long long n, double* out, cudaStream_t s) {
-  k_reduce_sum<<<1, 1024, 0, s>>>(part, n, out);
-  return cudaGetLastError();
+  if (n <= 8192) {
+    k_reduce_sum<1><<<1, 1024, 0, s>>>(part, n, out);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(8);
+  cfg.blockDim = dim3(1024);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 8;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_reduce_sum<8>, part, n, out);
+  const cudaError_t last = cudaGetLastError();
+  return e != cudaSuccess ? e : last;
 }
 
 cudaError_t launch_kinetic_energy_fp64(const double* f, double* out, double* part, const StepArgs& a,

@@ -487,9 +487,9 @@ int32_t lbm_adjoint_step(const lbm_params* p, const void* f_n, const void* lam_n
   if (!params_valid(p) || p->precision != LBM_FP64 || !a16(f_n) || !a16(lam_next) || !a16(lam_n) ||
       !a8(dtau_accum) || !a16(work))
     return LBM_EINVAL;
-  const int64_t need = lbm_adjoint_work_bytes(p);
-  if ((int64_t)work_bytes < need || lam_next == lam_n || f_n == lam_n) return LBM_EINVAL;
   const StepArgs a = make_step_args(p);
+  const int64_t need = (adjoint_side_count(a) + adjoint_partial_count(a)) * (int64_t)sizeof(double);
+  if ((int64_t)work_bytes < need || lam_next == lam_n || f_n == lam_n) return LBM_EINVAL;
   double* side = (double*)work;
   double* part = side + adjoint_side_count(a);
   return status_of(launch_adjoint_step((const double*)f_n, (const double*)lam_next, (double*)lam_n, side, part,

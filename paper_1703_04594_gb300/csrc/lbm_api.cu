@@ -72,6 +72,32 @@ double wall_multiplier(int i, double T) {
 
 }  // namespace
 
+// Constants of the FP32 collision that depend on the model alone.
+namespace {
+struct FloatModel {
+  double c2_iso, corr_iw, corr_m, corr_ivar;
+  FloatModel() {
+    double s = 0.0;  // sum_s w_s M_s with the float32 weights of the FP32 collision
+    for (int i = 0; i < Q; ++i) s += (double)(float)weight(i) * (double)(vx(i) * vx(i));
+    c2_iso = 1.0 / s;
+    // the mass and energy correction's basis: all 37 populations, float32 weights
+    double sw = 0.0, swq = 0.0;
+    for (int i = 0; i < Q; ++i) {
+      const double w = (double)(float)weight(i);
+      sw += w;
+      swq += w * v2(i);
+    }
+    const double m = swq / sw;
+    double var = 0.0;
+    for (int i = 0; i < Q; ++i) var += (double)(float)weight(i) * (v2(i) - m) * (v2(i) - m);
+    corr_iw = 1.0 / sw;
+    corr_m = m;
+    corr_ivar = 1.0 / var;
+  }
+};
+const FloatModel kFloatModel;
+}  // namespace
+
 StepArgs d2q37::make_step_args(const lbm_params* p) {
   StepArgs a;
   memset(&a, 0, sizeof(a));
@@ -92,24 +118,10 @@ StepArgs d2q37::make_step_args(const lbm_params* p) {
   a.f_om1 = 1.0f - a.f_omega;  // exact for 1/2 <= omega <= 2
   a.f_cgx = (float)a.cc.cgx;
   a.f_cgy = (float)a.cc.cgy;
-  {
-    double s = 0.0;  // sum_s w_s M_s with the float32 weights of the FP32 collision
-    for (int i = 0; i < Q; ++i) s += (double)(float)weight(i) * (double)(vx(i) * vx(i));
-    a.c2_iso = 1.0 / s;
-    // the mass and energy correction's basis: all 37 populations, float32 weights
-    double sw = 0.0, swq = 0.0;
-    for (int i = 0; i < Q; ++i) {
-      const double w = (double)(float)weight(i);
-      sw += w;
-      swq += w * v2(i);
-    }
-    const double m = swq / sw;
-    double var = 0.0;
-    for (int i = 0; i < Q; ++i) var += (double)(float)weight(i) * (v2(i) - m) * (v2(i) - m);
-    a.corr_iw = 1.0 / sw;
-    a.corr_m = m;
-    a.corr_ivar = 1.0 / var;
-  }
+  a.c2_iso = kFloatModel.c2_iso;
+  a.corr_iw = kFloatModel.corr_iw;
+  a.corr_m = kFloatModel.corr_m;
+  a.corr_ivar = kFloatModel.corr_ivar;
   a.corr_gx = p->gx / C;
   a.corr_gy = p->gy / C;
   a.corr_g2 = (p->gx * p->gx + p->gy * p->gy) / C2;

@@ -8,6 +8,7 @@ missing library raises ``RuntimeError``: there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 from dataclasses import dataclass
 
@@ -50,6 +51,22 @@ class Params:
     def c(self) -> CParams:
         return CParams(self.lx, self.ly, self.precision, self.bc, self.tau, self.gx, self.gy,
                        self.t_bottom, self.t_top, self.rho0)
+
+    # What every call needs of one parameter set, formed on its first use (the fields are frozen):
+    # the C struct's reference, and the state's bytes and type.  Left out of copies and pickles.
+    @functools.cached_property
+    def _call(self):
+        return _Call(ctypes.byref(self.c()), buffer_bytes(self), state_dtype(self))
+
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k != "_call"}
+
+
+class _Call:
+    __slots__ = ("ref", "bytes", "dtype")
+
+    def __init__(self, ref, nbytes, dtype):
+        self.ref, self.bytes, self.dtype = ref, nbytes, dtype
 
 
 class LbmError(RuntimeError):
@@ -136,7 +153,8 @@ def _ptr(t):
 
 def _stream(stream=None):
     if stream is None:
-        stream = torch.cuda.current_stream()
+        torch.cuda.init()
+        return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
     return ctypes.c_void_p(stream.cuda_stream)
 
 
@@ -175,12 +193,15 @@ def state_dtype(p: Params):
 
 def empty_state(p: Params, device="cuda") -> torch.Tensor:
     """An uninitialised state buffer [37, lx, pitch] of the storage type."""
-    return torch.empty((Q, p.lx, pitch(p)), dtype=state_dtype(p), device=device)
+    call = p._call
+    item = 4 if call.dtype == torch.float32 else 8
+    return torch.empty((Q, p.lx, call.bytes // (Q * p.lx * item)), dtype=call.dtype, device=device)
 
 
 def _state(p: Params, t: torch.Tensor, name: str):
-    if not (t.is_cuda and t.is_contiguous() and t.dtype == state_dtype(p)
-            and t.numel() * t.element_size() >= buffer_bytes(p)):
+    call = p._call
+    if not (t.is_cuda and t.is_contiguous() and t.dtype == call.dtype
+            and t.numel() * t.element_size() >= call.bytes):
         raise ValueError(f"{name}: expected a contiguous CUDA {state_dtype(p)} tensor of "
                          f"{buffer_bytes(p)} bytes, got {t.dtype} {tuple(t.shape)} on {t.device}")
     return _ptr(t)
@@ -194,45 +215,45 @@ def _field(p: Params, t: torch.Tensor, name: str):
 
 # ------------------------------------------------------------------------- device calls
 def init(p: Params, rho, ux, uy, T, f, stream=None):
-    _check("lbm_init", _lib().lbm_init(ctypes.byref(p.c()), _field(p, rho, "rho"), _field(p, ux, "ux"),
+    _check("lbm_init", _lib().lbm_init(p._call.ref, _field(p, rho, "rho"), _field(p, ux, "ux"),
                                        _field(p, uy, "uy"), _field(p, T, "T"), _state(p, f, "f"),
                                        _stream(stream)))
     return f
 
 
 def step(p: Params, f_in, f_out, stream=None):
-    _check("lbm_step", _lib().lbm_step(ctypes.byref(p.c()), _state(p, f_in, "f_in"),
+    _check("lbm_step", _lib().lbm_step(p._call.ref, _state(p, f_in, "f_in"),
                                        _state(p, f_out, "f_out"), _stream(stream)))
     return f_out
 
 
 def run(p: Params, f_a, f_b, n_steps: int, stream=None):
     """n_steps fused steps; returns the tensor holding the result."""
-    _check("lbm_run", _lib().lbm_run(ctypes.byref(p.c()), _state(p, f_a, "f_a"), _state(p, f_b, "f_b"),
+    _check("lbm_run", _lib().lbm_run(p._call.ref, _state(p, f_a, "f_a"), _state(p, f_b, "f_b"),
                                      int(n_steps), _stream(stream)))
     return f_a if n_steps % 2 == 0 else f_b
 
 
 def propagate(p: Params, f_in, f_tmp, stream=None):
-    _check("lbm_propagate", _lib().lbm_propagate(ctypes.byref(p.c()), _state(p, f_in, "f_in"),
+    _check("lbm_propagate", _lib().lbm_propagate(p._call.ref, _state(p, f_in, "f_in"),
                                                  _state(p, f_tmp, "f_tmp"), _stream(stream)))
     return f_tmp
 
 
 def propagate_push(p: Params, f_in, f_tmp, stream=None):
-    _check("lbm_propagate_push", _lib().lbm_propagate_push(ctypes.byref(p.c()), _state(p, f_in, "f_in"),
+    _check("lbm_propagate_push", _lib().lbm_propagate_push(p._call.ref, _state(p, f_in, "f_in"),
                                                            _state(p, f_tmp, "f_tmp"), _stream(stream)))
     return f_tmp
 
 
 def bc(p: Params, f_in, f_tmp, stream=None):
-    _check("lbm_bc", _lib().lbm_bc(ctypes.byref(p.c()), _state(p, f_in, "f_in"), _state(p, f_tmp, "f_tmp"),
+    _check("lbm_bc", _lib().lbm_bc(p._call.ref, _state(p, f_in, "f_in"), _state(p, f_tmp, "f_tmp"),
                                    _stream(stream)))
     return f_tmp
 
 
 def collide(p: Params, f_tmp, f_out, stream=None):
-    _check("lbm_collide", _lib().lbm_collide(ctypes.byref(p.c()), _state(p, f_tmp, "f_tmp"),
+    _check("lbm_collide", _lib().lbm_collide(p._call.ref, _state(p, f_tmp, "f_tmp"),
                                              _state(p, f_out, "f_out"), _stream(stream)))
     return f_out
 
@@ -242,7 +263,7 @@ def moments(p: Params, f, out=None, stream=None):
     if out is None:
         out = [torch.empty((p.lx, p.ly), dtype=torch.float64, device=f.device) for _ in range(4)]
     rho, ux, uy, T = out
-    _check("lbm_moments", _lib().lbm_moments(ctypes.byref(p.c()), _state(p, f, "f"), _field(p, rho, "rho"),
+    _check("lbm_moments", _lib().lbm_moments(p._call.ref, _state(p, f, "f"), _field(p, rho, "rho"),
                                              _field(p, ux, "ux"), _field(p, uy, "uy"), _field(p, T, "T"),
                                              _stream(stream)))
     return rho, ux, uy, T
@@ -259,7 +280,7 @@ def kinetic_energy(p: Params, f, out=None, scratch=None, stream=None):
     if scratch is None:
         scratch = torch.empty(reduce_scratch_bytes(p) // 8, dtype=torch.float64, device=f.device)
     _check("lbm_kinetic_energy", _lib().lbm_kinetic_energy(
-        ctypes.byref(p.c()), _state(p, f, "f"), _ptr(out), _ptr(scratch),
+        p._call.ref, _state(p, f, "f"), _ptr(out), _ptr(scratch),
         scratch.numel() * scratch.element_size(), _stream(stream)))
     return out
 
@@ -273,7 +294,7 @@ def kinetic_energy_noalloc(p: Params, f, out=None, stream=None):
     if out is None:
         out = torch.empty((), dtype=torch.float64, device=f.device)
     _check("lbm_kinetic_energy_noalloc", _lib().lbm_kinetic_energy_noalloc(
-        ctypes.byref(p.c()), _state(p, f, "f"), _ptr(out), _stream(stream)))
+        p._call.ref, _state(p, f, "f"), _ptr(out), _stream(stream)))
     return out
 
 
@@ -288,7 +309,7 @@ def simulate_host(p: Params, fields_in, n_steps: int, fields_out, f_a, f_b, fiel
     fi = [_ptr(t) for t in fields_in]
     fo = [_ptr(t) for t in fields_out]
     _check("lbm_simulate_host", _lib().lbm_simulate_host(
-        ctypes.byref(p.c()), *fi, int(n_steps), *fo, _state(p, f_a, "f_a"), _state(p, f_b, "f_b"),
+        p._call.ref, *fi, int(n_steps), *fo, _state(p, f_a, "f_a"), _state(p, f_b, "f_b"),
         _ptr(fields_dev), _stream(stream)))
     return fields_out
 
@@ -298,20 +319,20 @@ LAYOUT_SOA, LAYOUT_AOS, LAYOUT_PSOA, LAYOUT_CAOSOA = 0, 1, 2, 3
 
 
 def convert_layout(p: Params, src, frm: int, dst, to: int, stream=None):
-    _check("lbm_convert_layout", _lib().lbm_convert_layout(ctypes.byref(p.c()), frm, _state(p, src, "src"), to,
+    _check("lbm_convert_layout", _lib().lbm_convert_layout(p._call.ref, frm, _state(p, src, "src"), to,
                                                            _state(p, dst, "dst"), _stream(stream)))
     return dst
 
 
 def step_layout(p: Params, layout: int, f_in, f_out, stream=None):
-    _check("lbm_step_layout", _lib().lbm_step_layout(ctypes.byref(p.c()), layout, _state(p, f_in, "f_in"),
+    _check("lbm_step_layout", _lib().lbm_step_layout(p._call.ref, layout, _state(p, f_in, "f_in"),
                                                      _state(p, f_out, "f_out"), _stream(stream)))
     return f_out
 
 
 # ------------------------------------------------------------------------- adjoint
 def adjoint_work(p: Params, device="cuda"):
-    n = _lib().lbm_adjoint_work_bytes(ctypes.byref(p.c()))
+    n = _lib().lbm_adjoint_work_bytes(p._call.ref)
     if n < 0:
         raise LbmError("lbm_adjoint_work_bytes", EINVAL)
     return torch.empty((n + 7) // 8, dtype=torch.float64, device=device)
@@ -320,13 +341,13 @@ def adjoint_work(p: Params, device="cuda"):
 def adjoint_step(p: Params, f_n, lam_next, lam_n, dtau_acc, work, stream=None):
     """lam_n = (d step/d f_n)^T lam_next; dtau_acc (0-d device float64) += dL/dtau part."""
     _check("lbm_adjoint_step", _lib().lbm_adjoint_step(
-        ctypes.byref(p.c()), _state(p, f_n, "f_n"), _state(p, lam_next, "lam_next"), _state(p, lam_n, "lam_n"),
+        p._call.ref, _state(p, f_n, "f_n"), _state(p, lam_next, "lam_next"), _state(p, lam_n, "lam_n"),
         _ptr(dtau_acc), _ptr(work), work.numel() * work.element_size(), _stream(stream)))
     return lam_n
 
 
 def kinetic_energy_grad(p: Params, f, lam, stream=None):
-    _check("lbm_kinetic_energy_grad", _lib().lbm_kinetic_energy_grad(ctypes.byref(p.c()), _state(p, f, "f"),
+    _check("lbm_kinetic_energy_grad", _lib().lbm_kinetic_energy_grad(p._call.ref, _state(p, f, "f"),
                                                                      _state(p, lam, "lam"), _stream(stream)))
     return lam
 
@@ -335,7 +356,7 @@ def init_adjoint(p: Params, rho, ux, uy, T, lam0, stream=None):
     """(g_rho, g_ux, g_uy, g_T): gradients of the initial fields against lam0."""
     out = [torch.empty((p.lx, p.ly), dtype=torch.float64, device=lam0.device) for _ in range(4)]
     _check("lbm_init_adjoint", _lib().lbm_init_adjoint(
-        ctypes.byref(p.c()), _field(p, rho, "rho"), _field(p, ux, "ux"), _field(p, uy, "uy"), _field(p, T, "T"),
+        p._call.ref, _field(p, rho, "rho"), _field(p, ux, "ux"), _field(p, uy, "uy"), _field(p, T, "T"),
         _state(p, lam0, "lam0"), *[_ptr(t) for t in out], _stream(stream)))
     return out
 

@@ -21,7 +21,7 @@
 //   2. (k_adj_walls) the wall rows: every population of (x_s, 0) receives the sum of the
 //      bottom slots of column x_s, each times its ghost's weight w_i P_i(T_wall) (the
 //      transpose of rho_w = sum_j f_j(x_s, 0)), and likewise at the top.
-// dL/dtau partials are summed per strip and then in a fixed order (deterministic).
+// dL/dtau partials are summed per block and then in a fixed order (deterministic).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -303,22 +303,32 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
                sf[i * 32]);
     }
   }
-  // one partial per strip (a sum over the block would hold its early warps' registers and slots)
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) contrib += __shfl_down_sync(0xffffffffu, contrib, off);
-  if (threadIdx.x == 0) dtau_part[(long long)x * ((a.ly + 31) >> 5) + (y0 >> 5)] = contrib;
+  __shared__ double warp_sum[4];
+  if (threadIdx.x == 0) warp_sum[threadIdx.y] = contrib;
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    double s = warp_sum[0];
+    for (int w = 1; w < 4 && x + w < a.lx; ++w) s += warp_sum[w];  // the warps past lx have returned
+    dtau_part[blockIdx.y * gridDim.x + blockIdx.x] = s;
+  }
 }
 
-// Adds sum(part[0..n)) to *acc in a fixed order; one block of 256 threads.  Eight independent sums
-// per thread keep as many loads in flight (one at a time, 16384 partials took ~20 us).
+// Adds sum(part[0..n)) to *acc in a fixed order; one block of 256 threads.  Sixteen independent
+// sums per thread keep as many loads in flight.
 __device__ __forceinline__ void reduce_add_256(const double* __restrict__ part, long long n, double* acc) {
-  double s[8] = {};
-  for (long long i = threadIdx.x; i < n; i += 8 * 256) {
+  double s[16] = {};
+  for (long long i = threadIdx.x; i < n; i += 16 * 256) {
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
+    for (int j = 0; j < 16; ++j)
       if (i + j * 256 < n) s[j] += part[i + j * 256];
   }
-  double v = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+#pragma unroll
+  for (int h = 8; h > 0; h >>= 1)
+#pragma unroll
+    for (int j = 0; j < h; ++j) s[j] += s[j + h];
+  double v = s[0];
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
   __shared__ double ws[8];
@@ -413,7 +423,8 @@ __global__ void __launch_bounds__(128) k_init_adjoint(const double* __restrict__
 static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, (a.lx + 3) / 4); }
 
 long long adjoint_partial_count(const StepArgs& a) {
-  return (long long)((a.ly + 31) / 32) * a.lx;  // one per strip
+  const dim3 g = site_grid(a);
+  return (long long)g.x * g.y;
 }
 
 long long adjoint_side_count(const StepArgs& a) { return 2LL * a.lx * kGhostSlots; }

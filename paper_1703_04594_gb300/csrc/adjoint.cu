@@ -297,10 +297,12 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
     if (PERIODIC || fix64_wall_strip<PERIODIC>(a, y0)) {
       push_strip_edge<PERIODIC>(sf, lam_out, side, a, x, y);
     } else {
+      double* col[7];  // row y of column x - vx
 #pragma unroll
-      for (int i = 0; i < Q; ++i)
-        __stcs(lam_out + (i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch) - vy(i) + (unsigned)y,
-               sf[i * 32]);
+      for (int d = 0; d < 7; ++d)
+        col[d] = lam_out + ((unsigned)wrap_index(x - (d - 3), a.lx) * (unsigned)a.pitch + (unsigned)y);
+#pragma unroll
+      for (int i = 0; i < Q; ++i) __stcs(col[vx(i) + 3] + i * a.pop - vy(i), sf[i * 32]);
     }
   }
 #pragma unroll

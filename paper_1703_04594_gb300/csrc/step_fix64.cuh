@@ -82,18 +82,25 @@ template <bool PERIODIC, class Ld>
 __device__ __forceinline__ void stage_strip(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
                                             int x, int y0, int yc, double* __restrict__ sf, Ld ld) {
   const bool wall = fix64_wall_strip<PERIODIC>(a, y0);
+  // one pointer per source column (planes < 2^32 elements); a plane's stride and a hop in y are then
+  // an addition and an immediate
+  const double* col[7];
+#pragma unroll
+  for (int d = 0; d < 7; ++d) col[d] = fin + (unsigned)wrap_index(x - (d - 3), a.lx) * (unsigned)a.pitch;
   if (wall || PERIODIC) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       const int ys = PERIODIC ? wrap_index(yc - vy(i), a.ly) : min(max(yc - vy(i), 0), a.ly - 1);
-      const double* src = fin + (i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch) + (unsigned)ys;
+      const double* src = col[vx(i) + 3] + i * a.pop + (unsigned)ys;
       if (Ld::kL1) cp_async8(sf + i * 32, src);
       else sf[i * 32] = ld(src);
     }
   } else {
 #pragma unroll
+    for (int d = 0; d < 7; ++d) col[d] += (unsigned)yc;
+#pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const double* src = fin + (i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch) - vy(i) + (unsigned)yc;
+      const double* src = col[vx(i) + 3] + i * a.pop - vy(i);
       if (Ld::kL1) cp_async8(sf + i * 32, src);
       else sf[i * 32] = ld(src);
     }

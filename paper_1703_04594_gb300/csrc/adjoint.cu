@@ -269,22 +269,23 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
   double* const sf = adj_staged + threadIdx.y * (Q * 32) + threadIdx.x;
   FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);
   const double* lam = lam_next + (long long)x * a.pitch + (unsigned)yc;
-  stage_strip<PERIODIC>(fin, a, a, x, y0, yc, sf, LdReadOnly());
+  stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, LdReadOnly());
   // the block exponent of lambda, from the high words alone (the values are loaded again below,
   // when their fixed-point forms can go to the slots at once)
   unsigned top = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i)
     top = max(top, __ldg(reinterpret_cast<const unsigned*>(lam + i * a.pop) + 1) & 0x7fffffffu);
+  stage_finish<PERIODIC>(fin, a, a, x, y0, yc, sf, LdReadOnly());
   __syncthreads();
-  const FixMoments m = fix_moments_rolled(c_fix_axes, c_fix_quads, [&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
+  const FixMoments m = fix_moments_rolled(c_fix_groups, [&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
   const FixScalars v = fix_scalars(m, a.fx);
   const unsigned E = top == 0u ? 512u : top >> 20;  // all zero: any exponent
   __syncthreads();
   const int K = (1080 - (int)E) << 20;
   const bool ok = v.ok && a.fx.usable && k.fx.usable && E - 100u < 978u;
   const AdjIo io = {sx, lam, (unsigned)a.pop, K};
-  const FixMu mm = fix_mu_moments(K + (1 << 20), c_fix_axes, c_fix_quads, io);
+  const FixMu mm = fix_mu_moments(K + (1 << 20), c_fix_groups, io);
   __syncthreads();
   FixVjp r = fix_vjp(m, v, mm, a.fx, k.fx);
   if (top == 0u) r = FixVjp{};  // lambda = 0: no rounding residue

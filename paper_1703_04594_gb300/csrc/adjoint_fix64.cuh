@@ -92,16 +92,15 @@ struct FixMu {
 
 // `io.at(i)` returns a handle of population i's pair (i, i + NPAIR), and for population i + k NPAIR
 // `io.mu(h, k)` its mu, `io.fixed(h, k)` the halves of f' (fix_moments); `io.keep(h, k, q)` takes the
-// halves of its mu 2^(K + 1), after the other two calls.  `axes` and `quads` are the tables above (the
-// host tests pass their own copies).
+// halves of its mu 2^(K + 1), after the other two calls.  
 template <class Io>
-__host__ __device__ __forceinline__ FixMu fix_mu_moments(int K1, const FixGroup* axes, const FixGroup* quads,
+__host__ __device__ __forceinline__ FixMu fix_mu_moments(int K1, const FixGroup* groups,
                                                                 Io&& io) {
   FixMu r;
   r.mf = 5;
   FxDot mf;
-  const auto get = [&](auto at, int k) {
-    const long long q = fx_block(io.mu(at, k), K1);
+  const auto get = [&](auto at, int k, double m) {
+    const long long q = fx_block(m, K1);
     const FxHalves h = fx_halves(q);
     mf.add(h, io.fixed(at, k));
     io.keep(at, k, h);
@@ -119,13 +118,22 @@ __host__ __device__ __forceinline__ FixMu fix_mu_moments(int K1, const FixGroup*
   // 2^-53 of max |mu|
   unsigned long long m00 = 6, m20 = 17, m02 = 17, m40 = 107, m04 = 107, m22 = 21, m11 = 7, m31 = 28, m13 = 28;
   unsigned long long m10 = 8, m01 = 8, m30 = 41, m03 = 41, m12 = 13, m21 = 13;
-  m00 += (unsigned long long)weigh(get(io.at(0), 0), fx_halves_ct(kCw(0)), shell_exp(0));
+  m00 += (unsigned long long)weigh(get(io.at(0), 0, io.mu(io.at(0), 0)), fx_halves_ct(kCw(0)), shell_exp(0));
   flush(shell_exp(0));
+  // each group's mu are loaded while the group before it is worked on
+  double m[4];
+  const auto fetch = [&](int n) {
+    const auto ai = io.at(groups[n].i), aj = io.at(groups[n].j);
+    m[0] = io.mu(ai, 0), m[1] = io.mu(ai, 1), m[2] = io.mu(aj, 0), m[3] = io.mu(aj, 1);
+  };
+  fetch(0);
 #pragma unroll 1
-  for (int n = 0; n < 3; ++n) {
-    const FixGroup& g = axes[n];
+  for (int n = 0; n < kFixAxes; ++n) {
+    const FixGroup& g = groups[n];
     const auto ai = io.at(g.i), aj = io.at(g.j);
-    const long long p = get(ai, 0), q = get(ai, 1), u = get(aj, 0), v = get(aj, 1);
+    const double m0 = m[0], m1 = m[1], m2 = m[2], m3 = m[3];
+    fetch(n + 1 < kFixGroups ? n + 1 : n);
+    const long long p = get(ai, 0, m0), q = get(ai, 1, m1), u = get(aj, 0, m2), v = get(aj, 1, m3);
     flush(g.sh);
     const unsigned long long ex = (unsigned long long)weigh(p + q, g.w, g.sh), ox = (unsigned long long)weigh(p - q, g.w, g.sh);
     const unsigned long long ey = (unsigned long long)weigh(u + v, g.w, g.sh), oy = (unsigned long long)weigh(u - v, g.w, g.sh);
@@ -140,10 +148,12 @@ __host__ __device__ __forceinline__ FixMu fix_mu_moments(int K1, const FixGroup*
     m03 += g.a3 * oy;
   }
 #pragma unroll 1
-  for (int n = 0; n < 6; ++n) {
-    const FixGroup& g = quads[n];
+  for (int n = kFixAxes; n < kFixGroups; ++n) {
+    const FixGroup& g = groups[n];
     const auto ai = io.at(g.i), aj = io.at(g.j);
-    const long long p = get(ai, 0), q = get(ai, 1), u = get(aj, 0), v = get(aj, 1);
+    const double m0 = m[0], m1 = m[1], m2 = m[2], m3 = m[3];
+    fetch(n + 1 < kFixGroups ? n + 1 : n);
+    const long long p = get(ai, 0, m0), q = get(ai, 1, m1), u = get(aj, 0, m2), v = get(aj, 1, m3);
     flush(g.sh);
     const long long pp = p + q, pm = p - q, up = u + v, um = u - v;
     const unsigned long long S = (unsigned long long)weigh(pp + up, g.w, g.sh), D = (unsigned long long)weigh(pp - up, g.w, g.sh);

@@ -154,13 +154,12 @@ struct FixGroup {
 __host__ __device__ constexpr FxHalves fx_halves_ct(long long a) {
   return FxHalves{(int)(unsigned)a, (int)((a >> 32) + ((unsigned)a >> 31))};
 }
-#define LBM_FIX_AXES                                                                               \
-  {LBM_FIX_GROUP(1, 0, pop_index(0, 1)), LBM_FIX_GROUP(2, 0, pop_index(0, 2)), LBM_FIX_GROUP(3, 0, pop_index(0, 3))}
-#define LBM_FIX_QUADS \
-  {LBM_FIX_GROUP(1, 1, pop_index(1, -1)), LBM_FIX_GROUP(2, 1, pop_index(2, -1)), LBM_FIX_GROUP(1, 2, pop_index(1, -2)), \
+#define LBM_FIX_GROUPS                                                                             \
+  {LBM_FIX_GROUP(1, 0, pop_index(0, 1)), LBM_FIX_GROUP(2, 0, pop_index(0, 2)), LBM_FIX_GROUP(3, 0, pop_index(0, 3)), \
+   LBM_FIX_GROUP(1, 1, pop_index(1, -1)), LBM_FIX_GROUP(2, 1, pop_index(2, -1)), LBM_FIX_GROUP(1, 2, pop_index(1, -2)), \
    LBM_FIX_GROUP(2, 2, pop_index(2, -2)), LBM_FIX_GROUP(3, 1, pop_index(3, -1)), LBM_FIX_GROUP(1, 3, pop_index(1, -3))}
-static __constant__ FixGroup c_fix_axes[3] = LBM_FIX_AXES;
-static __constant__ FixGroup c_fix_quads[6] = LBM_FIX_QUADS;
+constexpr int kFixAxes = 3, kFixGroups = 9;  // the axes first
+static __constant__ FixGroup c_fix_groups[kFixGroups] = LBM_FIX_GROUPS;
 
 // ---- 1. populations to fixed point, and the moments ---------------------------------------------
 struct FixMoments {
@@ -239,7 +238,7 @@ __host__ __device__ __forceinline__ FixMoments fix_moments(Load&& load, Keep&& k
 // The same in loops over the tables above, for kernels whose code overflows the instruction cache
 // (about 150 more instructions executed, 400 fewer stored).
 template <class Load, class Keep>
-__host__ __device__ __forceinline__ FixMoments fix_moments_rolled(const FixGroup* axes, const FixGroup* quads, Load&& load, Keep&& keep) {
+__host__ __device__ __forceinline__ FixMoments fix_moments_rolled(const FixGroup* groups, Load&& load, Keep&& keep) {
   const double f0 = load(0);
   const unsigned E0 = fx_hi_word(f0) >> 20;
   const unsigned base = 4u - E0;
@@ -255,8 +254,8 @@ __host__ __device__ __forceinline__ FixMoments fix_moments_rolled(const FixGroup
   m.kb = (int)((E0 - 1019u) << 20);
   unsigned long long R = (conv(0, 2, f0) + 2) >> 2, E = 0, X = 0, Y = 0;
 #pragma unroll 1
-  for (int n = 0; n < 3; ++n) {
-    const FixGroup& g = axes[n];
+  for (int n = 0; n < kFixAxes; ++n) {
+    const FixGroup& g = groups[n];
     const int e = g.sh;
     const unsigned long long half = 1ull << (e - 1);
     const double a = load(g.i), b = load(g.i + NPAIR), c = load(g.j), d = load(g.j + NPAIR);
@@ -268,8 +267,8 @@ __host__ __device__ __forceinline__ FixMoments fix_moments_rolled(const FixGroup
     Y += g.a * (unsigned long long)((long long)(r - s + half) >> e);
   }
 #pragma unroll 1
-  for (int n = 0; n < 6; ++n) {
-    const FixGroup& g = quads[n];
+  for (int n = kFixAxes; n < kFixGroups; ++n) {
+    const FixGroup& g = groups[n];
     const int e = g.sh;
     const unsigned long long half = 1ull << (e - 1);
     const double a = load(g.i), b = load(g.i + NPAIR), c = load(g.j), dd = load(g.j + NPAIR);

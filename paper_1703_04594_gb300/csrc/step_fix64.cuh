@@ -76,11 +76,12 @@ __device__ __forceinline__ bool fix64_wall_strip(const StepScalars& a, int y0) {
 }
 
 // The pull-gather of a strip into its slots sf[i * 32] (sf: the lane's first slot), walls
-// included; yc is the lane's row clamped into the lattice.  Asynchronous copies when Ld caches in
-// L1, waited for here.
+// included; yc is the lane's row clamped into the lattice.  First the copies are issued
+// (asynchronous when Ld caches in L1), then waited for and the ghosts of wall strips written over
+// the clamped rows; in between the caller can issue other loads.
 template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void stage_strip(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
-                                            int x, int y0, int yc, double* __restrict__ sf, Ld ld) {
+__device__ __forceinline__ void stage_issue(const double* __restrict__ fin, const StepScalars& a, int x, int y0, int yc,
+                                            double* __restrict__ sf, Ld ld) {
   const bool wall = fix64_wall_strip<PERIODIC>(a, y0);
   // one pointer per source column (planes < 2^32 elements); a plane's stride and a hop in y are then
   // an addition and an immediate
@@ -105,9 +106,13 @@ __device__ __forceinline__ void stage_strip(const double* __restrict__ fin, cons
       else sf[i * 32] = ld(src);
     }
   }
+}
+template <bool PERIODIC, class Ld>
+__device__ __forceinline__ void stage_finish(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
+                                             int x, int y0, int yc, double* __restrict__ sf, Ld ld) {
   if (Ld::kL1) cp_async_wait_all();
-  if (wall) {
-    // ghost values over the clamped rows copied above; each wall only where the strip reaches it
+  if (fix64_wall_strip<PERIODIC>(a, y0)) {
+    // each wall only where the strip reaches it
     if (y0 < 3) {
       const double b = wall_density_lane(fin, x, a, 0, ld);
 #pragma unroll
@@ -157,7 +162,8 @@ __device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin,
   const bool active = y < a.ly;
   const int yc = active ? y : a.ly - 1;
   sf += lane;
-  stage_strip<PERIODIC>(fin, a, w, x, y0, yc, sf, ld);
+  stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, ld);
+  stage_finish<PERIODIC>(fin, a, w, x, y0, yc, sf, ld);
   if (!active) return;
   FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);  // the same slots, as fixed point
   const FixMoments m = fix_moments([&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });

@@ -2,9 +2,9 @@
 //
 // Work unit: a tile of 32 rows x TX columns of one lattice, one warp per column, processed
 // by one block (TX = warps per block, the autotuned tile width).  All lattices of a batch
-// are laid end to end in one tile index space (prefix sums in BatchLattice::tile_begin, y
-// fastest inside a lattice) and a device table gives each tile's lattice, so everything a
-// block reads about its lattice is uniform across the block.  Each warp runs the same strip
+// are laid end to end in one tile index space (y fastest inside a lattice) and a device table
+// gives each tile's lattice and position, so everything a block reads about its lattice is
+// uniform across the block.  Each warp runs the same strip
 // step as the single-lattice kernels (step_fix64.cuh, which stages its strips in dynamic
 // shared memory, and step_fp32.cuh), so results are bit-identical to lbm_run per lattice.
 //
@@ -39,9 +39,14 @@ namespace d2q37 {
 struct BatchLattice {
   StepArgs a;
   void* f[2];            // state buffers; f[parity] holds the current state
-  long long tile_begin;  // first tile of this lattice in the batch index space
-  int tiles_y;           // ceil(ly / 32)
-  int tiles_x;           // ceil(lx / TX)
+  int tiles_y;  // ceil(ly / 32)
+  int tiles_x;  // ceil(lx / TX)
+};
+
+// One tile of the batch: its lattice and first site (the table spares every thread a search and a
+// 64-bit division).
+struct __align__(16) BatchTile {
+  int lattice, x0, y0, pad;
 };
 
 // The first three words are reset by every persistent launch; `sticky` is not.
@@ -88,26 +93,23 @@ inline size_t batch_smem_bytes(int kind, int warps) {
 }
 
 // Tile t of the batch (32 rows x TX columns, one warp per column, as the single-lattice
-// kernels): its lattice comes from a per-tile table, so everything that depends on the
-// lattice is uniform across the block.
+// kernels): its lattice and position come from the tile table, so everything that depends on
+// the lattice is uniform across the block.
 template <int KIND, bool PERIODIC, class Ld>
-__device__ __forceinline__ void batch_tile(const BatchLattice* __restrict__ L, const unsigned short* __restrict__ tl,
+__device__ __forceinline__ void batch_tile(const BatchLattice* __restrict__ L, const BatchTile* __restrict__ tiles,
                                            long long t, int parity, Ld ld, double* staged) {
   using T = typename KindOf<KIND>::T;
-  const int j = tl[t];
-  const BatchLattice& B = L[j];
-  const long long local = t - B.tile_begin;
-  const int tx = (int)(local / B.tiles_y);
-  const int ty = (int)(local - (long long)tx * B.tiles_y);
-  const int x = tx * (int)blockDim.y + (int)threadIdx.y;
+  const BatchTile tile = tiles[t];
+  const BatchLattice& B = L[tile.lattice];
+  const int x = tile.x0 + (int)threadIdx.y, y0 = tile.y0;
   if (x >= B.a.lx) return;  // uniform per warp
   const T* src = (const T*)B.f[parity];
   T* dst = (T*)B.f[parity ^ 1];
   if constexpr (KIND == kFix64)
-    step_strip_fix64<PERIODIC>(src, dst, B.a, B.a, x, ty * 32, ld, staged + threadIdx.y * (Q * 32));
+    step_strip_fix64<PERIODIC>(src, dst, B.a, B.a, x, y0, ld, staged + threadIdx.y * (Q * 32));
   else
     step_strip_fp32<PERIODIC, KIND == kFp32Scaled || KIND == kFp32ConsScaled, KIND == kFp32Cons || KIND == kFp32ConsScaled>(
-        src, dst, B.a, B.a, x, ty * 32, ld);
+        src, dst, B.a, B.a, x, y0, ld);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
@@ -166,24 +168,24 @@ extern __shared__ double batch_staged[];
 
 template <int KIND, bool PERIODIC>
 __global__ void __launch_bounds__(256) __maxnreg__(batch_max_regs(KIND)) k_batch_step(const BatchLattice* __restrict__ L,
-                                                    const unsigned short* __restrict__ tl, long long total,
+                                                    const BatchTile* __restrict__ tiles, long long total,
                                                     int parity) {
   pdl_trigger();
   pdl_wait();
   const long long t = blockIdx.x;
   if (t >= total) return;
-  batch_tile<KIND, PERIODIC>(L, tl, t, parity, LdReadOnly(), batch_staged);
+  batch_tile<KIND, PERIODIC>(L, tiles, t, parity, LdReadOnly(), batch_staged);
 }
 
 template <int KIND, bool PERIODIC>
 __global__ void __launch_bounds__(256) __maxnreg__(batch_max_regs(KIND)) k_batch_persistent(const BatchLattice* __restrict__ L,
-                                                          const unsigned short* __restrict__ tl, long long total,
+                                                          const BatchTile* __restrict__ tiles, long long total,
                                                           int parity0, int steps, BatchSync* sync, unsigned phantom,
                                                           long long timeout_ns) {
   for (int st = 0; st < steps; ++st) {
     const int parity = (parity0 + st) & 1;
     for (long long t = blockIdx.x; t < total; t += gridDim.x)
-      batch_tile<KIND, PERIODIC>(L, tl, t, parity, LdL2(), batch_staged);
+      batch_tile<KIND, PERIODIC>(L, tiles, t, parity, LdL2(), batch_staged);
     if (st + 1 < steps && !grid_barrier(sync, (unsigned)(st + 1) * gridDim.x + phantom, timeout_ns, st)) return;
   }
 }
@@ -198,7 +200,7 @@ struct lbm_batch {
   int periodic = 0;
   int fp32_scaled = 0;  // FP32 batch with some reference density of 2 or more
   long long total_tiles = 0;
-  unsigned short* dev_tile_lattice = nullptr;  // lattice of every tile
+  BatchTile* dev_tiles = nullptr;
   size_t tile_table_cap = 0;
   std::vector<BatchLattice> host;
   BatchLattice* dev_lattices = nullptr;
@@ -233,7 +235,7 @@ template <int K>
 void* persistent_fn(bool periodic) {
   return periodic ? (void*)k_batch_persistent<K, true> : (void*)k_batch_persistent<K, false>;
 }
-using PerStepKernel = void (*)(const BatchLattice*, const unsigned short*, long long, int);
+using PerStepKernel = void (*)(const BatchLattice*, const BatchTile*, long long, int);
 template <int K>
 PerStepKernel per_step_fn(bool periodic) {
   return periodic ? k_batch_step<K, true> : k_batch_step<K, false>;
@@ -284,12 +286,12 @@ int32_t launch_per_step(lbm_batch* b, int steps, cudaStream_t s) {
   if (b->total_tiles > 0x7fffffffLL) return LBM_EINVAL;
   const size_t smem = batch_smem_bytes(kind_of(b), b->warps_per_block);
   const BatchLattice* L = b->dev_lattices;
-  const unsigned short* tl = b->dev_tile_lattice;
+  const BatchTile* tiles = b->dev_tiles;
   long long total = b->total_tiles;
   for (int st = 0; st < steps; ++st) {
     int par = (b->parity + st) & 1;
     const int32_t st_ = cuda_status(launch_dependent(per_step_kernel(b), dim3((unsigned)total),
-                                                     dim3(32, b->warps_per_block), smem, s, L, tl, total, par));
+                                                     dim3(32, b->warps_per_block), smem, s, L, tiles, total, par));
     if (st_ != LBM_OK) return st_;
   }
   return LBM_OK;
@@ -305,13 +307,13 @@ int32_t launch_persistent(lbm_batch* b, int steps, cudaStream_t s) {
   int32_t st = cuda_status(cudaMemsetAsync(b->dev_sync, 0, kBatchSyncLaunchBytes, s));
   if (st != LBM_OK) return st;
   const BatchLattice* L = b->dev_lattices;
-  const unsigned short* tl = b->dev_tile_lattice;
+  const BatchTile* tiles = b->dev_tiles;
   long long total = b->total_tiles;
   int parity0 = b->parity;
   BatchSync* sync = b->dev_sync;
   unsigned phantom = b->phantom;
   long long timeout = b->timeout_ns;
-  void* args[] = {(void*)&L, (void*)&tl, &total, &parity0, &steps, &sync, &phantom, &timeout};
+  void* args[] = {(void*)&L, (void*)&tiles, &total, &parity0, &steps, &sync, &phantom, &timeout};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(32, wpb);
@@ -350,33 +352,29 @@ int32_t run(lbm_batch* b, int steps, cudaStream_t s) {
   return st;
 }
 
-// Tile layout for tiles of 32 rows x tx columns, and the per-tile lattice table, uploaded
+// Tile layout for tiles of 32 rows x tx columns, and the tile table, uploaded
 // to the device (synchronous; grows the table allocation when needed).
 int32_t relayout(lbm_batch* b, int tx) {
-  long long tiles = 0;
-  for (BatchLattice& L : b->host) {
+  std::vector<BatchTile> table;
+  for (int j = 0; j < b->n; ++j) {
+    BatchLattice& L = b->host[j];
     L.tiles_y = (L.a.ly + 31) / 32;
     L.tiles_x = (L.a.lx + tx - 1) / tx;
-    L.tile_begin = tiles;
-    tiles += (long long)L.tiles_y * L.tiles_x;
+    for (int x = 0; x < L.tiles_x; ++x)
+      for (int y = 0; y < L.tiles_y; ++y) table.push_back({j, x * tx, y * 32, 0});
   }
-  std::vector<unsigned short> table((size_t)tiles);
-  for (int j = 0; j < b->n; ++j) {
-    const BatchLattice& L = b->host[j];
-    std::fill(table.begin() + L.tile_begin, table.begin() + L.tile_begin + (long long)L.tiles_y * L.tiles_x,
-              (unsigned short)j);
-  }
+  const long long tiles = (long long)table.size();
   if ((size_t)tiles > b->tile_table_cap) {
-    if (b->dev_tile_lattice) cudaFree(b->dev_tile_lattice);
-    b->dev_tile_lattice = nullptr;
+    if (b->dev_tiles) cudaFree(b->dev_tiles);
+    b->dev_tiles = nullptr;
     b->tile_table_cap = 0;
-    if (cudaMalloc(&b->dev_tile_lattice, sizeof(unsigned short) * (size_t)tiles) != cudaSuccess) return LBM_ENOMEM;
+    if (cudaMalloc(&b->dev_tiles, sizeof(BatchTile) * (size_t)tiles) != cudaSuccess) return LBM_ENOMEM;
     b->tile_table_cap = (size_t)tiles;
   }
   b->total_tiles = tiles;
   b->warps_per_block = tx;
-  int32_t st = cuda_status(cudaMemcpy(b->dev_tile_lattice, table.data(), sizeof(unsigned short) * (size_t)tiles,
-                                      cudaMemcpyHostToDevice));
+  int32_t st = cuda_status(
+      cudaMemcpy(b->dev_tiles, table.data(), sizeof(BatchTile) * (size_t)tiles, cudaMemcpyHostToDevice));
   if (st != LBM_OK) return st;
   return cuda_status(cudaMemcpy(b->dev_lattices, b->host.data(), sizeof(BatchLattice) * b->n, cudaMemcpyHostToDevice));
 }
@@ -446,7 +444,7 @@ int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* 
   }
   if (relayout(b, 4) != LBM_OK || cudaMemset(b->dev_sync, 0, sizeof(BatchSync)) != cudaSuccess ||
       allow_batch_smem(b) != LBM_OK) {
-    cudaFree(b->dev_tile_lattice);
+    cudaFree(b->dev_tiles);
     cudaFree(b->dev_lattices);
     cudaFree(b->dev_sync);
     delete b;
@@ -563,7 +561,7 @@ int64_t lbm_batch_sites(const lbm_batch* b) {
 
 void lbm_batch_destroy(lbm_batch* b) {
   if (!b) return;
-  cudaFree(b->dev_tile_lattice);
+  cudaFree(b->dev_tiles);
   cudaFree(b->dev_lattices);
   cudaFree(b->dev_sync);
   delete b;

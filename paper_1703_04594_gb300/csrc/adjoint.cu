@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
   if (active) {
     if (ok) contrib = k.om2 * fx_lower_exponent(r.D, K + (1 << 20) - m.kb);
     else contrib = adj_site_float64<PERIODIC>(fin, lam, a, k, x, y, sf);
-    if (PERIODIC || fix64_wall_strip<PERIODIC>(a, y0)) {
+    if (edge_strip(a, y0)) {
       push_strip_edge<PERIODIC>(sf, lam_out, side, a, x, y);
     } else {
       double* col[7];  // row y of column x - vx

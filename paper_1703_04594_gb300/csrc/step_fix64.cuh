@@ -69,11 +69,8 @@ __device__ __forceinline__ double wall_density_lane(const double* __restrict__ f
   return r;
 }
 
-// Whether the strip at rows y0 .. y0 + 31 pulls from a ghost row.
-template <bool PERIODIC>
-__device__ __forceinline__ bool fix64_wall_strip(const StepScalars& a, int y0) {
-  return !PERIODIC && (y0 < 3 || y0 + 32 > a.ly - 3);
-}
+// Whether the strip at rows y0 .. y0 + 31 pulls from beyond the first or the last row.
+__device__ __forceinline__ bool edge_strip(const StepScalars& a, int y0) { return y0 < 3 || y0 + 32 > a.ly - 3; }
 
 // The pull-gather of a strip into its slots sf[i * 32] (sf: the lane's first slot), walls
 // included; yc is the lane's row clamped into the lattice.  First the copies are issued
@@ -82,13 +79,12 @@ __device__ __forceinline__ bool fix64_wall_strip(const StepScalars& a, int y0) {
 template <bool PERIODIC, class Ld>
 __device__ __forceinline__ void stage_issue(const double* __restrict__ fin, const StepScalars& a, int x, int y0, int yc,
                                             double* __restrict__ sf, Ld ld) {
-  const bool wall = fix64_wall_strip<PERIODIC>(a, y0);
   // one pointer per source column (planes < 2^32 elements); a plane's stride and a hop in y are then
   // an addition and an immediate
   const double* col[7];
 #pragma unroll
   for (int d = 0; d < 7; ++d) col[d] = fin + (unsigned)wrap_index(x - (d - 3), a.lx) * (unsigned)a.pitch;
-  if (wall || PERIODIC) {
+  if (edge_strip(a, y0)) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
       const int ys = PERIODIC ? wrap_index(yc - vy(i), a.ly) : min(max(yc - vy(i), 0), a.ly - 1);
@@ -111,7 +107,7 @@ template <bool PERIODIC, class Ld>
 __device__ __forceinline__ void stage_finish(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
                                              int x, int y0, int yc, double* __restrict__ sf, Ld ld) {
   if (Ld::kL1) cp_async_wait_all();
-  if (fix64_wall_strip<PERIODIC>(a, y0)) {
+  if (!PERIODIC && edge_strip(a, y0)) {
     // each wall only where the strip reaches it
     if (y0 < 3) {
       const double b = wall_density_lane(fin, x, a, 0, ld);

@@ -354,8 +354,8 @@ __device__ __forceinline__ void step_strip_fp32(const float* __restrict__ fin, f
 #pragma unroll
   for (int d = 0; d < 7; ++d) col[d] = fin + (unsigned)wrap_index(x - (d - 3), a.lx) * (unsigned)a.pitch;
   float g[Q];
-  const bool wall_warp = !PERIODIC && (y0 < 3 || y0 + 32 > a.ly - 3);
-  if (wall_warp) {
+  const bool edge = y0 < 3 || y0 + 32 > a.ly - 3;
+  if (!PERIODIC && edge) {
     // clamped rows, then the ghost values over them; each wall only where the strip reaches it
 #pragma unroll
     for (int i = 0; i < Q; ++i)
@@ -380,7 +380,7 @@ __device__ __forceinline__ void step_strip_fp32(const float* __restrict__ fin, f
         }
       }
     }
-  } else if (PERIODIC) {
+  } else if (PERIODIC && edge) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) g[i] = ld(col[vx(i) + 3] + i * a.pop + (unsigned)wrap_index(yc - vy(i), a.ly));
   } else {

@@ -61,7 +61,7 @@ constexpr size_t kBatchSyncLaunchBytes = 3 * sizeof(unsigned int);
 namespace {
 
 // Step kinds: the strip functions of the three storage/arithmetic forms.
-// kFp32Scaled: FP32 storage where some lattice has a reference density of 2 or more (the
+// kFp32Scaled: FP32 storage where some lattice has a reference density outside [1/2, 2) (the
 // moment sums read each lattice's scale constants; see step_fp32.cuh); kFp32Cons and
 // kFp32ConsScaled: the same with the conserved-moment correction (LBM_FP32_CONSERVED).
 enum BatchKind { kFp32 = 1, kFix64 = 2, kFp32Scaled = 3, kFp32Cons = 4, kFp32ConsScaled = 5 };
@@ -198,7 +198,7 @@ struct lbm_batch {
   int n = 0;
   int precision = LBM_FP64;
   int periodic = 0;
-  int fp32_scaled = 0;  // FP32 batch with some reference density of 2 or more
+  int fp32_scaled = 0;  // FP32 batch with some reference density outside [1/2, 2)
   long long total_tiles = 0;
   BatchTile* dev_tiles = nullptr;
   size_t tile_table_cap = 0;
@@ -406,7 +406,7 @@ int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* 
     BatchLattice L;
     memset(&L, 0, sizeof(L));
     L.a = make_step_args(p);
-    if (L.a.fix_back != 1.0 / 4503599627370496.0) b->fp32_scaled = 1;
+    if (L.a.fp32_scaled) b->fp32_scaled = 1;
     L.f[0] = f_a[j];
     L.f[1] = f_b[j];
     b->host.push_back(L);

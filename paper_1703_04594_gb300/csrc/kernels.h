@@ -42,6 +42,10 @@ struct StepScalars {
   float f_split_c1, f_split_c2, f_split_s, f_fix_range, f_fix_back;
   int i_split_b1, i_split_b2;  // bit patterns of f_split_c1, f_split_c2
   double fix_back;
+  // fp32_scaled: rho0 outside [1/2, 2), where a lattice's own constants are read; inside it, rho0 and
+  // its energy rho0 D / c^2 in units of 2^-52 (rounded by less than an ulp of rho0)
+  int fp32_scaled;
+  long long rho0_fix, e0_fix;
 };
 
 // Wall tables, read only by the warps next to a wall.

@@ -103,7 +103,7 @@ static cudaError_t launch_fp32(const float* fin, float* fout, const StepArgs& a,
 }
 
 cudaError_t launch_step_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {
-  const bool scaled = a.fix_back != 1.0 / 4503599627370496.0;
+  const bool scaled = a.fp32_scaled;
   if (a.periodic) return scaled ? launch_fp32<true, true>(fin, fout, a, s) : launch_fp32<true, false>(fin, fout, a, s);
   return scaled ? launch_fp32<false, true>(fin, fout, a, s) : launch_fp32<false, false>(fin, fout, a, s);
 }

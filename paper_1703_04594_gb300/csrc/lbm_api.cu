@@ -145,6 +145,11 @@ StepArgs d2q37::make_step_args(const lbm_params* p) {
   memcpy(&a.i_split_b2, &a.f_split_c2, sizeof(int));
   a.fix_back = std::ldexp(1.0, k - 52);
   a.f_fix_back = (float)a.fix_back;
+  a.fp32_scaled = !(p->rho0 >= 0.5 && p->rho0 < 2.0);
+  if (!a.fp32_scaled) {
+    a.rho0_fix = std::llrint(std::ldexp(p->rho0, 52));
+    a.e0_fix = std::llrint(std::ldexp(p->rho0 * (D / C2), 52));
+  }
   for (int i = 0; i < Q; ++i) {
     a.wall_b[i] = wall_multiplier(i, p->t_bottom);
     a.wall_t[i] = wall_multiplier(i, p->t_top);

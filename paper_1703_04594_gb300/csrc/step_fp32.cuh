@@ -19,6 +19,7 @@
 //    f_i^eq - w_i rho0 = w_i [ (rho - rho0) + rho (P_i(s) - 1) ],
 //    so float32 rounds deviations, not whole populations.
 #pragma once
+#include "fixed64.cuh"
 #include "step_fp64.cuh"
 
 namespace d2q37 {
@@ -119,7 +120,7 @@ __device__ __forceinline__ long long join3(int H, int R, int L) {
 // range of the form, |g_i| < 8 * 2^k: a site holding a larger deviation, an infinity or a
 // NaN gets NaN moments, so every population it produces is NaN.  (A float64 fallback for
 // such sites does not fit the step's 80-register budget.)
-// SCALED = false is the common case k = 0 (rho0 < 2), with every constant an immediate;
+// SCALED = false is the common case 1/2 <= rho0 < 2 (k = 0), with every constant an immediate;
 // SCALED = true reads the lattice's constants (a separate instantiation, so the common
 // one keeps its registers).
 // The four exact sums of v_i 2^(52-k) over the 37 values (the lattice's split constants):
@@ -217,11 +218,24 @@ __device__ __forceinline__ void collide_site_fp32(float (&g)[Q], const StepScala
   const SplitConst sc = split_const<SCALED>(a);
   const bool in_range = fix_in_range<SCALED>(g, a);
   const FixSums in = fix_sums(g, sc);
-  const DevMoments<float> m = moments_of<float, SCALED>(in, in_range, a);
-  // float64: density, energy, temperature
-  const double drho = m.drho;
-  const double rho = a.rho0 + drho;
-  const double etot = m.de + a.rho0 * (D / C2);  // sum |v|^2 f
+  // float64: density, energy, temperature.  Unscaled (1/2 <= rho0 < 2), the reference density and its
+  // energy join the integer sums and the sums' scale 2^-52 is an exponent, so that each takes one
+  // conversion of the float64 pipe.
+  const float back_f = SCALED ? a.f_fix_back : 1.0f / 4503599627370496.0f;
+  const float jx = (float)in.X * back_f, jy = (float)in.Y * back_f;
+  double rho, etot;  // etot: sum |v|^2 f
+  float drho_f;
+  if (SCALED) {
+    const double drho = (double)in.R * a.fix_back;
+    rho = a.rho0 + drho;
+    etot = (double)in.E * a.fix_back + a.rho0 * (D / C2);
+    drho_f = (float)drho;
+  } else {
+    rho = fx_lower_exponent(in.R + a.rho0_fix, 52 << 20);
+    etot = fx_lower_exponent(in.E + a.e0_fix, 52 << 20);
+    drho_f = (float)in.R * back_f;
+  }
+  if (!in_range) rho = __longlong_as_double(0x7FF8000000000000LL);  // so every output is NaN
   const float rho_f = (float)rho;
   const float r_f = __frcp_rn(rho_f);
   const double r0 = (double)r_f;
@@ -230,12 +244,11 @@ __device__ __forceinline__ void collide_site_fp32(float (&g)[Q], const StepScala
   // c u = c^2 j / rho with the velocity scale c2_iso in place of c^2 (see StepScalars):
   // with it the float32 equilibrium's first-order momentum is exactly rho u
   const float c2ir_f = (float)(a.c2_iso * inv);
-  const float Ux0 = (float)m.jx * c2ir_f, Uy0 = (float)m.jy * c2ir_f;
+  const float Ux0 = (float)jx * c2ir_f, Uy0 = (float)jy * c2ir_f;
   const float uu = fmaf(Ux0, Ux0, Uy0 * Uy0) * (float)(1.0 / C2);
   // t = T_s - 1 = (c^2 e / rho - |u|^2) / D + tau (1 - tau) |g|^2 / D - 1: the large part in
   // float64, the small |u|^2 / D correction in float32
-  const float t = (float)fma(etot, C2 * inv * (1.0 / D), a.cc.tshift) - uu * (float)(1.0 / D);
-  const float drho_f = (float)drho;
+  const float t = (float)fma(etot, (C2 / D) * inv, a.cc.tshift) - uu * (float)(1.0 / D);
   // float32: Hermite coefficients in deviation form and relaxation
   const float Ux = Ux0 + a.f_cgx, Uy = Uy0 + a.f_cgy;
   const float U = fmaf(Ux, Ux, Uy * Uy) * (float)(1.0 / C2);
@@ -300,7 +313,7 @@ __device__ __forceinline__ void collide_site_fp32(float (&g)[Q], const StepScala
     // energy: + 2 j.g / c + rho |g|^2 / c^2
     const float dJx = fmaf(rho_f, a.f_corr_gx_hi, fmaf(rho_f, a.f_corr_gx_lo, dX));
     const float dJy = fmaf(rho_f, a.f_corr_gy_hi, fmaf(rho_f, a.f_corr_gy_lo, dY));
-    const float dE = fmaf(rho_f, a.f_corr_g2, fmaf(2.0f * m.jx, a.f_corr_gx_hi, fmaf(2.0f * m.jy, a.f_corr_gy_hi, dEs)));
+    const float dE = fmaf(rho_f, a.f_corr_g2, fmaf(2.0f * jx, a.f_corr_gx_hi, fmaf(2.0f * jy, a.f_corr_gy_hi, dEs)));
     const float alpha = dM * a.f_corr_iw;
     const float mf = a.f_corr_m;
     const float gamma = fmaf(-dM, mf, dE) * a.f_corr_ivar;
@@ -318,29 +331,44 @@ __device__ __forceinline__ void collide_site_fp32(float (&g)[Q], const StepScala
   }
 }
 
-// Wall deviation sum_j g_j at (x_s, row) of the seven source columns, summed in float64: lane l takes
-// every fourth population of column l % 8, and two shuffles add the four parts (the same value in the
-// column's four lanes).
+// The unevaluated sum s + e of float32 values, each term's rounding error kept (Knuth's two-sum).
+struct FloatPair {
+  float s, e;
+  __host__ __device__ __forceinline__ void add(float v) {
+    const float t = s + v, z = t - s;
+    e += (s - (t - z)) + (v - z);
+    s = t;
+  }
+};
+
+// Wall deviation sum_j g_j at (x_s, row) of the seven source columns: lane l sums every fourth
+// population of column l % 8, and two shuffles add the four parts (the same value in the column's
+// four lanes).  Compensated float32 sums, because the float64 pipe is busy with the site scalars:
+// summed there, the walls of small lattices took it to 66 %.
 template <class Ld>
 __device__ __forceinline__ float wall_drho_lane(const float* __restrict__ fin, int x, const StepScalars& a, int row, Ld ld) {
   const int lane = threadIdx.x & 31;
   const int d = lane & 7, part = lane >> 3;
-  double r = 0.0;
+  FloatPair r = {0.0f, 0.0f};
   if (d < 7) {
-    const float* src = fin + (long long)wrap_index(x - (d - 3), a.lx) * a.pitch + row;
+    const float* src = fin + ((unsigned)wrap_index(x - (d - 3), a.lx) * (unsigned)a.pitch + (unsigned)row);
 #pragma unroll
     for (int n = 0; n < 10; ++n) {
       const int i = 4 * n + part;
-      if (i < Q) r += (double)ld(src + i * a.pop);
+      if (i < Q) r.add(ld(src + i * a.pop));
     }
   }
-  r += __shfl_xor_sync(0xffffffffu, r, 8);
-  r += __shfl_xor_sync(0xffffffffu, r, 16);
-  return (float)r;
+#pragma unroll
+  for (int m = 8; m <= 16; m <<= 1) {
+    const float s = __shfl_xor_sync(0xffffffffu, r.s, m), e = __shfl_xor_sync(0xffffffffu, r.e, m);
+    r.add(s);
+    r.e += e;
+  }
+  return r.s + r.e;
 }
 
 // One warp-strip of the FP32 shifted step (see step_fp64.cuh for the strip contract).
-// SCALED: the lattice's reference density is 2 or more (see moments_fix); CONSERVE: the
+// SCALED: the lattice's reference density is outside [1/2, 2) (see moments_fix); CONSERVE: the
 // collision restores the exact conserved moments (collide_site_fp32).
 template <bool PERIODIC, bool SCALED, bool CONSERVE, class Ld>
 __device__ __forceinline__ void step_strip_fp32(const float* __restrict__ fin, float* __restrict__ fout,

@@ -103,32 +103,48 @@ __device__ __forceinline__ void stage_issue(const double* __restrict__ fin, cons
     }
   }
 }
+// The ghosts a wall gives one column: population i of the k-th row from the bottom wall, k < vy_i
+// (the opposite population from the top one), from source column d.
+struct WallGhost {
+  unsigned char i, k, opposite, d;
+};
+struct WallGhosts {
+  WallGhost g[32];
+  int n;
+};
+constexpr WallGhosts wall_ghosts() {
+  WallGhosts r = {};
+  for (int i = 0; i < Q; ++i)
+    for (int k = 0; k < vy(i); ++k) {
+      r.g[r.n++] = {(unsigned char)i, (unsigned char)k, (unsigned char)(i > NPAIR ? i - NPAIR : i + NPAIR),
+                    (unsigned char)(vx(i) + 3)};
+    }
+  return r;
+}
+static_assert(wall_ghosts().n <= 32, "one lane per ghost");
+static __constant__ WallGhosts c_wall_ghosts = wall_ghosts();
+
+// The wall sums are formed while the copies arrive, and one product per lane then gives all of a
+// wall's 26 ghosts (in the threads that pull them it took 15, at 64 cycles of the float64 pipe each).
 template <bool PERIODIC, class Ld>
 __device__ __forceinline__ void stage_finish(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
                                              int x, int y0, int yc, double* __restrict__ sf, Ld ld) {
-  if (Ld::kL1) cp_async_wait_all();
   if (!PERIODIC && edge_strip(a, y0)) {
-    // each wall only where the strip reaches it
-    if (y0 < 3) {
-      const double b = wall_density_lane(fin, x, a, 0, ld);
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        if (vy(i) > 0) {
-          const double r = __shfl_sync(0xffffffffu, b, vx(i) + 3);
-          if (yc < vy(i)) sf[i * 32] = r * w.wall_b[i];
-        }
-      }
-    }
-    if (y0 + 32 > a.ly - 3) {
-      const double t = wall_density_lane(fin, x, a, a.ly - 1, ld);
-#pragma unroll
-      for (int i = 0; i < Q; ++i) {
-        if (vy(i) < 0) {
-          const double r = __shfl_sync(0xffffffffu, t, vx(i) + 3);
-          if (yc >= a.ly + vy(i)) sf[i * 32] = r * w.wall_t[i];
-        }
-      }
-    }
+    const int lane = threadIdx.x & 31;
+    double rho[2] = {};  // each wall only where the strip reaches it
+    if (y0 < 3) rho[0] = wall_density_lane(fin, x, a, 0, ld);
+    if (y0 + 32 > a.ly - 3) rho[1] = wall_density_lane(fin, x, a, a.ly - 1, ld);
+    if (Ld::kL1) cp_async_wait_all();
+    __syncwarp();
+    const bool ghost = lane < wall_ghosts().n;
+    const WallGhost g = c_wall_ghosts.g[ghost ? lane : 0];
+    const double r0 = __shfl_sync(0xffffffffu, rho[0], g.d), r1 = __shfl_sync(0xffffffffu, rho[1], 6 - g.d);
+    if (ghost && y0 < 3) sf[g.i * 32 + (g.k - lane)] = r0 * w.wall_b[g.i];
+    const int top = a.ly - 1 - g.k - y0;  // the ghost's row in the strip
+    if (ghost && top >= 0 && top < 32) sf[g.opposite * 32 + (top - lane)] = r1 * w.wall_t[g.opposite];
+    __syncwarp();
+  } else if (Ld::kL1) {
+    cp_async_wait_all();
   }
 }
 

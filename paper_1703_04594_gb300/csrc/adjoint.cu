@@ -135,6 +135,22 @@ __host__ __device__ constexpr int ghost_base(int i, int sign) {
   return sign > 0 ? b[i] : t[i];
 }
 
+// The population of each slot.
+struct GhostSlots {
+  unsigned char bottom[32], top[32];
+};
+constexpr GhostSlots ghost_slots() {
+  GhostSlots r = {};
+  int b = 0, t = 0;
+  for (int i = 0; i < Q; ++i) {
+    for (int k = 0; k < vy(i); ++k) r.bottom[b++] = (unsigned char)i;
+    for (int k = 0; k < -vy(i); ++k) r.top[t++] = (unsigned char)i;
+  }
+  return r;
+}
+static_assert(kGhostSlots <= 32, "one lane per slot");
+__constant__ GhostSlots c_ghost_slots = ghost_slots();
+
 }  // namespace
 
 // The lattice-wide scalars of the adjoint collision, formed once on the host.
@@ -347,40 +363,36 @@ __device__ __forceinline__ void reduce_add_256(const double* __restrict__ part, 
 // Step 2: the wall rows' share of the transposed bc, after step 1 has written every
 // lambda entry: lambda_j(x, 0) += sum over the bottom slots of column x of the slot's value
 // times its ghost's weight w_i P_i(T_bottom), for all j (the ghost values' dependence on
-// rho_w(x) = sum_j f_j(x, 0)), and likewise for row ly - 1.  One thread per column, wall and
-// population j: each forms its column's wall sum in the same fixed order (so the 37 entries
-// of a column receive the same value; the column's 26 slots are read from cache) and adds
-// it to its own entry, so the launch spreads over the GPU instead of running 37 dependent
-// updates per column on a few blocks.  The grid's last block adds the step's dL/dtau
-// partials to *dtau (the reduction needs step 1 complete too, so it shares this launch).
+// rho_w(x) = sum_j f_j(x, 0)), and likewise for row ly - 1.  One warp per column and wall: a lane
+// per slot, a tree of shuffles, and each of the 37 entries receives the same value.  (One thread per
+// entry, each forming its column's sum from the 26 slots, took 41 operations of the float64
+// pipe a thread.)  The grid's last block adds the step's dL/dtau partials to *dtau (the reduction
+// needs step 1 complete too, so it shares this launch).
 __global__ void __launch_bounds__(256) k_adj_walls(const double* __restrict__ side, double* __restrict__ lam,
                                                    StepArgs a, const double* __restrict__ part, long long n_part,
                                                    double* dtau) {
+  pdl_trigger();
   pdl_wait();
   if (blockIdx.x == gridDim.x - 1) {  // uniform per block
     reduce_add_256(part, n_part, dtau);
     return;
   }
-  const long long item = (long long)blockIdx.x * 256 + threadIdx.x;  // (top * lx + x) * Q + j
-  if (item >= 2LL * a.lx * Q) return;
-  const int j = (int)(item % Q);
-  const long long col = item / Q;  // top * lx + x: the slot column of `side`
-  const int top = (int)(col / a.lx);
-  const int x = (int)(col - (long long)top * a.lx);
-  const double* src = side + col * kGhostSlots;
+  const int lane = threadIdx.x & 31;
+  const unsigned col = blockIdx.x * 8u + (threadIdx.x >> 5);  // top * lx + x: the slot column of `side`
+  if (col >= 2u * (unsigned)a.lx) return;  // uniform per warp
+  const bool top = col >= (unsigned)a.lx;
+  const unsigned x = top ? col - (unsigned)a.lx : col;
+  double* const dst = lam + ((long long)x * a.pitch + (top ? a.ly - 1 : 0));
+  const double l0 = dst[lane * a.pop], l1 = lane + 32 < Q ? dst[(lane + 32) * a.pop] : 0.0;
   double wall = 0.0;
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {  // rows in increasing y, then the ghost's weight
-    double t = 0.0;
-    if (top) {
-      for (int r = -vy(i) - 1; r >= 0; --r) t += src[ghost_base(i, -1) + r];
-      wall = vy(i) < 0 ? fma(t, a.wall_t[i], wall) : wall;
-    } else {
-      for (int r = 0; r < vy(i); ++r) t += src[ghost_base(i, 1) + r];
-      wall = vy(i) > 0 ? fma(t, a.wall_b[i], wall) : wall;
-    }
+  if (lane < kGhostSlots) {
+    const double v = side[(long long)col * kGhostSlots + lane];
+    wall = v * (top ? a.wall_t[c_ghost_slots.top[lane]] : a.wall_b[c_ghost_slots.bottom[lane]]);
   }
-  lam[j * a.pop + (long long)x * a.pitch + (top ? a.ly - 1 : 0)] += wall;
+#pragma unroll
+  for (int m = 16; m > 0; m >>= 1) wall += __shfl_xor_sync(0xffffffffu, wall, m);
+  dst[lane * a.pop] = l0 + wall;
+  if (lane + 32 < Q) dst[(lane + 32) * a.pop] = l1 + wall;
 }
 
 // Adds sum(part[0..n)) to *acc in a fixed order (one block of 256 threads).
@@ -458,8 +470,8 @@ cudaError_t launch_adjoint_step(const double* fin, const double* lam_next, doubl
     k_reduce_add<<<1, 256, 0, s>>>(part, adjoint_partial_count(a), dtau);
     return cudaGetLastError();
   }
-  const long long items = 2LL * a.lx * Q;  // (column, wall, population), plus one block for the dtau sum
-  return launch_dependent(k_adj_walls, dim3((unsigned)((items + 255) / 256) + 1), dim3(256), 0, s, side, lam, a, part,
+  const unsigned walls = (2u * (unsigned)a.lx + 7) / 8;  // 8 warps a block, plus one block for the dtau sum
+  return launch_dependent(k_adj_walls, dim3(walls + 1), dim3(256), 0, s, side, lam, a, part,
                           adjoint_partial_count(a), dtau);
 }
 

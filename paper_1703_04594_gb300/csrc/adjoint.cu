@@ -417,8 +417,27 @@ __global__ void __launch_bounds__(128) k_ke_grad(const double* __restrict__ f, d
   for (int i = 0; i < Q; ++i) lam[o + i * a.pop] = h + C * (ux * (double)vx(i) + uy * (double)vy(i));
 }
 
-// Gradient of f^0 = f^eq(rho, u, T) with respect to the four fields, against lambda^0.
-__global__ void __launch_bounds__(128) k_init_adjoint(const double* __restrict__ rho, const double* __restrict__ ux,
+__device__ __noinline__ EqVjp init_vjp_float64(double rho, double ux, double uy, double T, const double* __restrict__ lam,
+                                               long long pop) {
+  return eq_vjp_pairs(rho, ux, uy, T - 1.0, [&](int i) { return __ldg(lam + i * pop); });
+}
+
+// A site's lambda as fix_mu_moments reads it, without populations to weigh it with.
+struct InitIo {
+  const double* lam;
+  unsigned pop;
+  __device__ __forceinline__ const double* at(int i) const { return lam + (unsigned long long)pop * (unsigned)i; }
+  __device__ __forceinline__ double mu(const double* h, int k) const {
+    return __ldg(k ? h + (unsigned long long)pop * NPAIR : h);
+  }
+  __device__ __forceinline__ FxHalves fixed(const double*, int) const { return FxHalves{0, 0}; }
+  __device__ __forceinline__ void keep(const double*, int, FxHalves) const {}
+};
+
+// Gradient of f^0 = f^eq(rho, u, T) with respect to the four fields, against lambda^0: the moments of
+// lambda^0 in fixed point as in step 1 (256 x 512: 24 us; one float64 polynomial and its
+// derivatives per opposite pair, the route of sites out of its range, took 171 us).
+__global__ void __launch_bounds__(128, 4) k_init_adjoint(const double* __restrict__ rho, const double* __restrict__ ux,
                                                       const double* __restrict__ uy, const double* __restrict__ T,
                                                       const double* __restrict__ lam, double* __restrict__ g_rho,
                                                       double* __restrict__ g_ux, double* __restrict__ g_uy,
@@ -427,8 +446,27 @@ __global__ void __launch_bounds__(128) k_init_adjoint(const double* __restrict__
   const int y = blockIdx.x * 32 + threadIdx.x;
   if (x >= a.lx || y >= a.ly) return;
   const long long fi = (long long)x * a.ly + y;
-  const long long o = (long long)x * a.pitch + y;
-  const EqVjp G = eq_vjp_pairs(rho[fi], ux[fi], uy[fi], T[fi] - 1.0, [&](int i) { return __ldg(lam + o + i * a.pop); });
+  const double* l = lam + (long long)x * a.pitch + y;
+  unsigned top = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) top = max(top, __ldg(reinterpret_cast<const unsigned*>(l + i * a.pop) + 1) & 0x7fffffffu);
+  const unsigned E = top == 0u ? 512u : top >> 20;
+  const double r = rho[fi], u = ux[fi], v = uy[fi], t = T[fi];
+  int kb;
+  const FixScalars s = fix_scalars_of(r, u, v, t, kb);
+  EqVjp G = {};
+  if (s.ok && E - 100u < 978u) {
+    const int K = (1080 - (int)E) << 20;
+    const FixGradients g = fix_gradients(s, fix_mu_moments(K + (1 << 20), c_fix_groups, InitIo{l, (unsigned)a.pop}));
+    if (top != 0u) {  // lambda = 0: no rounding residue
+      const int K4 = K + (4 << 20);
+      const double rc = r * C;
+      G = {fx_lower_exponent(g.Gr, K4), rc * fx_lower_exponent(g.GX, K4), rc * fx_lower_exponent(g.GY, K4),
+           r * fx_lower_exponent(g.Gt, K4)};
+    }
+  } else {
+    G = init_vjp_float64(r, u, v, t, l, a.pop);
+  }
   g_rho[fi] = G.Grho;
   g_ux[fi] = G.Gux;
   g_uy[fi] = G.Guy;

@@ -189,8 +189,13 @@ struct FixVjp {
   long long D;       // tau^2 d/dtau of the site, in units of 2^(k - K - 1)
 };
 
-__host__ __device__ __forceinline__ FixVjp fix_vjp(const FixMoments& f, const FixScalars& v, const FixMu& m,
-                                                   const FixConsts& k, const AdjFixConsts& ka) {
+// The derivatives of sum_i mu_i f^eq_i / rho, in units of 2^(-4 - K): G_rho and, per unit density, those
+// with respect to X, Y and t.
+struct FixGradients {
+  long long Gr, GX, GY, Gt;
+};
+
+__host__ __device__ __forceinline__ FixGradients fix_gradients(const FixScalars& v, const FixMu& m) {
   const long long X = v.X, Y = v.Y, XX = v.XX, YY = v.YY, U = v.U, t = v.t;
   const FxHalves xh = fx_halves(X), yh = fx_halves(Y), xxh = fx_halves(XX), yyh = fx_halves(YY), th = fx_halves(t),
                  uh = fx_halves(U);
@@ -285,12 +290,20 @@ __host__ __device__ __forceinline__ FixVjp fix_vjp(const FixMoments& f, const Fi
   g.add(m02, fx_halves(e0 - (YY >> 4) - (YY >> 5)));
   g.add(m11, fx_halves(-((XY * 3) >> 4)));
   const long long Gt = g.high(7) + high2;
+  return {Gr, GX, GY, Gt};
+}
+
+__host__ __device__ __forceinline__ FixVjp fix_vjp(const FixMoments& f, const FixScalars& v, const FixMu& m,
+                                                   const FixConsts& k, const AdjFixConsts& ka) {
+  const FixGradients G = fix_gradients(v, m);
+  const long long Gr = G.Gr, GX = G.GX, GY = G.GY, Gt = G.Gt;
+  constexpr long long one = 1LL << 60;
   // nu = (d f^eq / d(rho, J, E))^T mu through u = J / rho, T = (E / rho - |u|^2) / D (per unit
   // density): nu_rho = G_rho - G_X X0 - G_Y Y0 + G_t (|u|^2 - D T) / 2 ..., with
   // |u|^2 - (E / rho) / 2 = kap; c nu_J = c^2 G_X - X0 G_t; nu_E = G_t / 2
   const FxHalves gxh = fx_halves(GX), gyh = fx_halves(GY), gth = fx_halves(Gt);
   const FxHalves x0 = fx_halves(v.X0), y0 = fx_halves(v.Y0);
-  const long long kap = (v.e + 2 * ka.tg - (t >> 3) - one) << 2;                 // [62], below 1.6
+  const long long kap = (v.e + 2 * ka.tg - (v.t >> 3) - one) << 2;                 // [62], below 1.6
   const long long nR = Gr - fx_smul(gxh, x0) - fx_smul(gyh, y0) + fx_smul(gth, fx_halves(kap)) * 4;
   const FxHalves c2 = fx_halves(kFxC2_62);
   const FxHalves nx = fx_halves(fx_smul(gxh, c2) * 4 - fx_smul(gth, x0));

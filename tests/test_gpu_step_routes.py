@@ -101,3 +101,28 @@ def test_initial_state_and_fields_on_both_routes(lx, ly, rho0):
         assert float((a.cpu() - b).abs().max()) <= 1e-12 * float(b.abs().max())
     ke = float(OL.kinetic_energy(host))
     assert abs(float(lbm.kinetic_energy(p, f)) - ke) <= 1e-12 * ke
+
+
+@pytest.mark.parametrize("lx,ly", [(4, 6), (5, 33), (70, 131)])
+@pytest.mark.parametrize("scale,wide", [(1.0, 0.1), (1e-200, 0.1), (3e5, 0.9)])
+def test_gradient_of_the_initial_state_on_both_routes(lx, ly, scale, wide):
+    """lbm_init_adjoint against reverse mode through the oracle's equilibrium, with fields inside the
+    fixed-point range (wide = 0.1) and on both sides of it: 1e-13 of what a field's term can reach
+    (sum_i |lambda_i| w_i times the density where the field is not the density, times 40)."""
+    require_gpu()
+    p = lbm.Params(lx, ly)
+    g = torch.Generator().manual_seed(29)
+    rho = 0.5 + torch.rand(lx, ly, dtype=torch.float64, generator=g)
+    ux, uy = ((torch.rand(2, lx, ly, dtype=torch.float64, generator=g) - 0.5) * wide).unbind(0)
+    T = 1.0 + (torch.rand(lx, ly, dtype=torch.float64, generator=g) - 0.5) * wide
+    fields = [t.contiguous().requires_grad_() for t in (rho, ux, uy, T)]
+    lam = torch.randn(37, lx, ly, dtype=torch.float64, generator=g)
+    lam[:, 1, 2] = 0.0
+    lam_dev = lbm.empty_state(p)
+    lam_dev[:, :, :ly] = lam.cuda() * scale
+    want = torch.autograd.grad((OL.init_equilibrium(*fields) * lam).sum(), fields)
+    got = lbm.init_adjoint(p, *[t.detach().cuda() for t in fields], lam_dev)
+    reach = 40.0 * (lam.abs() * torch.tensor(lbm.model()[1], dtype=torch.float64)[:, None, None]).sum(0) * rho.clamp(min=1.0)
+    for a, b in zip(got, want):
+        assert float(((a.cpu() / scale - b).abs() - 1e-13 * reach).max()) <= 0.0
+        assert float(a[1, 2]) == 0.0

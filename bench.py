@@ -9,7 +9,7 @@ lattice (one kernel launch).  Each state buffer is 9.9 GB, far larger than the 1
 L2, so no L2 flush is needed between steps.
 
 The default line also carries the other forms of the step, each with its own roofline,
-clock samples and baseline: ``fp64_fixed_relax`` (float64 states, fixed-point relaxation),
+clock samples and baseline: ``fp64_fixed_relax`` (LBM_FP64_FIXED, the same kernel today),
 ``fp32`` (FP32 shifted storage, same lattice), ``batch_fp64`` / ``batch_fp32`` (256
 independent RT lattices, Lx in 128..1024, Ly = 2 Lx, K steps, against looping the
 single-lattice kernel) and ``adjoint`` (gradient of the kinetic energy after 500 steps of a
@@ -41,9 +41,11 @@ sys.path.insert(0, ROOT)
 LX, LY, SEED = 4096, 8192, 2
 TAU, GY, T_BOTTOM, T_TOP = 0.8, -1e-4, 1.15, 0.85
 
-# Algorithmic work per site of the fused FP64 step: the factored collision (moments as
-# pair sums grouped by their integer velocity weights, per-shell Hermite coefficients, one
-# even/odd Horner pair per opposite pair, BGK relaxation), FMA = 2 flops:
+# Algorithmic work per site of a float64 step (what the separate and layout variants, which
+# collide in float64, are measured against; the fused step's collision is in integers and its
+# roofline is HBM): the factored collision (moments as pair sums grouped by their integer
+# velocity weights, per-shell Hermite coefficients, one even/odd Horner pair per opposite pair,
+# BGK relaxation), FMA = 2 flops:
 #   138 add + 97 mul + 138 fma + 1 div = 512 flops, 374 operations.
 # tests/test_flop_count.py counts it mechanically on a formulation checked against the
 # oracle's collision.
@@ -102,10 +104,10 @@ def _args():
     ap.add_argument("--precision", choices=["fp64", "fp32", "fp32c", "fp64fix"], default="fp64",
                     help="fp32 = FP32 shifted-deviation storage (fused only); fp32c = the same storage with "
                          "the conserved-moment correction; fp64fix = float64 storage "
-                         "with the fixed-point relaxation (fused only)")
+                         "as LBM_FP64_FIXED (fused only; the kernel of fp64)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-fixed", action="store_true",
-                    help="skip the extra timing of the fixed-point-relaxation FP64 step")
+                    help="skip the extra timing of the LBM_FP64_FIXED step")
     ap.add_argument("--no-forms", action="store_true",
                     help="skip the FP32, batched and adjoint forms that the default line adds")
     ap.add_argument("--batch-kind", choices=["uneven", "small"], default="uneven",
@@ -304,7 +306,7 @@ def run_ours(a):
     bufs = [fa, fb]
     # the float64 FMA rate measured by the library's probe kernel (TFLOP/s, FMA = 2 flops),
     # beside the peak derived from unit counts and the maximum clock
-    fp64_measured = 2 * lbm.probe_peak(lbm.PROBE_DFMA) / 1e12 if not (fp32 or fix) else None
+    fp64_measured = 2 * lbm.probe_peak(lbm.PROBE_DFMA) / 1e12 if a.variant != "fused" else None
     for k in range(a.warmup):
         one_step(bufs[k % 2], bufs[(k + 1) % 2])
     torch.cuda.synchronize()
@@ -329,10 +331,11 @@ def run_ours(a):
 
     # dominant kernel: the fused step is the only launch of a fused bench step
     kern_ms = statistics.mean(per_step)
-    if fp32 or fix:
+    hbm_bound = fp32 or fix or a.variant == "fused"
+    if hbm_bound:
         achieved = (BYTES_PER_SITE_FP32 if fp32 else BYTES_PER_SITE_FP64) * sites / (kern_ms * 1e-3) / 1e9
         roofline = {"bound": "hbm", "achieved": achieved, "peak": HBM_PEAK_GBS, "unit": "GB/s",
-                    "frac": achieved / HBM_PEAK_GBS, "traffic": traffic(a.precision, sites),
+                    "frac": achieved / HBM_PEAK_GBS, "traffic": traffic(a.precision if fp32 or fix else "fused", sites),
                     "kernel": "k_step_fp32" if fp32 else "k_step_fix64",
                     "peak_source": HBM_PEAK_SOURCE}
     else:
@@ -341,8 +344,7 @@ def run_ours(a):
                     "frac": achieved / FP64_PEAK_TFLOPS, "traffic": traffic(a.variant, sites),
                     "peak_measured": fp64_measured,
                     "frac_of_measured": achieved / fp64_measured if fp64_measured else None,
-                    "kernel": {"fused": "k_step_fp64", "separate": "whole step (3 kernels)",
-                               "push": "whole step (3 kernels)", "aos": "k_step_layout<AoS>",
+                    "kernel": {"separate": "whole step (3 kernels)", "push": "whole step (3 kernels)", "aos": "k_step_layout<AoS>",
                                "psoa": "k_step_layout<PSoA>", "caosoa": "k_step_layout<CAoSoA>"}[a.variant],
                     "peak_source": "152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz",
                     "hbm_gbs_equiv": BYTES_PER_SITE_FP64 * sites / (kern_ms * 1e-3) / 1e9}
@@ -389,8 +391,8 @@ def run_ours(a):
         f_gbs = BYTES_PER_SITE_FP64 * sites / (f_kern * 1e-3) / 1e9
         fixed_line = {"value": whole_job_mlups(sites, a.steps, world, f_ms), "unit": "MLUPS",
                       "ms_per_step": f_kern, "dtype": "f64+i64", "kernel": "k_step_fix64",
-                      "what": "float64 states; equilibrium and relaxation in 64-bit fixed point on the "
-                              "integer pipes (float64 outside its range); same parity bars as FP64",
+                      "what": "LBM_FP64_FIXED: float64 states, the collision in 64-bit fixed point on the integer "
+                              "pipes (float64 outside its range), the kernel that LBM_FP64 runs too",
                       "roofline": {"bound": "hbm", "achieved": f_gbs, "peak": HBM_PEAK_GBS, "unit": "GB/s",
                                    "frac": f_gbs / HBM_PEAK_GBS,
                                    "traffic": traffic("fp64fix", sites),
@@ -434,7 +436,7 @@ def run_ours(a):
     if rank == 0:
         line = {"metric": "D2Q37 MLUPS", "value": value, "unit": "MLUPS", "n_gpus": world, "steps": a.steps,
                 "warmup": a.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
-                "vs_baseline": None, "dtype": "f32+i64+f64" if fp32 else ("f64+i64" if fix else "f64"),
+                "vs_baseline": None, "dtype": "f32+i64+f64" if fp32 else ("f64+i64" if hbm_bound else "f64"),
                 "data": "synthetic",
                 "config": headline_config(lx, ly, a.variant, a.precision, world),
                 "roofline": roofline, "e2e": e2e,
@@ -452,7 +454,7 @@ def run_ours(a):
         dist.destroy_process_group()
 
 
-DTYPE = {"fp32": "f32+i64+f64", "fp32c": "f32+i64+f64", "fp64fix": "f64+i64", "fp64": "f64"}
+DTYPE = {"fp32": "f32+i64+f64", "fp32c": "f32+i64+f64", "fp64fix": "f64+i64", "fp64": "f64+i64"}
 
 
 def prec_enum(lbm, precision):
@@ -593,13 +595,11 @@ def time_batch(b, mode_cfg, steps, warmup, graph=False):
 def batch_roofline(precision, sites, ms_step, cfg):
     from paper_1703_04594_gb300 import lbm
 
-    kname = {"fp32": "fp32", "fp32c": "fp32 conserved", "fp64fix": "fix64", "fp64": "double"}[precision]
+    kname = {"fp32": "fp32", "fp32c": "fp32 conserved", "fp64fix": "fix64", "fp64": "fix64"}[precision]
     kernel = ("k_batch_persistent<" if cfg["mode"] == lbm.BATCH_PERSISTENT else "k_batch_step<") + kname + ">"
     # the captures are of the per-step kernel
-    tr = (traffic({"fp32": "batch_fp32", "fp64": "batch_fp64"}.get(precision, ""), sites)
+    tr = (traffic({"fp32": "batch_fp32", "fp64": "batch_fp64", "fp64fix": "batch_fp64"}.get(precision, ""), sites)
           if cfg["mode"] == lbm.BATCH_PER_STEP else None)
-    if precision == "fp64":
-        return kernel_roofline("alu", FLOPS_PER_SITE_FP64, sites, ms_step, kernel, tr)
     return kernel_roofline("hbm", BYTES_PER_SITE_FP32 if precision in ("fp32", "fp32c") else BYTES_PER_SITE_FP64, sites,
                            ms_step, kernel, tr)
 
@@ -786,8 +786,8 @@ def adjoint_form(a, repeats, precision="fp64", seed=5):
         return tg / repeats, tf / repeats
 
     # the default schedule, and the same gradient under two others: the segments recomputed
-    # with the float64 step (the default recomputes them with the fixed-point relaxation),
-    # and every state kept in HBM (no recomputation)
+    # as LBM_FP64 (the default recomputes them as LBM_FP64_FIXED, the same kernel), and every
+    # state kept in HBM (no recomputation)
     with ClockSampler(0) as clk:
         t_grad, t_fwd = timed_against_forward(gradient)
     other = {"float64_recomputation": timed_against_forward(lambda: gradient(recompute=lbm.FP64)),
@@ -802,8 +802,8 @@ def adjoint_form(a, repeats, precision="fp64", seed=5):
                     "adjoint step per segment, per site and forward step",
             "workload": f"dE/d(a_1..a_8, tau), E = kinetic energy after {n} steps of {lx}x{ly}, checkpoints "
                         f"every {every}", "repeats": repeats,
-            "forward_steps": "fixed-point relaxation" if precision == "fp64fix" else "float64",
-            "recomputed_steps": "fixed-point relaxation",
+            "forward_steps": "LBM_FP64_FIXED" if precision == "fp64fix" else "LBM_FP64",
+            "recomputed_steps": "LBM_FP64_FIXED",
             "gradient_s": t_grad, "forward_s": t_fwd, "gradient_over_forward": t_grad / t_fwd,
             "forward_baseline": {"value": whole_job_mlups(sites, n, 1, t_fwd * 1e3), "unit": "MLUPS",
                                  "what": "the same 500 forward steps and the energy, no gradient"},
@@ -827,7 +827,7 @@ def run_adjoint(a):
         line = {"metric": "D2Q37 MLUPS (gradient: forward + checkpointed adjoint)", "value": r["value"],
                 "unit": "MLUPS", "n_gpus": world, "steps": a.steps, "warmup": a.warmup,
                 "ms_per_step": r["gradient_s"] * 1e3 / ADJ_N, "higher_is_better": True, "scaling": "weak",
-                "vs_baseline": None, "dtype": "f64+i64" if a.precision == "fp64fix" else "f64",
+                "vs_baseline": None, "dtype": "f64+i64",
                 "data": "synthetic",
                 "config": {"workload": r["workload"], "checkpoint_every": ADJ_EVERY, "repeats": r["repeats"],
                            "forward_steps": r["forward_steps"], "recomputed_steps": r["recomputed_steps"]},

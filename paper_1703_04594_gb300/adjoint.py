@@ -8,14 +8,10 @@ the library's hand-written adjoint kernels (``lbm_adjoint_step``, ``lbm_init_adj
 example ``inputs.rt_fields`` with ``modes.a.requires_grad_()``) to get gradients with
 respect to interface-mode amplitudes.
 
-The forward steps run in the precision of ``params``: FP64, or FP64 with the fixed-point
-relaxation (LBM_FP64_FIXED, the same states within rounding), so the energy is that of the
-plain forward run bit for bit; the recomputation runs in ``recompute_precision``, by
-default the fixed-point relaxation (2.8x faster on GB300 than the float64 step): the
-recomputed states are only the points the adjoint linearises at, and they agree with the
-forward pass's to float64 rounding (the gradient agrees with a float64 recomputation's
-to ~1e-12).  ``recompute_precision=LBM_FP64`` recomputes with the float64 step; the
-adjoint steps are the FP64 ones either way.
+The forward steps run in the precision of ``params`` (LBM_FP64 or LBM_FP64_FIXED, which run
+the same kernel), so the energy is that of the plain forward run bit for bit; the
+recomputation runs in ``recompute_precision``, by default LBM_FP64_FIXED, so the recomputed
+states are the forward pass's.  The adjoint steps are the FP64 ones either way.
 
 Memory: the forward pass keeps a checkpoint every ``every`` steps (default ceil(sqrt(N)));
 the backward pass recomputes each segment's states from its checkpoint, newest segment

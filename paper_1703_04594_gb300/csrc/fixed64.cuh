@@ -4,8 +4,10 @@
 // its integer pipes issue 64 operations per clock per SM.  A signed or unsigned 64 x 64 ->
 // high-64 product (a handful of IMAD instructions) then costs a fraction of one DFMA.  The
 // helpers below move values between float64 and signed 64-bit fixed point (value = X * 2^-k)
-// with integer instructions, except fx_to_double_dp, which uses the float64 pipe's I2F on
-// purpose (that pipe is otherwise idle in the fixed-point kernels).
+// with integer instructions, except fx_lower_exponent, which uses the float64 pipe's I2F on
+// purpose (that pipe is otherwise nearly idle in the fixed-point kernels).  The kernels form their
+// products with fx_smul (site_fix64.cuh); the high-64 products and fx_to_double here are the exact
+// forms that the host tests hold them and each other to.
 #pragma once
 #include <stdint.h>
 
@@ -36,9 +38,7 @@ __host__ __device__ __forceinline__ long long fx_from_double(double v, int k, in
   return (x ^ s) - s;
 }
 
-// X * 2^-k as a float64, rounded half up in magnitude; integer instructions only.  (The
-// kernels use fx_to_double_dp below, which balances their pipes better; this form is the
-// integer-pipe alternative.)
+// X * 2^-k as a float64, rounded half up in magnitude; integer instructions only.
 // Valid for 0 < 1086 - clz(|X|) - k < 2047 (normal results), which holds for every use here.
 __host__ __device__ __forceinline__ double fx_to_double(long long X, int k) {
   const long long s = X >> 63;
@@ -63,15 +63,7 @@ __host__ __device__ __forceinline__ double fx_to_double(long long X, int k) {
 #endif
 }
 
-// X * 2^-k through the float64 pipe: one I2F (exact round to nearest) and an integer
-// subtraction from the exponent field.  Valid for normal results; 0 stays 0.  Used to move
-// part of the conversion work from the integer pipes to the otherwise idle float64 pipe.
-__device__ __forceinline__ double fx_to_double_dp(long long X, int k) {
-  const long long b = __double_as_longlong(__ll2double_rn(X)) - ((long long)k << 52);
-  return X == 0 ? 0.0 : __longlong_as_double(b);
-}
-
-// The same for 0 <= k <= 1022 without a test for zero: the I2F result's high word h is 0
+// X * 2^-k for 0 <= k <= 1022 through the float64 pipe, without a test for zero: the I2F result's high word h is 0
 // for X = 0 and at least 0x3FF00000 otherwise (|X| >= 1; a sign bit makes it larger
 // still), so subtracting min(h, k << 20) leaves 0 at 0 and lowers the exponent field of
 // every other value by k.

@@ -60,8 +60,11 @@ __device__ __forceinline__ Fix3 split3(float v, const SplitConst& k) {
 }
 
 // Two float32 in one 64-bit register: one instruction issues both operations (the same roundings).
-// The FP32 forms are bound by issue before memory, so the splits of an opposite pair share theirs:
-// 1021 x 2050 conserved, 4 steps: 0.546 -> 0.528 ms; 2048 x 8192, 4 steps: 3.29 -> 3.24 ms.
+// The FP32 forms are bound by issue before memory, so the splits of an opposite pair share theirs,
+// and two pairs of a shell share their relaxation (the populations are listed so that pairs j and
+// j + 1, j odd, are of one shell).  1021 x 2050 conserved, 4 steps: 0.546 -> 0.514 ms; 2048 x 8192,
+// 4 steps: 3.29 -> 3.16 ms.  (Splitting by the relaxation's pairs too: 0.510 and 3.16 ms, but 256
+// small lattices, where the 80 registers spill, 1.77 -> 1.86 ms.)
 __device__ __forceinline__ unsigned long long f2_pack(float a, float b) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
@@ -77,6 +80,11 @@ __device__ __forceinline__ unsigned long long f2_sub(unsigned long long a, unsig
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b, unsigned long long c) {
   unsigned long long r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
@@ -84,6 +92,13 @@ __device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsig
 }
 __device__ __forceinline__ int f2_lo(unsigned long long v) { return (int)(unsigned)v; }
 __device__ __forceinline__ int f2_hi(unsigned long long v) { return (int)(unsigned)(v >> 32); }
+
+constexpr bool shells_in_twos() {
+  for (int j = 1; j < NPAIR; j += 2)
+    if (shell(j) != shell(j + 1)) return false;
+  return true;
+}
+static_assert(shells_in_twos(), "the relaxation takes two opposite pairs of a shell at once");
 
 // split3 of two values at once.
 __device__ __forceinline__ void split3_pair(float a, float b, const SplitConst& k, Fix3& za, Fix3& zb) {
@@ -112,8 +127,8 @@ __device__ __forceinline__ Fix2 split2(float v, const SplitConst& k) {
   return {__float_as_int(h1) - k.b1, __float_as_int(h2) - k.b2};
 }
 
-__device__ __forceinline__ void split2_pair(float a, float b, const SplitConst& k, Fix2& za, Fix2& zb) {
-  const unsigned long long v = f2_pack(a, b), c1 = f2_pack(k.c1, k.c1);
+__device__ __forceinline__ void split2_packed(unsigned long long v, const SplitConst& k, Fix2& za, Fix2& zb) {
+  const unsigned long long c1 = f2_pack(k.c1, k.c1);
   const unsigned long long h1 = f2_add(v, c1);
   const unsigned long long h2 = f2_add(f2_sub(v, f2_sub(h1, c1)), f2_pack(k.c2, k.c2));
   za = {f2_lo(h1) - k.b1, f2_lo(h2) - k.b2};
@@ -124,10 +139,15 @@ __device__ __forceinline__ void split2_pair(float a, float b, const SplitConst& 
 // two lanes of split2.
 struct OutSums {
   int rH = 0, rR = 0, eH = 0, eR = 0, xH = 0, xR = 0, yH = 0, yR = 0;
-  // one opposite pair (v, -v): the sum and difference of the two values' lanes
-  __device__ __forceinline__ void add_pair(float a, float b, int vx, int vy, const SplitConst& k) {
-    Fix2 za, zb;
-    split2_pair(a, b, k, za, zb);
+  // two opposite pairs (v, -v), packed: p holds the values at v, m those at -v
+  __device__ __forceinline__ void add_pairs(unsigned long long p, unsigned long long m, int j, int l, const SplitConst& k) {
+    Fix2 p1, p2, m1, m2;
+    split2_packed(p, k, p1, p2);
+    split2_packed(m, k, m1, m2);
+    add(p1, m1, rep_vx(j), rep_vy(j));
+    add(p2, m2, rep_vx(l), rep_vy(l));
+  }
+  __device__ __forceinline__ void add(Fix2 za, Fix2 zb, int vx, int vy) {
     const int PH = za.H + zb.H, PR = za.R + zb.R, MH = za.H - zb.H, MR = za.R - zb.R;
     const int q = vx * vx + vy * vy;
     rH += PH;
@@ -335,19 +355,28 @@ __device__ __forceinline__ void collide_site_fp32(float (&g)[Q], const StepScala
   };
   out(0, fmaf(om1, g[0], K0[0]));
   if (CONSERVE) os.add_rest(g[0], sc);
+  const unsigned long long om1_2 = f2_pack(om1, om1);
 #pragma unroll
-  for (int j = 1; j <= NPAIR; ++j) {
-    const int sh = shell(j), vxk = rep_vx(j), vyk = rep_vy(j);
-    float s;
-    if (vyk == 0) s = X[vxk];
-    else if (vxk == 0) s = Y[vyk];
-    else s = vyk > 0 ? X[vxk] + Y[vyk] : X[vxk] - Y[-vyk];
-    const float s2 = s * s;
-    const float E = fmaf(fmaf(K4[sh], s2, K2[sh]), s2, K0[sh]);
-    const float O = s * fmaf(K3[sh], s2, K1[sh]);
-    out(j, fmaf(om1, g[j], E + O));
-    out(j + NPAIR, fmaf(om1, g[j + NPAIR], E - O));
-    if (CONSERVE) os.add_pair(g[j], g[j + NPAIR], vxk, vyk, sc);
+  for (int j = 1; j < NPAIR; j += 2) {
+    const int l = j + 1;  // two pairs, of one shell, at once
+    const int sh = shell(j);
+    const auto along = [&](int k) {
+      const int vxk = rep_vx(k), vyk = rep_vy(k);
+      if (vyk == 0) return X[vxk];
+      if (vxk == 0) return Y[vyk];
+      return vyk > 0 ? X[vxk] + Y[vyk] : X[vxk] - Y[-vyk];
+    };
+    const unsigned long long s = f2_pack(along(j), along(l)), s2 = f2_mul(s, s);
+    const auto dup = [](float v) { return f2_pack(v, v); };
+    const unsigned long long E = f2_fma(f2_fma(dup(K4[sh]), s2, dup(K2[sh])), s2, dup(K0[sh]));
+    const unsigned long long O = f2_mul(s, f2_fma(dup(K3[sh]), s2, dup(K1[sh])));
+    const unsigned long long p = f2_fma(om1_2, f2_pack(g[j], g[l]), f2_add(E, O));
+    const unsigned long long m = f2_fma(om1_2, f2_pack(g[j + NPAIR], g[l + NPAIR]), f2_sub(E, O));
+    out(j, __int_as_float(f2_lo(p)));
+    out(j + NPAIR, __int_as_float(f2_lo(m)));
+    out(l, __int_as_float(f2_hi(p)));
+    out(l + NPAIR, __int_as_float(f2_hi(m)));
+    if (CONSERVE) os.add_pairs(p, m, j, l, sc);
   }
   if constexpr (CONSERVE) {
     // What the outputs lack, in integers: the exact input sums (units of 2^(k-52)) minus the
@@ -370,12 +399,18 @@ __device__ __forceinline__ void collide_site_fp32(float (&g)[Q], const StepScala
     const float bx = a.f_c2_iso * dJx, by = a.f_c2_iso * dJy;
     store(0, g[0] + (float)w_shell(0) * fmaf(gamma, -mf, alpha));
 #pragma unroll
-    for (int j = 1; j <= NPAIR; ++j) {
+    for (int j = 1; j < NPAIR; j += 2) {
+      const int l = j + 1;
       const float ws = (float)w_shell(shell(j));
-      const float A = ws * fmaf(gamma, (float)v2(j) - mf, alpha);
-      const float B = fmaf(ws * (float)rep_vx(j), bx, (ws * (float)rep_vy(j)) * by);
-      store(j, g[j] + (A + B));
-      store(j + NPAIR, g[j + NPAIR] + (A - B));
+      const float A1 = ws * fmaf(gamma, (float)v2(j) - mf, alpha);
+      const auto along = [&](int k) { return fmaf(ws * (float)rep_vx(k), bx, (ws * (float)rep_vy(k)) * by); };
+      const unsigned long long A = f2_pack(A1, A1), B = f2_pack(along(j), along(l));
+      const unsigned long long p = f2_add(f2_pack(g[j], g[l]), f2_add(A, B));
+      const unsigned long long m = f2_add(f2_pack(g[j + NPAIR], g[l + NPAIR]), f2_sub(A, B));
+      store(j, __int_as_float(f2_lo(p)));
+      store(l, __int_as_float(f2_hi(p)));
+      store(j + NPAIR, __int_as_float(f2_lo(m)));
+      store(l + NPAIR, __int_as_float(f2_hi(m)));
     }
   }
 }

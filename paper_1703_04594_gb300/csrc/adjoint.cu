@@ -264,11 +264,12 @@ struct AdjIo {
 // (block 32 x 4 as the forward kernels).  `side` holds 2 * lx * kGhostSlots doubles: the bottom slots of
 // every column, then the top slots.  The strip's pull-gather is staged in shared memory (9.5 KB
 // per warp); a slot holds f~_i, then its fixed-point form, then mu_i's, then the output.  What bounds
-// it: 6.1 k instructions per strip, more code than the instruction cache holds (hit rate 83 %), and
-// latency at 16 warps per SM.  So the loops over populations are rolled, and block barriers keep a
-// block's four warps, one per scheduler, on the same code (512 x 1024: 0.236 ms without them,
-// 0.221 with; fully unrolled 0.247; blocks of 8 to 20 warps 0.238 to 0.338; the float64-pipe
-// version it replaces 0.334).
+// it: latency at 16 warps per SM (128 registers), and 5.8 k instructions per strip, more code than
+// the instruction cache holds unless the loops over populations are rolled and block barriers keep
+// a block's four warps, one per scheduler, on the same code (512 x 1024: 0.236 ms without the
+// barriers, 0.221 with, fully unrolled 0.247; blocks of 8 to 20 warps 0.238 to 0.338).  With lambda's
+// scan under the gather's copies and each group's lambda loaded a group ahead 0.157 ms, 2.9 TB/s; the
+// version in float64 and fixed point it replaces took 0.314.
 extern __shared__ double adj_staged[];
 template <bool PERIODIC>
 __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict__ fin,

@@ -30,7 +30,11 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 
 // ---------------------------------------------------------------------------------------
 // Fused step of float64 states: gather (propagate + bc) -> collide -> streaming store
-// (step_fix64.cuh).
+// (step_fix64.cuh).  4096 x 8192: 3.72 ms, 5.3 TB/s (0.80 of the copy rate); colliding in float64, bound by
+// that pipe, 15.4 ms.  Bound now by latency at 20 warps per SM with the multiply-add, ALU and float64
+// pipes and issue each 54 to 57 % busy: 96 registers, and 37.9 KB of staging per block.  Six blocks
+// (80 registers, the largest carveout) left too little L1 for the gather: 4.35 -> 5.41 ms for
+// 2160 x 8192, 2 steps.
 #ifndef LBM_FIX64_MIN_BLOCKS
 #define LBM_FIX64_MIN_BLOCKS 5
 #endif

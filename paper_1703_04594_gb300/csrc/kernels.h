@@ -65,11 +65,22 @@ struct StepArgs : StepScalars, StepWalls {};
 // kernel before it in the stream drains, which hides the launch; pdl_wait(), its first statement before
 // any access to global memory, waits until that kernel has completed and its writes are visible.
 // pdl_trigger() lets the next kernel in as soon as every block of this one has started: 64 x 128, 10
-// steps 104 -> 84 us, 501 x 1003 78.0 -> 74.7 us.  The adjoint's kernels do without it (their
+// steps 104 -> 84 us, 501 x 1003 78.0 -> 74.7 us.  The adjoint's collision does without it (its
 // successors' blocks then hold slots that the recomputation on the other stream could use: gradient
 // 5.92 against 6.10 ms, adjoint step 0.195 against 0.209).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// The fused steps' blocks: 32 rows of two columns.  Smaller blocks retire and spread more evenly than ones
+// of four (64 x 128, 10 steps: 77 -> 69.5 us; 2160 x 8192 float64, 2 steps: 3.87 -> 3.85 ms; 2048 x 8192
+// FP32, 4 steps: 3.140 -> 3.120 ms; 512 x 512 0.4 % slower); one column leaves its neighbours' source
+// columns to other blocks (3.87 -> 4.91 ms), five and more retire too coarsely (3.90 to 5.15).  Four
+// where two would exceed the grid's 65535 in y.
+inline dim3 step_block(const StepArgs& a) { return dim3(32, a.lx <= 2 * 65535 ? 2 : 4); }
+inline dim3 step_grid(const StepArgs& a) {
+  const unsigned w = step_block(a).y;
+  return dim3((a.ly + 31) / 32, (a.lx + w - 1) / w);
+}
 
 template <class... P, class... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

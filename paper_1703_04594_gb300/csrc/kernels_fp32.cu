@@ -24,7 +24,7 @@ __global__ void __launch_bounds__(128, CONSERVE ? LBM_FP32C_MIN_BLOCKS : LBM_FP3
                                                                        float* __restrict__ fout, StepArgs a) {
   pdl_trigger();
   pdl_wait();
-  const int x = blockIdx.y * 4 + threadIdx.y;
+  const int x = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
   step_strip_fp32<PERIODIC, SCALED, CONSERVE>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly());
 }
@@ -101,7 +101,7 @@ static const dim3 kSiteBlock(32, 4);
 template <bool PERIODIC, bool SCALED>
 static cudaError_t launch_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {
   return launch_dependent(a.conserve ? k_step_fp32<PERIODIC, SCALED, true> : k_step_fp32<PERIODIC, SCALED, false>,
-                          site_grid(a), kSiteBlock, 0, s, fin, fout, a);
+                          step_grid(a), step_block(a), 0, s, fin, fout, a);
 }
 
 cudaError_t launch_step_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {

@@ -32,7 +32,7 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 // Fused step of float64 states: gather (propagate + bc) -> collide -> streaming store
 // (step_fix64.cuh).  4096 x 8192: 3.72 ms, 5.3 TB/s (0.80 of the copy rate); colliding in float64, bound by
 // that pipe, 15.4 ms.  Bound now by latency at 20 warps per SM with the multiply-add, ALU and float64
-// pipes and issue each 54 to 57 % busy: 96 registers, and 37.9 KB of staging per block.  Six blocks
+// pipes and issue each 54 to 57 % busy: 96 registers, and 9.5 KB of staging per warp.  24 warps
 // (80 registers, the largest carveout) left too little L1 for the gather: 4.35 -> 5.41 ms for
 // 2160 x 8192, 2 steps.
 #ifndef LBM_FIX64_MIN_BLOCKS
@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(128, LBM_FIX64_MIN_BLOCKS) k_step_fix64(const 
                                                                          double* __restrict__ fout, StepArgs a) {
   pdl_trigger();
   pdl_wait();
-  const int x = blockIdx.y * 4 + threadIdx.y;
+  const int x = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
   step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly(), step_staged + threadIdx.y * (Q * 32));
 }
@@ -281,9 +281,10 @@ static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, 
 static const dim3 kSiteBlock(32, 4);
 
 cudaError_t launch_step_fix64(const double* fin, double* fout, const StepArgs& a, cudaStream_t s) {
-  constexpr size_t smem = 4 * Q * 32 * sizeof(double);
-  return launch_dependent(a.periodic ? k_step_fix64<true> : k_step_fix64<false>, site_grid(a), kSiteBlock, smem, s, fin,
-                          fout, a);
+  const dim3 block = step_block(a);
+  const size_t smem = block.y * Q * 32 * sizeof(double);
+  return launch_dependent(a.periodic ? k_step_fix64<true> : k_step_fix64<false>, step_grid(a), block, smem, s, fin, fout,
+                          a);
 }
 
 cudaError_t launch_propagate_fp64(const double* fin, double* ftmp, const StepArgs& a, cudaStream_t s) {

@@ -126,3 +126,22 @@ def test_gradient_of_the_initial_state_on_both_routes(lx, ly, scale, wide):
     for a, b in zip(got, want):
         assert float(((a.cpu() / scale - b).abs() - 1e-13 * reach).max()) <= 0.0
         assert float(a[1, 2]) == 0.0
+
+
+@pytest.mark.parametrize("precision", [lbm.FP64, lbm.FP32_SHIFTED])
+@pytest.mark.parametrize("lx", [5, 6, 131070, 131071])
+def test_columns_on_both_sides_of_the_block_width_rule(lx, precision):
+    """Blocks of two columns up to lx = 131070, of four beyond: a state uniform in x stays so, and its
+    columns are those of a small lattice, bit for bit."""
+    require_gpu()
+    small = lbm.Params(4, 6, tau=0.8, gx=1e-4, precision=precision)
+    rho, ux, uy, T = rt_fields(small, seed=3)
+    fields = [t[:1].expand(4, 6).contiguous() for t in (rho, ux, uy, T)]
+    f = device_init(small, fields)
+    p = lbm.Params(lx, 6, tau=0.8, gx=1e-4, precision=precision)
+    wide = lbm.empty_state(p)
+    wide[:, :, :6] = f[:, :1, :6]
+    out, want = lbm.empty_state(p), lbm.empty_state(small)
+    lbm.step(small, f, want)
+    lbm.step(p, wide, out)
+    assert torch.equal(out[:, :, :6], want[:, :1, :6].expand(37, lx, 6))

@@ -30,7 +30,7 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 
 // ---------------------------------------------------------------------------------------
 // Fused step of float64 states: gather (propagate + bc) -> collide -> streaming store
-// (step_fix64.cuh).  4096 x 8192: 3.72 ms, 5.3 TB/s (0.80 of the copy rate); colliding in float64, bound by
+// (step_fix64.cuh).  4096 x 8192: 3.70 ms, 5.3 TB/s (0.80 of the copy rate); colliding in float64, bound by
 // that pipe, 15.4 ms.  Bound now by latency at 20 warps per SM with the multiply-add, ALU and float64
 // pipes and issue each 54 to 57 % busy: 96 registers, and 9.5 KB of staging per warp.  24 warps
 // (80 registers, the largest carveout) left too little L1 for the gather: 4.35 -> 5.41 ms for

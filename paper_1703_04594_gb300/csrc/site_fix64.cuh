@@ -108,7 +108,9 @@ inline FixConsts make_fix_consts(double tau, double gx, double gy) {
   const double tc = tau * (1.0 - tau) * (gx * gx + gy * gy) / 2.0 - (sx * sx + sy * sy) / (2.0 * C2);
   const double om1 = 1.0 - om;  // as CollideConst::om1
   const auto small = [](double v) { return v > -0.125 && v < 0.125; };
-  r.usable = om > 0.0 && om < 2.0 && om1 > -1.0 && om1 < 1.0 && small(sx) && small(sy) && small(tc);
+  // omega [62] up to 2 - 2^-30 (tau from 0.5 + 2.4e-10): from 2 - 2^-31 on its high half would round up
+  // to 2^31
+  r.usable = om > 0.0 && om <= 2.0 - 0x1p-30 && om1 > -1.0 && om1 < 1.0 && small(sx) && small(sy) && small(tc);
   if (!r.usable) return r;
   // (doubles of this size are multiples of 2^-60 or round there; conversions are exact or
   // round to nearest)
@@ -355,7 +357,7 @@ __host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, 
   ok = ok & ((unsigned long long)(t + kT) < 2ull * kT);
   s.t = t << 4;
   s.R = fx_smul(m.R << 3, k.om);
-  ok = ok & (s.R < (9LL << 58) / 5 * 8);
+  ok = ok & ((unsigned long long)s.R < (9ull << 58) / 5 * 8);
   s.X0 = X0 << 4;
   s.Y0 = Y0 << 4;
   s.e = e2;

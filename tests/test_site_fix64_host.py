@@ -128,3 +128,28 @@ def test_sites_outside_the_range_are_refused(model, probe):
     assert [g[0] for g in got] == ["0"] * len(bad) + ["1"]
     # constants outside the formats: a forcing of tau g = 0.4
     assert probe([" ".join([bits(0.8), bits(0.5), bits(0.0)] + [bits(v) for v in base])])[0][0] == "0"
+
+
+def results_or_refused(model, probe, sites):
+    """Each site is refused or within the bound; returns how many were taken."""
+    _, _, vx, vy = model
+    got = probe([" ".join([bits(tau), bits(gx), bits(gy)] + [bits(v) for v in f]) for f, tau, gx, gy in sites])
+    inside = 0
+    for (f, tau, gx, gy), line in zip(sites, got):
+        if line[0] == "0":
+            continue
+        inside += 1
+        k = int(line[1])
+        for i, (h, want) in enumerate(zip(line[2:], collided(model, f, tau, gx, gy))):
+            unit = F(2) ** (k - SHELL_EXP[vx[i] ** 2 + vy[i] ** 2] - 57)
+            assert abs(F(from_bits(h)) - want) <= abs(want) * F(2) ** -53 + 12 * unit, (i, tau)
+    return inside
+
+
+@pytest.mark.parametrize("above", [2.0 ** -53, 1e-15, 1e-12, 1e-10, 1.1e-10, 1.2e-10, 2.3e-10, 2.4e-10, 1e-9, 1e-6])
+def test_relaxation_times_just_above_one_half(model, probe, above):
+    """omega close to 2, the end of its format: from 2 - 2^-31 on its high half would round up to 2^31."""
+    rng = random.Random(7)
+    sites = [(state(model, rng, rng.uniform(0.7, 1.4), 0.1, 0.15), 0.5 + above, 0.0, -1e-4) for _ in range(20)]
+    inside = results_or_refused(model, probe, sites)
+    assert inside == (20 if above >= 1e-9 else 0 if above <= 2e-10 else inside)

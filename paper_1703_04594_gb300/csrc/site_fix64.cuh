@@ -330,13 +330,14 @@ __host__ __device__ __forceinline__ long long fx_reciprocal(long long R) {
 __host__ __device__ __forceinline__ FixScalars fix_scalars(const FixMoments& m, const FixConsts& k) {
   FixScalars s;
   // rho in [9/64, 1), |j| < 1/4, |sum |v|^2 f - 2 rho / c^2| < 1/2 (2 rho |t| / c^2 + ... < 0.4 in
-  // range): what the formats below hold; unsigned compares of the offset values
+  // range): what the formats below hold; unsigned compares of the offset values.  The upper ends lie
+  // 2^-30 lower, where the high half of the shifted value still rounds to less than 2^31.
   const long long W = fx_smul(m.R << 3, fx_halves(kFxInvC2_63));  // rho / c^2 [62] = 2 rho / c^2 [61]
   const long long dev = m.E * 2 - W;                               // [61]
-  bool ok = m.ok & ((unsigned long long)(m.R - (9LL << 54)) < (55ull << 54)) &
-            ((unsigned long long)(m.X + (1LL << 58)) < (1ull << 59)) &
-            ((unsigned long long)(m.Y + (1LL << 58)) < (1ull << 59)) &
-            ((unsigned long long)(dev + (1LL << 60)) < (1ull << 61));
+  bool ok = m.ok & ((unsigned long long)(m.R - (9LL << 54)) < (55ull << 54) - (1ull << 30)) &
+            ((unsigned long long)(m.X + (1LL << 58)) < (1ull << 59) - (1ull << 28)) &
+            ((unsigned long long)(m.Y + (1LL << 58)) < (1ull << 59) - (1ull << 28)) &
+            ((unsigned long long)(dev + (1LL << 60)) < (1ull << 61) - (1ull << 30));
   const long long yc = fx_smul(fx_reciprocal(m.R) , fx_halves(kFxC2_62)) * 2;  // c^2 / rho [58] -> [59]
   const FxHalves y = fx_halves(yc);
   const long long X0 = fx_smul(m.X << 5, y), Y0 = fx_smul(m.Y << 5, y);  // [60]

@@ -153,3 +153,32 @@ def test_relaxation_times_just_above_one_half(model, probe, above):
     sites = [(state(model, rng, rng.uniform(0.7, 1.4), 0.1, 0.15), 0.5 + above, 0.0, -1e-4) for _ in range(20)]
     inside = results_or_refused(model, probe, sites)
     assert inside == (20 if above >= 1e-9 else 0 if above <= 2e-10 else inside)
+
+
+def edge_site(model, rho, jx, energy):
+    """Populations with f_0 just below 1/8, so that the site's scale is 1, inside their own ranges, of
+    density rho, momentum (jx, 0) and sum |v|^2 f = energy up to 2^-40."""
+    from scipy.optimize import linprog
+    _, _, vx, vy = model
+    shell = [a * a + b * b for a, b in zip(vx, vy)]
+    top = [2.0 / 2 ** SHELL_EXP[s] for s in shell]
+    bounds = [(0.0626, 0.1249)] + [(v * 1.05 / 256, v * 0.95) for v in top[1:]]
+    sol = linprog([0.0] * 37, A_eq=[[1.0] * 37, vx, vy, shell], b_eq=[rho, jx, 0.0, energy], bounds=bounds)
+    assert sol.success
+    return [round(v * 2.0 ** 50) * 2.0 ** -50 for v in sol.x]
+
+
+@pytest.mark.parametrize("gap", [2.0 ** -12, 2.0 ** -29, 2.0 ** -35])
+@pytest.mark.parametrize("rho", [0.97, 0.98, 0.995])
+def test_sums_at_the_ends_of_their_formats(model, probe, rho, gap):
+    """Momentum just below 1/4 and energy just below 1/2 above that of T = 1 at the site's scale: the
+    ends of the formats, where a high half would round up past them."""
+    c2 = model[0] ** 2
+    sites = []
+    for t in (-0.3, -0.1, 0.0, 0.1):
+        jx = 0.25 - gap
+        sites.append((edge_site(model, rho, jx, (2.0 * (1.0 + t) * rho + c2 * jx * jx / rho) / c2), 0.8, 0.0, 0.0))
+    for jx in (0.0, 0.05):
+        sites.append((edge_site(model, rho, jx, 2.0 * rho / c2 + 0.5 - gap), 0.8, 0.0, 0.0))
+    inside = results_or_refused(model, probe, sites)
+    assert gap < 2.0 ** -12 or inside >= 4

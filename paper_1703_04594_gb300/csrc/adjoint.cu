@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
   fix_adj_outputs(r, k.fx.om1, c_pair_fix, io);
   double contrib = 0.0;
   if (active) {
-    if (ok) contrib = k.om2 * fx_lower_exponent(r.D, K + (1 << 20) - m.kb);
+    if (ok) contrib = fix_dtau(r.D, k.om2, K, m.kb);
     else contrib = adj_site_float64<PERIODIC>(fin, lam, a, k, x, y, sf);
     if (edge_strip(a, y0)) {
       push_strip_edge<PERIODIC>(sf, lam_out, side, a, x, y);

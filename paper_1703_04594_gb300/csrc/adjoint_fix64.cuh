@@ -319,6 +319,21 @@ __host__ __device__ __forceinline__ FixVjp fix_vjp(const FixMoments& f, const Fi
   return r;
 }
 
+// The site's part of dL/dtau, D omega^2 2^(k - K - 1): K and kb = k in units of the exponent field.  Two
+// exact scalings: either exponent alone is within what the first or a float64 factor holds, their sum
+// is not (lambda and the density both large, or both small).
+__host__ __device__ __forceinline__ double fix_dtau(long long D, double om2, int K, int kb) {
+  const double v = om2 * fx_lower_exponent(D, K + (1 << 20));
+#ifdef __CUDA_ARCH__
+  return v * __hiloint2double(0x3FF00000 + kb, 0);
+#else
+  const unsigned long long b = (unsigned long long)(0x3FF00000 + kb) << 32;
+  double s;
+  __builtin_memcpy(&s, &b, 8);
+  return v * s;
+#endif
+}
+
 // ---- 3. the outputs ----------------------------------------------------------------------------------
 // `io.held(i)` returns the halves of mu_i 2^(K + 1); `io.out(i, v)` takes the site's out_i in units
 // of 2^-K.  One rolled loop over the opposite pairs (v, -v), out = (1 - w) mu + A +- B; `pairs` is

@@ -85,12 +85,23 @@ __host__ __device__ __forceinline__ double fx_to_double_dp_pos(long long X, int 
 #endif
 }
 
-// X 2^-(K / 2^20) for a float64 conversion of X and K >= 0 in units of the exponent field, as
+// X 2^-(K / 2^20) for a float64 conversion of X and 0 <= K <= 1022 2^20 in units of the exponent field, as
 // fx_to_double_dp_pos.
-__device__ __forceinline__ double fx_lower_exponent(long long X, int K) {
+__host__ __device__ __forceinline__ double fx_lower_exponent(long long X, int K) {
+#ifdef __CUDA_ARCH__
   const double d = __ll2double_rn(X);
   const unsigned h = (unsigned)__double2hiint(d);
   return __hiloint2double((int)(h - min(h, (unsigned)K)), __double2loint(d));
+#else
+  const double d = (double)X;
+  unsigned long long b;
+  __builtin_memcpy(&b, &d, 8);
+  const unsigned h = (unsigned)(b >> 32);
+  b = ((unsigned long long)(h - (h < (unsigned)K ? h : (unsigned)K)) << 32) | (b & 0xFFFFFFFFull);
+  double r;
+  __builtin_memcpy(&r, &b, 8);
+  return r;
+#endif
 }
 
 // f' = f 2^(59 + e) for a population whose value is an integer there: with the exponent

@@ -145,3 +145,25 @@ def test_columns_on_both_sides_of_the_block_width_rule(lx, precision):
     lbm.step(small, f, want)
     lbm.step(p, wide, out)
     assert torch.equal(out[:, :, :6], want[:, :1, :6].expand(37, lx, 6))
+
+
+@pytest.mark.parametrize("rho0,scale", [(1600.0, 1e14), (1600.0, 1e16), (16.0, 2.0 ** 55), (1e-250, 1e-270), (1e-250, 1e3)])
+def test_adjoint_step_at_large_and_small_scales_together(rho0, scale):
+    """lambda and the density both far from 1: the step is linear in lambda and its part of dL/dtau in the
+    density too, so both follow from the oracle's at 1 (bars as above)."""
+    require_gpu()
+    p = lbm.Params(6, 97, tau=0.7, gx=1e-4, gy=-2e-4)
+    rho, ux, uy, T = rt_fields(p, seed=5)
+    lam = torch.randn(37, p.lx, p.ly, dtype=torch.float64, generator=torch.Generator().manual_seed(17))
+    one = device_init(p, (rho, ux, uy, T))
+    want, want_tau = oracle_vjp(p, to_host(p, one), lam)
+    f = device_init(p, (rho * rho0, ux, uy, T))
+    lam_dev = torch.zeros_like(f)
+    lam_dev[:, :, :p.ly] = lam.cuda() * scale
+    lam_n = torch.zeros_like(f)
+    dtau = torch.zeros((), dtype=torch.float64, device="cuda")
+    lbm.adjoint_step(p, f, lam_dev, lam_n, dtau, lbm.adjoint_work(p))
+    got = to_host(p, lam_n) / scale
+    assert float(((got - want).abs() / reach_max(lam.abs().amax(0), p.bc)[None]).max()) <= 1e-13
+    reach = max(abs(want_tau), float(lam.abs().sum()) * 1e-3)
+    assert abs(float(dtau) - want_tau * scale * rho0) <= 1e-10 * reach * scale * rho0

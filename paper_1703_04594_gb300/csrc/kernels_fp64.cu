@@ -252,7 +252,8 @@ __device__ __forceinline__ double block_sum_1024(const double* __restrict__ part
 }
 
 // One cluster of CLUSTER blocks, each summing its part of the array; block 0 adds their sums in order
-// through distributed shared memory.
+// through distributed shared memory, which may be written once every block of the cluster has started
+// (the first barrier: arrived at on entry, waited for after the loads).
 template <int CLUSTER>
 __global__ void __launch_bounds__(1024) k_reduce_sum(const double* __restrict__ part, long long n,
                                                     double* __restrict__ out) {
@@ -262,9 +263,11 @@ __global__ void __launch_bounds__(1024) k_reduce_sum(const double* __restrict__ 
   } else {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
+    cluster.barrier_arrive();
     __shared__ double sums[CLUSTER];
     const long long each = (n + CLUSTER - 1) / CLUSTER, begin = each * blockIdx.x;
     const double t = block_sum_1024(part + begin, begin < n ? (n - begin < each ? n - begin : each) : 0);
+    cluster.barrier_wait();
     if (threadIdx.x == 0) cluster.map_shared_rank(sums, 0)[blockIdx.x] = t;
     cluster.sync();
     if (blockIdx.x == 0 && threadIdx.x == 0) {

@@ -170,16 +170,16 @@ struct AdjConsts {
 // so that its arithmetic does not weigh on the register allocation of the fixed-point path: the
 // site's outputs to its slots, and its part of dL/dtau returned.
 template <bool PERIODIC>
-__device__ __noinline__ double adj_site_float64(const double* __restrict__ fin, const double* __restrict__ lam,
+__device__ __noinline__ double adj_site_float64(const double* fin, const double* lam,
                                                 const StepArgs& a, const AdjConsts& k, int x, int y, double* sf) {
   double mu_ft = 0.0, rho, jx, jy, e;
   {
     double f[Q];
-    gather_site<PERIODIC>(fin, a, a, x, y, f, LdReadOnly());
+    gather_site<PERIODIC>(fin, a, a, x, y, f, LdCached());
     moments_int(f, rho, jx, jy, e);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
-      const double l = __ldg(lam + i * a.pop);
+      const double l = lam[i * a.pop];
       mu_ft = fma(l, f[i], mu_ft);
       sf[i * 32] = l;
     }
@@ -251,7 +251,7 @@ struct AdjIo {
     const double* lam;
   };
   __device__ __forceinline__ At at(int i) const { return At{slots + i * 32, lam + (unsigned long long)pop * (unsigned)i}; }
-  __device__ __forceinline__ double mu(At h, int k) const { return __ldg(k ? h.lam + (unsigned long long)pop * NPAIR : h.lam); }
+  __device__ __forceinline__ double mu(At h, int k) const { return *(k ? h.lam + (unsigned long long)pop * NPAIR : h.lam); }
   __device__ __forceinline__ FxHalves fixed(At h, int k) const { return h.f[k * (NPAIR * 32)]; }
   __device__ __forceinline__ void keep(At h, int k, FxHalves q) const { h.f[k * (NPAIR * 32)] = q; }
   __device__ __forceinline__ FxHalves held(int i) const { return slots[i * 32]; }
@@ -272,10 +272,8 @@ struct AdjIo {
 // version in float64 and fixed point it replaces took 0.314.
 extern __shared__ double adj_staged[];
 template <bool PERIODIC>
-__global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict__ fin,
-                                                     const double* __restrict__ lam_next, double* __restrict__ lam_out,
-                                                     double* __restrict__ side, double* __restrict__ dtau_part,
-                                                     StepArgs a, AdjConsts k) {
+__global__ void __launch_bounds__(128, 4) k_adj_collide(const double* fin, const double* lam_next, double* lam_out,
+                                                     double* side, double* dtau_part, StepArgs a, AdjConsts k) {
   pdl_wait();
   const int x = blockIdx.y * 4 + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
@@ -286,14 +284,14 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
   double* const sf = adj_staged + threadIdx.y * (Q * 32) + threadIdx.x;
   FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);
   const double* lam = lam_next + (long long)x * a.pitch + (unsigned)yc;
-  stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, LdReadOnly());
+  stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, LdCached());
   // the block exponent of lambda, from the high words alone (the values are loaded again below,
   // when their fixed-point forms can go to the slots at once)
   unsigned top = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i)
-    top = max(top, __ldg(reinterpret_cast<const unsigned*>(lam + i * a.pop) + 1) & 0x7fffffffu);
-  stage_finish<PERIODIC>(fin, a, a, x, y0, yc, sf, LdReadOnly());
+    top = max(top, reinterpret_cast<const unsigned*>(lam + i * a.pop)[1] & 0x7fffffffu);
+  stage_finish<PERIODIC>(fin, a, a, x, y0, yc, sf, LdCached());
   __syncthreads();
   const FixMoments m = fix_moments_rolled(c_fix_groups, [&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
   const FixScalars v = fix_scalars(m, a.fx);
@@ -337,7 +335,7 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* __restrict
 
 // Adds sum(part[0..n)) to *acc in a fixed order; one block of 256 threads.  Sixteen independent
 // sums per thread keep as many loads in flight.
-__device__ __forceinline__ void reduce_add_256(const double* __restrict__ part, long long n, double* acc) {
+__device__ __forceinline__ void reduce_add_256(const double* part, long long n, double* acc) {
   double s[16] = {};
   for (long long i = threadIdx.x; i < n; i += 16 * 256) {
 #pragma unroll
@@ -369,8 +367,8 @@ __device__ __forceinline__ void reduce_add_256(const double* __restrict__ part, 
 // entry, each forming its column's sum from the 26 slots, took 41 operations of the float64
 // pipe a thread.)  The grid's last block adds the step's dL/dtau partials to *dtau (the reduction
 // needs step 1 complete too, so it shares this launch).
-__global__ void __launch_bounds__(256) k_adj_walls(const double* __restrict__ side, double* __restrict__ lam,
-                                                   StepArgs a, const double* __restrict__ part, long long n_part,
+__global__ void __launch_bounds__(256) k_adj_walls(const double* side, double* lam, StepArgs a,
+                                                   const double* part, long long n_part,
                                                    double* dtau) {
   pdl_trigger();
   pdl_wait();
@@ -397,7 +395,7 @@ __global__ void __launch_bounds__(256) k_adj_walls(const double* __restrict__ si
 }
 
 // Adds sum(part[0..n)) to *acc in a fixed order (one block of 256 threads).
-__global__ void __launch_bounds__(256) k_reduce_add(const double* __restrict__ part, long long n, double* acc) {
+__global__ void __launch_bounds__(256) k_reduce_add(const double* part, long long n, double* acc) {
   reduce_add_256(part, n, acc);
 }
 

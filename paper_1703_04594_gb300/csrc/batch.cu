@@ -168,6 +168,7 @@ constexpr int batch_max_regs(int kind) {
 
 extern __shared__ double batch_staged[];
 
+// (the two tables are written before any launch that reads them, so they may be read-only loads)
 template <int KIND, bool PERIODIC>
 __global__ void __launch_bounds__(256) __maxnreg__(batch_max_regs(KIND)) k_batch_step(const BatchLattice* __restrict__ L,
                                                     const BatchTile* __restrict__ tiles, long long total,
@@ -176,7 +177,7 @@ __global__ void __launch_bounds__(256) __maxnreg__(batch_max_regs(KIND)) k_batch
   pdl_wait();
   const long long t = blockIdx.x;
   if (t >= total) return;
-  batch_tile<KIND, PERIODIC>(L, tiles, t, parity, LdReadOnly(), batch_staged);
+  batch_tile<KIND, PERIODIC>(L, tiles, t, parity, LdCached(), batch_staged);
 }
 
 template <int KIND, bool PERIODIC>

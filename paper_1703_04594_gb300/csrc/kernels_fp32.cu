@@ -20,13 +20,12 @@ namespace d2q37 {
 #endif
 template <bool PERIODIC, bool SCALED, bool CONSERVE>
 __global__ void __launch_bounds__(128, CONSERVE ? LBM_FP32C_MIN_BLOCKS : LBM_FP32_MIN_BLOCKS) k_step_fp32(
-    const float* __restrict__ fin,
-                                                                       float* __restrict__ fout, StepArgs a) {
+    const float* fin, float* fout, StepArgs a) {
   pdl_trigger();
   pdl_wait();
   const int x = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
-  step_strip_fp32<PERIODIC, SCALED, CONSERVE>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly());
+  step_strip_fp32<PERIODIC, SCALED, CONSERVE>(fin, fout, a, a, x, blockIdx.x * 32, LdCached());
 }
 
 // g_i = f_i^eq(rho, u, T) - w_i rho0, equilibrium evaluated in float64 then rounded.

@@ -40,13 +40,12 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 #endif
 extern __shared__ double step_staged[];  // 37 populations x 32 sites per warp
 template <bool PERIODIC>
-__global__ void __launch_bounds__(128, LBM_FIX64_MIN_BLOCKS) k_step_fix64(const double* __restrict__ fin,
-                                                                         double* __restrict__ fout, StepArgs a) {
+__global__ void __launch_bounds__(128, LBM_FIX64_MIN_BLOCKS) k_step_fix64(const double* fin, double* fout, StepArgs a) {
   pdl_trigger();
   pdl_wait();
   const int x = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
-  step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdReadOnly(), step_staged + threadIdx.y * (Q * 32));
+  step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdCached(), step_staged + threadIdx.y * (Q * 32));
 }
 
 // ---------------------------------------------------------------------------------------

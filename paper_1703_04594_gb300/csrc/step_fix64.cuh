@@ -18,7 +18,7 @@ constexpr int kFixWarps = 4;  // warps per block (block = 32 x 4 threads)
 // The pulled populations of one site, wall values included, loaded from global memory: for
 // sites that leave the fixed-point path, whose staged slots hold their fixed-point forms by then.
 template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void gather_site(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
+__device__ __forceinline__ void gather_site(const double* fin, const StepScalars& a, const StepWalls& w,
                                             int x, int yc, double (&f)[Q], Ld ld) {
   const auto wall_density = [&](int i, int row) {  // of the source column of population i
     const double* src = fin + (long long)wrap_index(x - vx(i), a.lx) * a.pitch + row;
@@ -40,7 +40,7 @@ __device__ __forceinline__ void gather_site(const double* __restrict__ fin, cons
 // The float64 collision of such a site.  Not inlined, so that its 37 live float64 values do not
 // weigh on the register allocation of the fixed-point path.
 template <bool PERIODIC, class Ld>
-__device__ __noinline__ void collide_site_reloaded(const double* __restrict__ fin, double* __restrict__ fout,
+__device__ __noinline__ void collide_site_reloaded(const double* fin, double* __restrict__ fout,
                                                    const StepScalars& a, const StepWalls& w, int x, int yc,
                                                    unsigned self) {
   double f[Q];
@@ -51,7 +51,7 @@ __device__ __noinline__ void collide_site_reloaded(const double* __restrict__ fi
 // rho(x_s, row) of the seven source columns: lane l sums every fourth population of column
 // l % 8, and two shuffles add the four parts (the same value in the column's four lanes).
 template <class Ld>
-__device__ __forceinline__ double wall_density_lane(const double* __restrict__ fin, int x, const StepScalars& a, int row,
+__device__ __forceinline__ double wall_density_lane(const double* fin, int x, const StepScalars& a, int row,
                                                     Ld ld) {
   const int lane = threadIdx.x & 31;
   const int d = lane & 7, part = lane >> 3;
@@ -77,7 +77,7 @@ __device__ __forceinline__ bool edge_strip(const StepScalars& a, int y0) { retur
 // (asynchronous when Ld caches in L1), then waited for and the ghosts of wall strips written over
 // the clamped rows; in between the caller can issue other loads.
 template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void stage_issue(const double* __restrict__ fin, const StepScalars& a, int x, int y0, int yc,
+__device__ __forceinline__ void stage_issue(const double* fin, const StepScalars& a, int x, int y0, int yc,
                                             double* __restrict__ sf, Ld ld) {
   // one pointer per source column (planes < 2^32 elements); a plane's stride and a hop in y are then
   // an addition and an immediate
@@ -127,7 +127,7 @@ static __constant__ WallGhosts c_wall_ghosts = wall_ghosts();
 // The wall sums are formed while the copies arrive, and one product per lane then gives all of a
 // wall's 26 ghosts (in the threads that pull them it took 15, at 64 cycles of the float64 pipe each).
 template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void stage_finish(const double* __restrict__ fin, const StepScalars& a, const StepWalls& w,
+__device__ __forceinline__ void stage_finish(const double* fin, const StepScalars& a, const StepWalls& w,
                                              int x, int y0, int yc, double* __restrict__ sf, Ld ld) {
   if (!PERIODIC && edge_strip(a, y0)) {
     const int lane = threadIdx.x & 31;
@@ -166,7 +166,7 @@ struct StepIo {
 };
 
 template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void step_strip_fix64(const double* __restrict__ fin, double* __restrict__ fout,
+__device__ __forceinline__ void step_strip_fix64(const double* fin, double* __restrict__ fout,
                                                  const StepScalars& a, const StepWalls& w, int x, int y0, Ld ld,
                                                  double* __restrict__ sf) {
   const int lane = threadIdx.x & 31;

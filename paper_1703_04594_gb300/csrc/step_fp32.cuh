@@ -430,7 +430,7 @@ struct FloatPair {
 // four lanes).  Compensated float32 sums, because the float64 pipe is busy with the site scalars:
 // summed there, the walls of small lattices took it to 66 %.
 template <class Ld>
-__device__ __forceinline__ float wall_drho_lane(const float* __restrict__ fin, int x, const StepScalars& a, int row, Ld ld) {
+__device__ __forceinline__ float wall_drho_lane(const float* fin, int x, const StepScalars& a, int row, Ld ld) {
   const int lane = threadIdx.x & 31;
   const int d = lane & 7, part = lane >> 3;
   FloatPair r = {0.0f, 0.0f};
@@ -455,7 +455,7 @@ __device__ __forceinline__ float wall_drho_lane(const float* __restrict__ fin, i
 // SCALED: the lattice's reference density is outside [1/2, 2) (see moments_fix); CONSERVE: the
 // collision restores the exact conserved moments (collide_site_fp32).
 template <bool PERIODIC, bool SCALED, bool CONSERVE, class Ld>
-__device__ __forceinline__ void step_strip_fp32(const float* __restrict__ fin, float* __restrict__ fout,
+__device__ __forceinline__ void step_strip_fp32(const float* fin, float* __restrict__ fout,
                                                 const StepScalars& a, const StepWalls& w, int x, int y0, Ld ld) {
   const int y = y0 + (threadIdx.x & 31);
   const bool active = y < a.ly;

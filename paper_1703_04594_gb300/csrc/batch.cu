@@ -92,6 +92,16 @@ inline size_t batch_smem_bytes(int kind, int warps) {
   return kind == kFix64 ? (size_t)warps * Q * 32 * sizeof(double) : 0;
 }
 
+// The sites of tile t outside the fixed-point range (see step_float64_sites).
+template <bool PERIODIC, class Ld>
+__device__ __noinline__ void tile_float64_sites(const BatchLattice* L, const BatchTile* tiles, long long t, int parity,
+                                                bool left, double* staged) {
+  const BatchTile tile = tiles[t];
+  const BatchLattice& B = L[tile.lattice];
+  collide_strip_float64<PERIODIC, Ld>((const double*)B.f[parity], (double*)B.f[parity ^ 1], B.a, B.a,
+                                      tile.x0 + (int)threadIdx.y, tile.y0, staged + threadIdx.y * (Q * 32), left);
+}
+
 // Tile t of the batch (32 rows x TX columns, one warp per column, as the single-lattice
 // kernels): its lattice and position come from the tile table, so everything that depends on
 // the lattice is uniform across the block.
@@ -105,9 +115,10 @@ __device__ __forceinline__ void batch_tile(const BatchLattice* __restrict__ L, c
   if (x >= B.a.lx) return;  // uniform per warp
   const T* src = (const T*)B.f[parity];
   T* dst = (T*)B.f[parity ^ 1];
-  if constexpr (KIND == kFix64)
-    step_strip_fix64<PERIODIC>(src, dst, B.a, B.a, x, y0, ld, staged + threadIdx.y * (Q * 32));
-  else
+  if constexpr (KIND == kFix64) {
+    const bool left = step_strip_fix64<PERIODIC>(src, dst, B.a, B.a, x, y0, ld, staged + threadIdx.y * (Q * 32));
+    if (__any_sync(0xffffffffu, left)) tile_float64_sites<PERIODIC, Ld>(L, tiles, t, parity, left, staged);
+  } else
     step_strip_fp32<PERIODIC, KIND == kFp32Scaled || KIND == kFp32ConsScaled, KIND == kFp32Cons || KIND == kFp32ConsScaled>(
         src, dst, B.a, B.a, x, y0, ld);
 }

@@ -39,13 +39,25 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 #define LBM_FIX64_MIN_BLOCKS 5
 #endif
 extern __shared__ double step_staged[];  // 37 populations x 32 sites per warp
+// The sites outside the fixed-point range, by a function that forms its indices itself and is not
+// inlined, so that the kernel keeps neither its float64 values nor its arguments in registers (a vote
+// before the relaxation, and a second copy of that for mixed strips, cost 2 % of the other strips' time).
+template <bool PERIODIC>
+__device__ __noinline__ void step_float64_sites(const double* fin, double* fout, const StepArgs& a, bool left) {
+  const int x = blockIdx.y * blockDim.y + threadIdx.y;
+  collide_strip_float64<PERIODIC, LdCached>(fin, fout, a, a, x, blockIdx.x * 32, step_staged + threadIdx.y * (Q * 32),
+                                            left);
+}
+
 template <bool PERIODIC>
 __global__ void __launch_bounds__(128, LBM_FIX64_MIN_BLOCKS) k_step_fix64(const double* fin, double* fout, StepArgs a) {
   pdl_trigger();
   pdl_wait();
   const int x = blockIdx.y * blockDim.y + threadIdx.y;
   if (x >= a.lx) return;  // uniform per warp
-  step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdCached(), step_staged + threadIdx.y * (Q * 32));
+  const bool left = step_strip_fix64<PERIODIC>(fin, fout, a, a, x, blockIdx.x * 32, LdCached(),
+                                               step_staged + threadIdx.y * (Q * 32));
+  if (__any_sync(FULL, left)) step_float64_sites<PERIODIC>(fin, fout, a, left);
 }
 
 // ---------------------------------------------------------------------------------------

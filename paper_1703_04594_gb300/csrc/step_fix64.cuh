@@ -37,17 +37,6 @@ __device__ __forceinline__ void gather_site(const double* fin, const StepScalars
   }
 }
 
-// The float64 collision of such a site.  Not inlined, so that its 37 live float64 values do not
-// weigh on the register allocation of the fixed-point path.
-template <bool PERIODIC, class Ld>
-__device__ __noinline__ void collide_site_reloaded(const double* fin, double* __restrict__ fout,
-                                                   const StepScalars& a, const StepWalls& w, int x, int yc,
-                                                   unsigned self) {
-  double f[Q];
-  gather_site<PERIODIC>(fin, a, w, x, yc, f, Ld());
-  collide_site(f, a.cc, [&](int i, double val) { __stcs(fout + i * a.pop + self, val); });
-}
-
 // rho(x_s, row) of the seven source columns: lane l sums every fourth population of column
 // l % 8, and two shuffles add the four parts (the same value in the column's four lanes).
 template <class Ld>
@@ -165,27 +154,46 @@ struct StepIo {
   }
 };
 
+// Returns whether the lane's site is still to be collided, in float64 (collide_strip_float64).
 template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void step_strip_fix64(const double* fin, double* __restrict__ fout,
-                                                 const StepScalars& a, const StepWalls& w, int x, int y0, Ld ld,
-                                                 double* __restrict__ sf) {
+__device__ __forceinline__ bool step_strip_fix64(const double* fin, double* __restrict__ fout, const StepScalars& a,
+                                                 const StepWalls& w, int x, int y0, Ld ld, double* __restrict__ sf) {
   const int lane = threadIdx.x & 31;
   const int y = y0 + lane;
-  const bool active = y < a.ly;
+  const bool active = y < a.ly;  // the other lanes work on the last row's data and store nothing
   const int yc = active ? y : a.ly - 1;
   sf += lane;
   stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, ld);
   stage_finish<PERIODIC>(fin, a, w, x, y0, yc, sf, ld);
-  if (!active) return;
+  if (!a.fx.usable) return active;  // uniform: the lattice's constants are outside the formats
   FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);  // the same slots, as fixed point
   const FixMoments m = fix_moments([&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
   const FixScalars v = fix_scalars(m, a.fx);
-  const unsigned self = (unsigned)((long long)x * a.pitch + y);
-  if (!v.ok || !a.fx.usable) {
-    collide_site_reloaded<PERIODIC, Ld>(fin, fout, a, w, x, yc, self);
-    return;
-  }
+  if (!active) return false;
+  if (!v.ok) return true;
   fix_relax(v, a.fx.om1, StepIo{sx, fout + (long long)x * a.pitch + (unsigned)y, a.pop, m.kb});
+  return false;
+}
+
+// The float64 collision of the lanes that step_strip_fix64 left: the whole warp gathers the strip once
+// more, walls included, over the fixed-point forms.  T = 1.5 everywhere: 64 x 128 18.3 us, 501 x 1003
+// 267 us, 2048 x 4096 3.87 ms a step; with each lane gathering its own site, and summing 37 wall values
+// per ghost, 74, 374 and 4.26; a kernel of the float64 collision alone 18.6, 258 and 3.88.
+template <bool PERIODIC, class Ld>
+__device__ __forceinline__ void collide_strip_float64(const double* fin, double* fout, const StepScalars& a,
+                                                      const StepWalls& w, int x, int y0, double* sf, bool left) {
+  const int y = y0 + (threadIdx.x & 31), yc = min(y, a.ly - 1);
+  sf += threadIdx.x & 31;
+  __syncwarp();
+  if (a.fx.usable) {  // else the populations are still in the slots
+    stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, Ld());
+    stage_finish<PERIODIC>(fin, a, w, x, y0, yc, sf, Ld());
+  }
+  if (!left) return;
+  const auto f = [&](int i) { return sf[i * 32]; };
+  const SiteScalars v = site_scalars(f, a.cc, [](int, int) {});
+  double* const dst = fout + (long long)x * a.pitch + (unsigned)y;
+  relax_site_get(f, a.cc.om1, v.R, v.Ux, v.Uy, v.t, [&](int i, double val) { __stcs(dst + i * a.pop, val); });
 }
 
 }  // namespace d2q37

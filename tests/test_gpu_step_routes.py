@@ -167,3 +167,32 @@ def test_adjoint_step_at_large_and_small_scales_together(rho0, scale):
     assert float(((got - want).abs() / reach_max(lam.abs().amax(0), p.bc)[None]).max()) <= 1e-13
     reach = max(abs(want_tau), float(lam.abs().sum()) * 1e-3)
     assert abs(float(dtau) - want_tau * scale * rho0) <= 1e-10 * reach * scale * rho0
+
+
+@pytest.mark.parametrize("lx,ly", [(4, 6), (5, 31), (7, 33), (6, 97)])
+@pytest.mark.parametrize("bc", [lbm.BC_WALLS, lbm.BC_PERIODIC_Y])
+@pytest.mark.parametrize("hot", [False, True])
+def test_strips_collided_in_float64(lx, ly, bc, hot):
+    """A lattice whose forcing is outside the fixed-point formats, and one with every second column too
+    hot for them, against the separate kernels (the bar above); the same lattices in a batch, in both
+    modes, have the same bits."""
+    require_gpu()
+    p = lbm.Params(lx, ly, tau=0.8, gx=0.0 if hot else 0.2, gy=-2e-4, bc=bc)
+    rho, ux, uy, T = rt_fields(p, seed=3)
+    if hot:
+        T = T + 0.5 * (torch.arange(lx, dtype=torch.float64)[:, None] % 2)
+    f = device_init(p, [t.contiguous() for t in (rho, ux, uy, T)])
+    tmp, want, got = lbm.empty_state(p), lbm.empty_state(p), lbm.empty_state(p)
+    lbm.propagate(p, f, tmp)
+    lbm.bc(p, f, tmp)
+    lbm.collide(p, tmp, want)
+    lbm.step(p, f, got)
+    a, b = got[:, :, :ly], want[:, :, :ly]
+    w = torch.tensor(lbm.model()[1], dtype=torch.float64, device="cuda")[:, None, None]
+    assert float(((a - b).abs() / (w * b.sum(0).abs())).max()) <= 2e-12
+    for mode in (lbm.BATCH_PER_STEP, lbm.BATCH_PERSISTENT):
+        batch = lbm.Batch([p], [f.clone()], [lbm.empty_state(p)])
+        batch.configure(mode, 2)
+        batch.run(1)
+        assert torch.equal(batch.states()[0][:, :, :ly], a)
+        batch.close()

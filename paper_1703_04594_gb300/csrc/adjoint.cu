@@ -166,23 +166,58 @@ struct AdjConsts {
   AdjFixConsts fx;
 };
 
-// The adjoint collision of one site in float64 (sites outside the fixed-point range), not inlined
-// so that its arithmetic does not weigh on the register allocation of the fixed-point path: the
-// site's outputs to its slots, and its part of dL/dtau returned.
+// Scatter of a strip's outputs next to a wall or across the periodic seam.  out_i(z) is
+// lambda_i(z - v_i) of the previous step (the transposed pull), or goes to the wall slot of its
+// source column when z - v_i is a ghost; entries of the site whose source z + v_i lies beyond a
+// wall get no push and are set to zero.
 template <bool PERIODIC>
-__device__ __noinline__ double adj_site_float64(const double* fin, const double* lam,
-                                                const StepArgs& a, const AdjConsts& k, int x, int y, double* sf) {
-  double mu_ft = 0.0, rho, jx, jy, e;
-  {
-    double f[Q];
-    gather_site<PERIODIC>(fin, a, a, x, y, f, LdCached());
-    moments_int(f, rho, jx, jy, e);
+__device__ __noinline__ void push_strip_edge(const double* sf, double* __restrict__ lam_out, double* __restrict__ side,
+                                             const StepArgs& a, int x, int y) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const double l = lam[i * a.pop];
-      mu_ft = fma(l, f[i], mu_ft);
-      sf[i * 32] = l;
+  for (int i = 0; i < Q; ++i) {
+    const int xs = wrap_index(x - vx(i), a.lx), yd = y - vy(i);
+    const double val = sf[i * 32];
+    if (!PERIODIC && yd < 0) {
+      __stcs(side + ((long long)xs * kGhostSlots + ghost_base(i, 1) + y), val);
+    } else if (!PERIODIC && yd >= a.ly) {
+      __stcs(side + (((long long)a.lx + xs) * kGhostSlots + ghost_base(i, -1) + (a.ly - 1 - y)), val);
+    } else {
+      __stcs(lam_out + (i * a.pop + (long long)xs * a.pitch + (PERIODIC ? wrap_index(yd, a.ly) : yd)), val);
     }
+    const int ys = y + vy(i);
+    if (!PERIODIC && (ys < 0 || ys >= a.ly)) __stcs(lam_out + (i * a.pop + (long long)x * a.pitch + y), 0.0);
+  }
+}
+
+extern __shared__ double adj_staged[];
+
+// The adjoint collision, in float64, of the lanes of a strip that the fixed-point path left, called by
+// the whole warp: their outputs to their slots and from there on, and their parts of dL/dtau returned.
+// It forms its indices itself and is not inlined, so that neither they nor its arithmetic weigh on the
+// register allocation of the fixed-point path.  The warp gathers the strip once more as a whole, as
+// collide_strip_float64 does.  T = 1.5 everywhere: 64 x 128 56 us, 256 x 512 246, 512 x 1024 831 a step
+// (each lane gathering its own site, and the fixed-point part run for nothing: 104, 344, 1069; a kernel
+// that takes only the equilibrium's derivatives in float64: 54, 233, 824).
+template <bool PERIODIC>
+__device__ __noinline__ double adj_float64_sites(const double* fin, const double* lam_next, double* lam_out,
+                                                 double* side, const StepArgs& a, const AdjConsts& k, bool left) {
+  const int x = blockIdx.y * 4 + threadIdx.y, y0 = blockIdx.x * 32;
+  const int y = y0 + threadIdx.x, yc = min(y, a.ly - 1);
+  double* const sf = adj_staged + threadIdx.y * (Q * 32) + threadIdx.x;
+  __syncwarp();
+  if (a.fx.usable && k.fx.usable) {  // else the populations are still in the slots
+    stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, LdCached());
+    stage_finish<PERIODIC>(fin, a, a, x, y0, yc, sf, LdCached());
+  }
+  if (!left) return 0.0;
+  const double* const lam = lam_next + ((long long)x * a.pitch + (unsigned)y);
+  double mu_ft = 0.0, rho, jx, jy, e;
+  moments_get([&](int i) { return sf[i * 32]; }, rho, jx, jy, e, [](int, int) {});
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const double l = lam[i * a.pop];
+    mu_ft = fma(l, sf[i * 32], mu_ft);
+    sf[i * 32] = l;
   }
   const auto mu = [&](int i) { return sf[i * 32]; };
   const double inv = 1.0 / rho;
@@ -212,32 +247,10 @@ __device__ __noinline__ double adj_site_float64(const double* fin, const double*
     sf[j * 32] = fma(om1, mu(j), A + B);
     sf[(j + NPAIR) * 32] = fma(om1, mu(j + NPAIR), A - B);
   }
+  push_strip_edge<PERIODIC>(sf, lam_out, side, a, x, y);
   // sum_i mu_i f^eq_i = rho * Grho
   return fma(-k.om2, fma(rho, G.Grho, -mu_ft),
              (k.om * rho) * fma(G.Gux, k.gx, fma(G.Guy, k.gy, G.Gt * k.dts_dtau)));
-}
-
-// Scatter of a strip's outputs next to a wall or across the periodic seam.  out_i(z) is
-// lambda_i(z - v_i) of the previous step (the transposed pull), or goes to the wall slot of its
-// source column when z - v_i is a ghost; entries of the site whose source z + v_i lies beyond a
-// wall get no push and are set to zero.
-template <bool PERIODIC>
-__device__ __noinline__ void push_strip_edge(const double* sf, double* __restrict__ lam_out, double* __restrict__ side,
-                                             const StepArgs& a, int x, int y) {
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const int xs = wrap_index(x - vx(i), a.lx), yd = y - vy(i);
-    const double val = sf[i * 32];
-    if (!PERIODIC && yd < 0) {
-      __stcs(side + ((long long)xs * kGhostSlots + ghost_base(i, 1) + y), val);
-    } else if (!PERIODIC && yd >= a.ly) {
-      __stcs(side + (((long long)a.lx + xs) * kGhostSlots + ghost_base(i, -1) + (a.ly - 1 - y)), val);
-    } else {
-      __stcs(lam_out + (i * a.pop + (long long)xs * a.pitch + (PERIODIC ? wrap_index(yd, a.ly) : yd)), val);
-    }
-    const int ys = y + vy(i);
-    if (!PERIODIC && (ys < 0 || ys >= a.ly)) __stcs(lam_out + (i * a.pop + (long long)x * a.pitch + y), 0.0);
-  }
 }
 
 // The fixed-point adjoint's view of a site: its slots, and its lambda (planes below 2^32 elements).
@@ -270,7 +283,6 @@ struct AdjIo {
 // barriers, 0.221 with, fully unrolled 0.247; blocks of 8 to 20 warps 0.238 to 0.338).  With lambda's
 // scan under the gather's copies and each group's lambda loaded a group ahead 0.157 ms, 2.9 TB/s; the
 // version in float64 and fixed point it replaces took 0.314.
-extern __shared__ double adj_staged[];
 template <bool PERIODIC>
 __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* fin, const double* lam_next, double* lam_out,
                                                      double* side, double* dtau_part, StepArgs a, AdjConsts k) {
@@ -292,35 +304,42 @@ __global__ void __launch_bounds__(128, 4) k_adj_collide(const double* fin, const
   for (int i = 0; i < Q; ++i)
     top = max(top, reinterpret_cast<const unsigned*>(lam + i * a.pop)[1] & 0x7fffffffu);
   stage_finish<PERIODIC>(fin, a, a, x, y0, yc, sf, LdCached());
-  __syncthreads();
-  const FixMoments m = fix_moments_rolled(c_fix_groups, [&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
-  const FixScalars v = fix_scalars(m, a.fx);
-  const unsigned E = top == 0u ? 512u : top >> 20;  // all zero: any exponent
-  __syncthreads();
-  const int K = (1080 - (int)E) << 20;
-  const bool ok = v.ok && a.fx.usable && k.fx.usable && E - 100u < 978u;
-  const AdjIo io = {sx, lam, (unsigned)a.pop, K};
-  const FixMu mm = fix_mu_moments(K + (1 << 20), c_fix_groups, io);
-  __syncthreads();
-  FixVjp r = fix_vjp(m, v, mm, a.fx, k.fx);
-  if (top == 0u) r = FixVjp{};  // lambda = 0: no rounding residue
-  __syncthreads();
-  fix_adj_outputs(r, k.fx.om1, c_pair_fix, io);
+  bool left = active;  // the lane's site is still to be taken in float64
   double contrib = 0.0;
-  if (active) {
-    if (ok) contrib = fix_dtau(r.D, k.om2, K, m.kb);
-    else contrib = adj_site_float64<PERIODIC>(fin, lam, a, k, x, y, sf);
-    if (edge_strip(a, y0)) {
-      push_strip_edge<PERIODIC>(sf, lam_out, side, a, x, y);
-    } else {
-      double* col[7];  // row y of column x - vx
+  if (a.fx.usable && k.fx.usable) {  // uniform; else the lattice's constants are outside the formats
+    __syncthreads();
+    const FixMoments m = fix_moments_rolled(c_fix_groups, [&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
+    const FixScalars v = fix_scalars(m, a.fx);
+    const unsigned E = top == 0u ? 512u : top >> 20;  // all zero: any exponent
+    __syncthreads();
+    const int K = (1080 - (int)E) << 20;
+    const bool ok = v.ok && E - 100u < 978u;
+    const bool some = __any_sync(0xffffffffu, ok);  // else the rest is spared (831 against 947 us)
+    const AdjIo io = {sx, lam, (unsigned)a.pop, K};
+    FixMu mm = {};
+    if (some) mm = fix_mu_moments(K + (1 << 20), c_fix_groups, io);
+    __syncthreads();
+    FixVjp r = {};
+    if (some) r = fix_vjp(m, v, mm, a.fx, k.fx);
+    if (top == 0u) r = FixVjp{};  // lambda = 0: no rounding residue
+    __syncthreads();
+    if (some) fix_adj_outputs(r, k.fx.om1, c_pair_fix, io);
+    left = active && !ok;
+    if (active && ok) {
+      contrib = fix_dtau(r.D, k.om2, K, m.kb);
+      if (edge_strip(a, y0)) {
+        push_strip_edge<PERIODIC>(sf, lam_out, side, a, x, y);
+      } else {
+        double* col[7];  // row y of column x - vx
 #pragma unroll
-      for (int d = 0; d < 7; ++d)
-        col[d] = lam_out + ((unsigned)wrap_index(x - (d - 3), a.lx) * (unsigned)a.pitch + (unsigned)y);
+        for (int d = 0; d < 7; ++d)
+          col[d] = lam_out + ((unsigned)wrap_index(x - (d - 3), a.lx) * (unsigned)a.pitch + (unsigned)y);
 #pragma unroll
-      for (int i = 0; i < Q; ++i) __stcs(col[vx(i) + 3] + i * a.pop - vy(i), sf[i * 32]);
+        for (int i = 0; i < Q; ++i) __stcs(col[vx(i) + 3] + i * a.pop - vy(i), sf[i * 32]);
+      }
     }
   }
+  if (__any_sync(0xffffffffu, left)) contrib += adj_float64_sites<PERIODIC>(fin, lam_next, lam_out, side, a, k, left);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) contrib += __shfl_down_sync(0xffffffffu, contrib, off);
   __shared__ double warp_sum[4];

@@ -15,28 +15,6 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // Shared staging: one warp holds sf[i * 32 + lane] for its 32 sites.
 constexpr int kFixWarps = 4;  // warps per block (block = 32 x 4 threads)
 
-// The pulled populations of one site, wall values included, loaded from global memory: for
-// sites that leave the fixed-point path, whose staged slots hold their fixed-point forms by then.
-template <bool PERIODIC, class Ld>
-__device__ __forceinline__ void gather_site(const double* fin, const StepScalars& a, const StepWalls& w,
-                                            int x, int yc, double (&f)[Q], Ld ld) {
-  const auto wall_density = [&](int i, int row) {  // of the source column of population i
-    const double* src = fin + (long long)wrap_index(x - vx(i), a.lx) * a.pitch + row;
-    double r = 0.0;
-#pragma unroll 1
-    for (int j = 0; j < Q; ++j) r += ld(src + j * a.pop);
-    return r;
-  };
-#pragma unroll
-  for (int i = 0; i < Q; ++i) {
-    const double* src = fin + i * a.pop + (long long)wrap_index(x - vx(i), a.lx) * a.pitch;
-    const int ys = PERIODIC ? wrap_index(yc - vy(i), a.ly) : yc - vy(i);
-    if (!PERIODIC && vy(i) > 0 && ys < 0) f[i] = wall_density(i, 0) * w.wall_b[i];
-    else if (!PERIODIC && vy(i) < 0 && ys >= a.ly) f[i] = wall_density(i, a.ly - 1) * w.wall_t[i];
-    else f[i] = ld(src + ys);
-  }
-}
-
 // rho(x_s, row) of the seven source columns: lane l sums every fourth population of column
 // l % 8, and two shuffles add the four parts (the same value in the column's four lanes).
 template <class Ld>

@@ -196,3 +196,22 @@ def test_strips_collided_in_float64(lx, ly, bc, hot):
         batch.run(1)
         assert torch.equal(batch.states()[0][:, :, :ly], a)
         batch.close()
+
+
+@pytest.mark.parametrize("lx,ly", [(4, 6), (5, 33), (7, 97)])
+@pytest.mark.parametrize("bc", [lbm.BC_WALLS, lbm.BC_PERIODIC_Y])
+def test_adjoint_of_a_lattice_outside_the_formats(lx, ly, bc):
+    """A forcing outside the fixed-point formats, so that every site is taken in float64, from the first
+    gather (the bar above)."""
+    require_gpu()
+    p = lbm.Params(lx, ly, tau=0.8, gx=0.2, gy=-2e-4, bc=bc)
+    f = device_init(p, rt_fields(p, seed=5))
+    lam = torch.randn(37, lx, ly, dtype=torch.float64, generator=torch.Generator().manual_seed(17))
+    lam_dev = torch.zeros_like(f)
+    lam_dev[:, :, :ly] = lam.cuda()
+    lam_n = torch.zeros_like(f)
+    dtau = torch.zeros((), dtype=torch.float64, device="cuda")
+    lbm.adjoint_step(p, f, lam_dev, lam_n, dtau, lbm.adjoint_work(p))
+    want, want_tau = oracle_vjp(p, to_host(p, f), lam)
+    assert float(((to_host(p, lam_n) - want).abs() / reach_max(lam.abs().amax(0), bc)[None]).max()) <= 1e-13
+    assert abs(float(dtau) - want_tau) <= 1e-10 * max(abs(want_tau), float(lam.abs().sum()) * 1e-3)

@@ -166,35 +166,68 @@ __global__ void __launch_bounds__(128, 4) k_init_fp64(const double* __restrict__
   else init_site_float64(r, u, v, t, dst, a.pop);
 }
 
-// The fields of a site in float64, for sites outside the fixed-point range.
-__device__ __noinline__ void site_fields_float64(const double* __restrict__ f, long long pop, double& rho, double& ux,
-                                                 double& uy, double& T) {
-  double jx, jy, e;
-  moments_float64([&](int i) { return __ldg(f + i * pop); }, rho, jx, jy, e);
-  const double inv_rho = 1.0 / rho;
-  ux = C * jx * inv_rho;
-  uy = C * jy * inv_rho;
-  T = (C2 * e * inv_rho - fma(ux, ux, uy * uy)) / D;
+// The moments (integer velocity units) of a site outside the range of fix_moments' sums: sums in integers
+// at the exponent of its largest population.  Terms round to 2^-54 of that or less, so that the sums are
+// closer to exact than float64 ones, whose 126 operations of the float64 pipe took 1.89 ms for the fields of
+// 2048 x 4096 such sites and 2.11 for the energy (now 0.83 and 0.85), and which are left to sites with an
+// infinity or a NaN and to the ends of the exponent range.
+__device__ __noinline__ void moments_block(const double* __restrict__ f, long long pop, double& rho, double& jx,
+                                           double& jy, double& e) {
+  double g[Q];
+#pragma unroll
+  for (int i = 0; i < Q; ++i) g[i] = __ldg(f + i * pop);
+  unsigned top = 0;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) top = max(top, fx_hi_word(g[i]) & 0x7fffffffu);
+  const int E = (int)(top >> 20), k = 1077 - E;  // |g_i| 2^k < 2^55, and sum |v|^2 |g_i| 2^k < 216 2^55 < 2^63
+  if (E < 55 || E > 2037) {                      // k within fix_to_double_rn's range otherwise
+    moments_float64([&](int i) { return g[i]; }, rho, jx, jy, e);
+    return;
+  }
+  bool unused = false;
+  const auto fix = [&](int i) { return fx_from_double(g[i], k, 64, unused); };
+  long long R = fix(0), En = 0, X = 0, Y = 0;
+#pragma unroll
+  for (int i = 1; i <= NPAIR; ++i) {
+    const long long a = fix(i), b = fix(i + NPAIR), P = a + b, M = a - b;
+    R += P;
+    En += (long long)v2(i) * P;
+    if (rep_vx(i) != 0) X += (long long)rep_vx(i) * M;
+    if (rep_vy(i) != 0) Y += (long long)rep_vy(i) * M;
+  }
+  rho = fix_to_double_rn(R, k), jx = fix_to_double_rn(X, k), jy = fix_to_double_rn(Y, k), e = fix_to_double_rn(En, k);
 }
 
 // rho, c u and T of a site by the fixed-point moments and scalars of site_fix64.cuh: exact sums, four
-// conversions on the float64 pipe.  false outside their range.  The kernels below then run at the
+// conversions on the float64 pipe.  The kernels below then run at the
 // copy rate, given the 128 registers that keep a site's 37 loads in flight (left to itself the
-// compiler took 66 and 0.48 ms): k_moments_fp64 reads and writes 2.75 GB (2048 x 4096) in 0.405 ms, 6.8 TB/s; with
-// rounding sums and float64 scalars it took ~0.85 ms.
-__device__ __forceinline__ bool site_fields_fix(const double* __restrict__ f, long long pop, double& rho, double& cux,
-                                                double& cuy, double& T) {
+// compiler took 66 and 0.48 ms): k_moments_fp64 reads and writes 2.75 GB (2048 x 4096) in 0.395 ms, 7.0 TB/s; with
+// rounding sums and float64 scalars it took ~0.85 ms.  Outside the scalars' range the result is false, and
+// in their places stand rho, jx, jy and e: from the same sums (T = 1.5 everywhere: 0.43 ms for the
+// fields, 0.44 for the energy) or from moments_block.
+__device__ __forceinline__ bool site_fields_fix(const double* __restrict__ f, long long pop, double& rho, double& x,
+                                                double& y, double& T) {
   double g[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) g[i] = __ldg(f + i * pop);
   const FixMoments m = fix_moments([&](int i) { return g[i]; }, [](int, FxHalves) {});
   const FixConsts no_force = {1, {0, 0}, {0, 1 << 30}, {0, 0}, {0, 0}, 0, 0, 0};  // omega = 1, g = 0
   const FixScalars v = fix_scalars(m, no_force);
+  if (!v.ok) {
+    if (m.sums_ok) {  // 2 <= 60 - k <= 951
+      const int k = 60 - m.kb / (1 << 20);
+      rho = fix_to_double_rn(m.R, k), x = fix_to_double_rn(m.X, k), y = fix_to_double_rn(m.Y, k),
+      T = fix_to_double_rn(m.E, k);
+    } else {
+      moments_block(f, pop, rho, x, y, T);
+    }
+    return false;
+  }
   rho = fx_lower_exponent(m.R, (60 << 20) - m.kb);
-  cux = fx_lower_exponent(v.X, 64 << 20);
-  cuy = fx_lower_exponent(v.Y, 64 << 20);
+  x = fx_lower_exponent(v.X, 64 << 20);
+  y = fx_lower_exponent(v.Y, 64 << 20);
   T = fx_lower_exponent((1LL << 60) + (v.t >> 4), 60 << 20);
-  return v.ok;
+  return true;
 }
 
 __global__ void __launch_bounds__(128, 4) k_moments_fp64(const double* __restrict__ fin, double* __restrict__ rho,
@@ -203,17 +236,21 @@ __global__ void __launch_bounds__(128, 4) k_moments_fp64(const double* __restric
   const int x = blockIdx.y * 4 + threadIdx.y;
   const int y = blockIdx.x * 32 + threadIdx.x;
   if (x >= a.lx || y >= a.ly) return;
-  const double* src = fin + (long long)x * a.pitch + y;
   const long long fi = (long long)x * a.ly + y;
-  double r, cx, cy, t;
-  if (site_fields_fix(src, a.pop, r, cx, cy, t)) {
-    rho[fi] = r;
-    ux[fi] = cx * (1.0 / C);
-    uy[fi] = cy * (1.0 / C);
-    T[fi] = t;
+  double r, u, v, t;
+  if (site_fields_fix(fin + (long long)x * a.pitch + y, a.pop, r, u, v, t)) {
+    u *= 1.0 / C;
+    v *= 1.0 / C;
   } else {
-    site_fields_float64(src, a.pop, rho[fi], ux[fi], uy[fi], T[fi]);
+    const double inv_rho = 1.0 / r;
+    u = C * u * inv_rho;
+    v = C * v * inv_rho;
+    t = (C2 * t * inv_rho - fma(u, u, v * v)) / D;
   }
+  rho[fi] = r;
+  ux[fi] = u;
+  uy[fi] = v;
+  T[fi] = t;
 }
 
 // Kinetic energy: per-block partial sums (fixed order), then one block sums the partials.
@@ -223,13 +260,14 @@ __global__ void __launch_bounds__(128, 4) k_ke_partial_fp64(const double* __rest
   const int y = blockIdx.x * 32 + threadIdx.x;
   double ke = 0.0;
   if (x < a.lx && y < a.ly) {
-    const double* src = fin + (long long)x * a.pitch + y;
-    double rho, ux, uy, T;
-    if (site_fields_fix(src, a.pop, rho, ux, uy, T)) {
-      ke = (0.5 / C2) * (rho * fma(ux, ux, uy * uy));
+    double rho, u, v, T;
+    if (site_fields_fix(fin + (long long)x * a.pitch + y, a.pop, rho, u, v, T)) {
+      ke = (0.5 / C2) * (rho * fma(u, u, v * v));
     } else {
-      site_fields_float64(src, a.pop, rho, ux, uy, T);
-      ke = 0.5 * rho * fma(ux, ux, uy * uy);
+      const double inv_rho = 1.0 / rho;
+      u = C * u * inv_rho;
+      v = C * v * inv_rho;
+      ke = 0.5 * rho * fma(u, u, v * v);
     }
   }
 #pragma unroll

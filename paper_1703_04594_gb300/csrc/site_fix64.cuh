@@ -168,6 +168,7 @@ struct FixMoments {
   long long R, E, X, Y;  // sum f, sum |v|^2 f, sum vx f, sum vy f, times 2^-k [60]
   int kb;                // k << 20 (the exponent field's unit), for the results
   bool ok;               // every population in range
+  bool sums_ok;          // the four sums hold, populations up to twice the range among them
 };
 
 // `load(i)` returns f_i as a float64, `keep(i, h)` stores its fixed-point form as halves; each is
@@ -234,6 +235,8 @@ __host__ __device__ __forceinline__ FixMoments fix_moments(Load&& load, Keep&& k
   // k below 60 (fx_lower_exponent), and rules out a sign bit, zeros, infinities and NaNs (with
   // f_0 ordinary, the others' shifts rule theirs out)
   m.ok = worst <= 8u && E0 - 128u <= 950u;
+  // below 4: four of them stay below 2^64, and the sums below 8 (E, the largest, below 6.9)
+  m.sums_ok = worst <= 9u && E0 - 128u <= 950u;
   return m;
 }
 
@@ -287,6 +290,8 @@ __host__ __device__ __forceinline__ FixMoments fix_moments_rolled(const FixGroup
   m.X = (long long)X;
   m.Y = (long long)Y;
   m.ok = worst <= 8u && E0 - 128u <= 950u;
+  // below 4: four of them stay below 2^64, and the sums below 8 (E, the largest, below 6.9)
+  m.sums_ok = worst <= 9u && E0 - 128u <= 950u;
   return m;
 }
 

@@ -143,12 +143,12 @@ __global__ void __launch_bounds__(128) k_collide_fp64(const double* __restrict__
 // f_i = f_i^eq(rho, u, T) from [lx][ly] fields: the fixed-point equilibrium of site_fix64.cuh (the
 // float64 pipe converts the 37 results and little else; a float64 equilibrium's ~250 operations of
 // it took 5.5 times as long), float64 for fields outside its range.
-__device__ __noinline__ void init_site_float64(double rho, double ux, double uy, double T, double* __restrict__ dst,
+__device__ __noinline__ void init_site_float64(double rho, double X, double Y, double t, double* __restrict__ dst,
                                                long long pop) {
   double f[Q];
 #pragma unroll
   for (int i = 0; i < Q; ++i) f[i] = 0.0;
-  relax_site(f, 0.0, rho, C * ux, C * uy, T - 1.0, [&](int i, double v) { dst[i * pop] = v; });
+  relax_site(f, 0.0, rho, X, Y, t, [&](int i, double v) { dst[i * pop] = v; });
 }
 
 __global__ void __launch_bounds__(128, 4) k_init_fp64(const double* __restrict__ rho, const double* __restrict__ ux,
@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(128, 4) k_init_fp64(const double* __restrict__
   int kb;
   const FixScalars s = fix_scalars_of(r, u, v, t, kb);
   if (s.ok) fix_relax<true>(s, FxHalves{0, 0}, StepIo{nullptr, dst, a.pop, kb});
-  else init_site_float64(r, u, v, t, dst, a.pop);
+  else init_site_float64(r, C * u, C * v, t - 1.0, dst, a.pop);
 }
 
 // The moments (integer velocity units) of a site outside the range of fix_moments' sums: sums in integers

@@ -26,6 +26,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -61,31 +62,16 @@ constexpr size_t kBatchSyncLaunchBytes = 3 * sizeof(unsigned int);
 namespace {
 
 // Step kinds: the strip functions of the three storage/arithmetic forms.
-// kFp32Scaled: FP32 storage where some lattice has a reference density outside [1/2, 2) (the
-// moment sums read each lattice's scale constants; see step_fp32.cuh); kFp32Cons and
-// kFp32ConsScaled: the same with the conserved-moment correction (LBM_FP32_CONSERVED).
-enum BatchKind { kFp32 = 1, kFix64 = 2, kFp32Scaled = 3, kFp32Cons = 4, kFp32ConsScaled = 5 };
+// kFp32Scaled: FP32 storage where every lattice has a reference density outside [1/2, 2), kFp32Mixed:
+// where some have (see Fp32Scale); kFp32Cons...: the same with the conserved-moment correction
+// (LBM_FP32_CONSERVED).
+enum BatchKind {
+  kFix64 = 1, kFp32 = 2, kFp32Scaled = 3, kFp32Mixed = 4, kFp32Cons = 5, kFp32ConsScaled = 6, kFp32ConsMixed = 7
+};
 
-template <int K>
-struct KindOf {
-  using T = double;
-};
-template <>
-struct KindOf<kFp32> {
-  using T = float;
-};
-template <>
-struct KindOf<kFp32Scaled> {
-  using T = float;
-};
-template <>
-struct KindOf<kFp32Cons> {
-  using T = float;
-};
-template <>
-struct KindOf<kFp32ConsScaled> {
-  using T = float;
-};
+constexpr bool conserves(int kind) { return kind >= kFp32Cons; }
+constexpr int scale_of(int kind) { return (kind - (conserves(kind) ? kFp32Cons : kFp32)) + kUnscaled; }
+static_assert(scale_of(kFp32) == kUnscaled && scale_of(kFp32ConsScaled) == kScaled && scale_of(kFp32Mixed) == kMixed, "");
 
 // Shared memory of a block: the fixed-point form stages 37 x 32 doubles per warp.
 inline size_t batch_smem_bytes(int kind, int warps) {
@@ -108,7 +94,7 @@ __device__ __noinline__ void tile_float64_sites(const BatchLattice* L, const Bat
 template <int KIND, bool PERIODIC, class Ld>
 __device__ __forceinline__ void batch_tile(const BatchLattice* __restrict__ L, const BatchTile* __restrict__ tiles,
                                            long long t, int parity, Ld ld, double* staged) {
-  using T = typename KindOf<KIND>::T;
+  using T = std::conditional_t<KIND == kFix64, double, float>;
   const BatchTile tile = tiles[t];
   const BatchLattice& B = L[tile.lattice];
   const int x = tile.x0 + (int)threadIdx.y, y0 = tile.y0;
@@ -119,8 +105,7 @@ __device__ __forceinline__ void batch_tile(const BatchLattice* __restrict__ L, c
     const bool left = step_strip_fix64<PERIODIC>(src, dst, B.a, B.a, x, y0, ld, staged + threadIdx.y * (Q * 32));
     if (__any_sync(0xffffffffu, left)) tile_float64_sites<PERIODIC, Ld>(L, tiles, t, parity, left, staged);
   } else
-    step_strip_fp32<PERIODIC, KIND == kFp32Scaled || KIND == kFp32ConsScaled, KIND == kFp32Cons || KIND == kFp32ConsScaled>(
-        src, dst, B.a, B.a, x, y0, ld);
+    step_strip_fp32<PERIODIC, scale_of(KIND), conserves(KIND)>(src, dst, B.a, B.a, x, y0, ld);
 }
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
@@ -174,7 +159,7 @@ __device__ __forceinline__ bool grid_barrier(BatchSync* sync, unsigned target, l
 // lattices Lx 128..1024: float64 26.5 ms a step (106.7 colliding in float64), FP32 11.6 (13.0);
 // 256 of 32 to 128, where two strips of five touch a wall: FP32 0.177 ms (0.295).
 constexpr int batch_max_regs(int kind) {
-  return kind == kFix64 || kind == kFp32Cons || kind == kFp32ConsScaled ? 96 : 80;
+  return kind == kFix64 || conserves(kind) ? 96 : 80;
 }
 
 extern __shared__ double batch_staged[];
@@ -212,7 +197,7 @@ struct lbm_batch {
   int n = 0;
   int precision = LBM_FP64;
   int periodic = 0;
-  int fp32_scaled = 0;  // FP32 batch with some reference density outside [1/2, 2)
+  int scaled = 0;  // lattices of an FP32 batch with a reference density outside [1/2, 2)
   long long total_tiles = 0;
   BatchTile* dev_tiles = nullptr;
   size_t tile_table_cap = 0;
@@ -240,39 +225,34 @@ int32_t cuda_status(cudaError_t e) {
 }
 
 int kind_of(const lbm_batch* b) {
-  if (b->precision == LBM_FP32_SHIFTED) return b->fp32_scaled ? kFp32Scaled : kFp32;
-  if (b->precision == LBM_FP32_CONSERVED) return b->fp32_scaled ? kFp32ConsScaled : kFp32Cons;
-  return kFix64;  // LBM_FP64 and LBM_FP64_FIXED
+  if (b->precision != LBM_FP32_SHIFTED && b->precision != LBM_FP32_CONSERVED) return kFix64;
+  const int scale = b->scaled == 0 ? kUnscaled : b->scaled == b->n ? kScaled : kMixed;
+  return (b->precision == LBM_FP32_CONSERVED ? kFp32Cons : kFp32) + (scale - kUnscaled);
 }
 
-template <int K>
-void* persistent_fn(bool periodic) {
-  return periodic ? (void*)k_batch_persistent<K, true> : (void*)k_batch_persistent<K, false>;
-}
 using PerStepKernel = void (*)(const BatchLattice*, const BatchTile*, long long, int);
+struct BatchKernels {
+  PerStepKernel per_step;
+  void* persistent;
+};
 template <int K>
-PerStepKernel per_step_fn(bool periodic) {
-  return periodic ? k_batch_step<K, true> : k_batch_step<K, false>;
+BatchKernels kernels_of(bool periodic) {
+  return periodic ? BatchKernels{k_batch_step<K, true>, (void*)k_batch_persistent<K, true>}
+                  : BatchKernels{k_batch_step<K, false>, (void*)k_batch_persistent<K, false>};
 }
-
-void* persistent_kernel(const lbm_batch* b) {
+BatchKernels batch_kernels(const lbm_batch* b) {
   switch (kind_of(b)) {
-    case kFp32: return persistent_fn<kFp32>(b->periodic);
-    case kFp32Scaled: return persistent_fn<kFp32Scaled>(b->periodic);
-    case kFp32Cons: return persistent_fn<kFp32Cons>(b->periodic);
-    case kFp32ConsScaled: return persistent_fn<kFp32ConsScaled>(b->periodic);
-    default: return persistent_fn<kFix64>(b->periodic);
+    case kFp32: return kernels_of<kFp32>(b->periodic);
+    case kFp32Scaled: return kernels_of<kFp32Scaled>(b->periodic);
+    case kFp32Mixed: return kernels_of<kFp32Mixed>(b->periodic);
+    case kFp32Cons: return kernels_of<kFp32Cons>(b->periodic);
+    case kFp32ConsScaled: return kernels_of<kFp32ConsScaled>(b->periodic);
+    case kFp32ConsMixed: return kernels_of<kFp32ConsMixed>(b->periodic);
+    default: return kernels_of<kFix64>(b->periodic);
   }
 }
-PerStepKernel per_step_kernel(const lbm_batch* b) {
-  switch (kind_of(b)) {
-    case kFp32: return per_step_fn<kFp32>(b->periodic);
-    case kFp32Scaled: return per_step_fn<kFp32Scaled>(b->periodic);
-    case kFp32Cons: return per_step_fn<kFp32Cons>(b->periodic);
-    case kFp32ConsScaled: return per_step_fn<kFp32ConsScaled>(b->periodic);
-    default: return per_step_fn<kFix64>(b->periodic);
-  }
-}
+PerStepKernel per_step_kernel(const lbm_batch* b) { return batch_kernels(b).per_step; }
+void* persistent_kernel(const lbm_batch* b) { return batch_kernels(b).persistent; }
 
 // Raises both kernels' dynamic shared memory limit to the largest staging a block can
 // need (8 warps); called once per plan.
@@ -420,7 +400,7 @@ int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* 
     BatchLattice L;
     memset(&L, 0, sizeof(L));
     L.a = make_step_args(p);
-    if (L.a.fp32_scaled) b->fp32_scaled = 1;
+    b->scaled += L.a.fp32_scaled;
     L.f[0] = f_a[j];
     L.f[1] = f_b[j];
     b->host.push_back(L);

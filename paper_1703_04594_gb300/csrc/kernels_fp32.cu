@@ -18,7 +18,7 @@ namespace d2q37 {
 #ifndef LBM_FP32C_MIN_BLOCKS
 #define LBM_FP32C_MIN_BLOCKS 5
 #endif
-template <bool PERIODIC, bool SCALED, bool CONSERVE>
+template <bool PERIODIC, int SCALED, bool CONSERVE>
 __global__ void __launch_bounds__(128, CONSERVE ? LBM_FP32C_MIN_BLOCKS : LBM_FP32_MIN_BLOCKS) k_step_fp32(
     const float* fin, float* fout, StepArgs a) {
   pdl_trigger();
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(128) k_init_fp32(const double* __restrict__ rh
 __device__ __forceinline__ void site_fields_fp32(const float (&g)[Q], const StepScalars& a, double& rho, double& ux,
                                                  double& uy, double& T) {
   const double rho0 = a.rho0;
-  const DevMoments<double> m = moments_fix<double, true>(g, a);
+  const DevMoments<double> m = moments_fix<double, kScaled>(g, a);
   rho = m.drho + rho0;
   const double inv = 1.0 / rho;
   ux = C * m.jx * inv;
@@ -97,7 +97,7 @@ __global__ void __launch_bounds__(128) k_ke_partial_fp32(const float* __restrict
 static inline dim3 site_grid(const StepArgs& a) { return dim3((a.ly + 31) / 32, (a.lx + 3) / 4); }
 static const dim3 kSiteBlock(32, 4);
 
-template <bool PERIODIC, bool SCALED>
+template <bool PERIODIC, int SCALED>
 static cudaError_t launch_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {
   return launch_dependent(a.conserve ? k_step_fp32<PERIODIC, SCALED, true> : k_step_fp32<PERIODIC, SCALED, false>,
                           step_grid(a), step_block(a), 0, s, fin, fout, a);
@@ -105,8 +105,8 @@ static cudaError_t launch_fp32(const float* fin, float* fout, const StepArgs& a,
 
 cudaError_t launch_step_fp32(const float* fin, float* fout, const StepArgs& a, cudaStream_t s) {
   const bool scaled = a.fp32_scaled;
-  if (a.periodic) return scaled ? launch_fp32<true, true>(fin, fout, a, s) : launch_fp32<true, false>(fin, fout, a, s);
-  return scaled ? launch_fp32<false, true>(fin, fout, a, s) : launch_fp32<false, false>(fin, fout, a, s);
+  if (a.periodic) return scaled ? launch_fp32<true, kScaled>(fin, fout, a, s) : launch_fp32<true, kUnscaled>(fin, fout, a, s);
+  return scaled ? launch_fp32<false, kScaled>(fin, fout, a, s) : launch_fp32<false, kUnscaled>(fin, fout, a, s);
 }
 
 cudaError_t launch_init_fp32(const double* rho, const double* ux, const double* uy, const double* T, float* f,

@@ -54,3 +54,48 @@ def test_wall_sums_beyond_the_storage_range(ly):
         out.append(o[:, :, :ly].double())
     assert bool(torch.isfinite(out[0]).all())
     assert float((out[0] - out[1]).abs().max()) <= 1e-5 * float(out[1].abs().max())
+
+
+@pytest.mark.parametrize("precision", [lbm.FP32_SHIFTED, lbm.FP32_CONSERVED])
+@pytest.mark.parametrize("rho0", [0.9, 1.3])
+def test_batch_of_mixed_reference_densities(rho0, precision):
+    """One lattice with a reference density outside [1/2, 2) puts a batch on the kernel that reads each
+    lattice's constants; every lattice still has the bits of its own lbm_run.  A last bit of a float64
+    density decides a float32 rounding once in some 10^8 sites, hence the size."""
+    require_gpu()
+    params, fa, fb, want = [], [], [], []
+    for j, (lx, ly, r) in enumerate([(2048, 2048, rho0), (24, 50, 3.0), (27, 63, 0.3), (30, 76, 0.7)]):
+        p = lbm.Params(lx, ly, tau=0.7, gx=1e-4, rho0=r, precision=precision)
+        rho, ux, uy, T = rt_fields(p, seed=40 + j)
+        f = device_init(p, [t.contiguous() for t in (rho * r, ux + 0.02, uy - 0.01, T)])
+        params.append(p)
+        want.append(lbm.run(p, f.clone(), lbm.empty_state(p), 300).clone())
+        fa.append(f)
+        fb.append(lbm.empty_state(p))
+    b = lbm.Batch(params, fa, fb)
+    b.run(300)
+    for p, got, w in zip(params, b.states(), want):
+        assert torch.equal(got[:, :, :p.ly], w[:, :, :p.ly]), p.rho0
+    b.close()
+
+
+@pytest.mark.parametrize("precision", [lbm.FP32_SHIFTED, lbm.FP32_CONSERVED])
+@pytest.mark.parametrize("mode", [lbm.BATCH_PER_STEP, lbm.BATCH_PERSISTENT])
+@pytest.mark.parametrize("bc", [lbm.BC_WALLS, lbm.BC_PERIODIC_Y])
+@pytest.mark.parametrize("densities", [(0.7, 1.3, 1.0), (3.0, 0.3, 1600.0), (0.9, 3.0, 1.0, 0.3)])
+def test_batches_in_each_instantiation(densities, bc, mode, precision):
+    """Reference densities all inside [1/2, 2), all outside, and both: the bits of the single runs."""
+    require_gpu()
+    params, fa, want = [], [], []
+    for j, rho0 in enumerate(densities):
+        p = lbm.Params(11 + 3 * j, 33 + 13 * j, tau=0.7, gx=1e-4, rho0=rho0, precision=precision, bc=bc)
+        rho, ux, uy, T = rt_fields(p, seed=40 + j)
+        fa.append(device_init(p, [t.contiguous() for t in (rho * rho0, ux + 0.02, uy - 0.01, T)]))
+        params.append(p)
+        want.append(lbm.run(p, fa[-1].clone(), lbm.empty_state(p), 5).clone())
+    b = lbm.Batch(params, fa, [lbm.empty_state(p) for p in params])
+    b.configure(mode, 2)
+    b.run(5)
+    for p, got, w in zip(params, b.states(), want):
+        assert torch.equal(got[:, :, :p.ly], w[:, :, :p.ly]), p.rho0
+    b.close()

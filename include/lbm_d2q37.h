@@ -26,8 +26,8 @@
  * Conventions for every call:
  *   - Pointers named *_dev are device pointers; *_host are host pointers.  The caller
  *     owns every buffer and the stream; no entry point allocates device memory except
- *     lbm_batch_plan (its tables, freed by lbm_batch_destroy) and lbm_probe_peak (a result
- *     buffer it frees before returning).
+ *     lbm_batch_plan, lbm_batch_configure and lbm_batch_autotune (the batch's tables, freed by
+ *     lbm_batch_destroy) and lbm_probe_peak (a result buffer it frees before returning).
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default stream).  Calls
  *     are stream-ordered and asynchronous unless stated otherwise.
  *   - Return value: LBM_OK, or an lbm_status error code.  Invalid arguments are
@@ -233,14 +233,16 @@ enum lbm_batch_mode {
 /* Validates n lattices and binds their buffers (f_a_dev[j], f_b_dev[j]: device states of
  * lbm_buffer_bytes(&params[j]) bytes, current state in f_a; no two of the 2n buffers may
  * overlap, else LBM_EINVAL).  Allocates the batch's own
- * device descriptor table, tile table and barrier word (freed by lbm_batch_destroy).
+ * device descriptor table, tile table and barrier word (freed by lbm_batch_destroy, as are the
+ * tables that lbm_batch_configure and lbm_batch_autotune add).
  * Synchronous.  Default configuration: one launch per step, tiles of 32 x 4.  At most 65535
  * lattices. */
 int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a_dev, void* const* f_b_dev, int32_t n,
                        lbm_batch** out);
 /* Sets mode, tile shape (a block steps a tile of 32 rows x tile_columns columns, one warp
  * per column; tile_columns = 1, 2, 4 or 8) and blocks per SM (persistent only; 0 = all that
- * fit).  Synchronous when the tile shape changes (the tile table is rebuilt). */
+ * fit).  Synchronous on the first use of a tile shape, for which a tile table is made; runs in
+ * flight and captured graphs keep the shape they were launched with. */
 int32_t lbm_batch_configure(lbm_batch* b, int32_t mode, int32_t tile_columns, int32_t blocks_per_sm);
 /* Reads the configuration (blocks_per_sm: the value the persistent launch uses, else 0). */
 int32_t lbm_batch_config(const lbm_batch* b, int32_t* mode, int32_t* tile_columns, int32_t* blocks_per_sm);

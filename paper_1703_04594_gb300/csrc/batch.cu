@@ -40,8 +40,6 @@ namespace d2q37 {
 struct BatchLattice {
   StepArgs a;
   void* f[2];            // state buffers; f[parity] holds the current state
-  int tiles_y;  // ceil(ly / 32)
-  int tiles_x;  // ceil(lx / TX)
 };
 
 // One tile of the batch: its lattice and first site (the table spares every thread a search and a
@@ -164,7 +162,7 @@ constexpr int batch_max_regs(int kind) {
 
 extern __shared__ double batch_staged[];
 
-// (the two tables are written before any launch that reads them, so they may be read-only loads)
+// (the two tables are written once, before any launch that reads them, so they may be read-only loads)
 template <int KIND, bool PERIODIC>
 __global__ void __launch_bounds__(256) __maxnreg__(batch_max_regs(KIND)) k_batch_step(const BatchLattice* __restrict__ L,
                                                     const BatchTile* __restrict__ tiles, long long total,
@@ -198,15 +196,17 @@ struct lbm_batch {
   int precision = LBM_FP64;
   int periodic = 0;
   int scaled = 0;  // lattices of an FP32 batch with a reference density outside [1/2, 2)
-  long long total_tiles = 0;
-  BatchTile* dev_tiles = nullptr;
-  size_t tile_table_cap = 0;
+  // A table of tiles for each tile width of 1, 2, 4 and 8 columns, made on its first use and kept as it is:
+  // launches in flight and captured graphs go on reading the one that they were given.
+  BatchTile* tables[4] = {};
+  long long tiles[4] = {};
   std::vector<BatchLattice> host;
   BatchLattice* dev_lattices = nullptr;
   BatchSync* dev_sync = nullptr;
   int parity = 0;
   int mode = LBM_BATCH_PER_STEP;
   int warps_per_block = 4;  // = tile width TX
+  int table() const { return warps_per_block == 8 ? 3 : warps_per_block / 2; }
   int blocks_per_sm = 0;  // 0 = as many as fit
   long long timeout_ns = 2000000000LL;
   unsigned phantom = 0;
@@ -277,11 +277,11 @@ int max_blocks_per_sm(const lbm_batch* b, int wpb) {
 }
 
 int32_t launch_per_step(lbm_batch* b, int steps, cudaStream_t s) {
-  if (b->total_tiles > 0x7fffffffLL) return LBM_EINVAL;
+  long long total = b->tiles[b->table()];
+  if (total > 0x7fffffffLL) return LBM_EINVAL;
   const size_t smem = batch_smem_bytes(kind_of(b), b->warps_per_block);
   const BatchLattice* L = b->dev_lattices;
-  const BatchTile* tiles = b->dev_tiles;
-  long long total = b->total_tiles;
+  const BatchTile* tiles = b->tables[b->table()];
   for (int st = 0; st < steps; ++st) {
     int par = (b->parity + st) & 1;
     const int32_t st_ = cuda_status(launch_dependent(per_step_kernel(b), dim3((unsigned)total),
@@ -301,8 +301,8 @@ int32_t launch_persistent(lbm_batch* b, int steps, cudaStream_t s) {
   int32_t st = cuda_status(cudaMemsetAsync(b->dev_sync, 0, kBatchSyncLaunchBytes, s));
   if (st != LBM_OK) return st;
   const BatchLattice* L = b->dev_lattices;
-  const BatchTile* tiles = b->dev_tiles;
-  long long total = b->total_tiles;
+  const BatchTile* tiles = b->tables[b->table()];
+  long long total = b->tiles[b->table()];
   int parity0 = b->parity;
   BatchSync* sync = b->dev_sync;
   unsigned phantom = b->phantom;
@@ -346,31 +346,22 @@ int32_t run(lbm_batch* b, int steps, cudaStream_t s) {
   return st;
 }
 
-// Tile layout for tiles of 32 rows x tx columns, and the tile table, uploaded
-// to the device (synchronous; grows the table allocation when needed).
+// Tiles of 32 rows x tx columns from here on: their table is made, if it is not there yet, and uploaded
+// (synchronous).
 int32_t relayout(lbm_batch* b, int tx) {
-  std::vector<BatchTile> table;
-  for (int j = 0; j < b->n; ++j) {
-    BatchLattice& L = b->host[j];
-    L.tiles_y = (L.a.ly + 31) / 32;
-    L.tiles_x = (L.a.lx + tx - 1) / tx;
-    for (int x = 0; x < L.tiles_x; ++x)
-      for (int y = 0; y < L.tiles_y; ++y) table.push_back({j, x * tx, y * 32, 0});
-  }
-  const long long tiles = (long long)table.size();
-  if ((size_t)tiles > b->tile_table_cap) {
-    if (b->dev_tiles) cudaFree(b->dev_tiles);
-    b->dev_tiles = nullptr;
-    b->tile_table_cap = 0;
-    if (cudaMalloc(&b->dev_tiles, sizeof(BatchTile) * (size_t)tiles) != cudaSuccess) return LBM_ENOMEM;
-    b->tile_table_cap = (size_t)tiles;
-  }
-  b->total_tiles = tiles;
   b->warps_per_block = tx;
-  int32_t st = cuda_status(
-      cudaMemcpy(b->dev_tiles, table.data(), sizeof(BatchTile) * (size_t)tiles, cudaMemcpyHostToDevice));
-  if (st != LBM_OK) return st;
-  return cuda_status(cudaMemcpy(b->dev_lattices, b->host.data(), sizeof(BatchLattice) * b->n, cudaMemcpyHostToDevice));
+  const int which = b->table();
+  if (b->tables[which]) return LBM_OK;
+  std::vector<BatchTile> table;
+  for (int j = 0; j < b->n; ++j)
+    for (int x = 0; x < b->host[j].a.lx; x += tx)
+      for (int y = 0; y < b->host[j].a.ly; y += 32) table.push_back({j, x, y, 0});
+  const size_t bytes = sizeof(BatchTile) * table.size();
+  if (cudaMalloc(&b->tables[which], bytes) != cudaSuccess) return LBM_ENOMEM;
+  b->tiles[which] = (long long)table.size();
+  const int32_t st = cuda_status(cudaMemcpy(b->tables[which], table.data(), bytes, cudaMemcpyHostToDevice));
+  // (a copy from pageable memory may return before its last part has arrived)
+  return st != LBM_OK ? st : cuda_status(cudaStreamSynchronize(0));
 }
 
 bool overlap(const void* a, const void* b, int64_t bytes) {
@@ -436,9 +427,10 @@ int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* 
     delete b;
     return LBM_ENOMEM;
   }
-  if (relayout(b, 4) != LBM_OK || cudaMemset(b->dev_sync, 0, sizeof(BatchSync)) != cudaSuccess ||
-      allow_batch_smem(b) != LBM_OK) {
-    cudaFree(b->dev_tiles);
+  if (cudaMemset(b->dev_sync, 0, sizeof(BatchSync)) != cudaSuccess ||
+      cudaMemcpy(b->dev_lattices, b->host.data(), sizeof(BatchLattice) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
+      relayout(b, 4) != LBM_OK || allow_batch_smem(b) != LBM_OK) {
+    cudaFree(b->tables[b->table()]);
     cudaFree(b->dev_lattices);
     cudaFree(b->dev_sync);
     delete b;
@@ -555,7 +547,7 @@ int64_t lbm_batch_sites(const lbm_batch* b) {
 
 void lbm_batch_destroy(lbm_batch* b) {
   if (!b) return;
-  cudaFree(b->dev_tiles);
+  for (BatchTile* t : b->tables) cudaFree(t);
   cudaFree(b->dev_lattices);
   cudaFree(b->dev_sync);
   delete b;

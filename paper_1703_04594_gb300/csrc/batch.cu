@@ -26,6 +26,8 @@
 
 #include <algorithm>
 #include <cstring>
+#include <exception>
+#include <memory>
 #include <type_traits>
 #include <utility>
 #include <vector>
@@ -206,12 +208,19 @@ struct lbm_batch {
   int parity = 0;
   int mode = LBM_BATCH_PER_STEP;
   int warps_per_block = 4;  // = tile width TX
-  int table() const { return warps_per_block == 8 ? 3 : warps_per_block / 2; }
+  int table() const { return table_of(warps_per_block); }
+  static int table_of(int tx) { return tx == 8 ? 3 : tx / 2; }
   int blocks_per_sm = 0;  // 0 = as many as fit
   long long timeout_ns = 2000000000LL;
   unsigned phantom = 0;
   int device = 0;
   int sms = 0;
+  ~lbm_batch() {
+    for (BatchTile* t : tables)
+      if (t) cudaFree(t);
+    if (dev_lattices) cudaFree(dev_lattices);
+    if (dev_sync) cudaFree(dev_sync);
+  }
 };
 
 namespace {
@@ -346,22 +355,52 @@ int32_t run(lbm_batch* b, int steps, cudaStream_t s) {
   return st;
 }
 
+// Device memory for n values, or LBM_ENOMEM with the failed call's error taken back (the next launch would
+// report it).
+template <class T>
+int32_t device_alloc(T** p, size_t n) {
+  if (cudaMalloc(p, sizeof(T) * n) == cudaSuccess) return LBM_OK;
+  *p = nullptr;
+  cudaGetLastError();
+  return LBM_ENOMEM;
+}
+
+// `call()`, with running out of host memory as a status.
+template <class Call>
+int32_t without_exceptions(Call&& call) {
+  try {
+    return call();
+  } catch (const std::exception&) {  // bad_alloc, length_error
+    return LBM_ENOMEM;
+  }
+}
+
 // Tiles of 32 rows x tx columns from here on: their table is made, if it is not there yet, and uploaded
-// (synchronous).
+// (synchronous).  On an error the batch stays as it was.
 int32_t relayout(lbm_batch* b, int tx) {
+  BatchTile*& dev = b->tables[lbm_batch::table_of(tx)];
+  if (!dev) {
+    size_t tiles = 0;
+    for (const BatchLattice& L : b->host) tiles += (size_t)((L.a.lx + tx - 1) / tx) * ((L.a.ly + 31) / 32);
+    std::vector<BatchTile> table;
+    table.reserve(tiles);
+    for (int j = 0; j < b->n; ++j)
+      for (int x = 0; x < b->host[j].a.lx; x += tx)
+        for (int y = 0; y < b->host[j].a.ly; y += 32) table.push_back({j, x, y, 0});
+    int32_t st = device_alloc(&dev, tiles);
+    if (st != LBM_OK) return st;
+    st = cuda_status(cudaMemcpy(dev, table.data(), sizeof(BatchTile) * tiles, cudaMemcpyHostToDevice));
+    // (a copy from pageable memory may return before its last part has arrived)
+    if (st == LBM_OK) st = cuda_status(cudaStreamSynchronize(0));
+    if (st != LBM_OK) {
+      cudaFree(dev);
+      dev = nullptr;
+      return st;
+    }
+    b->tiles[lbm_batch::table_of(tx)] = (long long)tiles;
+  }
   b->warps_per_block = tx;
-  const int which = b->table();
-  if (b->tables[which]) return LBM_OK;
-  std::vector<BatchTile> table;
-  for (int j = 0; j < b->n; ++j)
-    for (int x = 0; x < b->host[j].a.lx; x += tx)
-      for (int y = 0; y < b->host[j].a.ly; y += 32) table.push_back({j, x, y, 0});
-  const size_t bytes = sizeof(BatchTile) * table.size();
-  if (cudaMalloc(&b->tables[which], bytes) != cudaSuccess) return LBM_ENOMEM;
-  b->tiles[which] = (long long)table.size();
-  const int32_t st = cuda_status(cudaMemcpy(b->tables[which], table.data(), bytes, cudaMemcpyHostToDevice));
-  // (a copy from pageable memory may return before its last part has arrived)
-  return st != LBM_OK ? st : cuda_status(cudaStreamSynchronize(0));
+  return LBM_OK;
 }
 
 bool overlap(const void* a, const void* b, int64_t bytes) {
@@ -369,14 +408,8 @@ bool overlap(const void* a, const void* b, int64_t bytes) {
   return x < y + (uintptr_t)bytes && y < x + (uintptr_t)bytes;
 }
 
-}  // namespace
-
-extern "C" {
-
-int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* f_b, int32_t n, lbm_batch** out) {
-  if (!params || !f_a || !f_b || !out || n <= 0 || n > 65535) return LBM_EINVAL;
-  *out = nullptr;
-  lbm_batch* b = new lbm_batch();
+int32_t make_batch(const lbm_params* params, void* const* f_a, void* const* f_b, int32_t n, lbm_batch** out) {
+  std::unique_ptr<lbm_batch> b(new lbm_batch());
   b->n = n;
   b->precision = params[0].precision;
   b->periodic = params[0].bc == LBM_BC_PERIODIC_Y;
@@ -384,10 +417,8 @@ int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* 
     const lbm_params* p = &params[j];
     const int64_t bytes = lbm_buffer_bytes(p);
     if (!params_valid(p) || p->precision != b->precision || p->bc != params[0].bc || bytes <= 0 || !f_a[j] ||
-        !f_b[j] || ((uintptr_t)f_a[j] % 16) || ((uintptr_t)f_b[j] % 16) || overlap(f_a[j], f_b[j], bytes)) {
-      delete b;
+        !f_b[j] || ((uintptr_t)f_a[j] % 16) || ((uintptr_t)f_b[j] % 16) || overlap(f_a[j], f_b[j], bytes))
       return LBM_EINVAL;
-    }
     BatchLattice L;
     memset(&L, 0, sizeof(L));
     L.a = make_step_args(p);
@@ -407,46 +438,41 @@ int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* 
     }
     std::sort(ranges.begin(), ranges.end());
     for (size_t k = 1; k < ranges.size(); ++k)
-      if (ranges[k].first < ranges[k - 1].second) {
-        delete b;
-        return LBM_EINVAL;
-      }
+      if (ranges[k].first < ranges[k - 1].second) return LBM_EINVAL;
   }
   cudaDeviceProp prop;
-  if (cudaGetDevice(&b->device) != cudaSuccess || cudaGetDeviceProperties(&prop, b->device) != cudaSuccess) {
-    delete b;
+  if (cudaGetDevice(&b->device) != cudaSuccess || cudaGetDeviceProperties(&prop, b->device) != cudaSuccess)
     return LBM_ECUDA;
-  }
   b->sms = prop.multiProcessorCount;
-  if (cudaMalloc(&b->dev_lattices, sizeof(BatchLattice) * n) != cudaSuccess) {
-    delete b;
-    return LBM_ENOMEM;
-  }
-  if (cudaMalloc(&b->dev_sync, sizeof(BatchSync)) != cudaSuccess) {
-    cudaFree(b->dev_lattices);
-    delete b;
-    return LBM_ENOMEM;
-  }
+  int32_t st;
+  if ((st = device_alloc(&b->dev_lattices, n)) != LBM_OK || (st = device_alloc(&b->dev_sync, 1)) != LBM_OK) return st;
   if (cudaMemset(b->dev_sync, 0, sizeof(BatchSync)) != cudaSuccess ||
       cudaMemcpy(b->dev_lattices, b->host.data(), sizeof(BatchLattice) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      relayout(b, 4) != LBM_OK || allow_batch_smem(b) != LBM_OK) {
-    cudaFree(b->tables[b->table()]);
-    cudaFree(b->dev_lattices);
-    cudaFree(b->dev_sync);
-    delete b;
+      allow_batch_smem(b.get()) != LBM_OK)
     return LBM_ECUDA;
-  }
-  *out = b;
+  if ((st = relayout(b.get(), 4)) != LBM_OK) return st;
+  *out = b.release();
   return LBM_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int32_t lbm_batch_plan(const lbm_params* params, void* const* f_a, void* const* f_b, int32_t n, lbm_batch** out) {
+  if (!params || !f_a || !f_b || !out || n <= 0 || n > 65535) return LBM_EINVAL;
+  *out = nullptr;
+  return without_exceptions([&] { return make_batch(params, f_a, f_b, n, out); });
 }
 
 int32_t lbm_batch_configure(lbm_batch* b, int32_t mode, int32_t tile_columns, int32_t blocks_per_sm) {
   if (!b || (mode != LBM_BATCH_PER_STEP && mode != LBM_BATCH_PERSISTENT && mode != LBM_BATCH_LOOP)) return LBM_EINVAL;
   if (tile_columns != 1 && tile_columns != 2 && tile_columns != 4 && tile_columns != 8) return LBM_EINVAL;
   if (blocks_per_sm < 0 || blocks_per_sm > 64) return LBM_EINVAL;
+  const int32_t st = without_exceptions([&] { return relayout(b, tile_columns); });
+  if (st != LBM_OK) return st;
   b->mode = mode;
   b->blocks_per_sm = blocks_per_sm;
-  if (tile_columns != b->warps_per_block) return relayout(b, tile_columns);
   return LBM_OK;
 }
 
@@ -483,8 +509,9 @@ int32_t lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, void* stream) {
   struct Cand {
     int mode, tx, bps;
   };
-  std::vector<Cand> cands;
-  for (int tx : {2, 4, 8}) cands.push_back({LBM_BATCH_PER_STEP, tx, 0});
+  Cand cands[9];
+  int n = 0;
+  for (int tx : {2, 4, 8}) cands[n++] = {LBM_BATCH_PER_STEP, tx, 0};
   // The persistent launch saves one kernel boundary per step (a few microseconds) but its
   // loads must bypass L1 (other SMs rewrite the buffers between steps), which measured
   // 7 % (float64) to 32 % (FP32) slower per step on batches of millions of sites.  It is
@@ -492,7 +519,7 @@ int32_t lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, void* stream) {
   if (lbm_batch_sites(b) <= kPersistentCandidateSites) {
     for (int tx : {2, 4, 8}) {
       const int fit = max_blocks_per_sm(b, tx);
-      for (int bps = fit; bps >= 1 && bps >= fit - 1; --bps) cands.push_back({LBM_BATCH_PERSISTENT, tx, bps});
+      for (int bps = fit; bps >= 1 && bps >= fit - 1; --bps) cands[n++] = {LBM_BATCH_PERSISTENT, tx, bps};
     }
   }
   cudaEvent_t e0, e1;
@@ -504,7 +531,8 @@ int32_t lbm_batch_autotune(lbm_batch* b, int32_t trial_steps, void* stream) {
   float best = 1e30f;
   Cand best_c = {b->mode, b->warps_per_block, b->blocks_per_sm};
   int32_t st = LBM_OK;
-  for (const Cand& c : cands) {
+  for (const Cand* k = cands; k < cands + n; ++k) {
+    const Cand& c = *k;
     if ((st = lbm_batch_configure(b, c.mode, c.tx, c.bps)) != LBM_OK) break;
     if ((st = run(b, 1, s)) != LBM_OK) break;  // warm-up
     cudaEventRecord(e0, s);
@@ -546,10 +574,6 @@ int64_t lbm_batch_sites(const lbm_batch* b) {
 }
 
 void lbm_batch_destroy(lbm_batch* b) {
-  if (!b) return;
-  for (BatchTile* t : b->tables) cudaFree(t);
-  cudaFree(b->dev_lattices);
-  cudaFree(b->dev_sync);
   delete b;
 }
 

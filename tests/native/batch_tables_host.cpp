@@ -104,6 +104,30 @@ int main(int argc, char** argv) {
         expect(lbm_batch_configure(b, mode, tx, 0), LBM_OK, "configure");
         expect(lbm_batch_run(b, 2, nullptr), LBM_OK, "run");
       }
+  } else if (what == "no_device_memory") {  // the configuration before stays, and runs
+    expect(lbm_batch_plan(p, fa, fb, 2, &b), LBM_OK, "plan");
+    expect(lbm_batch_configure(b, LBM_BATCH_PER_STEP, 8, 0), LBM_OK, "configure");
+    g_fail_malloc = 1;
+    expect(lbm_batch_configure(b, LBM_BATCH_PERSISTENT, 1, 3), LBM_ENOMEM, "no device memory");
+    int32_t mode = 0, tx = 0;
+    lbm_batch_config(b, &mode, &tx, nullptr);
+    if (mode != LBM_BATCH_PER_STEP || tx != 8) wrong("the configuration changed");
+    expect(lbm_batch_run(b, 1, nullptr), LBM_OK, "run");
+    expect(lbm_batch_configure(b, LBM_BATCH_PERSISTENT, 1, 0), LBM_OK, "configure again");
+    expect(lbm_batch_run(b, 1, nullptr), LBM_OK, "run");
+  } else if (what == "no_host_memory") {  // an error, not an exception
+    try {
+      expect(lbm_batch_plan(p, fa, fb, 2, &b), LBM_OK, "plan");
+      g_new_limit = 256;
+      expect(lbm_batch_configure(b, LBM_BATCH_PER_STEP, 1, 0), LBM_ENOMEM, "no host memory");
+      lbm_batch* other = nullptr;
+      expect(lbm_batch_plan(p, fa, fb, 2, &other), LBM_ENOMEM, "no host memory for a plan");
+      if (other) wrong("a batch without memory");
+      g_new_limit = 0;
+      expect(lbm_batch_run(b, 1, nullptr), LBM_OK, "run");
+    } catch (...) {
+      wrong("an exception left the library");
+    }
   } else if (what == "plan") {  // every allocation of a plan failing in turn: nothing is left behind
     for (int n = 1; n <= 3; ++n) {
       g_fail_malloc = n;

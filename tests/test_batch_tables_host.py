@@ -1,5 +1,6 @@
 """The batch's tile tables against a fake of the CUDA runtime (tests/native/batch_tables_host.cpp): what a
-launch was given stays as it is until the batch is destroyed."""
+launch was given stays as it is until the batch is destroyed, and running out of memory is an error that
+leaves the batch as it was."""
 import os
 import shutil
 import subprocess
@@ -25,7 +26,7 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("what", ["in_flight", "plan"])
+@pytest.mark.parametrize("what", ["in_flight", "no_device_memory", "no_host_memory", "plan"])
 def test_tables(program, what):
     out = subprocess.run([program, what], capture_output=True, text=True, timeout=60)
     assert (out.returncode, out.stdout.strip()) == (0, "ok"), out.stderr

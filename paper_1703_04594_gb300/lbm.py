@@ -8,7 +8,6 @@ missing library raises ``RuntimeError``: there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes
-import functools
 import os
 from dataclasses import dataclass
 
@@ -32,8 +31,12 @@ class CParams(ctypes.Structure):
                 ("rho0", ctypes.c_double)]
 
 
+class _CallData:
+    __slots__ = ("_call_data",)
+
+
 @dataclass(frozen=True)
-class Params:
+class Params(_CallData):
     """Problem parameters (Sec. 3): lattice size, relaxation time, gravity (xi units per
     step), wall temperatures; ``precision`` and ``bc`` select the storage form and the
     y boundary."""
@@ -53,13 +56,19 @@ class Params:
                        self.t_bottom, self.t_top, self.rho0)
 
     # What every call needs of one parameter set, formed on its first use (the fields are frozen):
-    # the C struct's reference, and the state's bytes and type.  Left out of copies and pickles.
-    @functools.cached_property
+    # the C struct's reference, and the state's bytes and type.  Held beside the instance's
+    # attributes, and left out of copies and pickles.
+    @property
     def _call(self):
-        return _Call(ctypes.byref(self.c()), buffer_bytes(self), state_dtype(self))
+        try:
+            return self._call_data
+        except AttributeError:
+            call = _Call(ctypes.byref(self.c()), buffer_bytes(self), state_dtype(self))
+            object.__setattr__(self, "_call_data", call)
+            return call
 
     def __getstate__(self):
-        return {k: v for k, v in self.__dict__.items() if k != "_call"}
+        return dict(self.__dict__)
 
 
 class _Call:

@@ -24,3 +24,12 @@ def test_params_keep_their_call_data_to_themselves():
     assert struct.tau == 0.9 and struct.precision == lbm.FP64 and r._call.bytes == 2 * p._call.bytes
     with pytest.raises(lbm.LbmError):
         lbm.Params(3, 70)._call
+
+
+def test_params_hold_their_fields_alone():
+    """What a program makes of a parameter set's attributes does not depend on calls made with it."""
+    ensure_built()
+    p = lbm.Params(40, 70, tau=0.7)
+    before = dict(vars(p))
+    assert p._call.bytes > 0
+    assert dict(vars(p)) == before == dataclasses.asdict(p) and lbm.Params(**vars(p)) == p

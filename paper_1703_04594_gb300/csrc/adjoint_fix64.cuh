@@ -42,7 +42,9 @@ inline AdjFixConsts make_adj_fix_consts(double tau, double gx, double gy) {
   const double sx = C * tau * gx, sy = C * tau * gy, st = tau * (1.0 - 2.0 * tau) * gg / 2.0,
                tg = tau * (1.0 - tau) * gg / 2.0;
   const auto small = [](double v) { return v > -0.125 && v < 0.125; };
-  r.usable = om1 > -0.999 && om1 < 0.999 && small(sx) && small(sy) && small(st) && small(tg);
+  // 1 - omega [63] to 2^-30 of the format's ends, as omega in make_fix_consts
+  constexpr double end = 1.0 - 0x1p-30;
+  r.usable = om1 >= -end && om1 <= end && small(sx) && small(sy) && small(st) && small(tg);
   if (!r.usable) return r;
   const auto fix = [](double v, int k) {
     bool unused = false;

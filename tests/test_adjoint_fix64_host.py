@@ -85,3 +85,20 @@ def test_results_against_exact_arithmetic(model, probe, rho, lam_scale):  # noqa
             assert abs(F(from_bits(h)) - v) <= 64 * unit + abs(v) * F(2) ** -50
         bound = 64 * unit * F(2) ** k / F(tau) ** 2 + abs(want_tau) * F(2) ** -50 + F(2) ** -1074
         assert abs(F(from_bits(line[3])) - want_tau) <= bound, (float(want_tau), from_bits(line[3]))
+
+
+@pytest.mark.parametrize("tau", [0.5 + 2.4e-10, 0.5 + 1e-6, 0.5001, 0.50024, 900.0, 1100.0, 1e5, 5e5])
+def test_relaxation_times_at_both_ends(model, probe, tau):  # noqa: F811
+    """Wherever the forward step takes a relaxation time in fixed point, its adjoint does."""
+    rng = random.Random(12)
+    f = state(model, rng, 1.0, 0.1, 0.15)
+    lam = [rng.uniform(-1.0, 1.0) for _ in range(37)]
+    g = 1e-4 if tau < 1.0 else 0.0
+    line = probe([" ".join([bits(v) for v in [tau, g, -g] + f + lam])])[0]
+    assert line[0] == "1"
+    k, K = int(line[1]), int(line[2])
+    want, want_tau = exact(model, f, lam, tau, g, -g)
+    unit = F(2) ** -K
+    for h, v in zip(line[4:], want):
+        assert abs(F(from_bits(h)) - v) <= 64 * unit + abs(v) * F(2) ** -50
+    assert abs(F(from_bits(line[3])) - want_tau) <= 64 * unit * F(2) ** k / F(tau) ** 2 + abs(want_tau) * F(2) ** -50

@@ -80,7 +80,7 @@ def traffic(key, sites):
 
 
 def _hbm_peak(root=None):
-    """Measured STREAM-style copy bandwidth of the GB300s (GB/s) and where the
+    """Measured STREAM-style copy bandwidth of the GB300 (GB/s) and where the
     figure comes from: MEASURED_PEAKS.json, else one earlier GB300 measurement (6.8 TB/s)."""
     try:
         with open(os.path.join(root or ROOT, "MEASURED_PEAKS.json")) as fh:
@@ -759,11 +759,11 @@ def adjoint_form(a, repeats, precision="fp64", seed=5):
         res = lbm.run(p, f, lbm.empty_state(p), n)
         return float(lbm.kinetic_energy(p, res))
 
-    def gradient(every=every, recompute=None):
+    def gradient(every=every):
         amp = modes.a.clone().requires_grad_(True)
         tau = torch.tensor(TAU, dtype=torch.float64, requires_grad=True)
         fields = I.rt_fields(lx, ly, I.RTModes(a=amp, phi=modes.phi), T_BOTTOM, T_TOP, abs(GY), device="cuda")
-        e = A.kinetic_energy_after(*[t.contiguous() for t in fields], tau, p, n, every, recompute_precision=recompute)
+        e = A.kinetic_energy_after(*[t.contiguous() for t in fields], tau, p, n, every)
         e.backward()
         return amp.grad, tau.grad
 
@@ -785,13 +785,10 @@ def adjoint_form(a, repeats, precision="fp64", seed=5):
             tg += one(fn)
         return tg / repeats, tf / repeats
 
-    # the default schedule, and the same gradient under two others: the segments recomputed
-    # as LBM_FP64 (the default recomputes them as LBM_FP64_FIXED, the same kernel), and every
-    # state kept in HBM (no recomputation)
+    # the default schedule, and the same gradient with every state kept in HBM (no recomputation)
     with ClockSampler(0) as clk:
         t_grad, t_fwd = timed_against_forward(gradient)
-    other = {"float64_recomputation": timed_against_forward(lambda: gradient(recompute=lbm.FP64)),
-             "every_state_kept": timed_against_forward(lambda: gradient(every=1))}
+    other = {"every_state_kept": timed_against_forward(lambda: gradient(every=1))}
     torch.cuda.empty_cache()
     schedules = {k: {"gradient_s": g, "forward_s": f, "gradient_over_forward": g / f} for k, (g, f) in other.items()}
     schedules["every_state_kept"]["memory_gb"] = (n + 1) * lbm.buffer_bytes(p) / 1e9

@@ -49,9 +49,10 @@ extern "C" {
 enum lbm_status { LBM_OK = 0, LBM_EINVAL = 1, LBM_ECUDA = 2, LBM_ETIMEOUT = 3, LBM_ENOMEM = 4, LBM_ESIZE = 5 };
 /* LBM_FP64: float64 populations.  The fused step evaluates the collision (moments, site
  * scalars, equilibrium and relaxation) of a site in 64-bit fixed point scaled by the site's
- * density, with errors below one float64 rounding unit of each result (about a tenth of a
- * float64 evaluation's), when its populations are within a factor of the equilibrium at rest
- * and |u_s| < 0.31, |T_s - 1| < 0.4; every other site (fast or hot fluid, zero or negative
+ * density, with errors below one float64 rounding unit of the population's equilibrium at rest
+ * (about a tenth of a float64 evaluation's), when its populations are within a factor of that
+ * equilibrium, |u_s| < 0.31 and |T_s - 1| < 0.4, for tau >= 0.5 + 2.4e-10 and |tau g| < 0.1;
+ * every other site (fast or hot fluid, zero or negative
  * populations) is evaluated in float64, so every finite state is handled, and a non-finite
  * population makes its site's outputs NaN.  LBM_FP64_FIXED: the same step (the name is kept
  * for callers of earlier versions; the separate kernels, layouts and adjoint entry points take
@@ -117,7 +118,8 @@ int32_t lbm_run(const lbm_params* p, void* f_a_dev, void* f_b_dev, int32_t n_ste
  *   lbm_bc:        writes the wall equilibria into exactly those entries of f_tmp, with
  *                  rho_w taken from f_in;
  *   lbm_collide:   f_out = collide(f_tmp), site by site.
- * propagate -> bc -> collide equals lbm_step up to floating-point contraction order.
+ * propagate -> bc -> collide equals lbm_step up to the rounding of the float64 collision
+ * that lbm_collide evaluates.
  * FP64 only. */
 int32_t lbm_propagate(const lbm_params* p, const void* f_in_dev, void* f_tmp_dev, void* stream);
 /* The push form of the same propagate (Sec. 4, "push" vs "pull"): every site moves its own
@@ -140,7 +142,7 @@ int64_t lbm_reduce_scratch_bytes(const lbm_params* p);
 /* Total kinetic energy sum over fluid sites of rho |u|^2 / 2 (moments of eq. "macro"),
  * written to *out_dev.  Deterministic: per-block partial sums go to scratch_dev
  * (>= lbm_reduce_scratch_bytes bytes, device memory owned by the caller) and are then
- * summed in a fixed order by one block. */
+ * summed in a fixed order. */
 int32_t lbm_kinetic_energy(const lbm_params* p, const void* f_dev, double* out_dev,
                            void* scratch_dev, size_t scratch_bytes, void* stream);
 
@@ -192,9 +194,9 @@ enum lbm_layout { LBM_LAYOUT_SOA = 0, LBM_LAYOUT_AOS = 1, LBM_LAYOUT_PSOA = 2, L
  * and src must not be the same.  Exact copy. */
 int32_t lbm_convert_layout(const lbm_params* p, int32_t from, const void* src_dev, int32_t to, void* dst_dev,
                            void* stream);
-/* One fused step of a state stored in layout AOS, PSOA or CAOSOA (the same arithmetic as
- * lbm_step on the same gathered values; results agree with lbm_step up to the compiler's
- * contraction of multiply-adds). */
+/* One fused step of a state stored in layout AOS, PSOA or CAOSOA (lbm_collide's
+ * float64 collision of the values that lbm_step gathers; results agree with lbm_step up to its
+ * rounding). */
 int32_t lbm_step_layout(const lbm_params* p, int32_t layout, const void* f_in_dev, void* f_out_dev, void* stream);
 
 /* ---- Adjoint (reverse mode) of the FP64 step, for gradients of observables ----

@@ -155,7 +155,6 @@ __constant__ GhostSlots c_ghost_slots = ghost_slots();
 
 // The lattice-wide scalars of the adjoint collision, formed once on the host.
 struct AdjConsts {
-  double tau;
   double om, om2;       // w = 1/tau, w^2
   double om1;           // 1 - w
   double om_c, om_c2;   // w c, w c^2
@@ -505,7 +504,6 @@ cudaError_t launch_adjoint_step(const double* fin, const double* lam_next, doubl
   const dim3 blk(32, 4);
   constexpr size_t smem = 4 * Q * 32 * sizeof(double);
   AdjConsts k;
-  k.tau = tau;
   k.om = 1.0 / tau;
   k.om2 = k.om * k.om;
   k.om1 = 1.0 - k.om;

@@ -35,7 +35,8 @@ __host__ __device__ constexpr unsigned long long fx_const(double a, double b, in
 }
 // Shell constants with w' = w_s 2^e_s (signed formats need values below 2^63):
 //   cw = w' (Q0.63), cq = w' q_s (Q4.59), cq2 = w' q_s^2 (Q8.55, with q_s^2 rounded to
-//   64 bits first), cw6 = w' / 6 (unsigned Q0.64).
+//   64 bits first), cw6 = w' / 6 (unsigned Q0.64).  The kernels read cw; the others are what the
+//   host tests hold fx_const's roundings to.
 __host__ __device__ constexpr long long shell_cw(int s) {
   return (long long)fx_const(w_shell(s), 1.0, shell_exp(s) + 63);
 }

@@ -110,7 +110,7 @@ cudaError_t launch_init_fp64(const double* rho, const double* ux, const double* 
 cudaError_t launch_moments_fp64(const double* f, double* rho, double* ux, double* uy, double* T,
                                 const StepArgs& a, cudaStream_t s);
 long long ke_partial_count(const StepArgs& a);
-// Sums n doubles of part (one block, fixed order) into *out.
+// Sums n doubles of part into *out in a fixed order (one block, or a cluster of eight beyond 8192).
 cudaError_t launch_reduce_sum(const double* part, long long n, double* out, cudaStream_t s);
 cudaError_t launch_kinetic_energy_fp64(const double* f, double* out, double* part, const StepArgs& a,
                                        cudaStream_t s);

@@ -1,7 +1,7 @@
 // Kernels of float64 states: fused pull step, the separate propagate / bc / collide kernels,
 // equilibrium initialisation, moments and the kinetic-energy reduction.
 //
-// Thread mapping (all site kernels): block = 32 x 4 threads; threadIdx.x runs along y
+// Thread mapping: block = 32 x 4 threads (the fused step: step_block); threadIdx.x runs along y
 // (the contiguous axis, Sec. 4 "column-major, Y innermost"), so each warp owns 32
 // consecutive sites of one column x and every population load/store of a warp is one
 // contiguous 256-byte run (shifted by the hop's vy for loads).
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(128, 4) k_moments_fp64(const double* __restric
   T[fi] = t;
 }
 
-// Kinetic energy: per-block partial sums (fixed order), then one block sums the partials.
+// Kinetic energy: per-block partial sums (fixed order), then k_reduce_sum adds the partials.
 __global__ void __launch_bounds__(128, 4) k_ke_partial_fp64(const double* __restrict__ fin, double* __restrict__ part,
                                                          StepArgs a) {
   const int x = blockIdx.y * 4 + threadIdx.y;

@@ -1,7 +1,7 @@
 // Alternative population layouts for the fused FP64 step (the layout comparison of Sec. 4,
-// Tables "propagate-kernel"/"collide-kernel": AoS, SoA, CSoA, CAoSoA).  Same arithmetic as
-// the SoA step (collide_site) on the same gathered values; only the addresses of the 37
-// gathers and stores change.  Walls only (no periodic-y mode).
+// Tables "propagate-kernel"/"collide-kernel": AoS, SoA, CSoA, CAoSoA).  The float64
+// collision (collide_site) on the values that the SoA step gathers; only the addresses of the 37
+// gathers and stores differ between them.  Walls only (no periodic-y mode).
 //
 //   SoA:    the production layout.  With pitch a multiple of 32 it is the paper's CSoA with
 //           cluster width 32: a warp's 32 consecutive y are one aligned 256-byte cluster.
@@ -22,7 +22,7 @@
 
 #include "../../include/lbm_d2q37.h"
 #include "kernels.h"
-#include "step_fp64.cuh"
+#include "load_paths.cuh"
 
 namespace d2q37 {
 

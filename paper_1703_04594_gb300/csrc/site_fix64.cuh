@@ -35,7 +35,7 @@
 // integers multiply carry 61 to 64 bits.
 //
 // Range: 2^-8 <= f_i 2^(e_s - k) < 2, 9/64 <= rho 2^-k < 1, omega rho 2^-k < 1.8, |X|, |Y| < 3/8
-// (|u_s| < 0.31), |t| < 2/5, and |c tau g| < 1/8; other sites take the float64 collision.
+// (|u_s| < 0.31), |t| < 2/5, and |c tau g| < 1/8, omega <= 2 - 2^-30; other sites take the float64 collision.
 #pragma once
 #include "collide_fix64.cuh"
 
@@ -80,11 +80,6 @@ __host__ __device__ __forceinline__ long long fx_smul(long long a, FxHalves b) {
 __host__ __device__ __forceinline__ long long fx_smul(long long a, long long b) {
   return fx_smul(fx_halves(a), fx_halves(b));
 }
-// v 2^k as an integer, |v| 2^k < 2^62, at compile time or on the host.
-__host__ __device__ constexpr long long fx_signed(double v, int k) {
-  return v == 0.0 ? 0LL : v > 0.0 ? (long long)fx_const(v, 1.0, k) : -(long long)fx_const(-v, 1.0, k);
-}
-
 constexpr long long kFxC2_62 = (long long)fx_const(C2, 1.0, 62);
 constexpr long long kFxC2q_64 = (long long)fx_const(C2, 0.25, 64);          // c^2 / 4 [64]
 constexpr long long kFxC4_64 = (long long)fx_const(C2, C2 * 0.125, 64);    // c^4 / 8 [64]

@@ -1,7 +1,7 @@
 // One warp-strip of the fused float64 step with the fixed-point collision of site_fix64.cuh.
 #pragma once
 #include "site_fix64.cuh"
-#include "step_fp64.cuh"
+#include "load_paths.cuh"
 
 namespace d2q37 {
 
@@ -11,9 +11,6 @@ __device__ __forceinline__ void cp_async8(double* smem_dst, const double* gmem_s
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(gmem_src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-
-// Shared staging: one warp holds sf[i * 32 + lane] for its 32 sites.
-constexpr int kFixWarps = 4;  // warps per block (block = 32 x 4 threads)
 
 // rho(x_s, row) of the seven source columns: lane l sums every fourth population of column
 // l % 8, and two shuffles add the four parts (the same value in the column's four lanes).

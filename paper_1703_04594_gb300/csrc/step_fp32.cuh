@@ -20,7 +20,7 @@
 //    so float32 rounds deviations, not whole populations.
 #pragma once
 #include "fixed64.cuh"
-#include "step_fp64.cuh"
+#include "load_paths.cuh"
 
 namespace d2q37 {
 
@@ -455,7 +455,8 @@ __device__ __forceinline__ float wall_drho_lane(const float* fin, int x, const S
   return r.s + r.e;
 }
 
-// One warp-strip of the FP32 shifted step (see step_fp64.cuh for the strip contract).
+// One warp-strip of the FP32 steps, the sites (x, y0 .. y0 + 31): called by the whole warp, lane l for row
+// y0 + l; lanes beyond the last row gather clamped rows and store nothing.
 // SCALED: whether the lattice's reference density is outside [1/2, 2) (see Fp32Scale); CONSERVE: the
 // collision restores the exact conserved moments (collide_site_fp32).
 template <bool PERIODIC, int SCALED, bool CONSERVE, class Ld>

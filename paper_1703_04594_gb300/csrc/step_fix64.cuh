@@ -138,9 +138,10 @@ __device__ __forceinline__ bool step_strip_fix64(const double* fin, double* __re
   const bool active = y < a.ly;  // the other lanes work on the last row's data and store nothing
   const int yc = active ? y : a.ly - 1;
   sf += lane;
+  const int usable = a.fx.usable;  // read under the copies (48 lattices of a batch: 2.048 ms after them, 2.026 here)
   stage_issue<PERIODIC>(fin, a, x, y0, yc, sf, ld);
   stage_finish<PERIODIC>(fin, a, w, x, y0, yc, sf, ld);
-  if (!a.fx.usable) return active;  // uniform: the lattice's constants are outside the formats
+  if (!usable) return active;  // uniform: the lattice's constants are outside the formats
   FxHalves* const sx = reinterpret_cast<FxHalves*>(sf);  // the same slots, as fixed point
   const FixMoments m = fix_moments([&](int i) { return sf[i * 32]; }, [&](int i, FxHalves q) { sx[i * 32] = q; });
   const FixScalars v = fix_scalars(m, a.fx);

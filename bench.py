@@ -61,13 +61,13 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 # no capture of the current kernel exists.  Reads equal the algorithmic bytes; writes read
 # a little low on the captured cases because their tail is still in L2 when the kernel ends.
 TRAFFIC_BYTES_PER_SITE = {
-    "fused": 565.3,        # k_step_fix64, 1024 x 2048
-    "fp64fix": 565.3,      # the same kernel
+    "fused": 565.2,        # k_step_fix64, 1024 x 2048
+    "fp64fix": 565.2,      # the same kernel
     "fp32": 272.3,         # k_step_fp32 (shifted), 1024 x 2048
-    "fp32c": 272.5,        # k_step_fp32 (conserved moments), 1024 x 2048
-    "adjoint": 816.8,      # k_adj_collide, 512 x 1024 (the adjoint workload's own lattice)
-    "batch_fp32": 258.4,   # k_batch_step<fp32>, 64 small lattices
-    "batch_fp64": 587.5,   # k_batch_step<fix64>, 8 lattices Lx 128..1024
+    "fp32c": 272.4,        # k_step_fp32 (conserved moments), 1024 x 2048
+    "adjoint": 813.4,      # k_adj_collide, 512 x 1024 (the adjoint workload's own lattice)
+    "batch_fp32": 258.3,   # k_batch_step<fp32>, 64 small lattices
+    "batch_fp64": 587.2,   # k_batch_step<fix64>, 8 lattices Lx 128..1024
     "separate": None,
 }
 

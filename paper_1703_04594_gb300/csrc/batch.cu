@@ -156,7 +156,7 @@ __device__ __forceinline__ bool grid_barrier(BatchSync* sync, unsigned target, l
 // Register caps, with at most 256 threads per block (8 warps): the FP32 step keeps three
 // such blocks resident per SM (80 registers), the float64-state step and the conserved-moment
 // FP32 step the 96 registers of their single-lattice kernels (5 blocks of 4 warps per SM).  256
-// lattices Lx 128..1024: float64 26.5 ms a step (106.7 colliding in float64), FP32 11.6 (13.0);
+// lattices Lx 128..1024: float64 26.4 ms a step (106.7 colliding in float64), FP32 11.6 (13.0);
 // 256 of 32 to 128, where two strips of five touch a wall: FP32 0.177 ms (0.295).
 constexpr int batch_max_regs(int kind) {
   return kind == kFix64 || conserves(kind) ? 96 : 80;

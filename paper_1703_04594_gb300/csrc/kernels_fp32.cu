@@ -11,8 +11,8 @@ namespace d2q37 {
 #ifndef LBM_FP32_MIN_BLOCKS
 #define LBM_FP32_MIN_BLOCKS 6  // 80 registers; measured best among 4..8 blocks per SM
 #endif
-// 4096 x 8192: shifted 1.56 ms, 6.4 TB/s (0.95 of the copy rate; 1.75 before the walls' sums, the scalars
-// and the packed splits left the float64 pipe and the issue slots), conserved 1.90 ms (2.28), issue-bound.
+// 4096 x 8192: shifted 1.56 to 1.59 ms, 6.3 to 6.4 TB/s (0.93 to 0.95 of the copy rate; 1.75 before the walls' sums, the scalars
+// and the packed splits left the float64 pipe and the issue slots), conserved 1.92 ms (2.28), issue-bound.
 // The conserved-moment form holds all 37 outputs and eight sum lanes until its
 // correction: 5 blocks per SM (96 registers) instead of spilling at 80.
 #ifndef LBM_FP32C_MIN_BLOCKS

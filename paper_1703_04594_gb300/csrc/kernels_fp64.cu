@@ -30,9 +30,9 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 
 // ---------------------------------------------------------------------------------------
 // Fused step of float64 states: gather (propagate + bc) -> collide -> streaming store
-// (step_fix64.cuh).  4096 x 8192: 3.70 ms, 5.3 TB/s (0.80 of the copy rate); colliding in float64, bound by
+// (step_fix64.cuh).  4096 x 8192: 3.65 ms, 5.4 TB/s (0.81 of the copy rate); colliding in float64, bound by
 // that pipe, 15.4 ms.  Bound now by latency at 20 warps per SM with the multiply-add, ALU and float64
-// pipes and issue each 54 to 57 % busy: 96 registers, and 9.5 KB of staging per warp.  24 warps
+// pipes and issue each 55 to 58 % busy: 96 registers, and 9.5 KB of staging per warp.  24 warps
 // (80 registers, the largest carveout) left too little L1 for the gather: 4.35 -> 5.41 ms for
 // 2160 x 8192, 2 steps.
 #ifndef LBM_FIX64_MIN_BLOCKS
@@ -40,8 +40,9 @@ __device__ __forceinline__ void source_columns(int x, const StepArgs& a, long lo
 #endif
 extern __shared__ double step_staged[];  // 37 populations x 32 sites per warp
 // The sites outside the fixed-point range, by a function that forms its indices itself and is not
-// inlined, so that the kernel keeps neither its float64 values nor its arguments in registers (a vote
-// before the relaxation, and a second copy of that for mixed strips, cost 2 % of the other strips' time).
+// inlined, so that the kernel keeps neither its float64 values nor its arguments in registers (4096 x
+// 8192, 2 steps, of ordinary strips: 7.30 ms; with the vote before the relaxation, and a second copy of
+// that for mixed strips, 7.40; with the arguments kept, which spills, 7.52; no vote 7.26).
 template <bool PERIODIC>
 __device__ __noinline__ void step_float64_sites(const double* fin, double* fout, const StepArgs& a, bool left) {
   const int x = blockIdx.y * blockDim.y + threadIdx.y;
